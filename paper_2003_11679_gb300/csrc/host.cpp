@@ -382,6 +382,7 @@ void make_quad(const sie_params& p, QuadDev& q)
         q.n[r] = ns[r];
         gauss_legendre01(ns[r], q.x[r], q.w[r]);
     }
+    for (int n = 1; n < 64; n++) q.rn[n] = 1.0 / n;
     q.npan = p.q_npan;
     q.opan = p.q_opan;
     q.emupan = p.q_emupan;

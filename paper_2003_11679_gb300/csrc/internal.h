@@ -106,6 +106,7 @@ struct DevMesh {
 // quadrature description handed to the near-field kernel
 struct QuadDev {
     double x[7][32], w[7][32];  // far, out, ang, rad, olam, omu, emu
+    double rn[64];              // 1 / n
     int n[7];
     int npan, opan, emupan;
     double ratio, cf, kres, alen, oratio;

@@ -49,15 +49,24 @@ __device__ __forceinline__ cd cexpc(cd z)
     sincos(z.im, &s, &c);
     return {e * c, e * s};
 }
-__device__ __forceinline__ double cabsc(cd z) { return hypot(z.re, z.im); }
+// exp(-j k R), R real (a real k needs no exponential)
+__device__ __forceinline__ cd cexp_mjkr(cd k, double R)
+{
+    double s, c;
+    sincos(-k.re * R, &s, &c);
+    if (k.im == 0.0) return {c, s};
+    double e = exp(k.im * R);
+    return {e * c, e * s};
+}
+__device__ __forceinline__ double cnorm(cd z) { return z.re * z.re + z.im * z.im; }
 
 // (exp(z) - 1)/z
 __device__ cd phi1(cd z)
 {
-    if (cabsc(z) < 0.5) {
+    if (cnorm(z) < 0.25) {
         cd term = mk(1, 0), s = mk(1, 0);
-        for (int n = 1; n < 20; n++) {
-            term = term * z * (1.0 / (double)(n + 1));
+        for (int n = 2; n < 17; n++) {  // 0.5^16 / 17! < 1e-19
+            term = (term * z) * cq.rn[n];
             s = s + term;
         }
         return s;
@@ -65,21 +74,19 @@ __device__ cd phi1(cd z)
     return cdivc(cexpc(z) - mk(1, 0), z);
 }
 
-// (1 + z) exp(-z) - 1 with a series near 0
-__device__ cd hfun(cd z)
+// (1 + z) exp(-z) - 1 with a series near 0; e = exp(-z)
+__device__ cd hfun(cd z, cd e)
 {
-    if (cabsc(z) < 0.2) {
+    if (cnorm(z) < 0.04) {
+        // sum_{n >= 2} (-1)^(n+1) (n - 1) z^n / n!
         cd s = mk(0, 0), zn = z;
-        double fact = 1.0;
-        for (int n = 2; n < 16; n++) {
-            zn = zn * z;
-            fact *= n;
-            double sg = (n % 2 == 0) ? -1.0 : 1.0;
-            s = s + (sg * (double)(n - 1) / fact) * zn;
+        for (int n = 2; n < 15; n++) {
+            zn = (zn * z) * (-cq.rn[n]);
+            s = s + (double)(n - 1) * zn;
         }
         return s;
     }
-    return (mk(1, 0) + z) * cexpc(mk(-z.re, -z.im)) - mk(1, 0);
+    return (mk(1, 0) + z) * e - mk(1, 0);
 }
 
 struct v3 {
@@ -99,50 +106,44 @@ struct Inner {
     cd Ig[3];
 };
 
-__device__ __forceinline__ cd clogc(cd z) { return mk(log(hypot(z.re, z.im)), atan2(z.im, z.re)); }
-
-// Ein(z) = I_0^z (1 - exp(-t))/t dt for Re z >= 0: series for |z| < 2, else
-// E1(z) + log z + gamma, E1 by its continued fraction (modified Lentz)
-__device__ cd ein(cd z)
+// Ein(z) = I_0^z (1 - exp(-t))/t dt for Re z >= 0; e = exp(-z).  Series for
+// |z| < 2, else E1(z) + log z + gamma.  E1 = e / (z + 1 - 1 / (z + 3 - 4 /
+// (z + 5 - ...))) by the forward recurrence of numerator and denominator with
+// a term count from its convergence rate exp(-4 sqrt(n |z|) cos(arg z / 2)):
+// no division per term (n <= 104, terms below 1e180).  Beyond Re z = 40
+// E1 is below the rounding of log z.
+__device__ cd ein(cd z, cd e)
 {
-    if (cabsc(z) < 2.0) {
+    const double r2 = cnorm(z);
+    if (r2 < 4.0) {
         cd s = mk(0, 0), t = mk(1, 0);
         for (int n = 1; n < 60; n++) {
-            t = t * z * (1.0 / (double)n);
-            cd term = ((n & 1) ? 1.0 : -1.0) / (double)n * t;
+            t = (t * z) * cq.rn[n];
+            cd term = ((n & 1) ? cq.rn[n] : -cq.rn[n]) * t;
             s = s + term;
-            if (cabsc(term) < 1e-17 * cabsc(s)) break;
+            if (cnorm(term) < 1e-34 * cnorm(s)) break;
         }
         return s;
     }
-    const double tiny = 1e-300;
-    cd f = z, C = z, D = mk(0, 0);
-    for (int i = 1; i < 500; i++) {
-        double a = (double)((i + 1) / 2);
-        cd b = (i & 1) ? mk(1, 0) : z;
-        D = b + a * D;
-        if (cabsc(D) < tiny) D = mk(tiny, 0);
-        C = b + cdivc(mk(a, 0), C);
-        if (cabsc(C) < tiny) C = mk(tiny, 0);
-        D = cdivc(mk(1, 0), D);
-        cd delta = C * D;
-        f = f * delta;
-        if (cabsc(delta - mk(1, 0)) < 1e-16) break;
-    }
     const double euler = 0.57721566490153286061;
-    return cdivc(cexpc(mk(-z.re, -z.im)), f) + clogc(z) + mk(euler, 0);
+    cd o = mk(0.5 * log(r2) + euler, atan2(z.im, z.re));
+    if (z.re > 40.0) return o;
+    const int n = (int)(200.0 / (sqrt(r2) + z.re)) + 5;
+    cd A0 = mk(0, 0), A1 = mk(1, 0), B0 = mk(1, 0), B1 = mk(z.re + 1.0, z.im);
+    for (int i = 1; i <= n; i++) {
+        const cd b = mk(z.re + (double)(2 * i + 1), z.im);
+        const double a = -(double)(i * i);
+        cd A2 = b * A1 + a * A0, B2 = b * B1 + a * B0;
+        A0 = A1;
+        A1 = A2;
+        B0 = B1;
+        B1 = B2;
+    }
+    return o + e * cdivc(A1, B1);
 }
 
-// Numeric radial integrals over [0, rc] at height d.  Beyond R = RCUT/|Im k|
-// every direction whose edge lies farther away integrates the same truncated
-// range [0, rc(d)], so one evaluation serves all those directions of an
-// observation point (same sums, computed once).
-struct RadCache {
-    bool valid;
-    double rc;
-    cd a1, a2;
-};
-
+// Graded Gauss radial integrals of the lossy kernel over [0, rc] at height d
+// (|k| Rmax > 1): a1 = I rho^2/R exp(-jkR), a2 = I rho^2/R^3 [(1 + jkR) exp(-jkR) - 1]
 __device__ void radial_numeric(cd k, double rc, double d, cd* a1o, cd* a2o)
 {
     cd a1 = mk(0, 0), a2 = mk(0, 0);
@@ -152,169 +153,17 @@ __device__ void radial_numeric(cd k, double rc, double d, cd* a1o, cd* a2o)
         for (int qq = 0; qq < cq.n[QR_RAD]; qq++) {
             double rho = lo + (hi - lo) * cq.x[QR_RAD][qq];
             double wr = (hi - lo) * cq.w[QR_RAD][qq];
-            double R = sqrt(rho * rho + d * d);
+            double R2 = rho * rho + d * d, iR = rsqrt(R2), R = R2 * iR;
             cd z = mk(-k.im * R, k.re * R);  // j k R
             cd e = cexpc(mk(-z.re, -z.im));
-            cd hz = cabsc(z) < 0.2 ? hfun(z) : (mk(1, 0) + z) * e - mk(1, 0);
-            a1 = a1 + (wr * rho * rho / R) * e;
-            a2 = a2 + (wr * rho * rho / (R * R * R)) * hz;
+            double f = wr * rho * rho * iR;
+            a1 = a1 + f * e;
+            a2 = a2 + (f * iR * iR) * hfun(z, e);
         }
         hi = lo;
     }
     *a1o = a1;
     *a2o = a2;
-}
-
-// bounded radial remainders (series when |k| Rmax <= 1, else graded Gauss)
-__device__ void radial(cd k, double rhom, double d, double Rmax, cd* f1, cd* f2, RadCache* cache)
-{
-    if (cabsc(k) * Rmax <= 1.0) {
-        double rs = rhom / Rmax, ds = d / Rmax, Rs = sqrt(rs * rs + ds * ds), d2 = ds * ds;
-        cd ks = k * Rmax;
-        const int NT = 26;
-        double B[NT + 4];
-        B[0] = (d2 > 0.0) ? d2 * asinh(rs / fabs(ds)) : 0.0;  // d^2 B_-1
-        B[1] = rs;                                           // B_0
-        double Rp = 1.0, bodd = 0.0, beven = rs;
-        for (int m = 1; m <= NT + 2; m++) {
-            Rp *= Rs;
-            double bm;
-            if (m & 1) {
-                double d2b = (m == 1) ? B[0] : d2 * bodd;
-                bm = (rs * Rp + m * d2b) / (m + 1);
-                bodd = bm;
-            } else {
-                bm = (rs * Rp + m * d2 * beven) / (m + 1);
-                beven = bm;
-            }
-            B[m + 1] = bm;
-        }
-        double A[NT + 2];
-        A[0] = B[2] - B[0];
-        for (int m = 0; m <= NT; m++) A[m + 1] = B[m + 3] - d2 * B[m + 1];
-        cd s1 = mk(0, 0), s2 = mk(0, 0), t1 = mk(1, 0);
-        cd mjk = mk(ks.im, -ks.re);  // -j ks
-        for (int n = 0; n <= NT; n++) {
-            if (n > 0) t1 = t1 * mjk * (1.0 / (double)n);
-            s1 = s1 + A[n] * t1;
-            if (n >= 2) s2 = s2 + (-(double)(n - 1) * A[n - 2]) * t1;
-        }
-        *f1 = s1 * (Rmax * Rmax);
-        *f2 = s2;
-        return;
-    }
-    if (d == 0.0) {
-        // coplanar point: closed forms with z = j k rhom
-        cd z = mk(-k.im * rhom, k.re * rhom), e = cexpc(mk(-z.re, -z.im));
-        cd jk = mk(-k.im, k.re);
-        *f1 = cdivc(mk(1, 0) - e * (mk(1, 0) + z), jk * jk);
-        *f2 = mk(1, 0) - e - ein(z);
-        return;
-    }
-    // beyond R = RCUT/|Im k| the exponential is below 1e-15: f1 has no
-    // contribution there and (1 + jkR) exp(-jkR) - 1 = -1 integrates in closed form
-    double rc = rhom, tail = 0.0;
-    bool trunc = false;
-    double kim = fabs(k.im);
-    if (kim > 0.0) {
-        double Rc = RCUT / kim, Rm = sqrt(rhom * rhom + d * d);
-        if (Rc < Rm) {
-            trunc = true;
-            rc = Rc > fabs(d) ? sqrt(Rc * Rc - d * d) : 0.0;
-            double Rcc = sqrt(rc * rc + d * d);
-            tail = (log(rhom + Rm) - rhom / Rm) - (log(rc + Rcc) - rc / Rcc);
-        }
-    }
-    cd a1, a2;
-    if (trunc) {
-        // truncated: the range [0, rc] depends on d only
-        if (!cache->valid || cache->rc != rc) {
-            radial_numeric(k, rc, d, &cache->a1, &cache->a2);
-            cache->rc = rc;
-            cache->valid = true;
-        }
-        a1 = cache->a1;
-        a2 = cache->a2;
-    } else {
-        radial_numeric(k, rc, d, &a1, &a2);
-    }
-    a2 = a2 - mk(tail, 0);
-    *f1 = a1;
-    *f2 = a2;
-}
-
-__device__ void inner_polar(v3 r, v3 v0, v3 v1, v3 v2, cd k, Inner& o)
-{
-    v3 vv[3] = {v0, v1, v2};
-    v3 nm = cross(v1 - v0, v2 - v0);
-    nm = (1.0 / nrm(nm)) * nm;
-    double dd = dot(r - v0, nm);
-    v3 rho0 = r - dd * nm;
-    double Rmax = fmax(nrm(v0 - r), fmax(nrm(v1 - r), nrm(v2 - r)));
-    if (fabs(dd) < 1e-12 * Rmax) dd = 0.0;  // on the plane up to rounding
-    double ad = fabs(dd);
-    o.Is = mk(0, 0);
-    for (int d = 0; d < 3; d++) o.Iv[d] = o.Ig[d] = mk(0, 0);
-    if (k.im != 0.0) {  // whole triangle beyond RCUT/|Im k|: every term below exp(-RCUT)
-        v3 c = (1.0 / 3.0) * (v0 + v1 + v2);
-        double rc = fmax(nrm(v0 - c), fmax(nrm(v1 - c), nrm(v2 - c)));
-        if (nrm(r - c) - rc > RCUT / fabs(k.im)) return;
-    }
-    cd Is = mk(0, 0), Ign = mk(0, 0), Iv[3] = {mk(0, 0), mk(0, 0), mk(0, 0)}, Igt[3] = {mk(0, 0), mk(0, 0), mk(0, 0)};
-    RadCache rcache;
-    rcache.valid = false;
-    double Omega = 0.0;
-    cd mjk = mk(k.im, -k.re);  // -j k
-    for (int i = 0; i < 3; i++) {
-        v3 A = vv[i], B = vv[(i + 1) % 3];
-        v3 e = B - A;
-        double L = nrm(e);
-        v3 et = (1.0 / L) * e;
-        v3 m = cross(et, nm);
-        v3 Ar = A - rho0, Br = B - rho0;
-        double h = dot(Ar, m);
-        if (fabs(h) < 1e-12 * L) continue;
-        double sh = h > 0 ? 1.0 : -1.0, ah = fabs(h);
-        v3 u = sh * m;
-        double ta = dot(Ar, et), tb = dot(Br, et);
-        Omega += sh * (atan2(tb, ah) - atan2(ta, ah));
-        double sa = asinh(ta / ah), sb = asinh(tb / ah);
-        int npa = (int)ceil((sb - sa) / cq.alen);
-        if (npa < 1) npa = 1;
-        double ds = (sb - sa) / npa;
-        const int na = cq.n[QR_ANG];
-        for (int j = 0; j < na * npa; j++) {
-            int jp = j / na, jq = j % na;
-            double s = sa + ds * (jp + cq.x[QR_ANG][jq]);
-            double ch = cosh(s);
-            double wa = sh * ds * cq.w[QR_ANG][jq] / ch;
-            double ca = 1.0 / ch, sn = tanh(s);
-            v3 eh = ca * u + sn * et;
-            double rhom = ah * ch;
-            double Rm = sqrt(rhom * rhom + dd * dd);
-            cd is = cexpc(mjk * ad) * (Rm - ad) * phi1(mjk * (Rm - ad));
-            cd f1, f2;
-            radial(k, rhom, dd, Rmax, &f1, &f2, &rcache);
-            cd igt = mk(log(rhom + Rm) - rhom / Rm, 0) + f2;
-            cd ign = (-dd / Rm) * cexpc(mjk * Rm);
-            Is = Is + wa * is;
-            Ign = Ign + wa * ign;
-            double ehv[3] = {eh.x, eh.y, eh.z}, nmv[3] = {nm.x, nm.y, nm.z};
-            for (int d = 0; d < 3; d++) {
-                Iv[d] = Iv[d] + wa * (ehv[d] * f1 - (dd * nmv[d]) * is);
-                Igt[d] = Igt[d] + (wa * ehv[d]) * igt;
-            }
-        }
-    }
-    cd jump = mk(0, 0);
-    if (dd != 0.0) jump = (Omega * (dd > 0 ? 1.0 : -1.0)) * cexpc(mjk * ad);
-    const double f = 1.0 / (4.0 * M_PI);
-    double nmv[3] = {nm.x, nm.y, nm.z};
-    o.Is = f * Is;
-    for (int d = 0; d < 3; d++) {
-        o.Iv[d] = f * Iv[d];
-        o.Ig[d] = (-f) * (nmv[d] * (jump + Ign) - Igt[d]);
-    }
 }
 
 __device__ void inner_gauss(v3 r, v3 a, v3 b, v3 c, cd k, Inner& o)
@@ -324,6 +173,7 @@ __device__ void inner_gauss(v3 r, v3 a, v3 b, v3 c, cd k, Inner& o)
     o.Is = mk(0, 0);
     for (int d = 0; d < 3; d++) o.Iv[d] = o.Ig[d] = mk(0, 0);
     const int n = cq.n[QR_FAR];
+    const double f = 1.0 / (4.0 * M_PI);
     for (int i = 0; i < n; i++) {
         double u = cq.x[QR_FAR][i];
         for (int j = 0; j < n; j++) {
@@ -331,10 +181,10 @@ __device__ void inner_gauss(v3 r, v3 a, v3 b, v3 c, cd k, Inner& o)
             double w = twoA * (1.0 - u) * cq.w[QR_FAR][i] * cq.w[QR_FAR][j];
             v3 p = a + u * e1 + v * e2;
             v3 dv = p - r;
-            double R = nrm(dv);
-            cd e = cexpc(mk(k.im * R, -k.re * R));
-            cd G = (1.0 / (4.0 * M_PI * R)) * e;
-            cd g = (-1.0 / (4.0 * M_PI * R * R * R)) * (mk(1.0 - k.im * R, k.re * R) * e);
+            double R2 = dot(dv, dv), iR = rsqrt(R2), R = R2 * iR;
+            cd e = cexp_mjkr(k, R);
+            cd G = (f * iR) * e;
+            cd g = (-f * iR * iR * iR) * (mk(1.0 - k.im * R, k.re * R) * e);
             o.Is = o.Is + w * G;
             double dvv[3] = {dv.x, dv.y, dv.z};
             for (int d = 0; d < 3; d++) {
@@ -385,115 +235,554 @@ __device__ int graded_count(int toward_edge)
     return cq.opan * cq.n[QR_OLAM] * nmu;
 }
 
-// 14 moments per pair: Q0, Q1[3], Q2[3], Q3, U[3], V[3] (origin: centroid of t).
-// One warp per pair; lanes split the outer points.
-// obj_k: per-object wavenumbers of a several-object interior (null: kr + j ki)
-__global__ void __launch_bounds__(128) k_near_moments(const int32_t* __restrict__ pairs, int64_t np, DevMesh M,
-                                                      double kr, double ki, const double2* __restrict__ obj_k,
-                                                      double2* __restrict__ mom)
+// ------------------------------------------------------------------ pair classes
+// far (0): product Gauss on both triangles.  The others are close pairs, whose
+// outer rules have very different sizes: plain (1), vertex shared (2), edge
+// shared (3), self (4).
+enum { PC_FAR = 0, PC_PLAIN, PC_VERTEX, PC_EDGE, PC_SELF };
+
+__global__ void k_pair_class(const int32_t* __restrict__ pairs, int64_t np, DevMesh M, double kr, double ki,
+                             const double2* __restrict__ obj_k, uint8_t* __restrict__ cls)
 {
-    int64_t p = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    int lane = threadIdx.x & 31;
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
-    int t = pairs[2 * p], s = pairs[2 * p + 1];
+    const int t = pairs[2 * p], s = pairs[2 * p + 1];
     if (obj_k) {
         const double2 ko = obj_k[M.obj[t]];
         kr = ko.x;
         ki = ko.y;
     }
-    cd k = mk(kr, ki);
-    int tt[3] = {M.T[3 * t], M.T[3 * t + 1], M.T[3 * t + 2]};
-    int ss[3] = {M.T[3 * s], M.T[3 * s + 1], M.T[3 * s + 2]};
-    v3 a = ld3(M.V + 3 * tt[0]), b = ld3(M.V + 3 * tt[1]), c = ld3(M.V + 3 * tt[2]);
-    v3 a2 = ld3(M.V + 3 * ss[0]), b2 = ld3(M.V + 3 * ss[1]), c2 = ld3(M.V + 3 * ss[2]);
-    v3 ct = ld3(M.cen + 3 * t);
-    int shared[3], nsh = 0;
+    int nsh = 0;
     for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++)
-            if (tt[i] == ss[j]) shared[nsh++] = i;
-    bool close = nsh > 0;
-    if (!close) {
-        v3 cs = ld3(M.cen + 3 * s);
-        double D = nrm(ct - cs), Rt = M.rad[t], Rs = M.rad[s];
-        if (D < cq.cf * (Rt + Rs) || hypot(kr, ki) * (Rt + Rs) > cq.kres) close = true;
+        for (int j = 0; j < 3; j++) nsh += M.T[3 * t + i] == M.T[3 * s + j];
+    int c = PC_FAR;
+    if (t == s)
+        c = PC_SELF;
+    else if (nsh == 2)
+        c = PC_EDGE;
+    else if (nsh == 1)
+        c = PC_VERTEX;
+    else {
+        const double D = nrm(ld3(M.cen + 3 * t) - ld3(M.cen + 3 * s)), Rt = M.rad[t], Rs = M.rad[s];
+        if (nsh > 0 || D < cq.cf * (Rt + Rs) || hypot(kr, ki) * (Rt + Rs) > cq.kres) c = PC_PLAIN;
     }
-    // outer rule
-    int kind;  // 0 plain collapsed, 1 edge shared, 2 vertex shared, 3 self
-    int nout;
-    v3 ap, bp, cp;
-    if (t == s) {
-        kind = 3;
-        nout = 3 * graded_count(1);
-    } else if (nsh == 2) {
-        kind = 1;
-        int ia = 3 - shared[0] - shared[1];
-        v3 vt[3] = {a, b, c};
-        ap = vt[ia];
-        bp = vt[(ia + 1) % 3];
-        cp = vt[(ia + 2) % 3];
-        nout = graded_count(1);
-    } else if (nsh == 1) {
-        kind = 2;
-        int ia = shared[0];
-        v3 vt[3] = {a, b, c};
-        ap = vt[ia];
-        bp = vt[(ia + 1) % 3];
-        cp = vt[(ia + 2) % 3];
-        nout = graded_count(0);
-    } else {
-        kind = 0;
-        int n = close ? cq.n[QR_OUT] : cq.n[QR_FAR];
-        nout = n * n;
+    cls[p] = (uint8_t)c;
+}
+
+// 14 moments per pair: Q0, Q1[3], Q2[3], Q3, U[3], V[3] (origin: centroid of t).
+// Contribution of one outer point: weight w, rt = r - c_t, inner integrals
+__device__ __forceinline__ void add_moments(cd* acc, double w, const double* rt, bool self, cd Is, const cd* Iv,
+                                            const cd* Ig)
+{
+    cd I2[3];
+    for (int d = 0; d < 3; d++) I2[d] = Iv[d] + rt[d] * Is;
+    acc[0] = acc[0] + w * Is;
+    for (int d = 0; d < 3; d++) {
+        acc[1 + d] = acc[1 + d] + (w * rt[d]) * Is;
+        acc[4 + d] = acc[4 + d] + w * I2[d];
     }
-    cd acc[14];
-    for (int i = 0; i < 14; i++) acc[i] = mk(0, 0);
-    double twoA = nrm(cross(b - a, c - a));
-    for (int qo = lane; qo < nout; qo += 32) {
-        v3 r;
-        double w;
-        if (kind == 0) {
-            int ridx = close ? QR_OUT : QR_FAR;
-            int n = cq.n[ridx];
-            int i = qo / n, j = qo % n;
-            double u = cq.x[ridx][i], v = cq.x[ridx][j] * (1.0 - u);
-            r = a + u * (b - a) + v * (c - a);
-            w = twoA * (1.0 - u) * cq.w[ridx][i] * cq.w[ridx][j];
-        } else if (kind == 3) {
-            int per = graded_count(1), sub = qo / per;
-            v3 vt[3] = {a, b, c};
-            graded_point(ct, vt[sub], vt[(sub + 1) % 3], 1, qo % per, r, w);
-        } else {
-            graded_point(ap, bp, cp, kind == 1, qo, r, w);
-        }
-        Inner in;
-        if (close)
-            inner_polar(r, a2, b2, c2, k, in);
-        else
-            inner_gauss(r, a2, b2, c2, k, in);
-        v3 rt = r - ct;
-        double rtv[3] = {rt.x, rt.y, rt.z};
-        cd I2[3];
-        for (int d = 0; d < 3; d++) I2[d] = in.Iv[d] + rtv[d] * in.Is;
-        acc[0] = acc[0] + w * in.Is;
-        for (int d = 0; d < 3; d++) {
-            acc[1 + d] = acc[1 + d] + (w * rtv[d]) * in.Is;
-            acc[4 + d] = acc[4 + d] + w * I2[d];
-        }
-        acc[7] = acc[7] + w * (rtv[0] * I2[0] + rtv[1] * I2[1] + rtv[2] * I2[2]);
-        if (t != s) {
-            acc[8] = acc[8] + (-w) * (rtv[1] * in.Ig[2] - rtv[2] * in.Ig[1]);
-            acc[9] = acc[9] + (-w) * (rtv[2] * in.Ig[0] - rtv[0] * in.Ig[2]);
-            acc[10] = acc[10] + (-w) * (rtv[0] * in.Ig[1] - rtv[1] * in.Ig[0]);
-            for (int d = 0; d < 3; d++) acc[11 + d] = acc[11 + d] + w * in.Ig[d];
-        }
-    }
+    acc[7] = acc[7] + w * (rt[0] * I2[0] + rt[1] * I2[1] + rt[2] * I2[2]);
+    if (self) return;
+    acc[8] = acc[8] + (-w) * (rt[1] * Ig[2] - rt[2] * Ig[1]);
+    acc[9] = acc[9] + (-w) * (rt[2] * Ig[0] - rt[0] * Ig[2]);
+    acc[10] = acc[10] + (-w) * (rt[0] * Ig[1] - rt[1] * Ig[0]);
+    for (int d = 0; d < 3; d++) acc[11 + d] = acc[11 + d] + w * Ig[d];
+}
+
+__device__ __forceinline__ void store_moments(cd* acc, int lane, double2* __restrict__ mom)
+{
     for (int i = 0; i < 14; i++)
         for (int off = 16; off > 0; off >>= 1) {
             acc[i].re += __shfl_down_sync(0xffffffffu, acc[i].re, off);
             acc[i].im += __shfl_down_sync(0xffffffffu, acc[i].im, off);
         }
     if (lane == 0)
-        for (int i = 0; i < 14; i++) mom[14 * p + i] = make_double2(acc[i].re, acc[i].im);
+        for (int i = 0; i < 14; i++) mom[i] = make_double2(acc[i].re, acc[i].im);
+}
+
+// far pairs: one warp per pair, a lane per outer point
+__global__ void __launch_bounds__(128) k_near_far(const int32_t* __restrict__ pairs, int64_t np,
+                                                  const uint8_t* __restrict__ cls, DevMesh M, double kr, double ki,
+                                                  const double2* __restrict__ obj_k, double2* __restrict__ mom)
+{
+    const int64_t p = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    const int lane = threadIdx.x & 31;
+    if (p >= np || cls[p] != PC_FAR) return;
+    const int t = pairs[2 * p], s = pairs[2 * p + 1];
+    if (obj_k) {
+        const double2 ko = obj_k[M.obj[t]];
+        kr = ko.x;
+        ki = ko.y;
+    }
+    const v3 a = ld3(M.V + 3 * M.T[3 * t]), b = ld3(M.V + 3 * M.T[3 * t + 1]), c = ld3(M.V + 3 * M.T[3 * t + 2]);
+    const v3 a2 = ld3(M.V + 3 * M.T[3 * s]), b2 = ld3(M.V + 3 * M.T[3 * s + 1]), c2 = ld3(M.V + 3 * M.T[3 * s + 2]);
+    const v3 ct = ld3(M.cen + 3 * t);
+    const double twoA = nrm(cross(b - a, c - a));
+    const int n = cq.n[QR_FAR];
+    cd acc[14];
+    for (int i = 0; i < 14; i++) acc[i] = mk(0, 0);
+    for (int qo = lane; qo < n * n; qo += 32) {
+        const int i = qo / n, j = qo % n;
+        const double u = cq.x[QR_FAR][i], v = cq.x[QR_FAR][j] * (1.0 - u);
+        const v3 r = a + u * (b - a) + v * (c - a);
+        Inner in;
+        inner_gauss(r, a2, b2, c2, mk(kr, ki), in);
+        const v3 rt = r - ct;
+        const double rtv[3] = {rt.x, rt.y, rt.z};
+        add_moments(acc, twoA * (1.0 - u) * cq.w[QR_FAR][i] * cq.w[QR_FAR][j], rtv, false, in.Is, in.Iv, in.Ig);
+    }
+    store_moments(acc, lane, mom + 14 * p);
+}
+
+// ------------------------------------------------------------------ close pairs
+// One warp per unit = (pair, run of 32 or more outer points), a lane per outer
+// point.  FP64 arithmetic bounds it (2 FP64 lanes per SM), so the work is
+// arranged to keep all lanes on it and to spend few operations per direction:
+//  * a point near an edge has over ten angular panels, one at the centre three:
+//    the panels of the 32 points are listed, panel index by panel index, and
+//    the lanes take panels, whosever they are (the moments are linear in them);
+//    exp(s) is a product of the panel's start and tabulated steps;
+//  * |k| Rmax <= 1: every radial integral of a direction comes from the powers of
+//    R and the moments A_n = I rho^2 R^(n-1) drho, A_n = (rho R^(n+1) - t)/(n+2)
+//    with t = d^2 I R^(n-1), summed against the Taylor coefficients of
+//    exp(-jkR), as many orders as the largest |k| R of the 32 panels needs for 1e-18
+//    (4 to 8 of the graded panels next to an edge);
+//  * units of self and edge pairs come first, so no long unit ends the launch.
+// One warp per pair with the outer points split over lanes, 27 orders with a
+// division each and separate cosh, tanh, phi1 per direction took 364 ms for the
+// exterior near region of an 80-triangle sphere at 3 GHz; 27 ms now, 37 million
+// directions at 286 FP64 operations, the FP64 pipe 88% busy.
+constexpr int NC_W = 2;     // warps per CTA (42 KB of shared memory)
+constexpr int NC_NT = 24;   // largest order: 1 / 24! < 2e-24
+constexpr int NC_NA = 8;    // angular nodes with tabulated exp(+-ds x_q); more are evaluated
+constexpr int NC_LIST = 96; // (edge, panel index) entries listed at a time
+
+struct CloseSm {
+    double et[3][3], em[3][3], va[3][3], len[3];          // source triangle: edges, in-plane normals
+    double dd[32], lad[32], iad[32], w[32], rt[3][32];      // per outer point
+    double2 is0[32], ead[32], a1[32], a2[32];
+    double rc[32];
+    double h[3][32], sa[3][32], ds[3][32];                  // per edge and point
+    double ep[NC_NA][3][32], en[NC_NA][3][32];              // exp(+-ds x_q)
+    double2 u[NC_NT + 4], g[NC_NT + 2], b[NC_NT + 2];      // u_m = (-j k/|k|)^m / m!, -m u_(m+1), u_(m-1) / m
+    unsigned mask[NC_LIST];                                 // points of a list entry
+    int pre[NC_LIST + 1];                                   // items before it
+    int2 ent[NC_LIST];                                      // (edge, panel index)
+    unsigned char ser[32];
+};
+
+template <bool REALK>
+__global__ void __launch_bounds__(32 * NC_W, 4) k_near_close(const int2* __restrict__ unit, int nunit, int npts,
+                                                          const int32_t* __restrict__ pairs,
+                                                          const uint8_t* __restrict__ cls, DevMesh M, double kr,
+                                                          double ki, const double2* __restrict__ obj_k,
+                                                          double2* __restrict__ part)
+{
+    __shared__ CloseSm sm_[NC_W];
+    const int un = blockIdx.x * NC_W + threadIdx.x / 32;
+    const int lane = threadIdx.x & 31;
+    if (un >= nunit) return;
+    CloseSm& S = sm_[threadIdx.x / 32];
+    const int p = unit[un].x, q_lo = unit[un].y;
+    const int t = pairs[2 * (int64_t)p], s = pairs[2 * (int64_t)p + 1], kind = cls[p];
+    if (!REALK && obj_k) {
+        const double2 ko = obj_k[M.obj[t]];
+        kr = ko.x;
+        ki = ko.y;
+    }
+    const cd k = mk(kr, REALK ? 0.0 : ki);
+    const double kabs = REALK ? kr : sqrt(kr * kr + ki * ki);
+    const cd mjk = mk(k.im, -k.re);  // -j k
+    const int tt[3] = {M.T[3 * t], M.T[3 * t + 1], M.T[3 * t + 2]};
+    const v3 a = ld3(M.V + 3 * tt[0]), b = ld3(M.V + 3 * tt[1]), c = ld3(M.V + 3 * tt[2]);
+    const v3 ct = ld3(M.cen + 3 * t);
+    const v3 vs[3] = {ld3(M.V + 3 * M.T[3 * s]), ld3(M.V + 3 * M.T[3 * s + 1]), ld3(M.V + 3 * M.T[3 * s + 2])};
+    v3 nm = cross(vs[1] - vs[0], vs[2] - vs[0]);
+    nm = (1.0 / nrm(nm)) * nm;
+    if (lane < 3) {
+        const v3 A = lane == 0 ? vs[0] : (lane == 1 ? vs[1] : vs[2]);
+        const v3 B = lane == 0 ? vs[1] : (lane == 1 ? vs[2] : vs[0]);
+        const v3 e = B - A;
+        const double L = nrm(e);
+        const v3 et = (1.0 / L) * e, m = cross(et, nm);
+        S.len[lane] = L;
+        S.et[lane][0] = et.x, S.et[lane][1] = et.y, S.et[lane][2] = et.z;
+        S.em[lane][0] = m.x, S.em[lane][1] = m.y, S.em[lane][2] = m.z;
+        S.va[lane][0] = A.x, S.va[lane][1] = A.y, S.va[lane][2] = A.z;
+    }
+    if (lane < NC_NT + 4) {
+        const cd z = mk(mjk.re / kabs, mjk.im / kabs);
+        cd u = mk(1, 0);
+        for (int i = 1; i <= lane; i++) u = (u * z) * cq.rn[i];
+        S.u[lane] = make_double2(u.re, u.im);
+    }
+    __syncwarp();
+    if (lane >= 1 && lane < NC_NT + 2) {
+        const double2 u0 = S.u[lane - 1], u2 = S.u[lane + 1];
+        S.g[lane] = make_double2(-(double)lane * u2.x, -(double)lane * u2.y);
+        S.b[lane] = make_double2(cq.rn[lane] * u0.x, cq.rn[lane] * u0.y);
+    }
+    // outer rule
+    int nout;
+    v3 ap = a, bp = b, cp = c;
+    if (kind == PC_SELF)
+        nout = 3 * graded_count(1);
+    else if (kind == PC_PLAIN)
+        nout = cq.n[QR_OUT] * cq.n[QR_OUT];
+    else {
+        int sum = 0, first = -1;
+        for (int i = 0; i < 3; i++)
+            for (int j = 0; j < 3; j++)
+                if (tt[i] == M.T[3 * s + j]) {
+                    sum += i;
+                    if (first < 0) first = i;
+                }
+        const int ia = kind == PC_EDGE ? 3 - sum : first;  // apex: the vertex off the shared edge, or the shared one
+        ap = ia == 0 ? a : (ia == 1 ? b : c);
+        bp = ia == 0 ? b : (ia == 1 ? c : a);
+        cp = ia == 0 ? c : (ia == 1 ? a : b);
+        nout = graded_count(kind == PC_EDGE);
+    }
+    const int per = graded_count(1);
+    const double twoA = nrm(cross(b - a, c - a));
+    const double f4 = 1.0 / (4.0 * M_PI);
+    const int na = cq.n[QR_ANG];
+    cd acc[14];
+    for (int i = 0; i < 14; i++) acc[i] = mk(0, 0);
+    const int q_hi = min(nout, q_lo + npts);
+    __syncwarp();
+    for (int q0 = q_lo; q0 < q_hi; q0 += 32) {
+        const int qo = q0 + lane;
+        int np3[3] = {0, 0, 0};
+        double dd = 0.0, ad = 0.0, lad = 0.0, iad = 1.0;
+        int ser = 1;
+        if (qo < q_hi) {
+            v3 r;
+            double w;
+            if (kind == PC_PLAIN) {
+                const int n = cq.n[QR_OUT], i = qo / n, j = qo % n;
+                const double u = cq.x[QR_OUT][i], v = cq.x[QR_OUT][j] * (1.0 - u);
+                r = a + u * (b - a) + v * (c - a);
+                w = twoA * (1.0 - u) * cq.w[QR_OUT][i] * cq.w[QR_OUT][j];
+            } else if (kind == PC_SELF) {
+                const int sub = qo / per;
+                graded_point(ct, sub == 0 ? a : (sub == 1 ? b : c), sub == 0 ? b : (sub == 1 ? c : a), 1, qo % per, r,
+                             w);
+            } else {
+                graded_point(ap, bp, cp, kind == PC_EDGE, qo, r, w);
+            }
+            const v3 rt = r - ct;
+            dd = dot(r - vs[0], nm);
+            const v3 rho0 = r - dd * nm;
+            const double Rmax = fmax(nrm(vs[0] - r), fmax(nrm(vs[1] - r), nrm(vs[2] - r)));
+            if (fabs(dd) < 1e-12 * Rmax) dd = 0.0;  // on the plane up to rounding
+            ad = fabs(dd);
+            bool off = false;
+            if (!REALK && k.im != 0.0) {  // whole triangle beyond RCUT/|Im k|: every term below exp(-RCUT)
+                const v3 cc = (1.0 / 3.0) * (vs[0] + vs[1] + vs[2]);
+                const double rc = fmax(nrm(vs[0] - cc), fmax(nrm(vs[1] - cc), nrm(vs[2] - cc)));
+                off = nrm(r - cc) - rc > RCUT / fabs(k.im);
+            }
+            ser = kabs * Rmax <= 1.0;
+            double Omega = 0.0;
+            for (int i = 0; i < 3 && !off; i++) {
+                const v3 et = {S.et[i][0], S.et[i][1], S.et[i][2]}, m = {S.em[i][0], S.em[i][1], S.em[i][2]};
+                const v3 Ar = ld3(S.va[i]) - rho0, Br = ld3(S.va[i == 2 ? 0 : i + 1]) - rho0;
+                const double h = dot(Ar, m), ah = fabs(h);
+                if (ah < 1e-12 * S.len[i]) continue;
+                const double ta = dot(Ar, et), tb = dot(Br, et);
+                Omega += (h > 0 ? 1.0 : -1.0) * (atan2(tb, ah) - atan2(ta, ah));
+                const double sa = asinh(ta / ah), sb = asinh(tb / ah);
+                const int npa = max(1, (int)ceil((sb - sa) / cq.alen));
+                np3[i] = npa;
+                S.h[i][lane] = h;
+                S.sa[i][lane] = sa;
+                S.ds[i][lane] = (sb - sa) / npa;
+            }
+            S.w[lane] = w;
+            S.rt[0][lane] = rt.x;
+            S.rt[1][lane] = rt.y;
+            S.rt[2][lane] = rt.z;
+            if (dd != 0.0) {
+                lad = log(ad);
+                iad = 1.0 / ad;
+            }
+            cd ea = mk(1, 0);
+            if (dd != 0.0 && !off) {
+                ea = cexp_mjkr(k, ad);
+                const cd jump = (-f4 * Omega * (dd > 0 ? 1.0 : -1.0)) * ea;
+                const double rtv[3] = {rt.x, rt.y, rt.z};
+                const cd Ig[3] = {nm.x * jump, nm.y * jump, nm.z * jump};
+                const cd z3[3] = {mk(0, 0), mk(0, 0), mk(0, 0)};
+                add_moments(acc, w, rtv, kind == PC_SELF, mk(0, 0), z3, Ig);
+            }
+            S.ead[lane] = make_double2(ea.re, ea.im);
+            if (!REALK && !ser && !off && dd != 0.0) {
+                // beyond R = RCUT/|Im k| every direction whose edge lies farther
+                // away integrates the same truncated range: once per point
+                const double Rc = k.im != 0.0 ? RCUT / fabs(k.im) : 1e300;
+                double rc = -1.0;
+                if (Rc < Rmax) {
+                    rc = Rc > ad ? sqrt(Rc * Rc - dd * dd) : 0.0;
+                    cd a1, a2;
+                    radial_numeric(k, rc, dd, &a1, &a2);
+                    S.a1[lane] = make_double2(a1.re, a1.im);
+                    S.a2[lane] = make_double2(a2.re, a2.im);
+                }
+                S.rc[lane] = rc;
+            }
+        }
+        if (ser) {  // I_0^|d| of exp(-jkR) in units of 1/|k|
+            cd v = mk(0, 0);
+            const double da = kabs * ad;
+            double pw = da;
+            for (int m = 1; m <= NC_NT && pw > 1e-19 * da; m++, pw *= da) {
+                const double2 u = S.u[m - 1];
+                v = v + (pw * cq.rn[m]) * mk(u.x, u.y);
+            }
+            S.is0[lane] = make_double2(v.re, v.im);
+        }
+        S.dd[lane] = dd;
+        S.lad[lane] = lad;
+        S.iad[lane] = iad;
+        S.ser[lane] = (unsigned char)ser;
+        if (na <= NC_NA)
+            for (int i = 0; i < 3; i++)
+                for (int q = 0; q < na && np3[i] > 0; q++) {
+                    const double e = exp(S.ds[i][lane] * cq.x[QR_ANG][q]);
+                    S.ep[q][i][lane] = e;
+                    S.en[q][i][lane] = 1.0 / e;
+                }
+        // the panels in work: entry e = panel jp of edge i, held by the points of its mask
+        int li = 0, lj = 0;
+        while (li < 3) {
+            int nent = 0, total = 0;
+            for (; li < 3 && nent < NC_LIST; lj++) {
+                const unsigned m = __ballot_sync(0xffffffffu, np3[li] > lj);
+                if (m == 0) {
+                    li++;
+                    lj = -1;
+                    continue;
+                }
+                if (lane == 0) {
+                    S.mask[nent] = m;
+                    S.pre[nent] = total;
+                    S.ent[nent] = make_int2(li, lj);
+                }
+                total += __popc(m);
+                nent++;
+            }
+            if (lane == 0) S.pre[nent] = total;
+            __syncwarp();
+            for (int it0 = 0; it0 < total; it0 += 32) {
+                const int item = it0 + lane;
+                const bool on = item < total;
+                int lo = 0, hi = nent;  // last entry with pre <= item
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (S.pre[mid] <= item)
+                        lo = mid;
+                    else
+                        hi = mid;
+                }
+                const int2 en = S.ent[lo];
+                const int pt = on ? (int)__fns(S.mask[lo], 0, item - S.pre[lo] + 1) : 0, i = en.x;
+                const double h = on ? S.h[i][pt] : 1.0, ah = fabs(h), ds = on ? S.ds[i][pt] : 0.0;
+                const double dd = S.dd[pt], ad = fabs(dd), lad = S.lad[pt], iad = S.iad[pt];
+                const double s0 = on ? S.sa[i][pt] + ds * en.y : 0.0, e0 = exp(s0), i0 = 1.0 / e0;
+                const bool series = S.ser[pt];
+                // orders for 1e-18 at the largest |k| R of these panels
+                int NT = 4;
+                {
+                    const float kd = (float)(kabs * ad);
+                    const float top = 0.5f * (fmaxf((float)e0 * expf((float)ds), (float)i0) + 1.0f) * (float)(kabs * ah);
+                    const float xr = on && series ? sqrtf(top * top + kd * kd) : 0.0f;
+                    const float x = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(xr)));
+                    float v = x * x * x * x * (1.0f / 24.0f);
+                    for (; v > 1e-18f && NT < NC_NT; NT++) v *= x / (float)(NT + 1);
+                    NT = (NT + 1) & ~1;
+                }
+                if (!on) continue;
+                cd sis = mk(0, 0), sgn = mk(0, 0), fc = mk(0, 0), fs = mk(0, 0), gc = mk(0, 0), gs = mk(0, 0);
+                for (int q = 0; q < na; q++) {
+                    const double es = na <= NC_NA ? e0 * S.ep[q][i][pt] : exp(s0 + ds * cq.x[QR_ANG][q]);
+                    const double ei = na <= NC_NA ? i0 * S.en[q][i][pt] : 1.0 / es;
+                    const double c2 = es + ei, ca = 2.0 / c2, sn = 0.5 * (es - ei) * ca;
+                    const double rhom = 0.5 * ah * c2;
+                    const double R2 = rhom * rhom + dd * dd, iR = rsqrt(R2), Rm = R2 * iR;
+                    const double wa = ds * cq.w[QR_ANG][q] * ca;
+                    const double la = log((rhom + Rm) * iad);  // asinh(rhom/|d|), or log 2 rhom in the plane
+                    cd is, f1, f2, E;
+                    if (series) {
+                        const double rs = kabs * rhom, Rs = kabs * Rm, d2 = (kabs * dd) * (kabs * dd);
+                        double Rp = 1.0, to = d2 * la, te = d2 * rs;
+                        is = mk(0, 0), f1 = mk(0, 0), f2 = mk(0, 0), E = mk(1, 0);
+                        for (int m = 1; m <= NT; m += 2) {
+                            Rp *= Rs;
+                            double A = cq.rn[m + 1] * fma(rs, Rp, -to);
+                            to = d2 * (A + to);
+                            if (REALK) {  // even powers real, odd ones imaginary
+                                f1.re = fma(S.u[m - 1].x, A, f1.re);
+                                f2.re = fma(S.g[m].x, A, f2.re);
+                                E.im = fma(S.u[m].y, Rp, E.im);
+                                is.re = fma(S.b[m].x, Rp, is.re);
+                                Rp *= Rs;
+                                A = cq.rn[m + 2] * fma(rs, Rp, -te);
+                                te = d2 * (A + te);
+                                f1.im = fma(S.u[m].y, A, f1.im);
+                                f2.im = fma(S.g[m + 1].y, A, f2.im);
+                                E.re = fma(S.u[m + 1].x, Rp, E.re);
+                                is.im = fma(S.b[m + 1].y, Rp, is.im);
+                            } else {
+#pragma unroll
+                                for (int o = 0; o < 2; o++) {
+                                    if (o) {
+                                        Rp *= Rs;
+                                        A = cq.rn[m + 2] * fma(rs, Rp, -te);
+                                        te = d2 * (A + te);
+                                    }
+                                    const double2 u0 = S.u[m - 1 + o], u1 = S.u[m + o], g = S.g[m + o], b = S.b[m + o];
+                                    f1.re = fma(u0.x, A, f1.re);
+                                    f1.im = fma(u0.y, A, f1.im);
+                                    f2.re = fma(g.x, A, f2.re);
+                                    f2.im = fma(g.y, A, f2.im);
+                                    E.re = fma(u1.x, Rp, E.re);
+                                    E.im = fma(u1.y, Rp, E.im);
+                                    is.re = fma(b.x, Rp, is.re);
+                                    is.im = fma(b.y, Rp, is.im);
+                                }
+                            }
+                        }
+                        is = is - mk(S.is0[pt].x, S.is0[pt].y);
+                    } else {
+                        E = cexp_mjkr(k, Rm);
+                        is = mk(S.ead[pt].x, S.ead[pt].y) * (Rm - ad) * phi1(mjk * (Rm - ad));
+                        if (dd == 0.0) {
+                            // coplanar point: closed forms with z = j k rhom
+                            const cd z = mk(-k.im * rhom, k.re * rhom), jk = mk(-k.im, k.re);
+                            f1 = cdivc(mk(1, 0) - E * (mk(1, 0) + z), jk * jk);
+                            f2 = mk(1, 0) - E - ein(z, E);
+                        } else {
+                            // beyond R = RCUT/|Im k| the exponential is below 1e-15: f1 has no
+                            // contribution there and (1 + jkR) exp(-jkR) - 1 = -1 integrates in closed form
+                            const double Rc = (!REALK && k.im != 0.0) ? RCUT / fabs(k.im) : 1e300;
+                            if (Rc < Rm) {
+                                const double rc = S.rc[pt], Rcc = sqrt(rc * rc + dd * dd);
+                                const double tail = (la + lad - rhom * iR) - (log(rc + Rcc) - rc / Rcc);
+                                f1 = mk(S.a1[pt].x, S.a1[pt].y);
+                                f2 = mk(S.a2[pt].x - tail, S.a2[pt].y);
+                            } else {
+                                radial_numeric(k, rhom, dd, &f1, &f2);
+                            }
+                        }
+                    }
+                    f2.re += la + lad - rhom * iR;
+                    const double wn = -wa * dd * iR, wc = wa * ca, ws = wa * sn;
+                    sis = sis + wa * is;
+                    sgn = sgn + wn * E;
+                    fc = fc + wc * f1;
+                    fs = fs + ws * f1;
+                    gc = gc + wc * f2;
+                    gs = gs + ws * f2;
+                }
+                const double sh = h > 0 ? 1.0 : -1.0, f = sh * f4, si = series ? f / kabs : f, sf = series ? si / kabs : f;
+                const cd Is = si * sis;
+                fc = (sf * sh) * fc;  // u = sh m: the in-plane normal toward the edge
+                fs = sf * fs;
+                gc = f4 * gc;
+                gs = f * gs;
+                sgn = f * sgn;
+                cd Iv[3], Ig[3];
+                const double nmv[3] = {nm.x, nm.y, nm.z};
+                for (int d = 0; d < 3; d++) {
+                    Iv[d] = S.em[i][d] * fc + S.et[i][d] * fs - (dd * nmv[d]) * Is;
+                    Ig[d] = S.em[i][d] * gc + S.et[i][d] * gs - nmv[d] * sgn;
+                }
+                const double rtv[3] = {S.rt[0][pt], S.rt[1][pt], S.rt[2][pt]};
+                add_moments(acc, S.w[pt], rtv, kind == PC_SELF, Is, Iv, Ig);
+            }
+            __syncwarp();
+        }
+    }
+    store_moments(acc, lane, part + 14 * (int64_t)un);
+}
+
+// moments of each close pair: its units' parts in order
+__global__ void k_near_sum(int n, const int3* __restrict__ own, const double2* __restrict__ part,
+                           double2* __restrict__ mom)
+{
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 14 * n) return;
+    const int3 o = own[idx / 14];  // pair, first unit, units
+    const int i = idx % 14;
+    double2 s = make_double2(0, 0);
+    for (int u = 0; u < o.z; u++) {
+        const double2 v = part[14 * (int64_t)(o.y + u) + i];
+        s.x += v.x;
+        s.y += v.y;
+    }
+    mom[14 * (int64_t)o.x + i] = s;
+}
+
+// moments of all near pairs of a
+static sie_status near_moments(sie_op* op, const AimOp& a, const QuadDev& q, double2* mom)
+{
+    cudaStream_t st = op->mesh->ctx->stream;
+    const DevMesh& M = op->mesh->d;
+    const int64_t np = a.npairs;
+    if (np <= 0) return SIE_OK;
+    uint8_t* cls = nullptr;
+    std::vector<uint8_t> hc(np);
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&cls, np, st));
+    k_pair_class<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a.pairs, np, M, a.kr, a.ki, a.obj_k, cls);
+    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_CUDA_TRY(cudaMemcpyAsync(hc.data(), cls, np, cudaMemcpyDeviceToHost, st));
+    k_near_far<<<(unsigned)((np + 3) / 4), 128, 0, st>>>(a.pairs, np, cls, M, a.kr, a.ki, a.obj_k, mom);
+    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_CUDA_TRY(cudaStreamSynchronize(st));
+    // outer points of a class, as graded_count() on the device
+    const int ge = q.opan * q.n[QR_OLAM] * 2 * q.emupan * q.n[QR_EMU], gv = q.opan * q.n[QR_OLAM] * q.n[QR_OMU];
+    const int nout[5] = {0, q.n[QR_OUT] * q.n[QR_OUT], gv, ge, 3 * ge};
+    int64_t count[5] = {0, 0, 0, 0, 0}, total = 0;
+    for (int64_t p = 0; p < np; p++) count[hc[p]]++;
+    for (int c = 1; c < 5; c++) total += count[c] * ((nout[c] + 31) / 32);
+    // 32 outer points per unit while that keeps the list below 2^18 units (59 MB of parts), then up to 512
+    const int npts = 32 * (int)std::min<int64_t>(16, (total >> 18) + 1);
+    std::vector<int2> unit;
+    std::vector<int3> own;
+    for (int c = 4; c >= 1; c--)
+        for (int64_t p = 0; p < np && count[c] > 0; p++)
+            if (hc[p] == c) {
+                const int first = (int)unit.size();
+                for (int o = 0; o < nout[c]; o += npts) unit.push_back(make_int2((int)p, o));
+                own.push_back(make_int3((int)p, first, (int)unit.size() - first));
+            }
+    if (!unit.empty()) {
+        int2* du = nullptr;
+        int3* dow = nullptr;
+        double2* part = nullptr;
+        const int nu = (int)unit.size(), no = (int)own.size();
+        SIE_CUDA_TRY(cudaMallocAsync((void**)&du, sizeof(int2) * nu, st));
+        SIE_CUDA_TRY(cudaMallocAsync((void**)&dow, sizeof(int3) * no, st));
+        SIE_CUDA_TRY(cudaMallocAsync((void**)&part, sizeof(double2) * 14 * nu, st));
+        SIE_CUDA_TRY(cudaMemcpyAsync(du, unit.data(), sizeof(int2) * nu, cudaMemcpyHostToDevice, st));
+        SIE_CUDA_TRY(cudaMemcpyAsync(dow, own.data(), sizeof(int3) * no, cudaMemcpyHostToDevice, st));
+        const unsigned blocks = (unsigned)((nu + NC_W - 1) / NC_W);
+        if (!a.obj_k && a.ki == 0.0)
+            k_near_close<true><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, M, a.kr, 0.0, nullptr, part);
+        else
+            k_near_close<false><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, M, a.kr, a.ki, a.obj_k,
+                                                              part);
+        SIE_CUDA_TRY(cudaGetLastError());
+        k_near_sum<<<(14 * no + 127) / 128, 128, 0, st>>>(no, dow, part, mom);
+        SIE_CUDA_TRY(cudaGetLastError());
+        SIE_CUDA_TRY(cudaStreamSynchronize(st));  // the host lists outlive the copies
+        cudaFreeAsync(du, st);
+        cudaFreeAsync(dow, st);
+        cudaFreeAsync(part, st);
+    }
+    cudaFreeAsync(cls, st);
+    return SIE_OK;
 }
 
 // kernel values at integer lags |l_d| <= Lm: (G, dG/dx, dG/dy, dG/dz), zero at lag 0
@@ -533,62 +822,80 @@ __global__ void __launch_bounds__(128) k_near_local(const int32_t* __restrict__ 
     int lane = threadIdx.x & 31;
     if (p >= np) return;
     int t = pairs[2 * p], s = pairs[2 * p + 1];
-    // grid part: partial sums over the test nodes owned by this lane
-    cd gLA[9], gK[9], g0 = mk(0, 0);
-    for (int i = 0; i < 9; i++) gLA[i] = gK[i] = mk(0, 0);
+    // grid part: W_t^T G W_s and its curl form.  A lane owns a test node u and
+    // first sums over the source nodes v the four weights (w0, w1) of v times G
+    // and grad G (32 FMAs a node pair); the 3 x 3 local entries are then linear
+    // in a few sums over u (forming all 18 per node pair took 170).
+    // gs: LA: 0 sum_a w1_a|w1_a, 1..3 w1_a|w0, 4..6 w0|w1_a, 7 w0|w0 (also Lphi);
+    // K (curl form, D = grad G): 8 all weights w1, 9..11 w1 on the test side (by
+    // source component), 12..14 w1 on the source side (by test component), 15..17 w0|D|w0
+    cd gs[18];
+    for (int i = 0; i < 18; i++) gs[i] = mk(0, 0);
     if (has_grid) {
         const int Mp = Mord + 1;
         int bt[3] = {base[3 * t], base[3 * t + 1], base[3 * t + 2]};
         int bs[3] = {base[3 * s], base[3 * s + 1], base[3 * s + 2]};
-        const double* ct = M.coef + 3 * t;
-        const double* cs = M.coef + 3 * s;
-        const double* qt = M.q + 9 * t;
-        const double* qs = M.q + 9 * s;
         const int Wd = 2 * Lm + 1;
         for (int u = lane; u < S; u += 32) {
-            int ux = u % Mp, uy = (u / Mp) % Mp, uz = u / (Mp * Mp);
+            const int ux = u % Mp, uy = (u / Mp) % Mp, uz = u / (Mp * Mp);
             const double* wu = Wt + ((size_t)t * S + u) * 4;
-            double xt[3][3];  // test projection weights of slot i, component a
-            for (int i = 0; i < 3; i++)
-                for (int aa = 0; aa < 3; aa++) xt[i][aa] = ct[i] * (wu[1 + aa] + qt[3 * i + aa] * wu[0]);
-            for (int v = 0; v < S; v++) {
-                int vx = v % Mp, vy = (v / Mp) % Mp, vz = v / (Mp * Mp);
-                int lx = bt[0] + ux - bs[0] - vx, ly = bt[1] + uy - bs[1] - vy, lz = bt[2] + uz - bs[2] - vz;
-                const double2* kv = tab + 4 * (((lz + Lm) * Wd + (ly + Lm)) * Wd + (lx + Lm));
-                cd G = mk(kv[0].x, kv[0].y), Dx = mk(kv[1].x, kv[1].y), Dy = mk(kv[2].x, kv[2].y),
-                   Dz = mk(kv[3].x, kv[3].y);
-                const double* wv = Wt + ((size_t)s * S + v) * 4;
-                g0 = g0 + (wu[0] * wv[0]) * G;
-                for (int j = 0; j < 3; j++) {
-                    double xs[3];
-                    for (int cc = 0; cc < 3; cc++) xs[cc] = cs[j] * (wv[1 + cc] + qs[3 * j + cc] * wv[0]);
-                    for (int i = 0; i < 3; i++) {
-                        double la = xt[i][0] * xs[0] + xt[i][1] * xs[1] + xt[i][2] * xs[2];
-                        // sum_abc eps_abc xt_a D_b xs_c = D . (xs x xt)
-                        double wx = xs[1] * xt[i][2] - xs[2] * xt[i][1];
-                        double wy = xs[2] * xt[i][0] - xs[0] * xt[i][2];
-                        double wz = xs[0] * xt[i][1] - xs[1] * xt[i][0];
-                        gLA[3 * i + j] = gLA[3 * i + j] + la * G;
-                        gK[3 * i + j] = gK[3 * i + j] + wx * Dx + wy * Dy + wz * Dz;
+            cd Y[4][4];  // [G, Dx, Dy, Dz][w0, w1x, w1y, w1z]
+            for (int i = 0; i < 16; i++) Y[i / 4][i % 4] = mk(0, 0);
+            int v = 0;
+            for (int vz = 0; vz < Mp; vz++)
+                for (int vy = 0; vy < Mp; vy++)
+                    for (int vx = 0; vx < Mp; vx++, v++) {
+                        const int lx = bt[0] + ux - bs[0] - vx, ly = bt[1] + uy - bs[1] - vy,
+                                  lz = bt[2] + uz - bs[2] - vz;
+                        const double2* kv = tab + 4 * (((lz + Lm) * Wd + (ly + Lm)) * Wd + (lx + Lm));
+                        const double* wv = Wt + ((size_t)s * S + v) * 4;
+#pragma unroll
+                        for (int g = 0; g < 4; g++) {
+                            const double2 kg = kv[g];
+#pragma unroll
+                            for (int c = 0; c < 4; c++) {
+                                Y[g][c].re = fma(wv[c], kg.x, Y[g][c].re);
+                                Y[g][c].im = fma(wv[c], kg.y, Y[g][c].im);
+                            }
+                        }
                     }
-                }
+            const double w0 = wu[0], w1[3] = {wu[1], wu[2], wu[3]};
+            gs[0] = gs[0] + w1[0] * Y[0][1] + w1[1] * Y[0][2] + w1[2] * Y[0][3];
+            gs[7] = gs[7] + w0 * Y[0][0];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const int e = (d + 1) % 3, f = (d + 2) % 3;
+                gs[1 + d] = gs[1 + d] + w1[d] * Y[0][0];
+                gs[4 + d] = gs[4 + d] + w0 * Y[0][1 + d];
+                // eps_abc x_a D_b y_c, a = d: (b, c) = (e, f) minus (f, e)
+                const cd curl = Y[1 + e][1 + f] - Y[1 + f][1 + e];
+                gs[8] = gs[8] + w1[d] * curl;
+                gs[12 + d] = gs[12 + d] + w0 * curl;
+                // c = d: (a, b) = (e, f) minus (f, e)
+                gs[9 + d] = gs[9 + d] + w1[e] * Y[1 + f][0] - w1[f] * Y[1 + e][0];
+                gs[15 + d] = gs[15 + d] + w0 * Y[1 + d][0];
             }
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            for (int i = 0; i < 9; i++) {
-                gLA[i].re += __shfl_down_sync(0xffffffffu, gLA[i].re, off);
-                gLA[i].im += __shfl_down_sync(0xffffffffu, gLA[i].im, off);
-                gK[i].re += __shfl_down_sync(0xffffffffu, gK[i].re, off);
-                gK[i].im += __shfl_down_sync(0xffffffffu, gK[i].im, off);
+        for (int off = 16; off > 0; off >>= 1)
+            for (int i = 0; i < 18; i++) {
+                gs[i].re += __shfl_xor_sync(0xffffffffu, gs[i].re, off);
+                gs[i].im += __shfl_xor_sync(0xffffffffu, gs[i].im, off);
             }
-            g0.re += __shfl_down_sync(0xffffffffu, g0.re, off);
-            g0.im += __shfl_down_sync(0xffffffffu, g0.im, off);
-        }
     }
-    if (lane != 0) return;
-    // exact entries from the moments
+    if (lane >= 10) return;
     const double2* mm = mom + 14 * p;
-    cd Q0 = mk(mm[0].x, mm[0].y);
+    double2* o = out + NLOC * p;
+    const cd Q0 = mk(mm[0].x, mm[0].y);
+    if (lane == 9) {  // scalar potential
+        const double At = M.area[t], As = M.area[s];
+        const cd lp = (1.0 / (At * As)) * (Q0 - gs[7]);
+        o[18] = make_double2(lp.re, lp.im);
+        const cd lpe = (1.0 / (At * As)) * Q0;
+        o[28] = make_double2(lpe.re, lpe.im);  // exact
+        return;
+    }
+    // a lane per local entry (i, j): exact value from the moments, grid value from gs
+    const int i = lane / 3, j = lane % 3;
     cd Q1[3], Q2[3], U[3], Vv[3];
     for (int d = 0; d < 3; d++) {
         Q1[d] = mk(mm[1 + d].x, mm[1 + d].y);
@@ -596,32 +903,32 @@ __global__ void __launch_bounds__(128) k_near_local(const int32_t* __restrict__ 
         U[d] = mk(mm[8 + d].x, mm[8 + d].y);
         Vv[d] = mk(mm[11 + d].x, mm[11 + d].y);
     }
-    cd Q3 = mk(mm[7].x, mm[7].y);
-    v3 ctc = ld3(M.cen + 3 * t);
-    double At = M.area[t], As = M.area[s];
-    double2* o = out + NLOC * p;
-    for (int i = 0; i < 3; i++) {
-        double cm = M.coef[3 * t + i];
-        v3 pm = ld3(M.V + 3 * M.T[3 * t + i]) - ctc;
-        for (int j = 0; j < 3; j++) {
-            double cn = M.coef[3 * s + j];
-            v3 pn = ld3(M.V + 3 * M.T[3 * s + j]) - ctc;
-            cd la = Q3 - (pn.x * Q1[0] + pn.y * Q1[1] + pn.z * Q1[2]) - (pm.x * Q2[0] + pm.y * Q2[1] + pm.z * Q2[2]) +
-                    dot(pm, pn) * Q0;
-            v3 dl = pn - pm, cx = cross(pn, pm);
-            cd kk = dl.x * U[0] + dl.y * U[1] + dl.z * U[2] + cx.x * Vv[0] + cx.y * Vv[1] + cx.z * Vv[2];
-            la = (cm * cn) * la;
-            o[19 + 3 * i + j] = make_double2(la.re, la.im);  // exact
-            la = la - gLA[3 * i + j];
-            kk = (cm * cn) * kk - gK[3 * i + j];
-            o[3 * i + j] = make_double2(la.re, la.im);
-            o[9 + 3 * i + j] = make_double2(kk.re, kk.im);
-        }
+    const cd Q3 = mk(mm[7].x, mm[7].y);
+    const v3 ctc = ld3(M.cen + 3 * t);
+    const double cm = M.coef[3 * t + i], cn = M.coef[3 * s + j];
+    const v3 pm = ld3(M.V + 3 * M.T[3 * t + i]) - ctc, pn = ld3(M.V + 3 * M.T[3 * s + j]) - ctc;
+    cd la = Q3 - (pn.x * Q1[0] + pn.y * Q1[1] + pn.z * Q1[2]) - (pm.x * Q2[0] + pm.y * Q2[1] + pm.z * Q2[2]) +
+            dot(pm, pn) * Q0;
+    const v3 dl = pn - pm, cx = cross(pn, pm);
+    cd kk = dl.x * U[0] + dl.y * U[1] + dl.z * U[2] + cx.x * Vv[0] + cx.y * Vv[1] + cx.z * Vv[2];
+    la = (cm * cn) * la;
+    o[19 + 3 * i + j] = make_double2(la.re, la.im);  // exact
+    if (has_grid) {
+        const double* qt = M.q + 9 * t + 3 * i;
+        const double* qs = M.q + 9 * s + 3 * j;
+        // sum_a (w1 + qt w0)_a (w1 + qs w0)_a G
+        const cd gl = gs[0] + qs[0] * gs[1] + qs[1] * gs[2] + qs[2] * gs[3] + qt[0] * gs[4] + qt[1] * gs[5] +
+                      qt[2] * gs[6] + (qt[0] * qs[0] + qt[1] * qs[1] + qt[2] * qs[2]) * gs[7];
+        // sum_abc eps_abc (w1 + qt w0)_a D_b (w1 + qs w0)_c
+        const cd gk = gs[8] + qs[0] * gs[9] + qs[1] * gs[10] + qs[2] * gs[11] + qt[0] * gs[12] + qt[1] * gs[13] +
+                      qt[2] * gs[14] + (qs[1] * qt[2] - qs[2] * qt[1]) * gs[15] +
+                      (qs[2] * qt[0] - qs[0] * qt[2]) * gs[16] + (qs[0] * qt[1] - qs[1] * qt[0]) * gs[17];
+        la = la - (cm * cn) * gl;
+        kk = kk - gk;
     }
-    cd lp = (1.0 / (At * As)) * (Q0 - g0);
-    o[18] = make_double2(lp.re, lp.im);
-    cd lpe = (1.0 / (At * As)) * Q0;
-    o[28] = make_double2(lpe.re, lpe.im);  // exact
+    kk = (cm * cn) * kk;
+    o[3 * i + j] = make_double2(la.re, la.im);
+    o[9 + 3 * i + j] = make_double2(kk.re, kk.im);
 }
 
 // CSR values: entry (m, n) sums the local entries of the near pairs (t, s)
@@ -703,11 +1010,7 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&mom, sizeof(double2) * 14 * std::max<int64_t>(a.npairs, 1), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&loc, sizeof(double2) * NLOC * std::max<int64_t>(a.npairs, 1), st));
     const int wpb = 4;
-    if (a.npairs > 0) {
-        k_near_moments<<<(unsigned)((a.npairs + wpb - 1) / wpb), 32 * wpb, 0, st>>>(a.pairs, a.npairs, M, a.kr, a.ki,
-                                                                                    a.obj_k, mom);
-        SIE_CUDA_TRY(cudaGetLastError());
-    }
+    SIE_TRY(near_moments(op, a, q, mom));
     int Lm = a.g.Rnear + a.g.M;
     int S = (a.g.M + 1) * (a.g.M + 1) * (a.g.M + 1);
     if (a.has_grid) {
