@@ -1,9 +1,8 @@
 // AIM grid path of Eqs. (AIM_Lin), (AIM_Kin) on sm_103a:
 //   projection P / P_phi (moment-matching stencils, scatter),
-//   zero-padded 3D FFT (shared-memory radix-2 pencils, pruned passes),
-//   spectral multiply with the sampled Green's function and its gradient,
-//   pruned inverse FFT, interpolation W = P^T (gather), and the
-//   precorrected near-region CSR product (Eqs. LinNRP, KinNRP).
+//   zero-padded 3D FFT, spectral multiply with the sampled Green's function
+//   and its gradient and pruned inverse FFT (fft.cu), interpolation W = P^T
+//   (gather), and the precorrected near-region CSR product (Eqs. LinNRP, KinNRP).
 #include <algorithm>
 #include <chrono>
 #include <cstdlib>
@@ -15,7 +14,6 @@
 
 #include "internal.h"
 #include "spmv.cuh"
-#include "sysmul.cuh"
 
 namespace sie {
 
@@ -160,828 +158,6 @@ sie_status aim_weights(sie_op* op)
     k_to_f32<<<(unsigned)((4 * (size_t)nt * S + 255) / 256), 256, 0, st>>>(op->W, op->W32, 4 * (int64_t)nt * S);
     SIE_CUDA_TRY(cudaGetLastError());
     return SIE_OK;
-}
-
-// ------------------------------------------------------------------ FFT
-// Twiddles exp(-2 pi i k / n), k < n, for n = 2^l (l <= 10): one table per
-// device and length, made on first use (guarded: contexts may run in threads).
-constexpr int TW_MAXDEV = 64;
-static double2* g_tw[TW_MAXDEV][11] = {};
-static float2* g_tw32[TW_MAXDEV][11] = {};
-static std::mutex g_tw_mu;
-
-static sie_status twiddles_dev(int logn, int dev, double2** out, float2** out32)
-{
-    std::lock_guard<std::mutex> lk(g_tw_mu);
-    if (!g_tw[dev][logn]) {
-        int n = 1 << logn;
-        std::vector<double2> h(std::max(n, 1));
-        for (int k = 0; k < n; k++) {
-            long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)n;
-            h[k] = make_double2((double)cosl(a), (double)sinl(a));
-        }
-        double2* d = nullptr;
-        SIE_CUDA_TRY(cudaMalloc((void**)&d, sizeof(double2) * h.size()));
-        SIE_CUDA_TRY(cudaMemcpy(d, h.data(), sizeof(double2) * h.size(), cudaMemcpyHostToDevice));
-        std::vector<float2> hf(h.size());
-        for (size_t k = 0; k < h.size(); k++) hf[k] = make_float2((float)h[k].x, (float)h[k].y);
-        float2* f = nullptr;
-        SIE_CUDA_TRY(cudaMalloc((void**)&f, sizeof(float2) * hf.size()));
-        SIE_CUDA_TRY(cudaMemcpy(f, hf.data(), sizeof(float2) * hf.size(), cudaMemcpyHostToDevice));
-        g_tw[dev][logn] = d;
-        g_tw32[dev][logn] = f;
-    }
-    if (out) *out = g_tw[dev][logn];
-    if (out32) *out32 = g_tw32[dev][logn];
-    return SIE_OK;
-}
-
-static sie_status twiddles(int logn, cudaStream_t, double2** out)
-{
-    int dev = 0;
-    SIE_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= TW_MAXDEV) {
-        set_error("twiddles: device ordinal out of range");
-        return SIE_ERR_ARG;
-    }
-    return twiddles_dev(logn, dev, out, nullptr);
-}
-
-static sie_status twiddles(int logn, cudaStream_t, float2** out)
-{
-    int dev = 0;
-    SIE_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= TW_MAXDEV) {
-        set_error("twiddles: device ordinal out of range");
-        return SIE_ERR_ARG;
-    }
-    return twiddles_dev(logn, dev, nullptr, out);
-}
-
-struct PassGeom {
-    int n_in, n_out;       // elements read / written per pencil (zero padding / truncation)
-    int64_t npencil;       // pencils
-    int L;                 // pencil p -> lo = p % L, hi = p / L
-    int64_t slo_in, shi_in, st_in;
-    int64_t slo_out, shi_out, st_out;
-    int contig;            // 1: elements of a pencil are contiguous (x pass)
-    int64_t bs_in = 0, bs_out = 0;  // offsets between the grids of a batch (blockIdx.y)
-};
-
-// One CTA transforms PB pencils of length n = 2^LOGN held in shared memory.
-// Load at bit-reversed positions, log2(n) radix-2 DIT stages (the first two
-// fused into one radix-4 pass without multiplications), store.
-template <class C>
-__device__ __forceinline__ C cmake(double a, double b);
-template <>
-__device__ __forceinline__ double2 cmake<double2>(double a, double b) { return make_double2(a, b); }
-template <>
-__device__ __forceinline__ float2 cmake<float2>(double a, double b) { return make_float2((float)a, (float)b); }
-
-// C = double2 (FP64 path) or float2 (complex64 grid path)
-template <int LOGN, int PB, class C>
-__global__ void __launch_bounds__(256) k_fft_pass(const C* in, C* out,  // may alias (in place)
-                                                  const C* __restrict__ tw, int inv, PassGeom G)
-{
-    constexpr int n = 1 << LOGN;
-    constexpr int pitch = n + 1;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C* sm = reinterpret_cast<C*>(smraw);
-    const int64_t p0 = (int64_t)blockIdx.x * PB;
-    // load (zero padded)
-    for (int idx = threadIdx.x; idx < PB * n; idx += blockDim.x) {
-        int pl, j;
-        if (G.contig) {
-            pl = idx / n;
-            j = idx % n;
-        } else {
-            pl = idx % PB;
-            j = idx / PB;
-        }
-        int64_t p = p0 + pl;
-        C v = cmake<C>(0.0, 0.0);
-        if (p < G.npencil && j < G.n_in) {
-            int64_t b = (p % G.L) * G.slo_in + (p / G.L) * G.shi_in + blockIdx.y * G.bs_in;
-            v = in[b + (int64_t)j * G.st_in];
-        }
-        sm[pl * pitch + (__brev(j) >> (32 - LOGN))] = v;
-    }
-    __syncthreads();
-    // stages 1 and 2 have trivial twiddles (1 and -+j): adds and swaps only
-    for (int q = threadIdx.x; q < PB * (n / 4); q += blockDim.x) {
-        int pl = q / (n / 4), base = 4 * (q % (n / 4));
-        C* p = sm + pl * pitch + base;
-        C x0 = p[0], x1 = p[1], x2 = p[2], x3 = p[3];
-        C a0, a1, b0, b1;
-        a0.x = x0.x + x1.x;
-        a0.y = x0.y + x1.y;
-        a1.x = x0.x - x1.x;
-        a1.y = x0.y - x1.y;
-        b0.x = x2.x + x3.x;
-        b0.y = x2.y + x3.y;
-        b1.x = x2.x - x3.x;
-        b1.y = x2.y - x3.y;
-        // stage 2: w = 1 for (a0, b0); w = -j (forward) or +j (inverse) for (a1, b1)
-        C t;
-        if (inv) {
-            t.x = -b1.y;
-            t.y = b1.x;
-        } else {
-            t.x = b1.y;
-            t.y = -b1.x;
-        }
-        C y0, y1, y2, y3;
-        y0.x = a0.x + b0.x;
-        y0.y = a0.y + b0.y;
-        y2.x = a0.x - b0.x;
-        y2.y = a0.y - b0.y;
-        y1.x = a1.x + t.x;
-        y1.y = a1.y + t.y;
-        y3.x = a1.x - t.x;
-        y3.y = a1.y - t.y;
-        p[0] = y0;
-        p[1] = y1;
-        p[2] = y2;
-        p[3] = y3;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int s = 3; s <= LOGN; s++) {
-        const int half = 1 << (s - 1);
-        for (int bfly = threadIdx.x; bfly < PB * (n / 2); bfly += blockDim.x) {
-            int pl = bfly / (n / 2), bb = bfly % (n / 2);
-            int grp = bb >> (s - 1), pos = bb & (half - 1);
-            int i0 = grp * 2 * half + pos, i1 = i0 + half;
-            C w = tw[pos << (LOGN - s)];
-            if (inv) w.y = -w.y;
-            C u = sm[pl * pitch + i0], v = sm[pl * pitch + i1];
-            C vw;
-            vw.x = v.x * w.x - v.y * w.y;
-            vw.y = v.x * w.y + v.y * w.x;
-            C a0, a1;
-            a0.x = u.x + vw.x;
-            a0.y = u.y + vw.y;
-            a1.x = u.x - vw.x;
-            a1.y = u.y - vw.y;
-            sm[pl * pitch + i0] = a0;
-            sm[pl * pitch + i1] = a1;
-        }
-        __syncthreads();
-    }
-    for (int idx = threadIdx.x; idx < PB * n; idx += blockDim.x) {
-        int pl, j;
-        if (G.contig) {
-            pl = idx / n;
-            j = idx % n;
-        } else {
-            pl = idx % PB;
-            j = idx / PB;
-        }
-        int64_t p = p0 + pl;
-        if (p < G.npencil && j < G.n_out) {
-            int64_t b = (p % G.L) * G.slo_out + (p / G.L) * G.shi_out + blockIdx.y * G.bs_out;
-            out[b + (int64_t)j * G.st_out] = sm[pl * pitch + j];
-        }
-    }
-}
-
-
-// ------------------------------------------------------------------ Stockham FFT (register radix-8)
-// Self-sorting Stockham formulation (Govindaraju et al., SC'08): pass p with
-// current span Ns and radix R: thread j loads a[r] = x[j + r n/R], multiplies
-// by exp(-+2 pi i (j mod Ns) r / (Ns R)), does an R-point DFT in registers and
-// stores y[(j / Ns) Ns R + (j mod Ns) + r Ns].  n/8 threads per pencil; the
-// first pass reads the (zero padded) pencil straight from global memory, the
-// last writes the (truncated) output straight to global memory, the passes in
-// between exchange through shared memory.
-template <class C, int INV>
-__device__ __forceinline__ void cmulw(C& a, C w)
-{
-    C t;
-    if (INV) w.y = -w.y;
-    t.x = a.x * w.x - a.y * w.y;
-    t.y = a.x * w.y + a.y * w.x;
-    a = t;
-}
-
-template <class C, int INV>
-__device__ __forceinline__ void bfly2(C& a, C& b)
-{
-    C t = a;
-    a.x = t.x + b.x;
-    a.y = t.y + b.y;
-    b.x = t.x - b.x;
-    b.y = t.y - b.y;
-}
-
-// multiply by -j (forward) or +j (inverse)
-template <class C, int INV>
-__device__ __forceinline__ C mulmj(C a)
-{
-    C t;
-    if (INV) {
-        t.x = -a.y;
-        t.y = a.x;
-    } else {
-        t.x = a.y;
-        t.y = -a.x;
-    }
-    return t;
-}
-
-template <class C, int INV>
-__device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3)
-{
-    // X0 = (a0+a2)+(a1+a3), X2 = (a0+a2)-(a1+a3), X1 = (a0-a2) -+j (a1-a3), X3 = (a0-a2) +-j (a1-a3)
-    bfly2<C, INV>(a0, a2);
-    bfly2<C, INV>(a1, a3);
-    a3 = mulmj<C, INV>(a3);
-    bfly2<C, INV>(a0, a1);
-    bfly2<C, INV>(a2, a3);
-    // now a0 = X0, a1 = X2, a2 = X1, a3 = X3 -> reorder
-    C t = a1;
-    a1 = a2;
-    a2 = t;
-}
-
-template <class C, int INV>
-__device__ __forceinline__ void dft8(C* a)
-{
-    // even/odd split: E = DFT4(a0,a2,a4,a6), O = DFT4(a1,a3,a5,a7)
-    dft4<C, INV>(a[0], a[2], a[4], a[6]);
-    dft4<C, INV>(a[1], a[3], a[5], a[7]);
-    const double r = 0.70710678118654752440;
-    // O[k] *= W8^k : W8 = (1 -+ j)/sqrt2, W8^2 = -+j, W8^3 = (-1 -+ j)/sqrt2
-    C o1 = a[3], o2 = a[5], o3 = a[7];
-    C t;
-    if (!INV) {
-        t.x = (o1.x + o1.y) * r;
-        t.y = (o1.y - o1.x) * r;
-    } else {
-        t.x = (o1.x - o1.y) * r;
-        t.y = (o1.y + o1.x) * r;
-    }
-    o1 = t;
-    o2 = mulmj<C, INV>(o2);
-    if (!INV) {
-        t.x = (o3.y - o3.x) * r;
-        t.y = -(o3.x + o3.y) * r;
-    } else {
-        t.x = -(o3.x + o3.y) * r;
-        t.y = (o3.x - o3.y) * r;
-    }
-    o3 = t;
-    // E[k] in a[0], a[2], a[4], a[6]; O[k] (twiddled) in a[1], o1, o2, o3
-    C e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6], q0 = a[1];
-    a[0].x = e0.x + q0.x; a[0].y = e0.y + q0.y;
-    a[4].x = e0.x - q0.x; a[4].y = e0.y - q0.y;
-    a[1].x = e1.x + o1.x; a[1].y = e1.y + o1.y;
-    a[5].x = e1.x - o1.x; a[5].y = e1.y - o1.y;
-    a[2].x = e2.x + o2.x; a[2].y = e2.y + o2.y;
-    a[6].x = e2.x - o2.x; a[6].y = e2.y - o2.y;
-    a[3].x = e3.x + o3.x; a[3].y = e3.y + o3.y;
-    a[7].x = e3.x - o3.x; a[7].y = e3.y - o3.y;
-}
-
-template <class C, int INV, int R>
-__device__ __forceinline__ void dftR(C* a)
-{
-    if constexpr (R == 8)
-        dft8<C, INV>(a);
-    else if constexpr (R == 4)
-        dft4<C, INV>(a[0], a[1], a[2], a[3]);
-    else
-        bfly2<C, INV>(a[0], a[1]);
-}
-
-// one Stockham pass of radix R over the pencil held by (tp = thread in pencil);
-// SRC / DST: 0 = global, 1 = shared memory
-template <int LOGN, int R, int SRC, int DST, class C, int INV>
-__device__ __forceinline__ void stockham_pass(int Ns, int tp, const C* gin, int64_t gbase_in, int64_t gst_in,
-                                              int n_in, C* gout, int64_t gbase_out, int64_t gst_out, int n_out,
-                                              bool valid, const C* sin, C* sout, const C* __restrict__ tw)
-{
-    constexpr int n = 1 << LOGN;
-    constexpr int TPP = n / 8;  // threads per pencil
-    constexpr int NB = n / R;   // butterflies per pencil
-    constexpr int LR = R == 8 ? 3 : (R == 4 ? 2 : 1);
-    const int lns = __ffs(Ns) - 1;  // log2(Ns)
-    for (int jj = tp; jj < NB; jj += TPP) {
-        C a[R];
-        for (int r = 0; r < R; r++) {
-            int idx = jj + r * NB;
-            if (SRC == 0) {
-                C v;
-                v.x = 0;
-                v.y = 0;
-                if (valid && idx < n_in) v = gin[gbase_in + (int64_t)idx * gst_in];
-                a[r] = v;
-            } else {
-                a[r] = sin[idx];
-            }
-        }
-        // Ns and R are powers of two: masks and shifts instead of divisions
-        const int k = jj & (Ns - 1);
-        if (Ns > 1)
-            for (int r = 1; r < R; r++) cmulw<C, INV>(a[r], tw[(k * r) << (LOGN - lns - LR)]);
-        dftR<C, INV, R>(a);
-        const int o = ((jj >> lns) << (lns + LR)) + k;
-        for (int r = 0; r < R; r++) {
-            int idx = o + r * Ns;
-            if (DST == 0) {
-                if (valid && idx < n_out) gout[gbase_out + (int64_t)idx * gst_out] = a[r];
-            } else {
-                sout[idx] = a[r];
-            }
-        }
-    }
-}
-
-template <int LOGN, int PB, class C, int INV>
-__global__ void __launch_bounds__(PB*(1 << LOGN) / 8) k_fft_stockham(const C* in, C* out, const C* __restrict__ tw,
-                                                                     PassGeom G)
-{
-    constexpr int n = 1 << LOGN;
-    constexpr int TPP = n / 8;
-    constexpr int pitch = n + 1;
-    extern __shared__ __align__(16) unsigned char smraw2[];
-    C* sm0 = reinterpret_cast<C*>(smraw2);
-    C* sm1 = sm0 + PB * pitch;
-    // pencil-fastest thread order on strided passes keeps rows coalesced
-    int pl, tp;
-    if (G.contig) {
-        pl = threadIdx.x / TPP;
-        tp = threadIdx.x % TPP;
-    } else {
-        pl = threadIdx.x % PB;
-        tp = threadIdx.x / PB;
-    }
-    int64_t p = (int64_t)blockIdx.x * PB + pl;
-    bool valid = p < G.npencil;
-    int64_t bin = valid ? (p % G.L) * G.slo_in + (p / G.L) * G.shi_in + blockIdx.y * G.bs_in : 0;
-    int64_t bout = valid ? (p % G.L) * G.slo_out + (p / G.L) * G.shi_out + blockIdx.y * G.bs_out : 0;
-    C* s0 = sm0 + pl * pitch;
-    C* s1 = sm1 + pl * pitch;
-    // radix plan: 8^a x (1, 2 or 4)
-    constexpr int NP8 = LOGN / 3, REM = LOGN % 3;
-    constexpr int NPASS = NP8 + (REM ? 1 : 0);
-    int Ns = 1;
-    // pass 0 (global -> smem or global)
-    if constexpr (NPASS == 1) {
-        stockham_pass<LOGN, 8, 0, 0, C, INV>(Ns, tp, in, bin, G.st_in, G.n_in, out, bout, G.st_out, G.n_out, valid,
-                                             nullptr, nullptr, tw);
-        return;
-    } else {
-        stockham_pass<LOGN, 8, 0, 1, C, INV>(Ns, tp, in, bin, G.st_in, G.n_in, nullptr, 0, 0, 0, valid, nullptr, s0,
-                                             tw);
-    }
-    Ns *= 8;
-    __syncthreads();
-    C* cur = s0;
-    C* nxt = s1;
-    for (int ps = 1; ps < NP8; ps++) {
-        bool last = (ps == NPASS - 1);
-        if (last) {
-            stockham_pass<LOGN, 8, 1, 0, C, INV>(Ns, tp, nullptr, 0, 0, 0, out, bout, G.st_out, G.n_out, valid, cur,
-                                                 nullptr, tw);
-            return;
-        }
-        stockham_pass<LOGN, 8, 1, 1, C, INV>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, cur, nxt, tw);
-        Ns *= 8;
-        __syncthreads();
-        C* t = cur;
-        cur = nxt;
-        nxt = t;
-    }
-    if constexpr (REM == 1)
-        stockham_pass<LOGN, 2, 1, 0, C, INV>(Ns, tp, nullptr, 0, 0, 0, out, bout, G.st_out, G.n_out, valid, cur,
-                                             nullptr, tw);
-    else if constexpr (REM == 2)
-        stockham_pass<LOGN, 4, 1, 0, C, INV>(Ns, tp, nullptr, 0, 0, 0, out, bout, G.st_out, G.n_out, valid, cur,
-                                             nullptr, tw);
-}
-
-template <int LOGN, int PB, class C>
-static sie_status launch_pass_pb(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, const C* tw,
-                                 int nbatch)
-{
-    constexpr int n = 1 << LOGN;
-    size_t smem = sizeof(C) * PB * (n + 1);
-    // once per instantiation (thread-safe static initialisation)
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_fft_pass<LOGN, PB, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    SIE_CUDA_TRY(attr);
-    unsigned blocks = (unsigned)((G.npencil + PB - 1) / PB);
-    k_fft_pass<LOGN, PB, C><<<dim3(blocks, nbatch), 256, smem, st>>>(in, out, tw, inv, G);
-    SIE_CUDA_TRY(cudaGetLastError());
-    return SIE_OK;
-}
-
-// Pencils per CTA: as many as keep at least ~4 CTAs per SM in flight (more
-// pencils per CTA give longer coalesced rows on the strided passes, fewer
-// leave SMs idle on the small passes); SIE_FFT_PB overrides for tuning.
-static int pick_pb(int n, int64_t npencil)
-{
-    static int forced = -1;
-    if (forced < 0) {
-        const char* e = getenv("SIE_FFT_PB");
-        forced = e ? atoi(e) : 0;
-    }
-    if (forced == 4 || forced == 8 || forced == 16) return (n >= 512 && forced == 16) ? 8 : forced;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (!sms) sms = 152;
-    }
-    for (int pb : {16, 8, 4}) {
-        if (n >= 512 && pb == 16) continue;
-        if (npencil / pb >= 4LL * sms) return pb;
-    }
-    return 4;
-}
-
-template <int LOGN, int PB, class C>
-static sie_status launch_stockham(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, const C* tw,
-                                  int nbatch)
-{
-    constexpr int n = 1 << LOGN;
-    size_t smem = sizeof(C) * 2 * PB * (n + 1);
-    // once per instantiation (thread-safe static initialisation)
-    static const cudaError_t attr = [smem] {
-        cudaError_t e = cudaFuncSetAttribute(k_fft_stockham<LOGN, PB, C, 0>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(k_fft_stockham<LOGN, PB, C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
-    }();
-    SIE_CUDA_TRY(attr);
-    unsigned blocks = (unsigned)((G.npencil + PB - 1) / PB);
-    constexpr int threads = PB * n / 8;
-    if (inv)
-        k_fft_stockham<LOGN, PB, C, 1><<<dim3(blocks, nbatch), threads, smem, st>>>(in, out, tw, G);
-    else
-        k_fft_stockham<LOGN, PB, C, 0><<<dim3(blocks, nbatch), threads, smem, st>>>(in, out, tw, G);
-    SIE_CUDA_TRY(cudaGetLastError());
-    return SIE_OK;
-}
-
-// ------------------------------------------------------------------ fused z stage of the system product
-// Forward z-transforms of the seven source grids, the spectral products of
-// Eq. (sys) (sys_specmul) and the inverse z-transforms of the four result
-// grids, PB (x, y) columns per CTA: the full-length z spectra of a column
-// stay in shared memory, so the 7 + 4 grids of n^3 are neither written out by
-// the forward z pass nor read back by the spectral multiply and the inverse z
-// pass.  Reads z < nz_phys of the seven grids, writes z < nz_phys of grids
-// 0..3 (the inverse y pass reads nothing else).  Thread layout: grid g (7),
-// then pencil-fastest within the grid (coalesced rows along x).  Shared
-// memory: two pitch-(n + 1) arrays per (grid, pencil), the spectrum A and one
-// Stockham ping-pong buffer T; the passes alternate so that the forward chain
-// ends in A and the inverse chain starts from it.
-template <int LOGN, int PB, class C, class R>
-__global__ void __launch_bounds__(7 * PB * (1 << LOGN) / 8)
-    k_fft_z_sys(C* __restrict__ buf, const C* __restrict__ spec, const C* __restrict__ tw, int nz_phys,
-                int64_t ncol, int64_t plane, int64_t bnn, R k0)
-{
-    constexpr int n = 1 << LOGN;
-    constexpr int TPP = n / 8;
-    constexpr int pitch = n + 1;
-    constexpr int NP8 = LOGN / 3, REM = LOGN % 3;
-    constexpr int NPASS = NP8 + (REM ? 1 : 0);
-    extern __shared__ __align__(16) unsigned char smz[];
-    C* sm = reinterpret_cast<C*>(smz);
-    const int gi = threadIdx.x / (PB * TPP);
-    const int rr = threadIdx.x % (PB * TPP);
-    const int pl = rr % PB, tp = rr / PB;
-    const int64_t col = (int64_t)blockIdx.x * PB + pl;
-    const bool valid = col < ncol;
-    C* A = sm + (int64_t)(gi * PB + pl) * 2 * pitch;
-    C* T = A + pitch;
-    // pass ps writes A when (NPASS - 1 - ps) is even, so the last lands in A
-    auto dst_of = [&](int ps) { return ((NPASS - 1 - ps) & 1) ? T : A; };
-    // kernel spectra of this thread's spectral-product points
-    constexpr int NT = 7 * PB * TPP;
-    constexpr int NPT = (PB * n + NT - 1) / NT;
-    C sp[NPT][4];
-#pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        const int idx = threadIdx.x + k * NT;
-        const int p2 = idx % PB, kz = idx / PB;
-        const int64_t c2 = (int64_t)blockIdx.x * PB + p2;
-        if (idx < PB * n && c2 < ncol) {
-            const int64_t i = (int64_t)kz * plane + c2;
-#pragma unroll
-            for (int q = 0; q < 4; q++) sp[k][q] = spec[q * bnn + i];
-        }
-    }
-    // ---- forward: global (z < nz_phys, zero padded) -> ... -> A
-    int Ns = 1;
-    const int64_t gbase = gi * bnn + (valid ? col : 0);
-    stockham_pass<LOGN, 8, 0, 1, C, 0>(Ns, tp, buf, gbase, plane, nz_phys, nullptr, 0, 0, 0, valid, nullptr,
-                                       dst_of(0), tw);
-    Ns *= 8;
-    __syncthreads();
-    for (int ps = 1; ps < NP8; ps++) {
-        stockham_pass<LOGN, 8, 1, 1, C, 0>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, dst_of(ps - 1),
-                                           dst_of(ps), tw);
-        Ns *= 8;
-        __syncthreads();
-    }
-    if constexpr (REM == 1)
-        stockham_pass<LOGN, 2, 1, 1, C, 0>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, T, A, tw);
-    else if constexpr (REM == 2)
-        stockham_pass<LOGN, 4, 1, 1, C, 0>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, T, A, tw);
-    if constexpr (REM != 0) __syncthreads();
-    // ---- spectral products, in place into A of grids 0..3 (kernel spectra
-    // loaded before the forward passes, so their latency overlaps them)
-#pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        const int idx = threadIdx.x + k * NT;
-        if (idx >= PB * n) break;
-        const int p2 = idx % PB, kz = idx / PB;
-        const int64_t c2 = (int64_t)blockIdx.x * PB + p2;
-        if (c2 >= ncol) continue;
-        C in[7], out[4];
-#pragma unroll
-        for (int g = 0; g < 7; g++) in[g] = sm[(int64_t)(g * PB + p2) * 2 * pitch + kz];
-        sys_specmul(sp[k][0], sp[k][1], sp[k][2], sp[k][3], k0, in, out);
-#pragma unroll
-        for (int g = 0; g < 4; g++) sm[(int64_t)(g * PB + p2) * 2 * pitch + kz] = out[g];
-    }
-    __syncthreads();
-    // ---- inverse of grids 0..3: A -> T -> A ... -> global (z < nz_phys)
-    const bool act = gi < 4;
-    Ns = 1;
-    C* cur = A;
-    C* nxt = T;
-    if constexpr (NPASS == 1) {
-        if (act)
-            stockham_pass<LOGN, 8, 1, 0, C, 1>(Ns, tp, nullptr, 0, 0, 0, buf, gbase, plane, nz_phys, valid, A,
-                                               nullptr, tw);
-        return;
-    } else {
-        if (act)
-            stockham_pass<LOGN, 8, 1, 1, C, 1>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, cur, nxt, tw);
-    }
-    Ns *= 8;
-    __syncthreads();
-    {
-        C* t = cur;
-        cur = nxt;
-        nxt = t;
-    }
-    for (int ps = 1; ps < NP8; ps++) {
-        if (ps == NPASS - 1) {
-            if (act)
-                stockham_pass<LOGN, 8, 1, 0, C, 1>(Ns, tp, nullptr, 0, 0, 0, buf, gbase, plane, nz_phys, valid, cur,
-                                                   nullptr, tw);
-            return;
-        }
-        if (act)
-            stockham_pass<LOGN, 8, 1, 1, C, 1>(Ns, tp, nullptr, 0, 0, 0, nullptr, 0, 0, 0, valid, cur, nxt, tw);
-        Ns *= 8;
-        __syncthreads();
-        C* t = cur;
-        cur = nxt;
-        nxt = t;
-    }
-    if constexpr (REM == 1) {
-        if (act)
-            stockham_pass<LOGN, 2, 1, 0, C, 1>(Ns, tp, nullptr, 0, 0, 0, buf, gbase, plane, nz_phys, valid, cur,
-                                               nullptr, tw);
-    } else if constexpr (REM == 2) {
-        if (act)
-            stockham_pass<LOGN, 4, 1, 0, C, 1>(Ns, tp, nullptr, 0, 0, 0, buf, gbase, plane, nz_phys, valid, cur,
-                                               nullptr, tw);
-    }
-}
-
-template <int LOGN, int PB, class C, class R>
-static sie_status launch_z_sys_pb(cudaStream_t st, C* buf, const C* spec, const C* tw, int nz_phys, int64_t ncol,
-                                  int64_t plane, int64_t bnn, R k0)
-{
-    constexpr int n = 1 << LOGN;
-    const size_t smem = sizeof(C) * 7 * PB * 2 * (n + 1);
-    static const cudaError_t attr = cudaFuncSetAttribute(k_fft_z_sys<LOGN, PB, C, R>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    SIE_CUDA_TRY(attr);
-    const unsigned blocks = (unsigned)((ncol + PB - 1) / PB);
-    k_fft_z_sys<LOGN, PB, C, R><<<blocks, 7 * PB * n / 8, smem, st>>>(buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-    SIE_CUDA_TRY(cudaGetLastError());
-    return SIE_OK;
-}
-
-// columns per CTA of k_fft_z_sys: 4 (complex64) or 2 (complex128) by default,
-// 57.8 KB of shared memory at n = 128; SIE_ZSYS_PB = 2, 4 or 8 overrides
-// (complex64; complex128 takes half of it, at least 1), for tuning
-static int zsys_pb(bool c64)
-{
-    static int forced = -1;
-    if (forced < 0) {
-        const char* e = getenv("SIE_ZSYS_PB");
-        forced = e ? atoi(e) : 0;
-    }
-    int pb = (forced == 2 || forced == 4 || forced == 8) ? forced : 4;
-    return c64 ? pb : std::max(1, pb / 2);
-}
-
-template <int LOGN, class C, class R>
-static sie_status launch_z_sys(cudaStream_t st, C* buf, const C* spec, int nz_phys, int64_t ncol, int64_t plane,
-                               int64_t bnn, R k0)
-{
-    C* tw = nullptr;
-    SIE_TRY(twiddles(LOGN, st, &tw));
-    const int pb = zsys_pb(sizeof(C) == 8);
-    if constexpr (sizeof(C) == 8) {
-        if (pb == 2) return launch_z_sys_pb<LOGN, 2, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-        if (pb == 8 && LOGN <= 7) return launch_z_sys_pb<LOGN, 8, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-        return launch_z_sys_pb<LOGN, 4, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-    } else {
-        if (pb == 1) return launch_z_sys_pb<LOGN, 1, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-        if (pb == 4 && LOGN <= 7) return launch_z_sys_pb<LOGN, 4, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-        return launch_z_sys_pb<LOGN, 2, C, R>(st, buf, spec, tw, nz_phys, ncol, plane, bnn, k0);
-    }
-}
-
-static int fft_kernel_choice()
-{
-    static int k = -1;
-    if (k < 0) {
-        const char* e = getenv("SIE_FFT_KERNEL");
-        k = (e && e[0] == 'r') ? 1 : 0;  // 0: Stockham radix-8 (default), 1: shared-memory radix-2
-    }
-    return k;
-}
-
-template <int LOGN, class C>
-static sie_status launch_pass_n(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, int nbatch)
-{
-    C* tw = nullptr;
-    SIE_TRY(twiddles(LOGN, st, &tw));
-    if (fft_kernel_choice() == 0) {
-        // 256 threads per CTA (n/8 per pencil); halve the pencils per CTA when
-        // that leaves fewer than ~4 CTAs per SM
-        constexpr int PB = 2048 >> LOGN;
-        constexpr int PBh = PB >= 2 ? PB / 2 : 1;
-        int pb = pick_pb(1 << LOGN, G.npencil * nbatch);
-        if (pb >= 16 || G.npencil * nbatch / PB >= 4LL * 152)
-            return launch_stockham<LOGN, PB, C>(st, in, out, inv, G, tw, nbatch);
-        return launch_stockham<LOGN, PBh, C>(st, in, out, inv, G, tw, nbatch);
-    }
-    switch (pick_pb(1 << LOGN, G.npencil * nbatch)) {
-        case 16:
-            if constexpr (LOGN < 9) return launch_pass_pb<LOGN, 16, C>(st, in, out, inv, G, tw, nbatch);
-            [[fallthrough]];
-        case 8: return launch_pass_pb<LOGN, 8, C>(st, in, out, inv, G, tw, nbatch);
-        default: return launch_pass_pb<LOGN, 4, C>(st, in, out, inv, G, tw, nbatch);
-    }
-}
-
-template <class C>
-static sie_status launch_pass(cudaStream_t st, int n, const C* in, C* out, int inv, const PassGeom& G, int nb = 1)
-{
-    switch (n) {
-        case 16: return launch_pass_n<4>(st, in, out, inv, G, nb);
-        case 32: return launch_pass_n<5>(st, in, out, inv, G, nb);
-        case 64: return launch_pass_n<6>(st, in, out, inv, G, nb);
-        case 128: return launch_pass_n<7>(st, in, out, inv, G, nb);
-        case 256: return launch_pass_n<8>(st, in, out, inv, G, nb);
-        case 512: return launch_pass_n<9>(st, in, out, inv, G, nb);
-        case 1024: return launch_pass_n<10>(st, in, out, inv, G, nb);
-    }
-    set_error("unsupported FFT length");
-    return SIE_ERR_UNSUPPORTED;
-}
-
-// dir = -1: forward transform of the compact N grid `src` (or, prune = 0, of the
-// full n grid already in buf) into the full spectrum in buf.
-// dir = +1: inverse of the spectrum in buf; prune = 1 writes only the physical
-// N box into the compact array `src` (used as output), prune = 0 keeps n^3 in buf.
-// nbatch grids at once: grid k at buf + k n^3 and (compact) src + k N^3
-template <class C>
-static sie_status fft3d_t(cudaStream_t st, C* buf, const C* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
-                          int nbatch)
-{
-    const int64_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int64_t Nx = prune ? g.N[0] : nx, Ny = prune ? g.N[1] : ny, Nz = prune ? g.N[2] : nz;
-    const int64_t pyz = nx * ny;  // padded plane
-    const int64_t bnn = nx * ny * nz, bNg = (int64_t)g.N[0] * g.N[1] * g.N[2];
-    if (dir < 0) {
-        // x pass: pencils (y < Ny, z < Nz)
-        PassGeom X{(int)Nx, (int)nx, Ny * Nz, (int)Ny, prune ? Nx : nx, prune ? Nx * Ny : pyz, 1, nx, pyz, 1, 1,
-                   prune ? bNg : bnn, bnn};
-        {
-            Stage s_(pc, "fft_fwd_x");
-            SIE_TRY(launch_pass(st, (int)nx, prune ? src : buf, buf, 0, X, nbatch));
-        }
-        // y pass: pencils (x < nx, z < Nz)
-        PassGeom Y{(int)Ny, (int)ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
-        {
-            Stage s_(pc, "fft_fwd_y");
-            SIE_TRY(launch_pass(st, (int)ny, buf, buf, 0, Y, nbatch));
-        }
-        // z pass: pencils (x < nx, y < ny)
-        PassGeom Z{(int)Nz, (int)nz, nx * ny, (int)nx, 1, nx, pyz, 1, nx, pyz, 0, bnn, bnn};
-        {
-            Stage s_(pc, "fft_fwd_z");
-            SIE_TRY(launch_pass(st, (int)nz, buf, buf, 0, Z, nbatch));
-        }
-    } else {
-        PassGeom Z{(int)nz, (int)Nz, nx * ny, (int)nx, 1, nx, pyz, 1, nx, pyz, 0, bnn, bnn};
-        {
-            Stage s_(pc, "fft_inv_z");
-            SIE_TRY(launch_pass(st, (int)nz, buf, buf, 1, Z, nbatch));
-        }
-        PassGeom Y{(int)ny, (int)Ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
-        {
-            Stage s_(pc, "fft_inv_y");
-            SIE_TRY(launch_pass(st, (int)ny, buf, buf, 1, Y, nbatch));
-        }
-        C* dst = prune ? const_cast<C*>(src) : buf;
-        PassGeom X{(int)nx, (int)Nx, Ny * Nz, (int)Ny, nx, pyz, 1, prune ? Nx : nx, prune ? Nx * Ny : pyz, 1, 1,
-                   bnn, prune ? bNg : bnn};
-        {
-            Stage s_(pc, "fft_inv_x");
-            SIE_TRY(launch_pass(st, (int)nx, buf, dst, 1, X, nbatch));
-        }
-    }
-    return SIE_OK;
-}
-
-sie_status fft3d(cudaStream_t st, double2* buf, const double2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
-                 int nbatch)
-{
-    return fft3d_t(st, buf, src, g, dir, prune, pc, nbatch);
-}
-
-sie_status fft3d(cudaStream_t st, float2* buf, const float2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
-                 int nbatch)
-{
-    return fft3d_t(st, buf, src, g, dir, prune, pc, nbatch);
-}
-
-// Grid part of the system product (Eq. sys) with the fused z stage: forward x
-// and y passes of the seven compact source grids in src (into buf), the fused
-// forward-z / spectral-product / inverse-z kernel, then the inverse y and x
-// passes of the four result grids back into the compact src.  Same arithmetic
-// as fft3d(-1) + k_specmul_sys + fft3d(+1), in another order of memory passes.
-template <class C, class R>
-static sie_status fft_sys_t(cudaStream_t st, C* buf, C* src, const GridDesc& g, const C* spec, R k0, sie_ctx* pc)
-{
-    const int64_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int64_t Nx = g.N[0], Ny = g.N[1], Nz = g.N[2];
-    const int64_t pyz = nx * ny, bnn = nx * ny * nz, bNg = Nx * Ny * Nz;
-    PassGeom X{(int)Nx, (int)nx, Ny * Nz, (int)Ny, Nx, Nx * Ny, 1, nx, pyz, 1, 1, bNg, bnn};
-    {
-        Stage s_(pc, "fft_fwd_x");
-        SIE_TRY(launch_pass(st, (int)nx, src, buf, 0, X, 7));
-    }
-    PassGeom Y{(int)Ny, (int)ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
-    {
-        Stage s_(pc, "fft_fwd_y");
-        SIE_TRY(launch_pass(st, (int)ny, buf, buf, 0, Y, 7));
-    }
-    {
-        Stage s_(pc, "fft_z_specmul");
-        sie_status s;
-        switch (nz) {
-            case 16: s = launch_z_sys<4>(st, buf, spec, (int)Nz, pyz, pyz, bnn, k0); break;
-            case 32: s = launch_z_sys<5>(st, buf, spec, (int)Nz, pyz, pyz, bnn, k0); break;
-            case 64: s = launch_z_sys<6>(st, buf, spec, (int)Nz, pyz, pyz, bnn, k0); break;
-            case 128: s = launch_z_sys<7>(st, buf, spec, (int)Nz, pyz, pyz, bnn, k0); break;
-            case 256: s = launch_z_sys<8>(st, buf, spec, (int)Nz, pyz, pyz, bnn, k0); break;
-            default:
-                set_error("fused z stage: unsupported FFT length");
-                return SIE_ERR_UNSUPPORTED;
-        }
-        SIE_TRY(s);
-    }
-    PassGeom Yi{(int)ny, (int)Ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
-    {
-        Stage s_(pc, "fft_inv_y");
-        SIE_TRY(launch_pass(st, (int)ny, buf, buf, 1, Yi, 4));
-    }
-    PassGeom Xi{(int)nx, (int)Nx, Ny * Nz, (int)Ny, nx, pyz, 1, Nx, Nx * Ny, 1, 1, bnn, bNg};
-    {
-        Stage s_(pc, "fft_inv_x");
-        SIE_TRY(launch_pass(st, (int)nx, buf, src, 1, Xi, 4));
-    }
-    return SIE_OK;
-}
-
-bool fft_sys_supported(const GridDesc& g) { return g.n[2] >= 16 && g.n[2] <= 256; }
-
-sie_status fft_sys(cudaStream_t st, double2* buf, double2* src, const GridDesc& g, const double2* spec, double k0,
-                   sie_ctx* pc)
-{
-    return fft_sys_t(st, buf, src, g, spec, k0, pc);
-}
-
-sie_status fft_sys(cudaStream_t st, float2* buf, float2* src, const GridDesc& g, const float2* spec, float k0,
-                   sie_ctx* pc)
-{
-    return fft_sys_t(st, buf, src, g, spec, k0, pc);
 }
 
 // ------------------------------------------------------------------ kernel spectra
@@ -1225,13 +401,17 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
             k_project<<<(M.nt * S + 255) / 256, 256, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, x, g, ngrid, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
-        SIE_TRY(fft3d(st, buf, src, g, -1, 1, pc, ngrid));
-        {
-            Stage s_(pc, "specmul");
-            k_specmul<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(which_LK, a.spec, buf, nn);
-            SIE_CUDA_TRY(cudaGetLastError());
+        if (fft_fused_z(g)) {
+            SIE_TRY(fft_lk(st, which_LK, buf, src, g, a.spec, pc, 1));
+        } else {
+            SIE_TRY(fft3d(st, buf, src, g, -1, 1, pc, ngrid));
+            {
+                Stage s_(pc, "specmul");
+                k_specmul<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(which_LK, a.spec, buf, nn);
+                SIE_CUDA_TRY(cudaGetLastError());
+            }
+            SIE_TRY(fft3d(st, buf, src, g, +1, 1, pc, ngrid));
         }
-        SIE_TRY(fft3d(st, buf, src, g, +1, 1, pc, ngrid));
         std::complex<double> kk(a.kr, a.ki);
         std::complex<double> sc = -1.0 / (kk * kk);
         {

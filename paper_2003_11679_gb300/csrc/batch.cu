@@ -259,13 +259,17 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
                                                                            ngrid, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
-        SIE_TRY(fft3d(st, buf, src, g, -1, 1, pc, ngrid * nr));
-        {
-            Stage s_(pc, "specmul_block");
-            k_specmul_b<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(which_LK, nr, a.spec, buf, nn);
-            SIE_CUDA_TRY(cudaGetLastError());
+        if (fft_fused_z(g)) {
+            SIE_TRY(fft_lk(st, which_LK, buf, src, g, a.spec, pc, nr));
+        } else {
+            SIE_TRY(fft3d(st, buf, src, g, -1, 1, pc, ngrid * nr));
+            {
+                Stage s_(pc, "specmul_block");
+                k_specmul_b<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(which_LK, nr, a.spec, buf, nn);
+                SIE_CUDA_TRY(cudaGetLastError());
+            }
+            SIE_TRY(fft3d(st, buf, src, g, +1, 1, pc, ngrid * nr));
         }
-        SIE_TRY(fft3d(st, buf, src, g, +1, 1, pc, ngrid * nr));
         std::complex<double> kk(a.kr, a.ki);
         std::complex<double> sc = which_LK == 0 ? -1.0 / (kk * kk) : std::complex<double>(0.0);
         {

@@ -377,10 +377,12 @@ sie_status constraint_lu_build(sie_op* op);
 void constraint_lu_release(sie_op* op);
 // SIE_ERR_TIMEOUT when a triangular-solve wait of a constraint LU ran out (synchronises)
 sie_status constraint_lu_check(sie_op* op);
-// grid part of the system product: forward x, y; fused forward z + spectral
-// products + inverse z; inverse y, x (seven source grids in the compact src,
-// four result grids back into it)
-bool fft_sys_supported(const GridDesc& g);  // z length 16 .. 256
+// grid products: forward x, y; fused forward z + spectral products + inverse z;
+// inverse y, x (source grids in the compact src, result grids back into it):
+// the system product (7 grids -> 4), and nb products L (4 -> 4) or K (3 -> 3)
+bool fft_fused_z(const GridDesc& g);  // z length up to 256
+sie_status fft_lk(cudaStream_t st, int which_LK, double2* buf, double2* src, const GridDesc& g, const double2* spec,
+                  sie_ctx* pc, int nb);
 sie_status fft_sys(cudaStream_t st, double2* buf, double2* src, const GridDesc& g, const double2* spec, double k0,
                    sie_ctx* pc);
 sie_status fft_sys(cudaStream_t st, float2* buf, float2* src, const GridDesc& g, const float2* spec, float k0,

@@ -1406,7 +1406,7 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
                 op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W32, tc, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
-        if (fused_z() && fft_sys_supported(g)) {
+        if (fused_z() && fft_fused_z(g)) {
             SIE_TRY(fft_sys(st, buf, src, g, X.spec32, (float)op->k0, c));
         } else {
             SIE_TRY(fft3d(st, buf, src, g, -1, 1, c, 7));
@@ -1434,7 +1434,7 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
                 op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W, op->pm_tc, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
-        if (fused_z() && fft_sys_supported(g)) {
+        if (fused_z() && fft_fused_z(g)) {
             SIE_TRY(fft_sys(st, buf, src, g, X.spec, op->k0, c));
         } else {
             SIE_TRY(fft3d(st, buf, src, g, -1, 1, c, 7));
