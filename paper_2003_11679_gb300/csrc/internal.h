@@ -234,8 +234,6 @@ struct KrylovWork {
     int m = 0;
     double2 *V = nullptr, *Z = nullptr, *w = nullptr, *h = nullptr, *r = nullptr, *part = nullptr;
     double2* cgsp = nullptr;        // per-chunk partial sums of the fused Gram-Schmidt passes
-    double2* dv = nullptr;          // device-controlled cycle: v_j and z_j (2 n)
-    int* dj = nullptr;              // device-controlled cycle: iteration index, iterations done
     double2* Hd = nullptr;          // Hessenberg, rotations, g, y (device)
     double* sc = nullptr;           // |b|, beta, per-iteration relative residuals (device)
     double* resid_h = nullptr;      // pinned copies of the residuals
@@ -243,9 +241,9 @@ struct KrylovWork {
     sie_status alloc(cudaStream_t st, int64_t n_, int m_);
     void release(cudaStream_t st);
 };
-// Krylov workspace of a panel solve: R right-hand sides whose vectors sit side
-// by side (basis V[j][q][n], Z[j][q][n]); one launch per Gram-Schmidt step
-// serves all of them (gridDim.y = R)
+// Krylov workspace of R right-hand sides, each with its own basis (V: R of m + 1
+// vectors, Z: R of m; the cooperative grid form keeps them V[j][q][n]); one launch
+// per Gram-Schmidt step serves all of them (gridDim.y = R)
 struct PanelWork {
     int64_t n = 0;
     int m = 0, R = 0;
@@ -284,12 +282,13 @@ struct sie_op {
     float4* pk_he = nullptr;        // mixed near product: complex64 (H, E) side by side (ne)
     float2* pk_sig = nullptr;       // mixed near product: complex64 triangle charges (nt)
     sie::KrylovWork kin, kout, kcs_in, kcs_out;
-    sie::KrylovWork kmulti[8];      // lockstep solves: one Krylov basis per right-hand side
-    sie::KrylovWork kcs_multi[8];   // ... and per triangle system of their constraint preconditioner
+    sie::PanelWork kmulti;          // lockstep solves: one Krylov basis per right-hand side
+    sie::PanelWork kcs_multi;       // ... and per triangle system of their constraint preconditioner
     sie::PanelWork kzp;             // lockstep block products: the nested interior solves of the block
     double2* zp = nullptr;          // block products: H, E, rhs and scratch panels (4 x 8 ne)
     double2* mscr = nullptr;        // lockstep solves: per right-hand side scratch (8 blocks)
     double2* ir_multi = nullptr;    // lockstep refinement: residuals, corrections, products (3 x 8 (ne + nt))
+    double2* con_scr = nullptr;     // their constraint preconditioner in one kernel: 8 (ne + 2 nt)
     double2* mvec = nullptr;        // lockstep solves from host buffers: 2 x 8 (ne + nt)
     double2 *cs_e = nullptr, *cs_t = nullptr, *pc_e = nullptr, *pc_t = nullptr;  // preconditioner scratch
     // last solve: outer iters, relres; max nested iters, relres; max constraint iters, relres
@@ -301,7 +300,10 @@ struct sie_op {
     bool capturing = false;         // apply_Z emits the device-controlled nested solve
     cudaStream_t gs[2] = {nullptr, nullptr};  // capture streams: graph, while-loop body
     double2* g_io = nullptr;        // graph input x and output y, 2 (ne + nt)
-    double* gstat = nullptr;        // device: max nested iterations and residual of graph runs
+    // device (6): largest nested iteration count and residual since cleared, those of the
+    // the last nested solve (residual, count)
+    double* gstat = nullptr;
+    unsigned* res_bar = nullptr;    // resident kernels: barrier counter, error flag, lockstep flags (RES_WORDS)
     size_t gnodes[2] = {0, 0};      // nodes of the last captured graph: outside the loop, loop body
     double2* ir_buf = nullptr;      // iterative refinement: residual, correction, product (3 (ne + nt))
     double q_w = 0.0;               // charge-row weight of the GMRES residual norm (0: not yet computed)
@@ -330,6 +332,23 @@ struct sie_op {
 
 // ------------------------------------------------------------------ launchers (aim.cu, near.cu)
 namespace sie {
+// Krylov workspace of a grid-resident solve (resident.cuh) of R vectors
+struct ResWork {
+    int m = 0;
+    double2 *V = nullptr, *Z = nullptr, *W = nullptr, *H = nullptr, *part = nullptr;
+    int64_t ldh = 0;
+};
+// constraint preconditioner (ext: the exterior AEFIE form) of R vectors in one
+// cluster kernel (constraint.cu); v1, b, q: scratch of R ne, R nt, R nt.  false: not
+// taken (no dense inverse, too many triangles); *st_out: launch status
+bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, int R, const double2* const* x,
+                         double2* const* y, double tol, int maxit, int restart, const ResWork& w, double2* v1, double2* b,
+                         double2* q, sie_status* st_out);
+// E_q = f (or per edge) A^-1 b(H_q), q < R <= 8: nested interior solves of
+// near-region-only and SIBC operators (nested.cu); extra: iterations run past
+// the tolerance; statistics in op->gstat
+sie_status nested_solve(sie_op* op, int R, const double2* H, int64_t ldh, double2* E, int64_t lde, double2 f,
+                        int extra, const ResWork& w);
 sie_status dev_upload_mesh(sie_mesh* m);
 sie_status dev_free_mesh(sie_mesh* m);
 sie_status aim_weights(sie_op* op);

@@ -1,0 +1,591 @@
+// Resident FGMRES: one kernel runs a whole Krylov cycle.  The small systems
+// solved inside every system product and preconditioner (interior impedance,
+// charge system) need a few microseconds of arithmetic per iteration; as a graph
+// loop of nine kernels an iteration took 45 to 50 us.  Two forms:
+//
+//  * clu_fgmres (up to CLU_MAXN rows): a thread-block cluster of 8 or 16 CTAs per
+//    right-hand side.  The vector that the next product gathers from sits whole
+//    in every CTA's shared memory, written by its owners through distributed
+//    shared memory; so are the CTAs' partial sums.  An iteration meets at 3 or 4
+//    hardware cluster barriers (0.2 to 0.3 us) and reads no other memory than the
+//    matrix rows (L1) and own rows of the basis;
+//  * res_fgmres (more rows): a cooperative grid of up to one CTA per SM with
+//    barriers in global memory (about 1.5 us); what other CTAs wrote is read past
+//    L1 (ld.cg).  On 8 CTAs a copper bar's 504-row solve took 186 us this way.
+//
+// CTA c owns the rows [r0, r1) of every vector.  Every CTA sums the partial sums
+// in the same fixed order and repeats the Givens rotations, so all take the same
+// decisions and a run's rounding does not depend on timing.  Classical
+// Gram-Schmidt twice; the second pass's norm is |w|^2 - |h2|^2 (h2 is at rounding
+// level, so nothing cancels), which saves a reduction.
+//
+// Waits in global memory are bounded: a CTA that gives up sets *err and returns,
+// the others run out at their next wait, and the host reports SIE_ERR_TIMEOUT.
+// Launches whose CTAs wait on one another that way are cooperative.
+#pragma once
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "internal.h"
+
+namespace sie {
+
+constexpr int RES_T = 512;              // threads per CTA
+constexpr int RES_MAXCTA = 160;         // partial-sum slots
+constexpr int RES_WORDS = 2 + 8 * 16;   // counter, error flag, ring of lockstep flags
+constexpr int RES_SPIN = 1 << 20;       // polls of a barrier before it gives up (under a second)
+
+__device__ __forceinline__ double2 r_cm(double2 a, double2 b)
+{
+    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 r_cj(double2 a) { return make_double2(a.x, -a.y); }
+// c + a b
+__device__ __forceinline__ void r_fma(double2& c, double2 a, double2 b)
+{
+    c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
+    c.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
+}
+
+struct ResBar {
+    unsigned* cnt;   // zero at the launch
+    int* err;
+    unsigned target;
+};
+// false: the wait ran out
+__device__ __forceinline__ bool res_barrier(ResBar& b)
+{
+    __shared__ int bad;
+    b.target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.cnt) : "memory");
+        unsigned v = 0;
+        int it = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(b.cnt) : "memory");
+            if (++it > RES_SPIN) ok = 0;
+        } while (ok && v < b.target);
+        if (!ok) atomicExch(b.err, 1);
+        bad = !ok;
+    }
+    __syncthreads();
+    return !bad;
+}
+
+// Krylov arrays: vector q of step j at V + (j R + q) n; part: per-CTA sums
+struct ResKrylov {
+    int64_t n;
+    int m, R;           // largest cycle length, right-hand sides
+    double2 *V, *Z, *W; // (m + 1) R n, m R n, R n
+    double2* H;         // rotated Hessenberg columns: per right-hand side (m + 1) m
+    int64_t ldh;        // stride of H between right-hand sides
+    double2* part;      // RES_MAXCTA R 2 (m + 2)
+    double tol;
+    int extra;          // iterations run after every residual is below tol (host-checked cycles ran one)
+    double* stat;       // 0, 1: largest iteration count and residual so far; 2, 3: this run's residual and count
+};
+
+// dynamic shared memory of res_fgmres
+inline size_t res_smem(int m, int R) { return sizeof(double2) * (size_t)R * 5 * (m + 2); }
+
+__device__ __forceinline__ double2 warp_sum(double2 s)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    return s;
+}
+
+// part[(c R + q) ld + i] = sum over own rows of conj(V_i) w, i < nv, and of |w|^2 (slot nv) when norm
+__device__ __forceinline__ void res_dots(const ResKrylov& K, int64_t r0, int64_t r1, int nv, bool norm, double2* part,
+                                         int ld)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int cols = nv + (norm ? 1 : 0);
+    for (int t = warp; t < K.R * cols; t += nw) {
+        const int q = t / cols, i = t % cols;
+        const double2* w = K.W + q * K.n;
+        const double2* v = i < nv ? K.V + ((int64_t)i * K.R + q) * K.n : w;
+        double2 s = make_double2(0, 0);
+        for (int64_t k = r0 + lane; k < r1; k += 32) r_fma(s, r_cj(v[k]), w[k]);
+        s = warp_sum(s);
+        if (lane == 0) part[((int64_t)blockIdx.x * K.R + q) * ld + i] = s;
+    }
+}
+
+// h[q ldh + i] = sum over the CTAs of part (in CTA order per lane, then a fixed tree)
+__device__ __forceinline__ void res_reduce(const ResKrylov& K, int cols, const double2* part, int ld, double2* h, int ldh)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int t = warp; t < K.R * cols; t += nw) {
+        const int q = t / cols, i = t % cols;
+        double2 s = make_double2(0, 0);
+        for (int c = lane; c < (int)gridDim.x; c += 32) {
+            const double2 p = __ldcg(part + ((int64_t)c * K.R + q) * ld + i);
+            s.x += p.x;
+            s.y += p.y;
+        }
+        s = warp_sum(s);
+        if (lane == 0) h[q * ldh + i] = s;
+    }
+    __syncthreads();
+}
+
+// w -= sum_i V_i h_i on own rows
+__device__ __forceinline__ void res_update(const ResKrylov& K, int64_t r0, int64_t r1, int nv, const double2* h, int ldh)
+{
+    const int rows = (int)(r1 - r0);
+    for (int t = threadIdx.x; t < K.R * rows; t += blockDim.x) {
+        const int q = t / rows;
+        const int64_t k = r0 + t % rows;
+        double2 s = make_double2(0, 0);
+        const double2* v = K.V + (int64_t)q * K.n + k;
+        for (int i = 0; i < nv; i++) r_fma(s, v[(int64_t)i * K.R * K.n], h[q * ldh + i]);
+        double2* w = K.W + q * K.n + k;
+        *w = make_double2(w->x - s.x, w->y - s.y);
+    }
+    __syncthreads();
+}
+
+// column j of one right-hand side (one thread): h1 + h2 and the norm hn through
+// the previous rotations, rotation j (c real), g; the rotated column to Hq when
+// store; returns |g_{j+1}|
+__device__ __forceinline__ double res_givens(int j, int m, const double2* a1, const double2* a2, double hn, double2* c_,
+                                             double2* s_, double2* g_, double2* Hq, bool store)
+{
+    double2 a = make_double2(a1[0].x + a2[0].x, a1[0].y + a2[0].y);
+    for (int i = 0; i < j; i++) {
+        const double2 b = make_double2(a1[i + 1].x + a2[i + 1].x, a1[i + 1].y + a2[i + 1].y);
+        const double2 sb = r_cm(s_[i], b), ta = r_cm(r_cj(s_[i]), a);
+        if (store) Hq[i * m + j] = make_double2(c_[i].x * a.x + sb.x, c_[i].x * a.y + sb.y);
+        a = make_double2(c_[i].x * b.x - ta.x, c_[i].x * b.y - ta.y);
+    }
+    const double2 b = make_double2(hn, 0);
+    const double aa = hypot(a.x, a.y), den = hypot(aa, hn);
+    double2 c, s;
+    if (aa == 0.0) {
+        c = make_double2(0, 0);
+        s = make_double2(1, 0);
+    } else {
+        c = make_double2(aa / den, 0);
+        s = r_cm(make_double2(a.x / aa, a.y / aa), r_cj(b));
+        s.x /= den;
+        s.y /= den;
+    }
+    c_[j] = c;
+    s_[j] = s;
+    const double2 sb = r_cm(s, b);
+    if (store) Hq[j * m + j] = make_double2(c.x * a.x + sb.x, c.x * a.y + sb.y);
+    const double2 gj = g_[j], t = r_cm(r_cj(s), gj);
+    g_[j] = make_double2(c.x * gj.x, c.x * gj.y);
+    g_[j + 1] = make_double2(-t.x, -t.y);
+    return hypot(t.x, t.y);
+}
+
+// y = R^-1 g in place of g, j + 1 unknowns, by one warp (Hq complete)
+__device__ __forceinline__ void res_backsub(int j, int m, const double2* Hq, double2* g_, int lane)
+{
+    for (int i = j; i >= 0; i--) {
+        const double2 d = __ldcg(Hq + i * m + i), s = g_[i];
+        const double den = d.x * d.x + d.y * d.y;
+        const double2 y = den > 0 ? make_double2((s.x * d.x + s.y * d.y) / den, (s.y * d.x - s.x * d.y) / den)
+                                  : make_double2(0, 0);
+        __syncwarp();
+        if (lane == 0) g_[i] = y;
+        for (int k = lane; k < i; k += 32) {
+            const double2 t = r_cm(__ldcg(Hq + k * m + i), y);
+            g_[k] = make_double2(g_[k].x - t.x, g_[k].y - t.y);
+        }
+        __syncwarp();
+    }
+}
+
+__device__ __forceinline__ void res_stat(double* stat, int iters, double worst)
+{
+    stat[0] = fmax(stat[0], (double)iters);
+    stat[1] = worst != worst ? worst : fmax(stat[1], worst);
+    stat[2] = worst;
+    stat[3] = iters;
+}
+
+// relative residual; a NaN norm gives NaN
+__device__ __forceinline__ double res_rel(double r, double bn) { return bn > 0 ? r / bn : (bn == bn ? 0.0 : bn); }
+
+// norm of w - V h2 from |w|^2 and h2
+__device__ __forceinline__ double res_norm(double ww, const double2* h2, int nv)
+{
+    double s = ww;
+    for (int i = 0; i < nv; i++) s -= h2[i].x * h2[i].x + h2[i].y * h2[i].y;
+    return s != s ? s : sqrt(fmax(s, 0.0));
+}
+
+// The FGMRES cycle (zero initial guess, at most K.m iterations) on the residual
+// panel already in K.W (own rows, after a __syncthreads).  sys: rows r0, r1 of
+// this CTA; precond(j, bar): Z_j = M V_j, with the barrier that ends it; apply(j):
+// W = A Z_j on own rows; after_v(j): own rows of V_j are set (for a pointwise
+// preconditioner).  After it, the solutions' combinations: x_q = sum_i Z_i y_i,
+// y in shared memory at y[q (m + 2) + i], i <= jend.  Returns jend, -1 when a wait
+// ran out.
+template <class SYS>
+__device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* smem, double2** y_out)
+{
+    const int m = K.m, R = K.R, ld = m + 2;
+    const int64_t n = K.n, r0 = sys.r0, r1 = sys.r1;
+    const int rows = (int)(r1 - r0);
+    double2* cs = smem;
+    double2* sn = cs + R * ld;
+    double2* g = sn + R * ld;
+    double2* h1 = g + R * ld;
+    double2* h2 = h1 + R * ld;
+    __shared__ double bnorm[8], rel[8], wn[8];
+    __shared__ double2 nr[8];
+    double2* P1 = K.part;
+    double2* P2 = P1 + (int64_t)RES_MAXCTA * R * ld;
+    res_dots(K, r0, r1, 0, true, P1, ld);
+    if (!res_barrier(bar)) return -1;
+    res_reduce(K, 1, P1, ld, nr, 1);
+    if (threadIdx.x < R) {
+        const double d2 = nr[threadIdx.x].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
+        bnorm[threadIdx.x] = b;
+        wn[threadIdx.x] = b > 0 ? 1.0 / b : 0.0;
+        g[threadIdx.x * ld] = make_double2(b, 0);
+    }
+    __syncthreads();
+    auto set_v = [&](int j) {
+        for (int t = threadIdx.x; t < R * rows; t += blockDim.x) {
+            const int q = t / rows;
+            const int64_t k = r0 + t % rows;
+            const double2 w = K.W[q * n + k];
+            K.V[((int64_t)j * R + q) * n + k] = make_double2(w.x * wn[q], w.y * wn[q]);
+        }
+        sys.after_v(j);
+    };
+    set_v(0);
+    if (!res_barrier(bar)) return -1;
+    int j = 0, extra = K.extra;
+    for (;; j++) {
+        if (!sys.precond(j, bar)) return -1;
+        sys.apply(j);
+        __syncthreads();
+        res_dots(K, r0, r1, j + 1, false, P1, ld);
+        if (!res_barrier(bar)) return -1;
+        res_reduce(K, j + 1, P1, ld, h1, ld);
+        res_update(K, r0, r1, j + 1, h1, ld);
+        res_dots(K, r0, r1, j + 1, true, P2, ld);
+        if (!res_barrier(bar)) return -1;
+        res_reduce(K, j + 2, P2, ld, h2, ld);
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
+            const double hn = res_norm(h2[q * ld + j + 1].x, h2 + q * ld, j + 1);
+            wn[q] = hn > 0 ? 1.0 / hn : 0.0;
+            rel[q] = res_rel(res_givens(j, m, h1 + q * ld, h2 + q * ld, hn, cs + q * ld, sn + q * ld, g + q * ld,
+                                        K.H + q * K.ldh, blockIdx.x == 0),
+                             bnorm[q]);
+        }
+        __syncthreads();
+        bool more = false;
+        for (int q = 0; q < R; q++) more = more || rel[q] >= K.tol;
+        if (!more && extra > 0) {
+            extra--;
+            more = true;
+        }
+        more = more && j + 1 < m;
+        if (!more) break;
+        res_update(K, r0, r1, j + 1, h2, ld);
+        set_v(j + 1);
+        if (!res_barrier(bar)) return -1;
+    }
+    // y = R^-1 g: a warp per right-hand side (CTA 0's H is complete after a barrier)
+    if (!res_barrier(bar)) return -1;
+    if ((threadIdx.x >> 5) < R)
+        res_backsub(j, m, K.H + (threadIdx.x >> 5) * K.ldh, g + (threadIdx.x >> 5) * ld, threadIdx.x & 31);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double worst = 0;
+        for (int q = 0; q < R; q++) worst = rel[q] != rel[q] ? rel[q] : (worst != worst ? worst : fmax(worst, rel[q]));
+        res_stat(K.stat, j + 1, worst);
+    }
+    __syncthreads();
+    *y_out = g;
+    return j;
+}
+
+// the same from several clusters: maxima of nonnegative doubles by their bits (a NaN's exceed all)
+__device__ __forceinline__ void res_stat_max(double* stat, int iters, double rel)
+{
+    unsigned long long* st = (unsigned long long*)stat;
+    atomicMax(st + 0, (unsigned long long)__double_as_longlong((double)iters));
+    atomicMax(st + 1, (unsigned long long)__double_as_longlong(rel) & 0x7fffffffffffffffull);
+}
+
+// ------------------------------------------------------------------ cluster form
+constexpr int CLU_MAXN = 2048;  // rows: two gather vectors take 64 KB of shared memory then
+constexpr int CLU_MAXC = 16;
+
+// one right-hand side per cluster; shared memory of a CTA:
+//   x[2][n] gather vectors (v, z), w[rows], pr[2][C][m + 2] partial sums, cs, sn, g, h1, h2 [m + 2]
+int clu_ctas(int64_t n);
+int res_group(int64_t rows, int64_t nrow, int64_t nnz);
+bool clu_fits(const void* fn, int C, int R, size_t smem);
+sie_status clu_launch(const void* fn, int C, int R, size_t smem, void** args, cudaStream_t st);
+inline size_t clu_smem(int64_t n, int m, int C)
+{
+    return sizeof(double2) * (size_t)(2 * n + (n + C - 1) / C + 2 * C * (m + 2) + 5 * (m + 2));
+}
+
+struct CluMem {
+    double2 *xv, *xz, *w, *pr, *cs, *sn, *g, *h1, *h2;
+    int C, rank, ld;
+    __device__ CluMem(double2* s, int64_t n, int m)
+    {
+        auto c = cooperative_groups::this_cluster();
+        C = (int)c.num_blocks();
+        rank = (int)c.block_rank();
+        ld = m + 2;
+        xv = s;
+        xz = xv + n;
+        w = xz + n;
+        pr = w + (n + C - 1) / C;
+        cs = pr + 2 * C * ld;
+        sn = cs + ld;
+        g = sn + ld;
+        h1 = g + ld;
+        h2 = h1 + ld;
+    }
+    // *p in every CTA's shared memory (p: this CTA's address)
+    __device__ __forceinline__ void put(double2* p, double2 v) const
+    {
+        auto c = cooperative_groups::this_cluster();
+        for (int r = 0; r < C; r++) *c.map_shared_rank(p, r) = v;
+    }
+};
+
+__device__ __forceinline__ void clu_sync() { cooperative_groups::this_cluster().sync(); }
+
+// partial sums of conj(V_i) w, i < nv, and of |w|^2 (slot nv) when norm, to every CTA's pr[buf][rank]
+__device__ __forceinline__ void clu_dots(const CluMem& M, const double2* V, int64_t n, int64_t r0, int rows, int nv,
+                                         bool norm, int buf)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int i = warp; i < nv + (norm ? 1 : 0); i += nw) {
+        const double2* v = i < nv ? V + (int64_t)i * n + r0 : M.w;
+        double2 s = make_double2(0, 0);
+        for (int k = lane; k < rows; k += 32) r_fma(s, r_cj(v[k]), M.w[k]);
+        s = warp_sum(s);
+        if (lane < M.C)
+            *cooperative_groups::this_cluster().map_shared_rank(M.pr + (buf * M.C + M.rank) * M.ld + i, lane) = s;
+    }
+}
+// h[i] = sum over the CTAs
+__device__ __forceinline__ void clu_reduce(const CluMem& M, int cols, int buf, double2* h)
+{
+    for (int i = threadIdx.x; i < cols; i += blockDim.x) {
+        double2 s = make_double2(0, 0);
+        for (int c = 0; c < M.C; c++) {
+            const double2 p = M.pr[(buf * M.C + c) * M.ld + i];
+            s.x += p.x;
+            s.y += p.y;
+        }
+        h[i] = s;
+    }
+    __syncthreads();
+}
+
+// coupling of the clusters of a lockstep block: a cluster goes on while any
+// right-hand side was above tol lag iterations ago (lag 1: the flags it reads
+// were written an iteration ago, nothing waits).  flag: a ring of CLU_RING
+// iterations x 8 right-hand sides, zero at the launch, holding 2 (iteration + 1) +
+// (above tol); the clusters are never two iterations apart.
+constexpr int CLU_RING = 16;
+struct CluLock {
+    int R = 1, lag = 1;
+    unsigned* flag = nullptr;
+    int* err = nullptr;
+};
+// publish iteration it of right-hand side q (one CTA of its cluster); then 1: go on, 0: all below, -1: a wait ran out
+__device__ __forceinline__ int clu_vote(const CluLock& lock, int q, int it, bool above, bool publish)
+{
+    if (publish)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(lock.flag + (it % CLU_RING) * 8 + q),
+                     "r"(2u * (unsigned)(it + 1) + (above ? 1u : 0u))
+                     : "memory");
+    const int at = it - lock.lag;
+    if (at < 0) return 1;
+    int more = 0;
+    for (int p = 0; p < lock.R; p++) {
+        unsigned v = 0;
+        int n = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                         : "=r"(v)
+                         : "l"(lock.flag + (at % CLU_RING) * 8 + p)
+                         : "memory");
+        } while ((int)(v >> 1) < at + 1 && ++n < RES_SPIN);
+        if ((int)(v >> 1) < at + 1) {
+            atomicExch(lock.err, 1);
+            return -1;
+        }
+        if (v & 1) more = 1;
+    }
+    return more;
+}
+
+// The cycle for this cluster's right-hand side, whose residual is in M.w (own
+// rows, after a __syncthreads).  sys: r0, rows; precond(j): from M.xv, Z_j (own
+// rows) and M.xz of every CTA, false for a pointwise one done by set_v; set_v(j,
+// k, v): own row k of V_j is v (puts what the next product gathers); apply(j): M.w
+// = A z from M.xz.  After it y in M.g; returns jend, -1 when a wait ran out.
+// Restarted solves call it again with the new residual: it0 iterations done, at
+// most maxit in all, bnorm0 the norm of the right-hand side (below 0 in the first
+// cycle); *above: a residual is still above tol; rel_out: this one's.
+struct CluRun {
+    int it = 0, maxit = 1 << 30;
+    double bnorm = -1.0, rel = 0.0;
+    bool above = true;
+};
+template <class SYS>
+__device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const CluLock& lock, CluRun& run)
+{
+    const int m = K.m, rows = sys.rows;
+    const int64_t n = K.n, r0 = sys.r0;
+    double2* V = K.V + (int64_t)q * (m + 1) * n;  // this right-hand side's basis
+    double2* H = K.H + q * K.ldh;
+    __shared__ double bnorm, rel, wn;
+    __shared__ int go, above_s;
+    clu_sync();  // every CTA of the cluster has started, or is done with the last cycle
+    clu_dots(M, V, n, r0, rows, 0, true, 0);
+    clu_sync();
+    clu_reduce(M, 1, 0, M.h1);
+    if (threadIdx.x == 0) {
+        const double d2 = M.h1[0].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
+        bnorm = run.bnorm < 0 ? b : run.bnorm;
+        wn = b > 0 ? 1.0 / b : 0.0;
+        M.g[0] = make_double2(b, 0);
+    }
+    __syncthreads();
+    run.bnorm = bnorm;
+    auto set_v = [&](int j) {
+        for (int k = threadIdx.x; k < rows; k += blockDim.x) {
+            const double2 v = make_double2(M.w[k].x * wn, M.w[k].y * wn);
+            V[(int64_t)j * n + r0 + k] = v;
+            sys.set_v(j, k, v);
+        }
+        clu_sync();
+    };
+    set_v(0);
+    int j = 0, extra = K.extra;
+    for (;; j++) {
+        if (sys.precond(j)) clu_sync();
+        sys.apply(j);
+        __syncthreads();
+        clu_dots(M, V, n, r0, rows, j + 1, false, 0);
+        clu_sync();
+        clu_reduce(M, j + 1, 0, M.h1);
+        for (int k = threadIdx.x; k < rows; k += blockDim.x) {
+            double2 s = make_double2(0, 0);
+            for (int i = 0; i <= j; i++) r_fma(s, V[(int64_t)i * n + r0 + k], M.h1[i]);
+            M.w[k] = make_double2(M.w[k].x - s.x, M.w[k].y - s.y);
+        }
+        __syncthreads();
+        clu_dots(M, V, n, r0, rows, j + 1, true, 1);
+        clu_sync();
+        clu_reduce(M, j + 2, 1, M.h2);
+        if (threadIdx.x == 0) {
+            const double hn = res_norm(M.h2[j + 1].x, M.h2, j + 1);
+            wn = hn > 0 ? 1.0 / hn : 0.0;
+            rel = res_rel(res_givens(j, m, M.h1, M.h2, hn, M.cs, M.sn, M.g, H, M.rank == 0), bnorm);
+            int more = rel >= K.tol;
+            if (lock.R > 1) {
+                more = clu_vote(lock, q, run.it + j, rel >= K.tol, M.rank == 0);
+            } else if (!more && extra > 0) {
+                extra--;
+                more = 1;
+            }
+            above_s = more > 0;
+            go = more > 0 && j + 1 < m && run.it + j + 1 < run.maxit ? 1 : (more < 0 ? -1 : 0);
+        }
+        __syncthreads();
+        // the CTAs of a cluster read the same flags, but one of them may give up alone: agree first
+        int decide = go;
+        if (lock.R > 1) {
+            if (threadIdx.x < M.C)
+                *cooperative_groups::this_cluster().map_shared_rank(
+                    M.pr + M.rank * M.ld, threadIdx.x) = make_double2((double)go, 0);
+            clu_sync();
+            for (int c = 0; c < M.C; c++)
+                if (M.pr[c * M.ld].x < 0) decide = -1;
+        }
+        if (decide < 0) return -1;
+        if (!decide) break;
+        for (int k = threadIdx.x; k < rows; k += blockDim.x) {
+            double2 s = make_double2(0, 0);
+            for (int i = 0; i <= j; i++) r_fma(s, V[(int64_t)i * n + r0 + k], M.h2[i]);
+            M.w[k] = make_double2(M.w[k].x - s.x, M.w[k].y - s.y);
+        }
+        set_v(j + 1);
+    }
+    clu_sync();  // rank 0's H
+    if (threadIdx.x < 32) res_backsub(j, m, H, M.g, threadIdx.x);
+    run.rel = rel;
+    run.above = above_s != 0;
+    run.it += j + 1;
+    __syncthreads();
+    return j;
+}
+
+// sum over a CSR row of val x (x of R vectors ldx apart), by the G lanes of a
+// group: every lane ends with the sums.  CG: x was written by other CTAs of this
+// kernel.  All lanes of the warp call it (rows beyond the end with e0 = e1).
+template <int RM, bool CG>
+__device__ __forceinline__ void res_row(int64_t e0, int64_t e1, const int32_t* __restrict__ col,
+                                        const double2* __restrict__ val, const double2* x, int64_t ldx, int R, int l,
+                                        int G, double2* s)
+{
+#pragma unroll
+    for (int q = 0; q < RM; q++) s[q] = make_double2(0, 0);
+    int64_t e = e0 + l;
+    if constexpr (RM == 1) {
+        for (; e + 3 * G < e1; e += 4 * G) {  // four loads in flight
+            double2 v[4], xv[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int c = __ldg(col + e + u * G);
+                v[u] = __ldg(val + e + u * G);
+                xv[u] = CG ? __ldcg(x + c) : x[c];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) r_fma(s[0], v[u], xv[u]);
+        }
+    }
+    for (; e < e1; e += G) {
+        const int c = __ldg(col + e);
+        const double2 v = __ldg(val + e);
+#pragma unroll
+        for (int q = 0; q < RM; q++)
+            if (q < R) r_fma(s[q], v, CG ? __ldcg(x + q * ldx + c) : x[q * ldx + c]);
+    }
+#pragma unroll
+    for (int q = 0; q < RM; q++)
+        if (q < R)
+            for (int off = G >> 1; off > 0; off >>= 1) {
+                s[q].x += __shfl_xor_sync(0xffffffffu, s[q].x, off);
+                s[q].y += __shfl_xor_sync(0xffffffffu, s[q].y, off);
+            }
+}
+
+// for the rows [r0, r1) by groups of G lanes: body(row or -1, lane in group); all lanes of a warp run together
+template <class F>
+__device__ __forceinline__ void res_rows(int64_t r0, int64_t r1, int G, F body)
+{
+    const int per = blockDim.x / G, grp = threadIdx.x / G, l = threadIdx.x % G;
+    for (int64_t b = r0; b < r1; b += per) {
+        const int64_t k = b + grp;
+        body(k < r1 ? k : -1, l);
+    }
+}
+
+}  // namespace sie

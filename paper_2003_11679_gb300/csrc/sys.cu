@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "resident.cuh"
 #include "spmv.cuh"
 #include "sysmul.cuh"
 
@@ -66,7 +67,7 @@ __global__ void k_jacobi(int64_t n, const double2* __restrict__ x, const double2
 // order (deterministic, and spread over the whole GPU for long vectors)
 constexpr int MULTI_RHS = 8;    // right-hand sides per lockstep solve
 constexpr int DOT_CHUNKS = 64;
-constexpr int CGS_CHUNKS = 128;  // row chunks of the fused Gram-Schmidt kernels
+constexpr int CGS_CHUNKS = 128;  // row chunks of the fused Gram-Schmidt kernels (at most RES_MAXCTA)
 constexpr int CGS_TILE = 32;     // columns per shared-memory tile there
 __global__ void __launch_bounds__(256) k_dots_part(int64_t n, const double2* __restrict__ V, int64_t ld,
                                                    const double2* __restrict__ w, double2* __restrict__ part)
@@ -176,9 +177,7 @@ sie_status KrylovWork::alloc(cudaStream_t st, int64_t n_, int m_)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&r, sizeof(double2) * n, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&h, sizeof(double2) * 4 * (m + 2), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&part, sizeof(double2) * DOT_CHUNKS * (m + 1), st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&cgsp, sizeof(double2) * CGS_CHUNKS * (2 * (m + 1) + 1), st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&dv, sizeof(double2) * 2 * n, st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&dj, sizeof(int) * 4, st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&cgsp, sizeof(double2) * RES_MAXCTA * 2 * (m + 2), st));
     // Hessenberg (m+1) x m, rotations cs, sn, rhs g, solution y
     SIE_CUDA_TRY(cudaMallocAsync((void**)&Hd, sizeof(double2) * ((m + 1) * m + 2 * m + 2 * (m + 1)), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&sc, sizeof(double) * (8 + m + 1), st));
@@ -190,9 +189,7 @@ sie_status KrylovWork::alloc(cudaStream_t st, int64_t n_, int m_)
 
 void KrylovWork::release(cudaStream_t st)
 {
-    if (dj) cudaFreeAsync(dj, st);
-    dj = nullptr;
-    for (double2* p : {V, Z, w, h, r, part, cgsp, dv, Hd})
+    for (double2* p : {V, Z, w, h, r, part, cgsp, Hd})
         if (p) cudaFreeAsync(p, st);
     if (sc) cudaFreeAsync(sc, st);
     if (resid_h) {
@@ -201,7 +198,7 @@ void KrylovWork::release(cudaStream_t st)
     }
     for (auto& e : ev) cudaEventDestroy(e);
     ev.clear();
-    V = Z = w = h = r = part = cgsp = dv = Hd = nullptr;
+    V = Z = w = h = r = part = cgsp = Hd = nullptr;
     sc = nullptr;
     resid_h = nullptr;
     n = 0;
@@ -321,31 +318,24 @@ __device__ void cgs_partials(int64_t k0, int64_t k1, int nv, const double2* __re
 
 // Several right-hand sides in one launch (gridDim.y = R, panel Krylov solves):
 // the pointers of right-hand side q = blockIdx.y are offset by q times these
-// strides -- v: basis vectors and w (a panel of R vectors of n), p: partial
+// strides -- v: basis vectors, w: the vector being orthogonalised, p: partial
 // sums, h: the two Gram-Schmidt coefficient columns, d: Hessenberg, rotations
 // and g, s: scalars.  All zero for one right-hand side.
 struct PanelStrides {
-    int64_t v = 0, p = 0, h = 0, d = 0, s = 0;
+    int64_t v = 0, w = 0, p = 0, h = 0, d = 0, s = 0;
 };
 
-// pass 1: partial sums of V^H w.  With jd (device-controlled iteration, jd[0]
-// = j) nv = j + 1 is read on the device and zsrc is stored as column j of Z.
+// pass 1: partial sums of V^H w
 __global__ void __launch_bounds__(256) k_cgs_part(int64_t n, int nv, const double2* __restrict__ V, int64_t ld,
                                                   const double2* __restrict__ w, double2* __restrict__ P, int ldp,
-                                                  const int* __restrict__ jd, const double2* __restrict__ zsrc,
-                                                  double2* __restrict__ Z, PanelStrides ps = PanelStrides())
+                                                  PanelStrides ps = PanelStrides())
 {
     const int64_t q = blockIdx.y;
     V += q * ps.v;
-    w += q * ps.v;
+    w += q * ps.w;
     P += q * ps.p;
     int64_t k0, k1;
     cgs_rows(n, k0, k1);
-    if (jd) {
-        const int j = jd[0];
-        nv = j + 1;
-        for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) Z[(int64_t)j * ld + k] = zsrc[k];
-    }
     cgs_partials(k0, k1, nv, V, ld, w, P, ldp);
 }
 
@@ -355,7 +345,7 @@ __global__ void __launch_bounds__(256) k_cgs_update(int64_t n, int nv, const dou
                                                     const double2* __restrict__ Pin, int ldp,
                                                     double2* __restrict__ hout, double2* __restrict__ w,
                                                     double2* __restrict__ Pout, int last,
-                                                    const int* __restrict__ jd, PanelStrides ps = PanelStrides())
+                                                    PanelStrides ps = PanelStrides())
 {
     __shared__ double2 h[CGS_TILE];
     {
@@ -363,10 +353,9 @@ __global__ void __launch_bounds__(256) k_cgs_update(int64_t n, int nv, const dou
         V += q * ps.v;
         Pin += q * ps.p;
         hout += q * ps.h;
-        w += q * ps.v;
+        w += q * ps.w;
         Pout += q * ps.p;
     }
-    if (jd) nv = jd[0] + 1;
     int64_t k0, k1;
     cgs_rows(n, k0, k1);
     for (int i0 = 0; i0 < nv; i0 += CGS_TILE) {
@@ -410,22 +399,21 @@ __global__ void __launch_bounds__(256) k_cgs_update(int64_t n, int nv, const dou
 
 // |w| = sqrt(sum_c P[c]); V_{j+1} = w / |w| on this chunk's rows; block 0
 // writes column j of H (h1 + h2 and |w|) and applies the Givens step
-// (V: the basis, column stride ld (0: n); with jd, j = jd[0] is read on the
-// device; res, when given: the relative residual also to res[j gridDim.y + q])
+// (V: the basis, column stride ld (0: n); res, when given: the relative residual
+// also to res[j gridDim.y + q])
 __global__ void __launch_bounds__(256) k_cgs_finish(int64_t n, int j, int m, const double2* __restrict__ h1,
                                                     const double2* __restrict__ h2, const double2* __restrict__ P,
                                                     const double2* __restrict__ w, double2* __restrict__ V,
                                                     double2* __restrict__ H, double2* __restrict__ cs,
                                                     double2* __restrict__ sn, double2* __restrict__ g,
-                                                    double* __restrict__ sc, const int* __restrict__ jd,
-                                                    PanelStrides ps = PanelStrides(), int64_t ld = 0,
+                                                    double* __restrict__ sc, PanelStrides ps = PanelStrides(), int64_t ld = 0,
                                                     double* __restrict__ res = nullptr)
 {
     const int64_t q = blockIdx.y;
     h1 += q * ps.h;
     h2 += q * ps.h;
     P += q * ps.p;
-    w += q * ps.v;
+    w += q * ps.w;
     V += q * ps.v;
     H += q * ps.d;
     cs += q * ps.d;
@@ -433,7 +421,6 @@ __global__ void __launch_bounds__(256) k_cgs_finish(int64_t n, int j, int m, con
     g += q * ps.d;
     sc += q * ps.s;
     if (ld == 0) ld = n;
-    if (jd) j = jd[0];
     double2* Vn = V + (int64_t)(j + 1) * ld;
     __shared__ double hn_s;
     if (threadIdx.x < 32) {
@@ -456,72 +443,6 @@ __global__ void __launch_bounds__(256) k_cgs_finish(int64_t n, int j, int m, con
         gm_givens(j, m, H, cs, sn, g, sc);
         if (res) res[(int64_t)j * gridDim.y + q] = sc[3 + j];
     }
-}
-
-// ---- device-controlled cycle (the body of a CUDA-graph while loop).  jd[0]
-// is the iteration index j of the running cycle; jd[1] the iterations done.
-__global__ void k_gmd_init(int* __restrict__ jd)
-{
-    jd[0] = 0;
-    jd[1] = 0;
-}
-
-// vj = V[j]
-__global__ void k_gmd_fetch(int64_t n, const double2* __restrict__ V, const int* __restrict__ jd,
-                            double2* __restrict__ vj)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) vj[i] = V[(int64_t)jd[0] * n + i];
-}
-
-// after iteration j: continue while the relative residual sc[3 + j] is not
-// below tol and fewer than min(m, maxit) iterations ran (so the loop always ends)
-__global__ void k_gmd_cond(int* __restrict__ jd, const double* __restrict__ sc, double tol, int m, int maxit,
-                           cudaGraphConditionalHandle h)
-{
-    const int j = jd[0];
-    const bool more = sc[3 + j] >= tol && j + 1 < m && j + 1 < maxit;
-    jd[1] = j + 1;
-    if (more) jd[0] = j + 1;
-    cudaGraphSetConditional(h, more ? 1u : 0u);
-}
-
-// after the loop: jd[0] = last iteration jend; y = R^-1 g; out = (iterations, residual)
-__global__ void k_gmd_backsub(const int* __restrict__ jd, int m, const double2* __restrict__ H,
-                              const double2* __restrict__ g, double2* __restrict__ y, const double* __restrict__ sc,
-                              double* __restrict__ out)
-{
-    const int jend = jd[0];
-    for (int i = jend; i >= 0; i--) {
-        double2 s = g[i];
-        for (int k = i + 1; k <= jend; k++) {
-            double2 t = cm(H[i * m + k], y[k]);
-            s.x -= t.x;
-            s.y -= t.y;
-        }
-        double2 d = H[i * m + i];
-        double den = d.x * d.x + d.y * d.y;
-        y[i] = den > 0 ? make_double2((s.x * d.x + s.y * d.y) / den, (s.y * d.x - s.x * d.y) / den)
-                       : make_double2(0, 0);
-    }
-    out[0] = fmax(out[0], (double)jd[1]);
-    out[1] = fmax(out[1], sc[3 + jend]);
-}
-
-// x += Z[0..jend] y
-__global__ void k_gmd_update(int64_t n, const int* __restrict__ jd, const double2* __restrict__ Z,
-                             const double2* __restrict__ y, double2* __restrict__ x)
-{
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int nv = jd[0] + 1;
-    double sr = 0, si = 0;
-    for (int j = 0; j < nv; j++) {
-        double2 a = Z[(int64_t)j * n + k], b = y[j];
-        sr += a.x * b.x - a.y * b.y;
-        si += a.x * b.y + a.y * b.x;
-    }
-    x[k] = make_double2(x[k].x + sr, x[k].y + si);
 }
 
 // y = R^-1 g (upper triangular, size jend + 1)
@@ -586,10 +507,10 @@ static sie_status fgmres(sie_ctx* c, KrylovWork& K, int64_t n, const Apply& A, c
             double2* P1 = K.cgsp;
             double2* P2 = K.cgsp + (int64_t)CGS_CHUNKS * (m + 1);
             double2* P3 = K.cgsp + (int64_t)2 * CGS_CHUNKS * (m + 1);
-            k_cgs_part<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, K.w, P1, m + 1, nullptr, nullptr, nullptr);
-            k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, P1, m + 1, h1, K.w, P2, 0, nullptr);
-            k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, P2, m + 1, h2, K.w, P3, 1, nullptr);
-            k_cgs_finish<<<CGS_CHUNKS, 256, 0, st>>>(n, j, m, h1, h2, P3, K.w, K.V, H, cs, sn, g, K.sc, nullptr);
+            k_cgs_part<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, K.w, P1, m + 1);
+            k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, P1, m + 1, h1, K.w, P2, 0);
+            k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K.V, n, P2, m + 1, h2, K.w, P3, 1);
+            k_cgs_finish<<<CGS_CHUNKS, 256, 0, st>>>(n, j, m, h1, h2, P3, K.w, K.V, H, cs, sn, g, K.sc);
             SIE_CUDA_TRY(cudaGetLastError());
             SIE_CUDA_TRY(cudaMemcpyAsync(K.resid_h + j, K.sc + 3 + j, sizeof(double), cudaMemcpyDeviceToHost, st));
             SIE_CUDA_TRY(cudaEventRecord(K.ev[j], st));
@@ -634,96 +555,6 @@ static sie_status fgmres(sie_ctx* c, KrylovWork& K, int64_t n, const Apply& A, c
     if (iters_out) *iters_out = it;
     if (relres_out) *relres_out = rel;
     return rel < tol ? SIE_OK : SIE_ERR_NOT_CONVERGED;
-}
-
-// One FGMRES cycle (x0 = 0, at most min(m, maxit) iterations) emitted into the
-// stream c->stream while it is being captured into a CUDA graph: the
-// iterations form a conditional while node whose body ends with k_gmd_cond,
-// so the device decides when to stop and no host round trip is needed.  The
-// operators A and Minv are captured on the body stream body_st (c->stream is
-// switched to it while they run).  K must already be allocated for (n, m).
-// stat (device, 2 doubles) keeps the maximum iteration count and final
-// relative residual.  Same arithmetic as fgmres, without its lagged check.
-static sie_status fgmres_dev(sie_ctx* c, cudaStream_t body_st, KrylovWork& K, int64_t n, const Apply& A,
-                             const Apply& Minv, const double2* b, double2* x, double tol, int maxit, int m,
-                             double* stat, size_t* body_nodes)
-{
-    if (K.n != n || K.m != m) {
-        set_error("fgmres_dev: Krylov workspace not allocated");
-        return SIE_ERR_STATE;
-    }
-    cudaStream_t st = c->stream;
-    double2* H = K.Hd;
-    double2* cs = K.Hd + (m + 1) * m;
-    double2* sn = cs + m;
-    double2* g = sn + m;
-    double2* y = g + (m + 1);
-    double2* h1 = K.h;
-    double2* h2 = K.h + (m + 2);
-    double2* wd = K.h + 2 * (m + 2);
-    double2* vj = K.dv;
-    double2* zj = K.dv + n;
-    double2* P1 = K.cgsp;
-    double2* P2 = K.cgsp + (int64_t)CGS_CHUNKS * (m + 1);
-    double2* P3 = K.cgsp + (int64_t)2 * CGS_CHUNKS * (m + 1);
-    SIE_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double2) * n, st));
-    SIE_TRY(dots(st, n, 1, b, n, b, K.part, wd));
-    k_gm_start<<<nb(n), 256, 0, st>>>(n, b, wd, K.V, g, m, K.sc, 1);
-    k_gmd_init<<<1, 1, 0, st>>>(K.dj);
-    SIE_CUDA_TRY(cudaGetLastError());
-    // while node after the current capture frontier
-    cudaStreamCaptureStatus cst;
-    cudaGraph_t graph = nullptr;
-    const cudaGraphNode_t* deps = nullptr;
-    const cudaGraphEdgeData* edges = nullptr;
-    size_t ndeps = 0;
-    SIE_CUDA_TRY(cudaStreamGetCaptureInfo(st, &cst, nullptr, &graph, &deps, &edges, &ndeps));
-    if (cst != cudaStreamCaptureStatusActive) {
-        set_error("fgmres_dev: stream is not being captured");
-        return SIE_ERR_STATE;
-    }
-    cudaGraphConditionalHandle hc;
-    SIE_CUDA_TRY(cudaGraphConditionalHandleCreate(&hc, graph, 1, cudaGraphCondAssignDefault));
-    cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};  // the rest zero
-    cp.conditional.handle = hc;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t wnode;
-    SIE_CUDA_TRY(cudaGraphAddNode(&wnode, graph, deps, edges, ndeps, &cp));
-    SIE_CUDA_TRY(cudaStreamUpdateCaptureDependencies(st, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    // body: one Arnoldi step
-    SIE_CUDA_TRY(cudaStreamBeginCaptureToGraph(body_st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    c->stream = body_st;
-    sie_status s = SIE_OK;
-    do {
-        k_gmd_fetch<<<nb(n), 256, 0, body_st>>>(n, K.V, K.dj, vj);
-        if ((s = Minv(vj, zj)) != SIE_OK) break;
-        if ((s = A(zj, K.w)) != SIE_OK) break;
-        k_cgs_part<<<CGS_CHUNKS, 256, 0, body_st>>>(n, 0, K.V, n, K.w, P1, m + 1, K.dj, zj, K.Z);
-        k_cgs_update<<<CGS_CHUNKS, 256, 0, body_st>>>(n, 0, K.V, n, P1, m + 1, h1, K.w, P2, 0, K.dj);
-        k_cgs_update<<<CGS_CHUNKS, 256, 0, body_st>>>(n, 0, K.V, n, P2, m + 1, h2, K.w, P3, 1, K.dj);
-        k_cgs_finish<<<CGS_CHUNKS, 256, 0, body_st>>>(n, 0, m, h1, h2, P3, K.w, K.V, H, cs, sn, g, K.sc, K.dj);
-        k_gmd_cond<<<1, 1, 0, body_st>>>(K.dj, K.sc, tol, m, maxit, hc);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) {
-            set_error(std::string("fgmres_dev: ") + cudaGetErrorString(e));
-            s = SIE_ERR_CUDA;
-        }
-    } while (0);
-    c->stream = st;
-    cudaGraph_t tmp = nullptr;
-    cudaError_t e = cudaStreamEndCapture(body_st, &tmp);
-    if (s != SIE_OK) return s;
-    if (e != cudaSuccess) {
-        set_error(std::string("fgmres_dev: body capture: ") + cudaGetErrorString(e));
-        return SIE_ERR_CUDA;
-    }
-    if (body_nodes) SIE_CUDA_TRY(cudaGraphGetNodes(body, nullptr, body_nodes));
-    k_gmd_backsub<<<1, 1, 0, st>>>(K.dj, m, H, g, y, K.sc, stat);
-    k_gmd_update<<<nb(n), 256, 0, st>>>(n, K.dj, K.Z, y, x);
-    SIE_CUDA_TRY(cudaGetLastError());
-    return SIE_OK;
 }
 
 // ------------------------------------------------------------------ system kernels
@@ -1219,13 +1050,50 @@ static sie_status constraint_solve(sie_op* op, AimOp& a, cplx kappa, KrylovWork&
 constexpr int INNER_BASIS_MAX = 128;
 static int inner_m(const sie_op* op) { return std::max(1, std::min(op->p.inner_maxit, INNER_BASIS_MAX)); }
 
-// interior impedance E' = Z' H = -(j k0 eps_r + sigma eta0)^-1 L_i^-1 (K_i - Ix/2) H
-// nested_res (stream path): relative residual the nested solve ended with
-static sie_status apply_Z_sibc(sie_op* op, const double2* H, double2* E, double* nested_res);
+// E' = Z' H of a near-region-only or SIBC interior: one grid-resident kernel
+// (nested.cu).  Outside a capture the call waits for its result: a residual that
+// is not finite is an error, as in fgmres.  nested_res: the residual it ended with.
+static sie_status apply_Z_resident(sie_op* op, const double2* H, double2* E, double* nested_res)
+{
+    sie_ctx* c = op->mesh->ctx;
+    const int64_t ne = op->mesh->h.ne;
+    cplx f;
+    if (op->p.interior_model == SIE_SIBC) {
+        f = cplx(op->eta_re, op->eta_im);
+    } else {
+        f = -1.0 / cplx(op->sigma * ETA0, op->k0 * op->eps_r);
+    }
+    KrylovWork& K = op->kin;
+    SIE_TRY(K.alloc(c->stream, ne, inner_m(op)));
+    ResWork w;
+    w.m = K.m, w.V = K.V, w.Z = K.Z, w.W = K.w, w.H = K.Hd, w.part = K.cgsp;
+    {
+        Stage s_(c, "inner_solve");
+        // one iteration past the tolerance outside the graph, as fgmres with its lagged check
+        SIE_TRY(nested_solve(op, 1, H, ne, E, ne, make_double2(f.real(), f.imag()), op->capturing ? 0 : 1, w));
+    }
+    if (op->capturing) return SIE_OK;
+    SIE_CUDA_TRY(cudaMemcpyAsync(K.resid_h, op->gstat + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    SIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    const double rr = K.resid_h[0];
+    if (std::isinf(rr)) {
+        set_error("nested interior solve: a grid barrier's wait ran out");
+        return SIE_ERR_TIMEOUT;
+    }
+    if (!std::isfinite(rr)) {
+        set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
+        return SIE_ERR_ARG;
+    }
+    if (nested_res) *nested_res = rr;
+    return SIE_OK;
+}
 
+// interior impedance E' = Z' H = -(j k0 eps_r + sigma eta0)^-1 L_i^-1 (K_i - Ix/2) H,
+// or (eta_i / eta0) G^-1 Ix H (SIBC)
+// nested_res (not inside a capture): relative residual the nested solve ended with
 static sie_status apply_Z(sie_op* op, const double2* H, double2* E, double* nested_res)
 {
-    if (op->p.interior_model == SIE_SIBC) return apply_Z_sibc(op, H, E, nested_res);
+    if (!op->inn.has_grid) return apply_Z_resident(op, H, E, nested_res);
     sie_ctx* c = op->mesh->ctx;
     cudaStream_t st = c->stream;
     const int64_t ne = op->mesh->h.ne;
@@ -1236,92 +1104,27 @@ static sie_status apply_Z(sie_op* op, const double2* H, double2* E, double* nest
     auto A = [&](const double2* x, double2* y) { return aim_apply(op, I, 0, x, y); };
     cplx ki(I.kr, I.ki);
     // Nested preconditioner M_i of Eq. (nest2pc) in its near-region form: the
-    // constraint form (diag LA_i + near Lphi_i, block elimination) when the
-    // object has an interior grid, and when it is near-region only (skin depth
-    // below the near region, L_i = L_i,NR) a sparse approximate inverse of
-    // L_i,NR on its own pattern, applied as one CSR product
-    auto Mconstraint = [&](const double2* x, double2* y) {
+    // constraint form (diag LA_i + near Lphi_i, block elimination)
+    auto Minv = [&](const double2* x, double2* y) {
         return constraint_solve(op, I, 1.0 / (ki * ki), op->kcs_in, op->p.tol_constraint_inner, x, y);
     };
-    auto Mspai = [&](const double2* x, double2* y) {
-        Stage s_(c, "spai_apply");
-        return csr_mv(c->stream, (int)ne, I.nnz, I.row_ptr, I.col, I.valM, x, y);
-    };
-    const Apply Minv = I.has_grid ? Apply(Mconstraint) : Apply(Mspai);
     // one unrestarted cycle of at most min(inner_maxit, INNER_BASIS_MAX) iterations
     const int m_in = inner_m(op);
     if (nested_res) *nested_res = 0.0;
-    if (op->capturing && !I.has_grid) {
-        // inside the system-product graph: device-controlled nested cycle
-        SIE_TRY(fgmres_dev(c, op->gs[1], op->kin, ne, A, Minv, a, E, op->p.tol_inner, m_in, m_in, op->gstat,
-                           &op->gnodes[1]));
-    } else {
-        int it = 0;
-        double rr = 0;
-        sie_status s;
-        {
-            Stage s_(c, "inner_solve");
-            s = fgmres(c, op->kin, ne, A, Minv, a, E, op->p.tol_inner, m_in, m_in, &it, &rr);
-        }
-        if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
-        if (nested_res) *nested_res = rr;
-        op->stats[2] = std::max(op->stats[2], (double)it);
-        op->stats[3] = std::max(op->stats[3], rr);
+    int it = 0;
+    double rr = 0;
+    sie_status s;
+    {
+        Stage s_(c, "inner_solve");
+        s = fgmres(c, op->kin, ne, A, Minv, a, E, op->p.tol_inner, m_in, m_in, &it, &rr);
     }
-    if (op->edge_zf) {  // several objects: each edge scaled by its object's factor
-        k_scale_edges<<<nb(ne), 256, 0, st>>>(ne, op->edge_zf, E);
-        SIE_CUDA_TRY(cudaGetLastError());
-        return SIE_OK;
-    }
+    if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
+    if (nested_res) *nested_res = rr;
+    op->stats[2] = std::max(op->stats[2], (double)it);
+    op->stats[3] = std::max(op->stats[3], rr);
     cplx zs(0.0, op->k0 * op->eps_r);
     zs += op->sigma * ETA0;
     SIE_TRY(axpby(st, ne, -1.0 / zs, E, 0.0, E));
-    return SIE_OK;
-}
-
-// Surface impedance boundary condition: E' = (eta_i / eta0) G^-1 Ix H, the Gram
-// system solved by the same nested FGMRES (Jacobi preconditioned; G is
-// well conditioned), on the device inside the system-product graph
-static sie_status apply_Z_sibc(sie_op* op, const double2* H, double2* E, double* nested_res)
-{
-    sie_ctx* c = op->mesh->ctx;
-    cudaStream_t st = c->stream;
-    const int64_t ne = op->mesh->h.ne;
-    double2* a = op->sys_tmp;  // ne
-    SIE_TRY(spmv(st, (int)ne, op->ix_nnz, op->ix_row_ptr, op->ix_col, op->ix_val, H, cplx(1.0, 0.0), a, false));
-    auto A = [&](const double2* x, double2* y) {
-        return spmv(c->stream, (int)ne, op->gr_nnz, op->gr_row_ptr, op->gr_col, op->gr_val, x, cplx(1.0, 0.0), y,
-                    false);
-    };
-    auto Mj = [&](const double2* x, double2* y) {
-        k_jacobi<<<nb(ne), 256, 0, c->stream>>>(ne, x, op->gr_diag, make_double2(1.0, 0.0), y);
-        SIE_CUDA_TRY(cudaGetLastError());
-        return SIE_OK;
-    };
-    const int m_in = inner_m(op);
-    if (nested_res) *nested_res = 0.0;
-    if (op->capturing) {
-        SIE_TRY(fgmres_dev(c, op->gs[1], op->kin, ne, A, Mj, a, E, op->p.tol_inner, m_in, m_in, op->gstat,
-                           &op->gnodes[1]));
-    } else {
-        int it = 0;
-        double rr = 0;
-        sie_status s;
-        {
-            Stage s_(c, "inner_solve");
-            s = fgmres(c, op->kin, ne, A, Mj, a, E, op->p.tol_inner, m_in, m_in, &it, &rr);
-        }
-        if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
-        if (nested_res) *nested_res = rr;
-        op->stats[2] = std::max(op->stats[2], (double)it);
-        op->stats[3] = std::max(op->stats[3], rr);
-    }
-    if (op->edge_zf) {
-        k_scale_edges<<<nb(ne), 256, 0, st>>>(ne, op->edge_zf, E);
-        SIE_CUDA_TRY(cudaGetLastError());
-        return SIE_OK;
-    }
-    SIE_TRY(axpby(st, ne, cplx(op->eta_re, op->eta_im), E, 0.0, E));
     return SIE_OK;
 }
 
@@ -1516,10 +1319,6 @@ static sie_status build_sys_graph(sie_op* op)
     // everything the product touches exists before the capture starts
     SIE_TRY(op->kin.alloc(c->stream, ne, inner_m(op)));
     if (!op->g_io) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->g_io, sizeof(double2) * 2 * n, c->stream));
-    if (!op->gstat) {
-        SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * 2, c->stream));
-        SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 2, c->stream));
-    }
     for (int i = 0; i < 2; i++)
         if (!op->gs[i]) SIE_CUDA_TRY(cudaStreamCreateWithFlags(&op->gs[i], cudaStreamNonBlocking));
     SIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -1567,12 +1366,14 @@ static sie_status apply_sys_fast(sie_op* op, const double2* x, double2* y)
 void sys_stats_fold(sie_op* op)
 {
     if (!op->gstat) return;
-    double h[2] = {0, 0};
+    double h[6] = {0, 0, 0, 0, 0, 0};
     cudaStream_t st = op->mesh->ctx->stream;
     if (cudaMemcpyAsync(h, op->gstat, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess) return;
     if (cudaStreamSynchronize(st) != cudaSuccess) return;
     op->stats[2] = std::max(op->stats[2], h[0]);
     op->stats[3] = std::max(op->stats[3], h[1]);
+    op->stats[4] = std::max(op->stats[4], h[4]);
+    op->stats[5] = std::max(op->stats[5], h[5]);
 }
 
 // Constraint preconditioner (the near-region form of the AEFIE constraint
@@ -1596,6 +1397,16 @@ static sie_status constraint_solve(sie_op* op, AimOp& a, cplx kappa, KrylovWork&
     double2* q = op->cs_t + nt;   // nt: solution
     double2* ph = op->cs_t + 2 * nt;
     double2* te = op->cs_e + ne;  // ne scratch
+    {
+        SIE_TRY(K.alloc(st, nt, op->p.constraint_restart));
+        ResWork w;
+        w.m = K.m, w.V = K.V, w.Z = K.Z, w.H = K.Hd;
+        sie_status s = SIE_OK;
+        Stage s_(c, "constraint_solve");
+        if (constraint_resident(op, a, make_double2(kappa.real(), kappa.imag()), false, 1, &v, &y, tol,
+                                op->p.constraint_maxit, op->p.constraint_restart, w, t1, rq, q, &s))
+            return s;
+    }
     k_jacobi<<<nb(ne), 256, 0, st>>>(ne, v, a.dLA, make_double2(1.0, 0.0), t1);
     k_D<<<nb(nt), 256, 0, st>>>((int)nt, M, t1, rq);
     SIE_CUDA_TRY(cudaGetLastError());
@@ -1660,6 +1471,17 @@ static sie_status precond_sys(sie_op* op, const double2* x, double2* y)
     double2* v1p = op->pc_e;          // ne
     double2* sig = op->pc_t;          // nt
     double2* ph = op->pc_t + nt;      // nt
+    {
+        KrylovWork& K = op->kcs_out;
+        SIE_TRY(K.alloc(st, nt, op->p.constraint_restart));
+        ResWork w;
+        w.m = K.m, w.V = K.V, w.Z = K.Z, w.H = K.Hd;
+        sie_status s = SIE_OK;
+        Stage s_(op->mesh->ctx, "constraint_solve");
+        if (constraint_resident(op, X, make_double2(1.0 / (op->k0 * op->k0), 0.0), true, 1, &x, &y, op->p.tol_constraint,
+                                op->p.constraint_maxit, op->p.constraint_restart, w, v1p, op->cs_t, op->cs_t + nt, &s))
+            return s;
+    }
     // v1' = v1 - (j k0)^-1 D^T Lphi B v2,  B v2 = -A v2
     k_sigma<<<nb(nt), 256, 0, st>>>((int)nt, M.area, x + ne, sig);
     SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphiNR, sig, 1.0, ph, false));
@@ -1871,6 +1693,10 @@ sie_status sys_prepare(sie_op* op)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_E, sizeof(double2) * h.ne, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_tmp, sizeof(double2) * (h.ne + 2 * h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_vec, sizeof(double2) * 4 * (h.ne + h.nt), st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * 6, st));
+    SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->res_bar, sizeof(unsigned) * RES_WORDS, st));
+    SIE_CUDA_TRY(cudaMemsetAsync(op->res_bar, 0, sizeof(unsigned) * RES_WORDS, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pk_he, sizeof(float4) * h.ne, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pk_sig, sizeof(float2) * h.nt, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->cs_e, sizeof(double2) * 2 * h.ne, st));
@@ -1896,18 +1722,21 @@ void sys_release(sie_op* op)
     op->ir_buf = nullptr;
     if (op->g_io) cudaFreeAsync(op->g_io, st);
     if (op->gstat) cudaFreeAsync(op->gstat, st);
+    if (op->res_bar) cudaFreeAsync(op->res_bar, st);
     op->g_io = nullptr;
     op->gstat = nullptr;
+    op->res_bar = nullptr;
     op->kin.release(st);
     op->kout.release(st);
-    for (KrylovWork& k : op->kmulti) k.release(st);
-    for (KrylovWork& k : op->kcs_multi) k.release(st);
+    op->kmulti.release(st);
+    op->kcs_multi.release(st);
     op->kzp.release(st);
     if (op->zp) cudaFreeAsync(op->zp, st);
     op->zp = nullptr;
     for (void* p : {(void*)op->mscr, (void*)op->ir_multi, (void*)op->mvec})
         if (p) cudaFreeAsync(p, st);
-    op->mscr = op->ir_multi = op->mvec = nullptr;
+    if (op->con_scr) cudaFreeAsync(op->con_scr, st);
+    op->mscr = op->ir_multi = op->mvec = op->con_scr = nullptr;
     op->kcs_in.release(st);
     op->kcs_out.release(st);
     for (void* p : {(void*)op->gr_row_ptr, (void*)op->gr_col, (void*)op->gr_val, (void*)op->gr_diag,
@@ -1935,6 +1764,14 @@ sie_status sys_matvec(sie_op* op, int which, const double2* x, double2* y)
 sie_status nested_check(sie_op* op, const char* who)
 {
     sys_stats_fold(op);
+    if (std::isinf(op->stats[3])) {
+        set_error(std::string(who) + ": a grid barrier's wait ran out in a nested interior solve");
+        return SIE_ERR_TIMEOUT;
+    }
+    if (std::isinf(op->stats[5])) {
+        set_error(std::string(who) + ": a wait ran out in a constraint preconditioner");
+        return SIE_ERR_TIMEOUT;
+    }
     if (op->stats[3] >= op->p.tol_inner) {
         set_error(std::string(who) + ": a nested interior solve ended at relative residual " +
                   std::to_string(op->stats[3]) + " >= tol_inner after min(inner_maxit, " +
@@ -2001,7 +1838,7 @@ sie_status sys_solve(sie_op* op, const double2* b, double2* x, int* iters, doubl
         return precond_sys(op, tw, v);
     };
     for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 2, op->mesh->ctx->stream));
+    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, op->mesh->ctx->stream));
     SIE_TRY(weight_rows(op, b, bw, false));
     int it = 0;
     double rr = 0;
@@ -2061,7 +1898,7 @@ sie_status sys_solve_refined(sie_op* op, const double2* b, double2* x, int* iter
         return precond_sys(op, tw, v);
     };
     for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 2, st));
+    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
     SIE_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double2) * n, st));
     double bn = 0, rel = 1.0;
     SIE_TRY(weight_rows(op, b, op->bal, false));
@@ -2190,9 +2027,9 @@ sie_status sys_far_sums(sie_op* op, const double2* x, const double* rhat_d, int 
     return SIE_OK;
 }
 
-// ------------------------------------------------------------------ panel Krylov solves
+// ------------------------------------------------------------------ Krylov workspace of several right-hand sides
 // per right-hand side sizes inside a PanelWork
-static int64_t pw_p(int m) { return (int64_t)CGS_CHUNKS * (2 * (m + 1) + 1); }
+static int64_t pw_p(int m) { return (int64_t)RES_MAXCTA * 2 * (m + 2); }
 static int64_t pw_h(int m) { return 2 * (int64_t)(m + 2); }
 static int64_t pw_d(int m) { return (int64_t)(m + 1) * m + 2 * m + 2 * (m + 1); }
 static int64_t pw_s(int m) { return 8 + m + 1; }
@@ -2239,184 +2076,23 @@ void PanelWork::release(cudaStream_t st)
     m = R = 0;
 }
 
-// Restarted flexible GMRES for R right-hand sides held as panels (B, X: R
-// contiguous vectors of n), zero initial guess: the arithmetic of fgmres per
-// right-hand side, with A and Minv applied to a whole panel and every
-// Gram-Schmidt / Givens step one launch for all R (PanelStrides).  Ends when
-// every residual is below tol (host check lagged by one iteration); iters,
-// relres[q] as for fgmres.
-static sie_status fgmres_panel(sie_ctx* c, PanelWork& K, int R, int64_t n, const Apply& A, const Apply& Minv,
-                               const double2* B, double2* X, double tol, int maxit, int restart, int* iters_out,
-                               double* relres_out)
-{
-    cudaStream_t st = c->stream;
-    const int m = restart;
-    SIE_TRY(K.alloc(st, n, m, R));
-    PanelStrides ps;
-    ps.v = n;
-    ps.p = pw_p(m);
-    ps.h = pw_h(m);
-    ps.d = pw_d(m);
-    ps.s = pw_s(m);
-    const int64_t ldv = (int64_t)R * n;
-    auto Hq = [&](int q) { return K.Hd + q * ps.d; };
-    auto gq = [&](int q) { return K.Hd + q * ps.d + (m + 1) * m + 2 * m; };
-    auto yq = [&](int q) { return K.Hd + q * ps.d + (m + 1) * m + 2 * m + (m + 1); };
-    SIE_CUDA_TRY(cudaMemsetAsync(X, 0, sizeof(double2) * R * n, st));
-    for (int q = 0; q < R; q++) {
-        SIE_TRY(dots(st, n, 1, B + q * n, n, B + q * n, K.part + q * DOT_CHUNKS, K.wd + q));
-        k_gm_start<<<nb(n), 256, 0, st>>>(n, B + q * n, K.wd + q, K.V + q * n, gq(q), m, K.sc + q * ps.s, 1);
-    }
-    SIE_CUDA_TRY(cudaGetLastError());
-    std::vector<double> rel(R, 1.0);
-    auto all_below = [&](const double* v) {
-        for (int q = 0; q < R; q++)
-            if (!(v[q] < tol)) return false;
-        return true;
-    };
-    int it = 0;
-    const int LAG = 1;
-    const dim3 grid(CGS_CHUNKS, R);
-    while (true) {
-        int j = 0;
-        bool conv = false;
-        for (; j < m && it < maxit; j++) {
-            double2* Vj = K.V + j * ldv;
-            double2* Zj = K.Z + j * ldv;
-            SIE_TRY(Minv(Vj, Zj));
-            SIE_TRY(A(Zj, K.W));
-            double2* P1 = K.P;
-            double2* P2 = K.P + (int64_t)CGS_CHUNKS * (m + 1);
-            double2* P3 = K.P + (int64_t)2 * CGS_CHUNKS * (m + 1);
-            k_cgs_part<<<grid, 256, 0, st>>>(n, j + 1, K.V, ldv, K.W, P1, m + 1, nullptr, nullptr, nullptr, ps);
-            k_cgs_update<<<grid, 256, 0, st>>>(n, j + 1, K.V, ldv, P1, m + 1, K.h, K.W, P2, 0, nullptr, ps);
-            k_cgs_update<<<grid, 256, 0, st>>>(n, j + 1, K.V, ldv, P2, m + 1, K.h + (m + 2), K.W, P3, 1, nullptr,
-                                               ps);
-            k_cgs_finish<<<grid, 256, 0, st>>>(n, j, m, K.h, K.h + (m + 2), P3, K.W, K.V, K.Hd,
-                                               K.Hd + (m + 1) * m, K.Hd + (m + 1) * m + m,
-                                               K.Hd + (m + 1) * m + 2 * m, K.sc, nullptr, ps, ldv, K.res);
-            SIE_CUDA_TRY(cudaGetLastError());
-            SIE_CUDA_TRY(cudaMemcpyAsync(K.res_h + (int64_t)j * R, K.res + (int64_t)j * R, sizeof(double) * R,
-                                         cudaMemcpyDeviceToHost, st));
-            SIE_CUDA_TRY(cudaEventRecord(K.ev[j], st));
-            it++;
-            if (j >= LAG) {
-                SIE_CUDA_TRY(cudaEventSynchronize(K.ev[j - LAG]));
-                const double* v = K.res_h + (int64_t)(j - LAG) * R;
-                for (int q = 0; q < R; q++)
-                    if (!std::isfinite(v[q])) {
-                        set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
-                        return SIE_ERR_ARG;
-                    }
-                if (all_below(v)) {
-                    conv = true;
-                    j++;
-                    break;
-                }
-            }
-        }
-        const int jend = j - 1;
-        SIE_CUDA_TRY(cudaEventSynchronize(K.ev[jend]));
-        for (int q = 0; q < R; q++) {
-            rel[q] = K.res_h[(int64_t)jend * R + q];
-            if (!std::isfinite(rel[q])) {
-                set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
-                return SIE_ERR_ARG;
-            }
-            k_gm_backsub<<<1, 1, 0, st>>>(jend, m, Hq(q), gq(q), yq(q));
-            k_gemv<<<nb(n), 256, 0, st>>>(n, jend + 1, K.Z + q * n, ldv, yq(q), 1.0, X + q * n);
-        }
-        SIE_CUDA_TRY(cudaGetLastError());
-        if (all_below(rel.data())) conv = true;
-        if (conv || it >= maxit) break;
-        // restart from the true residuals
-        SIE_TRY(A(X, K.W));
-        SIE_CUDA_TRY(cudaMemcpyAsync(K.Rv, B, sizeof(double2) * R * n, cudaMemcpyDeviceToDevice, st));
-        SIE_TRY(axpby(st, R * n, -1.0, K.W, 1.0, K.Rv));
-        std::vector<double> hb(2 * R);
-        for (int q = 0; q < R; q++) {
-            SIE_TRY(dots(st, n, 1, K.Rv + q * n, n, K.Rv + q * n, K.part + q * DOT_CHUNKS, K.wd + q));
-            k_gm_start<<<nb(n), 256, 0, st>>>(n, K.Rv + q * n, K.wd + q, K.V + q * n, gq(q), m, K.sc + q * ps.s, 0);
-            SIE_CUDA_TRY(cudaMemcpyAsync(K.res_h + 2 * q, K.sc + q * ps.s, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                         st));
-        }
-        SIE_CUDA_TRY(cudaGetLastError());
-        SIE_CUDA_TRY(cudaStreamSynchronize(st));
-        for (int q = 0; q < R; q++) rel[q] = K.res_h[2 * q] > 0 ? K.res_h[2 * q + 1] / K.res_h[2 * q] : 0.0;
-        if (all_below(rel.data())) break;
-    }
-    for (int q = 0; q < R; q++) {
-        if (iters_out) iters_out[q] = it;
-        if (relres_out) relres_out[q] = rel[q];
-    }
-    return all_below(rel.data()) ? SIE_OK : SIE_ERR_NOT_CONVERGED;
-}
-
-// E = Z' H for a panel of R vectors (near-region-only or SIBC interiors): the
-// right-hand sides of the nested solves by CSR x panel products, then one
-// panel FGMRES for all R (near-only: A = L_i,NR, M = its sparse approximate
-// inverse; SIBC: A = Gram, M = Jacobi), with the stream path's iteration cap
-// and tolerance; then the impedance factor.  Hp, Ep: R x ne.
-static sie_status apply_Z_panel(sie_op* op, int R, const double2* Hp, double2* Ep, double* nested_res)
+// E = Z' H for a panel of R vectors (near-region-only or SIBC interiors), one
+// grid-resident kernel; Hp, Ep: R x ne.  Does not wait: its statistics stay in op->gstat.
+static sie_status apply_Z_panel(sie_op* op, int R, const double2* Hp, double2* Ep)
 {
     sie_ctx* c = op->mesh->ctx;
-    cudaStream_t st = c->stream;
     const int64_t ne = op->mesh->h.ne;
-    AimOp& I = op->inn;
-    const bool sibc = op->p.interior_model == SIE_SIBC;
-    double2* a = op->zp + 2 * MULTI_RHS * ne;  // right-hand sides
-    double2* t = op->zp + 3 * MULTI_RHS * ne;  // scratch
-    // I-cross H (weight -1/2 for GIBC, +1 for SIBC)
-    SIE_TRY(csr_panel(st, (int)ne, op->ix_row_ptr, op->ix_col, op->ix_val, Hp, ne, R, false, t, ne));
-    if (sibc) {
-        SIE_CUDA_TRY(cudaMemcpyAsync(a, t, sizeof(double2) * R * ne, cudaMemcpyDeviceToDevice, st));
-    } else {
-        SIE_TRY(csr_panel(st, (int)ne, I.row_ptr, I.col, I.valK, Hp, ne, R, false, a, ne));
-        SIE_TRY(axpby(st, R * ne, -0.5, t, 1.0, a));
-    }
-    auto A = [&](const double2* x, double2* y) {
-        if (sibc) return csr_panel(st, (int)ne, op->gr_row_ptr, op->gr_col, op->gr_val, x, ne, R, false, y, ne);
-        return csr_panel(st, (int)ne, I.row_ptr, I.col, I.valL, x, ne, R, false, y, ne);
-    };
-    auto M = [&](const double2* x, double2* y) {
-        if (sibc) {
-            for (int q = 0; q < R; q++)
-                k_jacobi<<<nb(ne), 256, 0, st>>>(ne, x + q * ne, op->gr_diag, make_double2(1.0, 0.0), y + q * ne);
-            SIE_CUDA_TRY(cudaGetLastError());
-            return SIE_OK;
-        }
-        return csr_panel(st, (int)ne, I.row_ptr, I.col, I.valM, x, ne, R, false, y, ne);
-    };
-    const int m_in = inner_m(op);
-    int it[MULTI_RHS];
-    double rr[MULTI_RHS];
-    sie_status s;
-    {
-        Stage s_(c, "inner_solve");
-        s = fgmres_panel(c, op->kzp, R, ne, A, M, a, Ep, op->p.tol_inner, m_in, m_in, it, rr);
-    }
-    if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
-    double worst = 0;
-    for (int q = 0; q < R; q++) {
-        worst = std::max(worst, rr[q]);
-        op->stats[2] = std::max(op->stats[2], (double)it[q]);
-        op->stats[3] = std::max(op->stats[3], rr[q]);
-    }
-    if (nested_res) *nested_res = worst;
-    if (op->edge_zf) {
-        for (int q = 0; q < R; q++) k_scale_edges<<<nb(ne), 256, 0, st>>>(ne, op->edge_zf, Ep + q * ne);
-        SIE_CUDA_TRY(cudaGetLastError());
-        return SIE_OK;
-    }
     cplx f;
-    if (sibc) {
+    if (op->p.interior_model == SIE_SIBC)
         f = cplx(op->eta_re, op->eta_im);
-    } else {
-        cplx zs(0.0, op->k0 * op->eps_r);
-        zs += op->sigma * ETA0;
-        f = -1.0 / zs;
-    }
-    return axpby(st, R * ne, f, Ep, 0.0, Ep);
+    else
+        f = -1.0 / cplx(op->sigma * ETA0, op->k0 * op->eps_r);
+    PanelWork& K = op->kzp;
+    SIE_TRY(K.alloc(c->stream, ne, inner_m(op), R));
+    ResWork w;
+    w.m = K.m, w.V = K.V, w.Z = K.Z, w.W = K.W, w.H = K.Hd, w.ldh = pw_d(K.m), w.part = K.P;
+    Stage s_(c, "inner_solve");
+    return nested_solve(op, R, Hp, ne, Ep, ne, make_double2(f.real(), f.imag()), 1, w);
 }
 
 // y_q = SYS x_q for R vectors (block product): the R nested interior solves as
@@ -2435,7 +2111,7 @@ static sie_status apply_sys_multi(sie_op* op, int R, const double2* const* x, do
     double2* Ep = op->zp + MULTI_RHS * ne;
     for (int q = 0; q < R; q++)
         SIE_CUDA_TRY(cudaMemcpyAsync(Hp + q * ne, x[q], sizeof(double2) * ne, cudaMemcpyDeviceToDevice, st));
-    SIE_TRY(apply_Z_panel(op, R, Hp, Ep, nullptr));
+    SIE_TRY(apply_Z_panel(op, R, Hp, Ep));
     for (int q = 0; q < R; q++) SIE_TRY(apply_sys_rest(op, x[q], Ep + q * ne, x[q] + ne, y[q]));
     return SIE_OK;
 }
@@ -2458,30 +2134,38 @@ public:
 };
 
 // R restarted flexible GMRES iterations in lockstep: one Krylov basis per
-// right-hand side (K[q]), the operator and the preconditioner applied to the
-// R current vectors at once (so a block implementation reads its data once
-// for all of them), the Gram-Schmidt, Givens and update steps of fgmres per
-// right-hand side.  The cycle ends when every residual is below tol (a
-// converged right-hand side keeps iterating with the others, which only lowers
-// its residual); restarts from the true residuals.  iters: iterations run
-// (the same for all), relres[q]: final relative residual of q.
-static sie_status fgmres_multi(sie_ctx* c, KrylovWork* K, int R, int64_t n, const BlockApply& A,
-                               const BlockApply& Minv, const double2* const* b, double2* const* x, double tol,
-                               int maxit, int restart, int* iters_out, double* relres_out, int lag = 1)
+// right-hand side (K.V + q (m + 1) n), the operator and the preconditioner applied
+// to the R current vectors at once (so a block implementation reads its data
+// once for all of them), every Gram-Schmidt and Givens step one launch for all R
+// (PanelStrides) and one residual copy.  The cycle ends when every residual is
+// below tol (a converged right-hand side keeps iterating with the others, which
+// only lowers its residual); restarts from the true residuals.  iters: iterations
+// run (the same for all), relres[q]: final relative residual of q.
+static sie_status fgmres_multi(sie_ctx* c, PanelWork& K, int R, int64_t n, const BlockApply& A, const BlockApply& Minv,
+                               const double2* const* b, double2* const* x, double tol, int maxit, int restart,
+                               int* iters_out, double* relres_out, int lag = 1)
 {
     cudaStream_t st = c->stream;
     const int m = restart;
-    for (int q = 0; q < R; q++) SIE_TRY(K[q].alloc(st, n, restart));
-    auto H = [&](int q) { return K[q].Hd; };
-    auto cs = [&](int q) { return K[q].Hd + (m + 1) * m; };
-    auto sn = [&](int q) { return K[q].Hd + (m + 1) * m + m; };
-    auto g = [&](int q) { return K[q].Hd + (m + 1) * m + 2 * m; };
-    auto y = [&](int q) { return K[q].Hd + (m + 1) * m + 2 * m + (m + 1); };
-    auto wd = [&](int q) { return K[q].h + 2 * (m + 2); };
+    SIE_TRY(K.alloc(st, n, m, R));
+    PanelStrides ps;
+    ps.v = (int64_t)(m + 1) * n;
+    ps.w = n;
+    ps.p = pw_p(m);
+    ps.h = pw_h(m);
+    ps.d = pw_d(m);
+    ps.s = pw_s(m);
+    double2* cs = K.Hd + (m + 1) * m;
+    double2* sn = cs + m;
+    double2* g = sn + m;
+    double2* y = g + (m + 1);
+    double2* h2 = K.h + (m + 2);
+    double2* P2 = K.P + (int64_t)CGS_CHUNKS * (m + 1);
+    double2* P3 = K.P + (int64_t)2 * CGS_CHUNKS * (m + 1);
     for (int q = 0; q < R; q++) {
         SIE_CUDA_TRY(cudaMemsetAsync(x[q], 0, sizeof(double2) * n, st));
-        SIE_TRY(dots(st, n, 1, b[q], n, b[q], K[q].part, wd(q)));
-        k_gm_start<<<nb(n), 256, 0, st>>>(n, b[q], wd(q), K[q].V, g(q), m, K[q].sc, 1);
+        SIE_TRY(dots(st, n, 1, b[q], n, b[q], K.part + q * DOT_CHUNKS, K.wd + q));
+        k_gm_start<<<nb(n), 256, 0, st>>>(n, b[q], K.wd + q, K.V + q * ps.v, g + q * ps.d, m, K.sc + q * ps.s, 1);
     }
     SIE_CUDA_TRY(cudaGetLastError());
     int it = 0;
@@ -2493,6 +2177,15 @@ static sie_status fgmres_multi(sie_ctx* c, KrylovWork* K, int R, int64_t n, cons
             if (!(v[q] < tol)) return false;
         return true;
     };
+    auto finite = [&](const double* v) {
+        for (int q = 0; q < R; q++)
+            if (!std::isfinite(v[q])) {
+                set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
+                return false;
+            }
+        return true;
+    };
+    const dim3 grid(CGS_CHUNKS, R);
     while (true) {
         int j = 0;
         bool conv = false;
@@ -2500,40 +2193,25 @@ static sie_status fgmres_multi(sie_ctx* c, KrylovWork* K, int R, int64_t n, cons
             const double2* vj[MULTI_RHS];
             double2 *zj[MULTI_RHS], *wq[MULTI_RHS];
             for (int q = 0; q < R; q++) {
-                vj[q] = K[q].V + (int64_t)j * n;
-                zj[q] = K[q].Z + (int64_t)j * n;
-                wq[q] = K[q].w;
+                vj[q] = K.V + q * ps.v + (int64_t)j * n;
+                zj[q] = K.Z + ((int64_t)q * m + j) * n;
+                wq[q] = K.W + q * n;
             }
             SIE_TRY(Minv(R, vj, zj));
             SIE_TRY(A(R, zj, wq));
-            for (int q = 0; q < R; q++) {
-                double2* P1 = K[q].cgsp;
-                double2* P2 = K[q].cgsp + (int64_t)CGS_CHUNKS * (m + 1);
-                double2* P3 = K[q].cgsp + (int64_t)2 * CGS_CHUNKS * (m + 1);
-                double2* h1 = K[q].h;
-                double2* h2 = K[q].h + (m + 2);
-                k_cgs_part<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K[q].V, n, K[q].w, P1, m + 1, nullptr, nullptr,
-                                                       nullptr);
-                k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K[q].V, n, P1, m + 1, h1, K[q].w, P2, 0, nullptr);
-                k_cgs_update<<<CGS_CHUNKS, 256, 0, st>>>(n, j + 1, K[q].V, n, P2, m + 1, h2, K[q].w, P3, 1, nullptr);
-                k_cgs_finish<<<CGS_CHUNKS, 256, 0, st>>>(n, j, m, h1, h2, P3, K[q].w, K[q].V, H(q), cs(q), sn(q),
-                                                         g(q), K[q].sc, nullptr);
-                SIE_CUDA_TRY(cudaMemcpyAsync(K[q].resid_h + j, K[q].sc + 3 + j, sizeof(double),
-                                             cudaMemcpyDeviceToHost, st));
-            }
+            k_cgs_part<<<grid, 256, 0, st>>>(n, j + 1, K.V, n, K.W, K.P, m + 1, ps);
+            k_cgs_update<<<grid, 256, 0, st>>>(n, j + 1, K.V, n, K.P, m + 1, K.h, K.W, P2, 0, ps);
+            k_cgs_update<<<grid, 256, 0, st>>>(n, j + 1, K.V, n, P2, m + 1, h2, K.W, P3, 1, ps);
+            k_cgs_finish<<<grid, 256, 0, st>>>(n, j, m, K.h, h2, P3, K.W, K.V, K.Hd, cs, sn, g, K.sc, ps, n, K.res);
             SIE_CUDA_TRY(cudaGetLastError());
-            SIE_CUDA_TRY(cudaEventRecord(K[0].ev[j], st));
+            SIE_CUDA_TRY(cudaMemcpyAsync(K.res_h + (int64_t)j * R, K.res + (int64_t)j * R, sizeof(double) * R,
+                                         cudaMemcpyDeviceToHost, st));
+            SIE_CUDA_TRY(cudaEventRecord(K.ev[j], st));
             it++;
             if (j >= LAG) {
-                SIE_CUDA_TRY(cudaEventSynchronize(K[0].ev[j - LAG]));
-                double v[MULTI_RHS];
-                for (int q = 0; q < R; q++) {
-                    v[q] = K[q].resid_h[j - LAG];
-                    if (!std::isfinite(v[q])) {
-                        set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
-                        return SIE_ERR_ARG;
-                    }
-                }
+                SIE_CUDA_TRY(cudaEventSynchronize(K.ev[j - LAG]));
+                const double* v = K.res_h + (int64_t)(j - LAG) * R;
+                if (!finite(v)) return SIE_ERR_ARG;
                 if (all_below(v)) {
                     conv = true;
                     j++;
@@ -2542,33 +2220,32 @@ static sie_status fgmres_multi(sie_ctx* c, KrylovWork* K, int R, int64_t n, cons
             }
         }
         const int jend = j - 1;
-        SIE_CUDA_TRY(cudaEventSynchronize(K[0].ev[jend]));
+        SIE_CUDA_TRY(cudaEventSynchronize(K.ev[jend]));
+        for (int q = 0; q < R; q++) rel[q] = K.res_h[(int64_t)jend * R + q];
+        if (!finite(rel)) return SIE_ERR_ARG;
         for (int q = 0; q < R; q++) {
-            rel[q] = K[q].resid_h[jend];
-            if (!std::isfinite(rel[q])) {
-                set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
-                return SIE_ERR_ARG;
-            }
-            k_gm_backsub<<<1, 1, 0, st>>>(jend, m, H(q), g(q), y(q));
-            k_gemv<<<nb(n), 256, 0, st>>>(n, jend + 1, K[q].Z, n, y(q), 1.0, x[q]);
+            k_gm_backsub<<<1, 1, 0, st>>>(jend, m, K.Hd + q * ps.d, g + q * ps.d, y + q * ps.d);
+            k_gemv<<<nb(n), 256, 0, st>>>(n, jend + 1, K.Z + (int64_t)q * m * n, n, y + q * ps.d, 1.0, x[q]);
         }
         SIE_CUDA_TRY(cudaGetLastError());
         if (all_below(rel)) conv = true;
         if (conv || it >= maxit) break;
         // restart from the true residuals
         double2* wq[MULTI_RHS];
-        for (int q = 0; q < R; q++) wq[q] = K[q].w;
+        for (int q = 0; q < R; q++) wq[q] = K.W + q * n;
         SIE_TRY(A(R, x, wq));
+        double hb[2 * MULTI_RHS];
         for (int q = 0; q < R; q++) {
-            SIE_CUDA_TRY(cudaMemcpyAsync(K[q].r, b[q], sizeof(double2) * n, cudaMemcpyDeviceToDevice, st));
-            SIE_TRY(axpby(st, n, -1.0, K[q].w, 1.0, K[q].r));
-            SIE_TRY(dots(st, n, 1, K[q].r, n, K[q].r, K[q].part, wd(q)));
-            k_gm_start<<<nb(n), 256, 0, st>>>(n, K[q].r, wd(q), K[q].V, g(q), m, K[q].sc, 0);
-            SIE_CUDA_TRY(cudaMemcpyAsync(K[q].resid_h, K[q].sc, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+            double2* r = K.Rv + q * n;
+            SIE_CUDA_TRY(cudaMemcpyAsync(r, b[q], sizeof(double2) * n, cudaMemcpyDeviceToDevice, st));
+            SIE_TRY(axpby(st, n, -1.0, wq[q], 1.0, r));
+            SIE_TRY(dots(st, n, 1, r, n, r, K.part + q * DOT_CHUNKS, K.wd + q));
+            k_gm_start<<<nb(n), 256, 0, st>>>(n, r, K.wd + q, K.V + q * ps.v, g + q * ps.d, m, K.sc + q * ps.s, 0);
+            SIE_CUDA_TRY(cudaMemcpyAsync(hb + 2 * q, K.sc + q * ps.s, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
         }
         SIE_CUDA_TRY(cudaGetLastError());
         SIE_CUDA_TRY(cudaStreamSynchronize(st));
-        for (int q = 0; q < R; q++) rel[q] = K[q].resid_h[0] > 0 ? K[q].resid_h[1] / K[q].resid_h[0] : 0.0;
+        for (int q = 0; q < R; q++) rel[q] = hb[2 * q] > 0 ? hb[2 * q + 1] / hb[2 * q] : 0.0;
         if (all_below(rel)) break;
     }
     for (int q = 0; q < R; q++) {
@@ -2594,6 +2271,9 @@ static sie_status multi_scratch(sie_op* op)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->mscr, sizeof(double2) * MULTI_RHS * multi_stride(op),
                                  op->mesh->ctx->stream));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->ir_multi, sizeof(double2) * 3 * MULTI_RHS * n, op->mesh->ctx->stream));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->con_scr,
+                                 sizeof(double2) * MULTI_RHS * (op->mesh->h.ne + 2 * op->mesh->h.nt),
+                                 op->mesh->ctx->stream));
     return SIE_OK;
 }
 
@@ -2614,6 +2294,19 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
     const int64_t ne = M.ne, nt = M.nt, n = ne + nt;
     const cplx jk0(0.0, op->k0);
     const cplx kappa = 1.0 / (op->k0 * op->k0);
+    const int m = std::min(op->p.constraint_restart, 20);
+    {
+        PanelWork& K = op->kcs_multi;
+        SIE_TRY(K.alloc(st, nt, m, R));
+        ResWork w;
+        w.m = m, w.V = K.V, w.Z = K.Z, w.H = K.Hd, w.ldh = pw_d(m);
+        double2* v1 = op->con_scr;
+        sie_status s = SIE_OK;
+        Stage s_(c, "constraint_solve");
+        if (constraint_resident(op, X, make_double2(kappa.real(), kappa.imag()), true, R, x, y, op->p.tol_constraint,
+                                op->p.constraint_maxit, m, w, v1, v1 + R * ne, v1 + R * (ne + nt), &s))
+            return s;
+    }
     double2 *v1p[MULTI_RHS], *t1[MULTI_RHS], *te[MULTI_RHS], *sig[MULTI_RHS], *ph[MULTI_RHS];
     double2 *rq[MULTI_RHS], *qv[MULTI_RHS], *ste[MULTI_RHS], *sph[MULTI_RHS];
     for (int q = 0; q < R; q++) {
@@ -2661,7 +2354,7 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
         double rr[MULTI_RHS];
         Stage s_(c, "constraint_solve");
         sie_status s = fgmres_multi(c, op->kcs_multi, R, nt, S, LU, rq, qv, op->p.tol_constraint,
-                                    op->p.constraint_maxit, std::min(op->p.constraint_restart, 20), it, rr, 0);
+                                    op->p.constraint_maxit, m, it, rr, 0);
         if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
         for (int q = 0; q < R; q++) {
             op->stats[4] = std::max(op->stats[4], (double)it[q]);
@@ -2728,7 +2421,7 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
         return precond_sys_multi(op, Rn, tw, v);
     };
     for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 2, st));
+    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
     for (int q = 0; q < R; q++) SIE_TRY(weight_rows(op, b[q], bw[q], false));
     int it[MULTI_RHS];
     double rr[MULTI_RHS];
@@ -2744,10 +2437,10 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
             t[q] = op->ir_multi + (int64_t)(2 * MULTI_RHS + q) * n;
             SIE_CUDA_TRY(cudaMemsetAsync(x[q], 0, sizeof(double2) * n, st));
         }
-        KrylovWork& K0 = op->kmulti[0];
-        SIE_TRY(K0.alloc(st, n, op->p.restart));
+        PanelWork& K0 = op->kmulti;
+        SIE_TRY(K0.alloc(st, n, op->p.restart, R));
         double bn[MULTI_RHS], rel[MULTI_RHS], rel_prev = 1.0;
-        for (int q = 0; q < R; q++) SIE_TRY(norm2(st, n, bw[q], K0.part, K0.h, K0.resid_h, &bn[q]));
+        for (int q = 0; q < R; q++) SIE_TRY(norm2(st, n, bw[q], K0.part, K0.wd, K0.res_h, &bn[q]));
         const int saved = op->p.precision;
         const int SWEEPS = 10;
         bool fp64_corr = false;
@@ -2760,7 +2453,7 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
                 SIE_CUDA_TRY(cudaMemcpyAsync(r[q], bw[q], sizeof(double2) * n, cudaMemcpyDeviceToDevice, st));
                 if (sweep > 0) s = axpby(st, n, -1.0, t[q], 1.0, r[q]);
                 double rn = 0;
-                if (s == SIE_OK) s = norm2(st, n, r[q], K0.part, K0.h, K0.resid_h, &rn);
+                if (s == SIE_OK) s = norm2(st, n, r[q], K0.part, K0.wd, K0.res_h, &rn);
                 rel[q] = bn[q] > 0 ? rn / bn[q] : 0.0;
                 worst = std::max(worst, rel[q]);
             }
