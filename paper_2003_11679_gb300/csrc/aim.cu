@@ -11,7 +11,9 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
+#include "gridio.cuh"
 #include "internal.h"
 #include "spmv.cuh"
 
@@ -227,46 +229,6 @@ sie_status aim_spectra(sie_op* op, AimOp& a)
     return SIE_OK;
 }
 
-// ------------------------------------------------------------------ projection (P, P_phi)
-// one thread per (triangle, stencil node): J_t(r) = alpha (r - c_t) + beta,
-// alpha = sum_i c_i x_i, beta = sum_i c_i x_i (c_t - p_i), div J_t = 2 alpha.
-// mode 0: grids Jx, Jy, Jz, rho; mode 1: Jx, Jy, Jz only.
-__global__ void k_project(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
-                          const double* __restrict__ W, const double2* __restrict__ x, GridDesc g, int ngrid,
-                          double2* __restrict__ src, int64_t Ng)
-{
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nt * S) return;
-    int t = idx / S, u = idx % S;
-    const int Mp = Mord + 1;
-    double2 al = make_double2(0, 0);
-    double2 be[3] = {al, al, al};
-    for (int i = 0; i < 3; i++) {
-        double2 xv = x[M.tri_edge[3 * t + i]];
-        double c = M.coef[3 * t + i];
-        al.x += c * xv.x;
-        al.y += c * xv.y;
-        for (int a = 0; a < 3; a++) {
-            double qq = c * M.q[9 * t + 3 * i + a];
-            be[a].x += qq * xv.x;
-            be[a].y += qq * xv.y;
-        }
-    }
-    int nx = base[3 * t] + u % Mp, ny = base[3 * t + 1] + (u / Mp) % Mp, nz = base[3 * t + 2] + u / (Mp * Mp);
-    int64_t node = ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
-    const double* w = W + (size_t)idx * 4;
-    for (int a = 0; a < 3; a++) {
-        double2* d = src + a * Ng + node;
-        atomicAdd(&d->x, al.x * w[1 + a] + be[a].x * w[0]);
-        atomicAdd(&d->y, al.y * w[1 + a] + be[a].y * w[0]);
-    }
-    if (ngrid == 4) {
-        double2* d = src + 3 * Ng + node;
-        atomicAdd(&d->x, 2.0 * al.x * w[0]);
-        atomicAdd(&d->y, 2.0 * al.y * w[0]);
-    }
-}
-
 // ------------------------------------------------------------------ spectral multiply
 // mode 0 (L): J_a *= G, rho *= G.  mode 1 (K): J <- Ghat_grad x J.
 __global__ void k_specmul(int mode, const double2* __restrict__ spec, double2* __restrict__ buf, int64_t nn)
@@ -291,72 +253,6 @@ __global__ void k_specmul(int mode, const double2* __restrict__ spec, double2* _
     }
 }
 
-// ------------------------------------------------------------------ interpolation (W = P^T)
-// one warp per triangle; lanes gather stencil nodes; y[e] += c_{t,i}
-// [S1 + (c_t - p_i) . T0 + scal 2 P0]  (scal = -1/k^2 for L, 0 for K)
-__global__ void k_interp(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
-                         const double* __restrict__ W, const double2* __restrict__ out, GridDesc g, int has_phi,
-                         double2 scal, int64_t Ng, double2* __restrict__ y)
-{
-    int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    int lane = threadIdx.x & 31;
-    if (t >= nt) return;
-    const int Mp = Mord + 1;
-    double s1r = 0, s1i = 0, t0r[3] = {0, 0, 0}, t0i[3] = {0, 0, 0}, p0r = 0, p0i = 0;
-    for (int u = lane; u < S; u += 32) {
-        int nx = base[3 * t] + u % Mp, ny = base[3 * t + 1] + (u / Mp) % Mp, nz = base[3 * t + 2] + u / (Mp * Mp);
-        int64_t node = ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
-        const double* w = W + ((size_t)t * S + u) * 4;
-        for (int a = 0; a < 3; a++) {
-            double2 A = out[a * Ng + node];
-            s1r += w[1 + a] * A.x;
-            s1i += w[1 + a] * A.y;
-            t0r[a] += w[0] * A.x;
-            t0i[a] += w[0] * A.y;
-        }
-        if (has_phi) {
-            double2 P = out[3 * Ng + node];
-            p0r += w[0] * P.x;
-            p0i += w[0] * P.y;
-        }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        s1r += __shfl_down_sync(0xffffffffu, s1r, off);
-        s1i += __shfl_down_sync(0xffffffffu, s1i, off);
-        p0r += __shfl_down_sync(0xffffffffu, p0r, off);
-        p0i += __shfl_down_sync(0xffffffffu, p0i, off);
-        for (int a = 0; a < 3; a++) {
-            t0r[a] += __shfl_down_sync(0xffffffffu, t0r[a], off);
-            t0i[a] += __shfl_down_sync(0xffffffffu, t0i[a], off);
-        }
-    }
-    if (lane < 3) {
-        int i = lane;
-        // broadcast from lane 0
-        double S1r = __shfl_sync(0x7u, s1r, 0), S1i = __shfl_sync(0x7u, s1i, 0);
-        double P0r = __shfl_sync(0x7u, p0r, 0), P0i = __shfl_sync(0x7u, p0i, 0);
-        double T0r[3], T0i[3];
-        for (int a = 0; a < 3; a++) {
-            T0r[a] = __shfl_sync(0x7u, t0r[a], 0);
-            T0i[a] = __shfl_sync(0x7u, t0i[a], 0);
-        }
-        double vr = S1r, vi = S1i;
-        for (int a = 0; a < 3; a++) {
-            double qq = M.q[9 * t + 3 * i + a];
-            vr += qq * T0r[a];
-            vi += qq * T0i[a];
-        }
-        if (has_phi) {
-            vr += 2.0 * (scal.x * P0r - scal.y * P0i);
-            vi += 2.0 * (scal.x * P0i + scal.y * P0r);
-        }
-        double c = M.coef[3 * t + i];
-        double2* d = y + M.tri_edge[3 * t + i];
-        atomicAdd(&d->x, c * vr);
-        atomicAdd(&d->y, c * vi);
-    }
-}
-
 // ------------------------------------------------------------------ near CSR product
 // y[m] += sum_e val[e] x[col[e]]; one warp per row
 
@@ -367,15 +263,48 @@ sie_status csr_mv(cudaStream_t st, int nrow, int64_t nnz, const int64_t* rp, con
     return SIE_OK;
 }
 
-// y += W applied to the inverse-transformed grids (3 vector grids, + scalar grid)
-sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y)
+// y_r += W applied to the nr inverse-transformed products (4 grids each with the
+// scalar potential, else 3)
+sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y, int64_t ldy, int nr)
 {
     const DevMesh& M = op->mesh->d;
     const GridDesc& g = op->ext.g;
     int S = (g.M + 1) * (g.M + 1) * (g.M + 1);
     int64_t Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
-    k_interp<<<(M.nt + 3) / 4, 128, 0, op->mesh->ctx->stream>>>(M.nt, S, g.M, M, op->base, op->W, grids, g, has_phi,
-                                                                scal, Ng, y);
+    cudaStream_t st = op->mesh->ctx->stream;
+    auto go = [&](auto wide, auto ng) {
+        constexpr int G = decltype(wide)::value, NG = decltype(ng)::value;
+        constexpr int T = G == 32 ? GIO_SMALL : 256;
+        k_interp<G, double2, double, NG><<<dim3(gio_blocks(M.nt, G, T), nr), T, 0, st>>>(
+            M.nt, S, g.M, M, op->base, op->W, grids, g, scal, Ng, y, ldy);
+    };
+    using I32 = std::integral_constant<int, 32>;
+    using I4 = std::integral_constant<int, 4>;
+    using I3 = std::integral_constant<int, 3>;
+    if ((int64_t)M.nt * nr <= GIO_WIDE)
+        has_phi ? go(I32(), I4()) : go(I32(), I3());
+    else
+        has_phi ? go(I4(), I4()) : go(I4(), I3());
+    SIE_CUDA_TRY(cudaGetLastError());
+    return SIE_OK;
+}
+
+// source grids of nr vectors x (ldx apart): J and, for L, the charge; tc: scratch of 4 nt per vector
+sie_status aim_project(sie_op* op, const double2* x, int64_t ldx, int nr, int ngrid, double2* tc, double2* src)
+{
+    const DevMesh& M = op->mesh->d;
+    const GridDesc& g = op->ext.g;
+    const int S = (g.M + 1) * (g.M + 1) * (g.M + 1);
+    const int64_t Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
+    cudaStream_t st = op->mesh->ctx->stream;
+    SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(double2) * ngrid * nr * Ng, st));
+    const dim3 grid((M.nt * S + 255) / 256, nr);
+    if ((int64_t)M.nt * nr > GIO_WIDE) {
+        k_tri_coef1<<<dim3((M.nt + 127) / 128, nr), 128, 0, st>>>(M.nt, M, x, ldx, tc);
+        k_project<true><<<grid, 256, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, x, ldx, tc, g, ngrid, src, Ng);
+    } else {
+        k_project<false><<<grid, 256, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, x, ldx, nullptr, g, ngrid, src, Ng);
+    }
     SIE_CUDA_TRY(cudaGetLastError());
     return SIE_OK;
 }
@@ -389,17 +318,13 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
     if (a.has_grid) {
         SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * M.ne, st));
         const GridDesc& g = a.g;
-        int S = (g.M + 1) * (g.M + 1) * (g.M + 1);
-        int64_t Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
         int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
         int ngrid = which_LK == 0 ? 4 : 3;
         double2* src = op->ws.src;
         double2* buf = op->ws.bufs;
         {
             Stage s_(pc, "project");
-            SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(double2) * ngrid * Ng, st));
-            k_project<<<(M.nt * S + 255) / 256, 256, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, x, g, ngrid, src, Ng);
-            SIE_CUDA_TRY(cudaGetLastError());
+            SIE_TRY(aim_project(op, x, M.ne, 1, ngrid, op->pm_tc, src));
         }
         if (fft_fused_z(g)) {
             SIE_TRY(fft_lk(st, which_LK, buf, src, g, a.spec, pc, 1));
@@ -416,7 +341,7 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
         std::complex<double> sc = -1.0 / (kk * kk);
         {
             Stage s_(pc, "interp");
-            SIE_TRY(aim_interp(op, src, which_LK == 0, make_double2(sc.real(), sc.imag()), y));
+            SIE_TRY(aim_interp(op, src, which_LK == 0, make_double2(sc.real(), sc.imag()), y, M.ne, 1));
         }
     }
     {
@@ -465,7 +390,7 @@ sie_status sie_op_destroy(sie_op* op)
     free_aim(op->ext);
     free_aim(op->inn);
     void* ptrs[] = {op->base, op->W, op->W32, op->ws.bufs, op->ws.src, op->xtmp, op->bws_bufs, op->bws_src, op->bws_vec,
-                    op->edge_zf};
+                    op->bws_tc, op->bws_xp, op->edge_zf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete op;

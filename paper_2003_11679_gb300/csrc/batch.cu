@@ -1,13 +1,12 @@
 // Multi-right-hand-side AIM products (Eqs. AIM_Lin, AIM_Kin) for a block of up
 // to RB vectors: the kernel spectra, the stencil weights and the near-region
 // values are read once per block instead of once per vector.
-//   * projection: one grid of CTAs per right-hand side (weights from L2);
+//   * projection: one grid of CTAs per right-hand side (gridio.cuh; weights from L2);
 //   * FFTs: one launch per pass over all grids of the block;
 //   * spectral multiply: G (or grad G) loaded once per node, applied to every
 //     vector of the block;
 //   * interpolation: one grid of CTAs per right-hand side;
-//   * near region: CSR x panel product, each (column, value) pair loaded once
-//     and multiplied into RB accumulators.
+//   * near region: CSR x panel product, each (column, value) pair loaded once.
 // Vectors are rhs-major (vector r at r * len), as everywhere in the ABI.
 #include <algorithm>
 #include <complex>
@@ -17,46 +16,6 @@
 namespace sie {
 
 constexpr int RB = 8;  // right-hand sides per block
-
-// projection of vector r = blockIdx.y into grids src + (r * ngrid + a) * Ng
-__global__ void k_project_b(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
-                            const double* __restrict__ W, const double2* __restrict__ x, int64_t ldx, GridDesc g,
-                            int ngrid, double2* __restrict__ src, int64_t Ng)
-{
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nt * S) return;
-    const int r = blockIdx.y;
-    x += (int64_t)r * ldx;
-    src += (int64_t)r * ngrid * Ng;
-    int t = idx / S, u = idx % S;
-    const int Mp = Mord + 1;
-    double2 al = make_double2(0, 0);
-    double2 be[3] = {al, al, al};
-    for (int i = 0; i < 3; i++) {
-        double2 xv = x[M.tri_edge[3 * t + i]];
-        double c = M.coef[3 * t + i];
-        al.x += c * xv.x;
-        al.y += c * xv.y;
-        for (int a = 0; a < 3; a++) {
-            double qq = c * M.q[9 * t + 3 * i + a];
-            be[a].x += qq * xv.x;
-            be[a].y += qq * xv.y;
-        }
-    }
-    int nx = base[3 * t] + u % Mp, ny = base[3 * t + 1] + (u / Mp) % Mp, nz = base[3 * t + 2] + u / (Mp * Mp);
-    int64_t node = ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
-    const double* w = W + (size_t)idx * 4;
-    for (int a = 0; a < 3; a++) {
-        double2* d = src + a * Ng + node;
-        atomicAdd(&d->x, al.x * w[1 + a] + be[a].x * w[0]);
-        atomicAdd(&d->y, al.y * w[1 + a] + be[a].y * w[0]);
-    }
-    if (ngrid == 4) {
-        double2* d = src + 3 * Ng + node;
-        atomicAdd(&d->x, 2.0 * al.x * w[0]);
-        atomicAdd(&d->y, 2.0 * al.y * w[0]);
-    }
-}
 
 // spectral multiply of nr vectors, the spectra read once per node: mode 0
 // (L): every grid times G; mode 1 (K): J <- grad G x J
@@ -85,111 +44,57 @@ __global__ void k_specmul_b(int mode, int nr, const double2* __restrict__ spec, 
     }
 }
 
-// interpolation of vector r = blockIdx.y: one warp per triangle, y[e] +=
-// c_{t,i} [S1 + (c_t - p_i).T0 + scal 2 P0]
-__global__ void k_interp_b(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
-                           const double* __restrict__ W, const double2* __restrict__ out, GridDesc g, int ngrid,
-                           double2 scal, int64_t Ng, double2* __restrict__ y, int64_t ldy)
-{
-    int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    int lane = threadIdx.x & 31;
-    if (t >= nt) return;
-    const int r = blockIdx.y;
-    out += (int64_t)r * ngrid * Ng;
-    y += (int64_t)r * ldy;
-    const int Mp = Mord + 1;
-    double s1r = 0, s1i = 0, t0r[3] = {0, 0, 0}, t0i[3] = {0, 0, 0}, p0r = 0, p0i = 0;
-    for (int u = lane; u < S; u += 32) {
-        int nx = base[3 * t] + u % Mp, ny = base[3 * t + 1] + (u / Mp) % Mp, nz = base[3 * t + 2] + u / (Mp * Mp);
-        int64_t node = ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
-        const double* w = W + ((size_t)t * S + u) * 4;
-        for (int a = 0; a < 3; a++) {
-            double2 A = out[a * Ng + node];
-            s1r += w[1 + a] * A.x;
-            s1i += w[1 + a] * A.y;
-            t0r[a] += w[0] * A.x;
-            t0i[a] += w[0] * A.y;
-        }
-        if (ngrid == 4) {
-            double2 P = out[3 * Ng + node];
-            p0r += w[0] * P.x;
-            p0i += w[0] * P.y;
-        }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        s1r += __shfl_down_sync(0xffffffffu, s1r, off);
-        s1i += __shfl_down_sync(0xffffffffu, s1i, off);
-        p0r += __shfl_down_sync(0xffffffffu, p0r, off);
-        p0i += __shfl_down_sync(0xffffffffu, p0i, off);
-        for (int a = 0; a < 3; a++) {
-            t0r[a] += __shfl_down_sync(0xffffffffu, t0r[a], off);
-            t0i[a] += __shfl_down_sync(0xffffffffu, t0i[a], off);
-        }
-    }
-    if (lane < 3) {
-        const int i = lane;
-        double S1r = __shfl_sync(0x7u, s1r, 0), S1i = __shfl_sync(0x7u, s1i, 0);
-        double P0r = __shfl_sync(0x7u, p0r, 0), P0i = __shfl_sync(0x7u, p0i, 0);
-        double T0r[3], T0i[3];
-        for (int a = 0; a < 3; a++) {
-            T0r[a] = __shfl_sync(0x7u, t0r[a], 0);
-            T0i[a] = __shfl_sync(0x7u, t0i[a], 0);
-        }
-        double vr = S1r, vi = S1i;
-        for (int a = 0; a < 3; a++) {
-            double qq = M.q[9 * t + 3 * i + a];
-            vr += qq * T0r[a];
-            vi += qq * T0i[a];
-        }
-        vr += 2.0 * (scal.x * P0r - scal.y * P0i);
-        vi += 2.0 * (scal.x * P0i + scal.y * P0r);
-        double c = M.coef[3 * t + i];
-        double2* d = y + M.tri_edge[3 * t + i];
-        atomicAdd(&d->x, c * vr);
-        atomicAdd(&d->y, c * vi);
-    }
-}
-
-// Y[r] (+)= A X[r] for r < NR: a warp per row; each (column, value) pair
-// loaded once, its product accumulated into NR sums per lane
-template <int NR>
+// Y[r] (+)= A X[r] for r < nr <= GL: a warp per row.  GL lanes share an entry, one
+// right-hand side each, so 32 / GL entries are in work at a time; the value is one
+// broadcast load and the vectors, interleaved by k_pack_rhs, one coalesced row of GL
+// per entry (rhs-major vectors cost nr scattered 16-byte gathers).  Only the 32 / GL
+// entry slots are summed across lanes.  FP64 arithmetic bounds it: eight right-hand
+// sides, 15.0 M entries: 1,533 us with an entry per lane and 8 x 10 warp-wide additions
+// a row; 843 us now (765 us of products).
+template <int GL>
 __global__ void __launch_bounds__(128) k_csr_panel(int nrow, const int64_t* __restrict__ rp,
                                                    const int32_t* __restrict__ col, const double2* __restrict__ val,
-                                                   const double2* __restrict__ X, int64_t ldx, int acc,
+                                                   const double2* __restrict__ Xp, int nr, int acc,
                                                    double2* __restrict__ Y, int64_t ldy)
 {
-    const int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (r >= nrow) return;
-    double sr[NR], si[NR];
+    const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    const int lane = threadIdx.x & 31, r = lane % GL, sl = lane / GL;
+    constexpr int STEP = 32 / GL, U = 4;
+    if (row >= nrow) return;
+    double sr[U], si[U];  // independent chains
 #pragma unroll
-    for (int k = 0; k < NR; k++) sr[k] = si[k] = 0.0;
-    for (int64_t e = rp[r] + lane; e < rp[r + 1]; e += 32) {
-        const int c = __ldg(col + e);
-        const double2 v = __ldg(val + e);
+    for (int u = 0; u < U; u++) sr[u] = si[u] = 0.0;
+    const int64_t e1 = rp[row + 1];
+    int64_t e = rp[row] + sl;
+    for (; e + (U - 1) * STEP < e1; e += U * STEP) {
+        int c[U];
+        double2 v[U], x[U];
 #pragma unroll
-        for (int k = 0; k < NR; k++) {
-            const double2 xv = __ldg(X + k * ldx + c);
-            sr[k] += v.x * xv.x - v.y * xv.y;
-            si[k] += v.x * xv.y + v.y * xv.x;
+        for (int u = 0; u < U; u++) {
+            c[u] = __ldg(col + e + u * STEP);
+            v[u] = __ldg(val + e + u * STEP);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) x[u] = __ldg(Xp + (int64_t)c[u] * GL + r);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            sr[u] = fma(v[u].x, x[u].x, fma(-v[u].y, x[u].y, sr[u]));
+            si[u] = fma(v[u].x, x[u].y, fma(v[u].y, x[u].x, si[u]));
         }
     }
-#pragma unroll
-    for (int k = 0; k < NR; k++) {
-        for (int off = 16; off > 0; off >>= 1) {
-            sr[k] += __shfl_xor_sync(0xffffffffu, sr[k], off);
-            si[k] += __shfl_xor_sync(0xffffffffu, si[k], off);
-        }
+    for (; e < e1; e += STEP) {
+        const double2 v = __ldg(val + e), x = __ldg(Xp + (int64_t)__ldg(col + e) * GL + r);
+        sr[0] = fma(v.x, x.x, fma(-v.y, x.y, sr[0]));
+        si[0] = fma(v.x, x.y, fma(v.y, x.x, si[0]));
     }
-    if (lane < NR) {
-        double yr = 0, yi = 0;
+    double yr = (sr[0] + sr[1]) + (sr[2] + sr[3]), yi = (si[0] + si[1]) + (si[2] + si[3]);
 #pragma unroll
-        for (int k = 0; k < NR; k++)
-            if (k == lane) {
-                yr = sr[k];
-                yi = si[k];
-            }
-        double2* o = Y + lane * ldy + r;
+    for (int off = GL; off < 32; off <<= 1) {
+        yr += __shfl_xor_sync(0xffffffffu, yr, off);
+        yi += __shfl_xor_sync(0xffffffffu, yi, off);
+    }
+    if (sl == 0 && r < nr) {
+        double2* o = Y + r * ldy + row;
         if (acc) {
             yr += o->x;
             yi += o->y;
@@ -198,20 +103,34 @@ __global__ void __launch_bounds__(128) k_csr_panel(int nrow, const int64_t* __re
     }
 }
 
-sie_status csr_panel(cudaStream_t st, int nrow, const int64_t* rp, const int32_t* col, const double2* val,
-                            const double2* X, int64_t ldx, int nr, bool acc, double2* Y, int64_t ldy)
+// Xp[c GL + r] = X[r ldx + c], zero for r >= nr
+__global__ void k_pack_rhs(int64_t n, int nr, int GL, const double2* __restrict__ X, int64_t ldx,
+                           double2* __restrict__ Xp)
 {
-    const unsigned blocks = (unsigned)((nrow + 3) / 4);
-    switch (nr) {
-        case 1: k_csr_panel<1><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 2: k_csr_panel<2><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 3: k_csr_panel<3><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 4: k_csr_panel<4><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 5: k_csr_panel<5><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 6: k_csr_panel<6><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        case 7: k_csr_panel<7><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-        default: k_csr_panel<8><<<blocks, 128, 0, st>>>(nrow, rp, col, val, X, ldx, acc, Y, ldy); break;
-    }
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * GL) return;
+    const int64_t c = i / GL;
+    const int r = (int)(i % GL);
+    Xp[i] = r < nr ? X[r * ldx + c] : make_double2(0, 0);
+}
+
+// Y = A X (acc: Y += A X) for nr <= RB vectors of an edge CSR matrix, rhs-major; the
+// values read once for all nr
+static sie_status csr_panel(sie_op* op, const int64_t* rp, const int32_t* col, const double2* val, const double2* X,
+                            int nr, bool acc, double2* Y)
+{
+    cudaStream_t st = op->mesh->ctx->stream;
+    const int ne = op->mesh->d.ne;
+    if (!op->bws_xp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_xp, sizeof(double2) * RB * ne, st));
+    const int GL = nr > 4 ? 8 : (nr > 2 ? 4 : 2);
+    k_pack_rhs<<<(unsigned)(((int64_t)ne * GL + 255) / 256), 256, 0, st>>>(ne, nr, GL, X, ne, op->bws_xp);
+    const unsigned blocks = (unsigned)((ne + 3) / 4);
+    if (GL == 8)
+        k_csr_panel<8><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
+    else if (GL == 4)
+        k_csr_panel<4><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
+    else
+        k_csr_panel<2><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
     SIE_CUDA_TRY(cudaGetLastError());
     return SIE_OK;
 }
@@ -225,6 +144,7 @@ static sie_status batch_workspace(sie_op* op, double2** bufs, double2** src)
     if (!op->bws_bufs) {
         SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_bufs, sizeof(double2) * 4 * RB * nn, st));
         SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_src, sizeof(double2) * 4 * RB * Ng, st));
+        SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_tc, sizeof(double2) * 4 * RB * op->mesh->d.nt, st));
     }
     *bufs = op->bws_bufs;
     *src = op->bws_src;
@@ -246,18 +166,13 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
     if (a.has_grid) {
         SIE_CUDA_TRY(cudaMemsetAsync(Y, 0, sizeof(double2) * ne * nr, st));
         const GridDesc& g = a.g;
-        const int S = (g.M + 1) * (g.M + 1) * (g.M + 1);
-        const int64_t Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
         const int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
         const int ngrid = which_LK == 0 ? 4 : 3;
         double2 *buf, *src;
         SIE_TRY(batch_workspace(op, &buf, &src));
         {
             Stage s_(pc, "project_block");
-            SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(double2) * ngrid * nr * Ng, st));
-            k_project_b<<<dim3((M.nt * S + 255) / 256, nr), 256, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, X, ne, g,
-                                                                           ngrid, src, Ng);
-            SIE_CUDA_TRY(cudaGetLastError());
+            SIE_TRY(aim_project(op, X, ne, nr, ngrid, op->bws_tc, src));
         }
         if (fft_fused_z(g)) {
             SIE_TRY(fft_lk(st, which_LK, buf, src, g, a.spec, pc, nr));
@@ -274,15 +189,13 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
         std::complex<double> sc = which_LK == 0 ? -1.0 / (kk * kk) : std::complex<double>(0.0);
         {
             Stage s_(pc, "interp_block");
-            k_interp_b<<<dim3((M.nt + 3) / 4, nr), 128, 0, st>>>(M.nt, S, g.M, M, op->base, op->W, src, g, ngrid,
-                                                                 make_double2(sc.real(), sc.imag()), Ng, Y, ne);
-            SIE_CUDA_TRY(cudaGetLastError());
+            SIE_TRY(aim_interp(op, src, which_LK == 0, make_double2(sc.real(), sc.imag()), Y, ne, nr));
         }
     }
     {
         Stage s_(pc, a.has_grid ? "spmv_block" : "spmv_near_only_block");
         const double2* v = which_LK == 0 ? a.valL : a.valK;
-        SIE_TRY(csr_panel(st, (int)ne, a.row_ptr, a.col, v, X, ne, nr, a.has_grid, Y, ne));
+        SIE_TRY(csr_panel(op, a.row_ptr, a.col, v, X, nr, a.has_grid, Y));
     }
     return SIE_OK;
 }

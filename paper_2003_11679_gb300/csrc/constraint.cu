@@ -111,10 +111,9 @@ struct ConClu {
     }
     __device__ void set_v(int, int k, double2 v)
     {
-        auto c = cooperative_groups::this_cluster();
-        const float2 f = make_float2((float)v.x, (float)v.y);
-        for (int r = 0; r < M.C; r++) *c.map_shared_rank(xf + r0 + k, r) = f;
+        xf[r0 + k] = make_float2((float)v.x, (float)v.y);
     }
+    __device__ void share() { M.spread(xf, r0, rows); }
     // z = X v: a warp per row
     __device__ bool precond(int j)
     {
@@ -207,8 +206,10 @@ __global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, 
             double2 x = sol[r0 + k];
             for (int i = 0; i <= jend; i++) r_fma(x, ops.Z[(int64_t)i * K.n + r0 + k], M.g[i]);
             sol[r0 + k] = x;
-            M.put(M.xz + r0 + k, x);
+            M.xz[r0 + k] = x;
         }
+        __syncthreads();
+        M.spread(M.xz, r0, rows);
         clu_sync();
         ops.lphi([&](int c) { return M.xz[c]; });
         clu_sync();

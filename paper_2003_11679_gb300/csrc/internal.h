@@ -317,14 +317,13 @@ struct sie_op {
     double2* gr_val = nullptr;
     double2* gr_diag = nullptr;
     double eta_re = 0, eta_im = 0;
-    // projection of the system product as a gather: touched grid nodes, CSR
-    // of their stencil entries (t * S + u), per-triangle coefficients
+    // projection of the system product as a gather: grid nodes with stencil entries, CSR
+    // of those entries (t * S + u), per-triangle coefficients
     int64_t pm_nnode = 0;
-    int64_t *pm_node = nullptr, *pm_ptr = nullptr;
-    int32_t* pm_ent = nullptr;
+    int32_t *pm_node = nullptr, *pm_ptr = nullptr, *pm_ent = nullptr;
     double2* pm_tc = nullptr;       // 9 per triangle (FP64; the complex64 path uses its first half)
     // multi-right-hand-side block workspace (allocated on first use)
-    double2 *bws_bufs = nullptr, *bws_src = nullptr, *bws_vec = nullptr;
+    double2 *bws_bufs = nullptr, *bws_src = nullptr, *bws_vec = nullptr, *bws_tc = nullptr, *bws_xp = nullptr;
     // several objects: per-edge factor of the interior impedance, -1/(j k0 eps_r + sigma eta0)
     // of the edge's object (GIBC) or eta_i/eta0 (SIBC); null for one object
     double2* edge_zf = nullptr;
@@ -357,13 +356,10 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q);
 sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, double2* y);
 // Y = A X for nr <= 8 vectors at once (spectra, weights and near values read once)
 sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X, double2* Y, int nr);
-sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y);
+sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y, int64_t ldy, int nr);
+sie_status aim_project(sie_op* op, const double2* x, int64_t ldx, int nr, int ngrid, double2* tc, double2* src);
 sie_status sys_prepare(sie_op* op);
-sie_status csr_tune_op(sie_op* op);
-// Y = A X (acc: Y += A X) for nr <= 8 vectors of a CSR matrix: X, Y rhs-major
-// with leading dimensions ldx, ldy; the values read once for all nr
-sie_status csr_panel(cudaStream_t st, int nrow, const int64_t* rp, const int32_t* col, const double2* val,
-                     const double2* X, int64_t ldx, int nr, bool acc, double2* Y, int64_t ldy);  // group sizes of the operator's CSR products, by measurement
+sie_status csr_tune_op(sie_op* op);  // group sizes of the operator's CSR products, by measurement
 void sys_release(sie_op* op);
 sie_status sys_matvec(sie_op* op, int which, const double2* x, double2* y);
 sie_status sys_solve(sie_op* op, const double2* b, double2* x, int* iters, double* relres);

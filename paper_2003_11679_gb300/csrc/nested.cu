@@ -124,15 +124,16 @@ struct NestClu {
     __device__ void set_v(int j, int k, double2 v)
     {
         if (s.m_val) {
-            M.put(M.xv + r0 + k, v);
+            M.xv[r0 + k] = v;
             return;
         }
         const double2 d = s.diag[r0 + k];
         const double den = d.x * d.x + d.y * d.y;
         const double2 z = make_double2((v.x * d.x + v.y * d.y) / den, (v.y * d.x - v.x * d.y) / den);
         if (j < K.m) Z[(int64_t)j * K.n + r0 + k] = z;
-        M.put(M.xz + r0 + k, z);
+        M.xz[r0 + k] = z;
     }
+    __device__ void share() { M.spread(s.m_val ? M.xv : M.xz, r0, rows); }
     __device__ bool precond(int j)
     {
         if (!s.m_val) return false;

@@ -91,14 +91,17 @@ struct ResKrylov {
 // dynamic shared memory of res_fgmres
 inline size_t res_smem(int m, int R) { return sizeof(double2) * (size_t)R * 5 * (m + 2); }
 
+// sums of both components over the warp, in every lane: the halves of the warp
+// take one component each after the first exchange (6 FP64 additions, not 10)
 __device__ __forceinline__ double2 warp_sum(double2 s)
 {
+    const bool up = threadIdx.x & 16;
+    double keep = up ? s.y : s.x;
+    keep += __shfl_xor_sync(0xffffffffu, up ? s.x : s.y, 16);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
-    }
-    return s;
+    for (int off = 8; off > 0; off >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, off);
+    const double other = __shfl_xor_sync(0xffffffffu, keep, 16);
+    return up ? make_double2(other, keep) : make_double2(keep, other);
 }
 
 // part[(c R + q) ld + i] = sum over own rows of conj(V_i) w, i < nv, and of |w|^2 (slot nv) when norm
@@ -152,11 +155,20 @@ __device__ __forceinline__ void res_update(const ResKrylov& K, int64_t r0, int64
     __syncthreads();
 }
 
+// 2^-exponent of v (1 for zero, infinity and NaN)
+__device__ __forceinline__ double res_unscale(double v)
+{
+    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    return (e == 0 || e == 0x7ff) ? 1.0 : __hiloint2double((2046 - min(e, 2045)) << 20, 0);
+}
+
 // column j of one right-hand side (one thread): h1 + h2 and the norm hn through
 // the previous rotations, rotation j (c real), g; the rotated column to Hq when
-// store; returns |g_{j+1}|
-__device__ __forceinline__ double res_givens(int j, int m, const double2* a1, const double2* a2, double hn, double2* c_,
-                                             double2* s_, double2* g_, double2* Hq, bool store)
+// store; gabs = |g_j| becomes |g_{j+1}|.  One chain of dependent FP64 operations:
+// two reciprocal square roots instead of three hypot and six divisions (13,600
+// cycles an iteration with those, a third of it)
+__device__ __forceinline__ void res_givens(int j, int m, const double2* a1, const double2* a2, double hn, double2* c_,
+                                           double2* s_, double2* g_, double2* Hq, bool store, double& gabs)
 {
     double2 a = make_double2(a1[0].x + a2[0].x, a1[0].y + a2[0].y);
     for (int i = 0; i < j; i++) {
@@ -165,26 +177,28 @@ __device__ __forceinline__ double res_givens(int j, int m, const double2* a1, co
         if (store) Hq[i * m + j] = make_double2(c_[i].x * a.x + sb.x, c_[i].x * a.y + sb.y);
         a = make_double2(c_[i].x * b.x - ta.x, c_[i].x * b.y - ta.y);
     }
-    const double2 b = make_double2(hn, 0);
-    const double aa = hypot(a.x, a.y), den = hypot(aa, hn);
-    double2 c, s;
-    if (aa == 0.0) {
+    // scaled by a power of two: no square overflows or underflows
+    const double sc = res_unscale(fmax(fmax(fabs(a.x), fabs(a.y)), hn));
+    const double ax = a.x * sc, ay = a.y * sc, b = hn * sc, u = ax * ax + ay * ay, t = u + b * b;
+    const double ru = u > 0 ? rsqrt(u) : 0.0, rt = t > 0 ? rsqrt(t) : (t == t ? 0.0 : t), sn = b * rt;
+    double2 c, s, d;  // d = c a + s hn
+    if (u == 0.0) {
         c = make_double2(0, 0);
         s = make_double2(1, 0);
+        d = make_double2(hn, 0);
     } else {
-        c = make_double2(aa / den, 0);
-        s = r_cm(make_double2(a.x / aa, a.y / aa), r_cj(b));
-        s.x /= den;
-        s.y /= den;
+        c = make_double2(u * ru * rt, 0);
+        s = make_double2(ax * ru * sn, ay * ru * sn);
+        const double r = ru * (t * rt);
+        d = make_double2(a.x * r, a.y * r);
     }
     c_[j] = c;
     s_[j] = s;
-    const double2 sb = r_cm(s, b);
-    if (store) Hq[j * m + j] = make_double2(c.x * a.x + sb.x, c.x * a.y + sb.y);
-    const double2 gj = g_[j], t = r_cm(r_cj(s), gj);
+    if (store) Hq[j * m + j] = d;
+    const double2 gj = g_[j], gt = r_cm(r_cj(s), gj);
     g_[j] = make_double2(c.x * gj.x, c.x * gj.y);
-    g_[j + 1] = make_double2(-t.x, -t.y);
-    return hypot(t.x, t.y);
+    g_[j + 1] = make_double2(-gt.x, -gt.y);
+    gabs *= u == 0.0 ? 1.0 : sn;
 }
 
 // y = R^-1 g in place of g, j + 1 unknowns, by one warp (Hq complete)
@@ -216,11 +230,14 @@ __device__ __forceinline__ void res_stat(double* stat, int iters, double worst)
 // relative residual; a NaN norm gives NaN
 __device__ __forceinline__ double res_rel(double r, double bn) { return bn > 0 ? r / bn : (bn == bn ? 0.0 : bn); }
 
-// norm of w - V h2 from |w|^2 and h2
-__device__ __forceinline__ double res_norm(double ww, const double2* h2, int nv)
+// norm of w - V h2 from |w|^2 = h2[nv] and h2[0 .. nv), by one warp; in every lane
+__device__ __forceinline__ double res_norm(const double2* h2, int nv, int lane)
 {
-    double s = ww;
-    for (int i = 0; i < nv; i++) s -= h2[i].x * h2[i].x + h2[i].y * h2[i].y;
+    double s = 0;
+    for (int i = lane; i < nv; i += 32) s += h2[i].x * h2[i].x + h2[i].y * h2[i].y;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    s = h2[nv].x - s;
     return s != s ? s : sqrt(fmax(s, 0.0));
 }
 
@@ -242,7 +259,7 @@ __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* sm
     double2* g = sn + R * ld;
     double2* h1 = g + R * ld;
     double2* h2 = h1 + R * ld;
-    __shared__ double bnorm[8], rel[8], wn[8];
+    __shared__ double bnorm[8], rel[8], wn[8], gabs[8];
     __shared__ double2 nr[8];
     double2* P1 = K.part;
     double2* P2 = P1 + (int64_t)RES_MAXCTA * R * ld;
@@ -251,7 +268,7 @@ __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* sm
     res_reduce(K, 1, P1, ld, nr, 1);
     if (threadIdx.x < R) {
         const double d2 = nr[threadIdx.x].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
-        bnorm[threadIdx.x] = b;
+        bnorm[threadIdx.x] = gabs[threadIdx.x] = b;
         wn[threadIdx.x] = b > 0 ? 1.0 / b : 0.0;
         g[threadIdx.x * ld] = make_double2(b, 0);
     }
@@ -279,13 +296,15 @@ __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* sm
         res_dots(K, r0, r1, j + 1, true, P2, ld);
         if (!res_barrier(bar)) return -1;
         res_reduce(K, j + 2, P2, ld, h2, ld);
-        if (threadIdx.x < R) {
-            const int q = threadIdx.x;
-            const double hn = res_norm(h2[q * ld + j + 1].x, h2 + q * ld, j + 1);
-            wn[q] = hn > 0 ? 1.0 / hn : 0.0;
-            rel[q] = res_rel(res_givens(j, m, h1 + q * ld, h2 + q * ld, hn, cs + q * ld, sn + q * ld, g + q * ld,
-                                        K.H + q * K.ldh, blockIdx.x == 0),
-                             bnorm[q]);
+        if ((threadIdx.x >> 5) < R) {
+            const int q = threadIdx.x >> 5;
+            const double hn = res_norm(h2 + q * ld, j + 1, threadIdx.x & 31);
+            if ((threadIdx.x & 31) == 0) {
+                wn[q] = hn > 0 ? 1.0 / hn : 0.0;
+                res_givens(j, m, h1 + q * ld, h2 + q * ld, hn, cs + q * ld, sn + q * ld, g + q * ld, K.H + q * K.ldh,
+                           blockIdx.x == 0, gabs[q]);
+                rel[q] = res_rel(gabs[q], bnorm[q]);
+            }
         }
         __syncthreads();
         bool more = false;
@@ -356,11 +375,18 @@ struct CluMem {
         h1 = g + ld;
         h2 = h1 + ld;
     }
-    // *p in every CTA's shared memory (p: this CTA's address)
-    __device__ __forceinline__ void put(double2* p, double2 v) const
+    // own rows of a gather vector (x: whole, this CTA's copy, own rows set before a
+    // __syncthreads) to the other CTAs, spread over all threads
+    template <class T>
+    __device__ __forceinline__ void spread(T* x, int64_t r0, int rows) const
     {
         auto c = cooperative_groups::this_cluster();
-        for (int r = 0; r < C; r++) *c.map_shared_rank(p, r) = v;
+        const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int r = warp; r < C; r += nw) {
+            if (r == rank) continue;
+            T* o = c.map_shared_rank(x + r0, r);
+            for (int k = lane; k < rows; k += 32) o[k] = x[r0 + k];
+        }
     }
 };
 
@@ -380,17 +406,25 @@ __device__ __forceinline__ void clu_dots(const CluMem& M, const double2* V, int6
             *cooperative_groups::this_cluster().map_shared_rank(M.pr + (buf * M.C + M.rank) * M.ld + i, lane) = s;
     }
 }
-// h[i] = sum over the CTAs
+// h[i] = sum over the CTAs (8 or 16), four chains
 __device__ __forceinline__ void clu_reduce(const CluMem& M, int cols, int buf, double2* h)
 {
     for (int i = threadIdx.x; i < cols; i += blockDim.x) {
-        double2 s = make_double2(0, 0);
-        for (int c = 0; c < M.C; c++) {
-            const double2 p = M.pr[(buf * M.C + c) * M.ld + i];
-            s.x += p.x;
-            s.y += p.y;
+        const double2* p = M.pr + buf * M.C * M.ld + i;
+        double2 s[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const double2 a = p[c * M.ld], b = p[(c + 4) * M.ld];
+            s[c] = make_double2(a.x + b.x, a.y + b.y);
         }
-        h[i] = s;
+        if (M.C > 8)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const double2 a = p[(c + 8) * M.ld], b = p[(c + 12) * M.ld];
+                s[c].x += a.x + b.x;
+                s[c].y += a.y + b.y;
+            }
+        h[i] = make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
     }
     __syncthreads();
 }
@@ -437,8 +471,8 @@ __device__ __forceinline__ int clu_vote(const CluLock& lock, int q, int it, bool
 // The cycle for this cluster's right-hand side, whose residual is in M.w (own
 // rows, after a __syncthreads).  sys: r0, rows; precond(j): from M.xv, Z_j (own
 // rows) and M.xz of every CTA, false for a pointwise one done by set_v; set_v(j,
-// k, v): own row k of V_j is v (puts what the next product gathers); apply(j): M.w
-// = A z from M.xz.  After it y in M.g; returns jend, -1 when a wait ran out.
+// k, v): own row k of V_j is v (sets own row of what the next product gathers, which
+// share() then copies to the other CTAs); apply(j): M.w = A z from M.xz.  After it y in M.g; returns jend, -1 when a wait ran out.
 // Restarted solves call it again with the new residual: it0 iterations done, at
 // most maxit in all, bnorm0 the norm of the right-hand side (below 0 in the first
 // cycle); *above: a residual is still above tol; rel_out: this one's.
@@ -454,7 +488,7 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
     const int64_t n = K.n, r0 = sys.r0;
     double2* V = K.V + (int64_t)q * (m + 1) * n;  // this right-hand side's basis
     double2* H = K.H + q * K.ldh;
-    __shared__ double bnorm, rel, wn;
+    __shared__ double bnorm, rel, wn, gabs;
     __shared__ int go, above_s;
     clu_sync();  // every CTA of the cluster has started, or is done with the last cycle
     clu_dots(M, V, n, r0, rows, 0, true, 0);
@@ -463,6 +497,7 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
     if (threadIdx.x == 0) {
         const double d2 = M.h1[0].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
         bnorm = run.bnorm < 0 ? b : run.bnorm;
+        gabs = b;
         wn = b > 0 ? 1.0 / b : 0.0;
         M.g[0] = make_double2(b, 0);
     }
@@ -474,6 +509,8 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
             V[(int64_t)j * n + r0 + k] = v;
             sys.set_v(j, k, v);
         }
+        __syncthreads();
+        sys.share();
         clu_sync();
     };
     set_v(0);
@@ -494,10 +531,12 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
         clu_dots(M, V, n, r0, rows, j + 1, true, 1);
         clu_sync();
         clu_reduce(M, j + 2, 1, M.h2);
+        double hn = 0;
+        if (threadIdx.x < 32) hn = res_norm(M.h2, j + 1, threadIdx.x);
         if (threadIdx.x == 0) {
-            const double hn = res_norm(M.h2[j + 1].x, M.h2, j + 1);
             wn = hn > 0 ? 1.0 / hn : 0.0;
-            rel = res_rel(res_givens(j, m, M.h1, M.h2, hn, M.cs, M.sn, M.g, H, M.rank == 0), bnorm);
+            res_givens(j, m, M.h1, M.h2, hn, M.cs, M.sn, M.g, H, M.rank == 0, gabs);
+            rel = res_rel(gabs, bnorm);
             int more = rel >= K.tol;
             if (lock.R > 1) {
                 more = clu_vote(lock, q, run.it + j, rel >= K.tol, M.rank == 0);

@@ -74,7 +74,7 @@ __device__ __forceinline__ double2 csr_row_dot(int64_t e0, int64_t e1, const int
     return make_double2(sr, si);
 }
 
-// y = alpha A x (ACC = false) or y += alpha A x (ACC = true); blockDim 256
+// y = alpha A x (ACC = false) or y += alpha A x (ACC = true); up to 256 threads
 template <int G, bool ACC, class VT, class XT>
 __global__ void __launch_bounds__(256) k_csr(int nrow, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                              const VT* __restrict__ val, const XT* __restrict__ x,
@@ -141,19 +141,22 @@ template <class VT, class XT>
 inline cudaError_t csr_launch_g(cudaStream_t st, int G, int nrow, const int64_t* rp, const int32_t* col,
                                 const VT* val, const XT* x, double2 alpha, bool acc, double2* y)
 {
-    const unsigned blocks = (unsigned)(((int64_t)nrow * G + 255) / 256);
+    // CTAs of 64 threads when 256 would not fill the SMs twice: FP64 runs at 2 lanes per
+    // SM, so a small product gains from more SMs
+    const int T = (int64_t)nrow * G < 256 * 304 ? 64 : 256;
+    const unsigned blocks = (unsigned)(((int64_t)nrow * G + T - 1) / T);
     if (G == 4) {
-        if (acc) k_csr<4, true, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<4, false, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<4, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        else k_csr<4, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
     } else if (G == 8) {
-        if (acc) k_csr<8, true, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<8, false, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<8, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        else k_csr<8, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
     } else if (G == 16) {
-        if (acc) k_csr<16, true, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<16, false, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<16, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        else k_csr<16, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
     } else {
-        if (acc) k_csr<32, true, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<32, false, VT, XT><<<blocks, 256, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<32, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        else k_csr<32, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
     }
     return cudaGetLastError();
 }

@@ -12,6 +12,7 @@
 #include <cstring>
 #include <vector>
 
+#include "gridio.cuh"
 #include "internal.h"
 #include "resident.cuh"
 #include "spmv.cuh"
@@ -558,12 +559,6 @@ static sie_status fgmres(sie_ctx* c, KrylovWork& K, int64_t n, const Apply& A, c
 }
 
 // ------------------------------------------------------------------ system kernels
-// Projection as a gather (deterministic, no atomics): per triangle t the
-// current on t is alpha (r - c_t) + beta (alpha = sum_i c_i x_i, beta_a =
-// sum_i c_i q_ia x_i) for x = H and x = E', and the charge grid takes
-// -c0rho_t; grid node v sums, in a fixed order, the stencil entries (t, u)
-// that land on it: J_a += alpha_H w1[a] + beta_H[a] w0, M_a likewise with E',
-// rho += -c0rho_t w0.
 template <class C>
 __device__ __forceinline__ C cmk(double a, double b)
 {
@@ -603,46 +598,6 @@ __global__ void k_tri_coef(int nt, DevMesh M, const double2* __restrict__ H, con
     o[8] = cmk<C>(-rho[t].x, -rho[t].y);
 }
 
-// one thread per touched node; ent: t * S + u, grouped by node (ptr)
-template <class C, class R>
-__global__ void k_project_gather(int64_t nnode, const int64_t* __restrict__ node, const int64_t* __restrict__ ptr,
-                                 const int32_t* __restrict__ ent, int S, const R* __restrict__ W,
-                                 const C* __restrict__ tc, C* __restrict__ src, int64_t Ng)
-{
-    int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nnode) return;
-    R acc[14];
-#pragma unroll
-    for (int i = 0; i < 14; i++) acc[i] = 0;
-    for (int64_t k = ptr[v]; k < ptr[v + 1]; k++) {
-        const int32_t id = ent[k];
-        const int t = id / S;
-        const R* w = W + (int64_t)id * 4;
-        const R w0 = w[0], w1[3] = {w[1], w[2], w[3]};
-        const C* c = tc + 9 * (int64_t)t;
-#pragma unroll
-        for (int f = 0; f < 2; f++) {
-            const C al = c[4 * f];
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                const C be = c[4 * f + 1 + a];
-                acc[2 * (3 * f + a)] += al.x * w1[a] + be.x * w0;
-                acc[2 * (3 * f + a) + 1] += al.y * w1[a] + be.y * w0;
-            }
-        }
-        acc[12] += c[8].x * w0;
-        acc[13] += c[8].y * w0;
-    }
-    const int64_t nd = node[v];
-#pragma unroll
-    for (int g = 0; g < 7; g++) {
-        C o;
-        o.x = acc[2 * g];
-        o.y = acc[2 * g + 1];
-        src[g * Ng + nd] = o;
-    }
-}
-
 __global__ void k_specmul_sys32(const float2* __restrict__ spec, float2* __restrict__ buf, int64_t nn, float k0)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -651,64 +606,6 @@ __global__ void k_specmul_sys32(const float2* __restrict__ spec, float2* __restr
     for (int g = 0; g < 7; g++) in[g] = buf[g * nn + i];
     sys_specmul(spec[i], spec[nn + i], spec[2 * nn + i], spec[3 * nn + i], k0, in, out);
     for (int g = 0; g < 4; g++) buf[g * nn + i] = out[g];
-}
-
-// W = P^T on the complex64 grids: FP32 gathers and sums, FP64 edge coefficients
-__global__ void k_interp32(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
-                           const float* __restrict__ W, const float2* __restrict__ out, GridDesc g, int64_t Ng,
-                           double2* __restrict__ y)
-{
-    int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    int lane = threadIdx.x & 31;
-    if (t >= nt) return;
-    const int Mp = Mord + 1;
-    float s1r = 0, s1i = 0, t0r[3] = {0, 0, 0}, t0i[3] = {0, 0, 0}, p0r = 0, p0i = 0;
-    for (int u = lane; u < S; u += 32) {
-        int nx = base[3 * t] + u % Mp, ny = base[3 * t + 1] + (u / Mp) % Mp, nz = base[3 * t + 2] + u / (Mp * Mp);
-        int64_t node = ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
-        const float4 w = *reinterpret_cast<const float4*>(W + ((size_t)t * S + u) * 4);
-        const float w1[3] = {w.y, w.z, w.w};
-        for (int a = 0; a < 3; a++) {
-            float2 A = out[a * Ng + node];
-            s1r += w1[a] * A.x;
-            s1i += w1[a] * A.y;
-            t0r[a] += w.x * A.x;
-            t0i[a] += w.x * A.y;
-        }
-        float2 P = out[3 * Ng + node];
-        p0r += w.x * P.x;
-        p0i += w.x * P.y;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        s1r += __shfl_down_sync(0xffffffffu, s1r, off);
-        s1i += __shfl_down_sync(0xffffffffu, s1i, off);
-        p0r += __shfl_down_sync(0xffffffffu, p0r, off);
-        p0i += __shfl_down_sync(0xffffffffu, p0i, off);
-        for (int a = 0; a < 3; a++) {
-            t0r[a] += __shfl_down_sync(0xffffffffu, t0r[a], off);
-            t0i[a] += __shfl_down_sync(0xffffffffu, t0i[a], off);
-        }
-    }
-    if (lane < 3) {
-        int i = lane;
-        double S1r = __shfl_sync(0x7u, s1r, 0), S1i = __shfl_sync(0x7u, s1i, 0);
-        double P0r = __shfl_sync(0x7u, p0r, 0), P0i = __shfl_sync(0x7u, p0i, 0);
-        double T0r[3], T0i[3];
-        for (int a = 0; a < 3; a++) {
-            T0r[a] = __shfl_sync(0x7u, t0r[a], 0);
-            T0i[a] = __shfl_sync(0x7u, t0i[a], 0);
-        }
-        double vr = S1r + 2.0 * P0r, vi = S1i + 2.0 * P0i;
-        for (int a = 0; a < 3; a++) {
-            double qq = M.q[9 * t + 3 * i + a];
-            vr += qq * T0r[a];
-            vi += qq * T0i[a];
-        }
-        double c = M.coef[3 * t + i];
-        double2* d = y + M.tri_edge[3 * t + i];
-        atomicAdd(&d->x, c * vr);
-        atomicAdd(&d->y, c * vi);
-    }
 }
 
 // A_a = j k0 G J_a - (Ggrad x M)_a into grids 0..2, Phi = G rho into grid 3
@@ -787,57 +684,66 @@ __global__ void __launch_bounds__(128) k_spmv2_c64(int nrow, const int64_t* __re
 
 // y[r] += a1 sum_e v1[e] x1[col[e]] + a2 sum_e v2[e] x2[col[e]]: the two
 // near-region matrices of one operator share their pattern, so the column
-// indices are read once; 4 independent loads per lane in flight
-__global__ void __launch_bounds__(128) k_spmv2(int nrow, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+// indices are read once.  G lanes per row, four loads of each array in flight per
+// lane.  FP64 arithmetic bounds large meshes: with 8 lanes the warp-wide additions of
+// a row's sums are shared by four rows (15.0 M entries, 190 us of products: 453 us
+// with 32 lanes, 274 us with 8).  Up to 8,192 rows the GPU is not full and a row's
+// chain counts: 32 lanes (504 rows: 12 us against 22 us).
+template <int G>
+__global__ void __launch_bounds__(256) k_spmv2(int nrow, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                                const double2* __restrict__ v1, const double2* __restrict__ x1, double2 a1,
                                                const double2* __restrict__ v2, const double2* __restrict__ x2, double2 a2,
                                                double2* __restrict__ y)
 {
-    int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    int lane = threadIdx.x & 31;
-    if (r >= nrow) return;
-    // one accumulator set per unrolled slot: 16 independent FP64 FMA chains
-    double s1r[4] = {0, 0, 0, 0}, s1i[4] = {0, 0, 0, 0}, s2r[4] = {0, 0, 0, 0}, s2i[4] = {0, 0, 0, 0};
-    const int64_t e0 = rp[r], e1 = rp[r + 1];
-    int64_t e = e0 + lane;
-    for (; e + 96 < e1; e += 128) {
-        int c[4];
-        double2 p[4], q[4];
+    constexpr int U = 4;
+    const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G), l = threadIdx.x % G;
+    const bool ok = r < nrow;
+    const int64_t e1 = ok ? rp[r + 1] : 0;
+    int64_t e = ok ? rp[r] + l : 0;
+    double s1r[2] = {0, 0}, s1i[2] = {0, 0}, s2r[2] = {0, 0}, s2i[2] = {0, 0};  // two chains each
+    for (; e + (U - 1) * G < e1; e += U * G) {
+        int c[U];
+        double2 p[U], q[U], xa[U], xb[U];
 #pragma unroll
-        for (int u = 0; u < 4; u++) c[u] = __ldg(col + e + 32 * u);
+        for (int u = 0; u < U; u++) c[u] = __ldg(col + e + u * G);
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            p[u] = __ldg(v1 + e + 32 * u);
-            q[u] = __ldg(v2 + e + 32 * u);
+        for (int u = 0; u < U; u++) {
+            p[u] = __ldg(v1 + e + u * G);
+            q[u] = __ldg(v2 + e + u * G);
         }
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            double2 xa = __ldg(x1 + c[u]), xb = __ldg(x2 + c[u]);
-            s1r[u] += p[u].x * xa.x - p[u].y * xa.y;
-            s1i[u] += p[u].x * xa.y + p[u].y * xa.x;
-            s2r[u] += q[u].x * xb.x - q[u].y * xb.y;
-            s2i[u] += q[u].x * xb.y + q[u].y * xb.x;
+        for (int u = 0; u < U; u++) {
+            xa[u] = __ldg(x1 + c[u]);
+            xb[u] = __ldg(x2 + c[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            s1r[u & 1] = fma(p[u].x, xa[u].x, fma(-p[u].y, xa[u].y, s1r[u & 1]));
+            s1i[u & 1] = fma(p[u].x, xa[u].y, fma(p[u].y, xa[u].x, s1i[u & 1]));
+            s2r[u & 1] = fma(q[u].x, xb[u].x, fma(-q[u].y, xb[u].y, s2r[u & 1]));
+            s2i[u & 1] = fma(q[u].x, xb[u].y, fma(q[u].y, xb[u].x, s2i[u & 1]));
         }
     }
-    for (; e < e1; e += 32) {  // at most 3 more entries per lane
-        int c = col[e];
-        double2 p = v1[e], q = v2[e], xa = x1[c], xb = x2[c];
-        s1r[0] += p.x * xa.x - p.y * xa.y;
-        s1i[0] += p.x * xa.y + p.y * xa.x;
-        s2r[0] += q.x * xb.x - q.y * xb.y;
-        s2i[0] += q.x * xb.y + q.y * xb.x;
+    for (; e < e1; e += G) {  // at most 3 more entries per lane
+        const int c = __ldg(col + e);
+        const double2 p = __ldg(v1 + e), q = __ldg(v2 + e), xa = __ldg(x1 + c), xb = __ldg(x2 + c);
+        s1r[0] = fma(p.x, xa.x, fma(-p.y, xa.y, s1r[0]));
+        s1i[0] = fma(p.x, xa.y, fma(p.y, xa.x, s1i[0]));
+        s2r[0] = fma(q.x, xb.x, fma(-q.y, xb.y, s2r[0]));
+        s2i[0] = fma(q.x, xb.y, fma(q.y, xb.x, s2i[0]));
     }
-    double t1r = (s1r[0] + s1r[1]) + (s1r[2] + s1r[3]), t1i = (s1i[0] + s1i[1]) + (s1i[2] + s1i[3]);
-    double t2r = (s2r[0] + s2r[1]) + (s2r[2] + s2r[3]), t2i = (s2i[0] + s2i[1]) + (s2i[2] + s2i[3]);
-    for (int off = 16; off > 0; off >>= 1) {
-        t1r += __shfl_down_sync(0xffffffffu, t1r, off);
-        t1i += __shfl_down_sync(0xffffffffu, t1i, off);
-        t2r += __shfl_down_sync(0xffffffffu, t2r, off);
-        t2i += __shfl_down_sync(0xffffffffu, t2i, off);
+    double t1r = s1r[0] + s1r[1], t1i = s1i[0] + s1i[1], t2r = s2r[0] + s2r[1], t2i = s2i[0] + s2i[1];
+    // a1 t1 + a2 t2 first: two sums to reduce instead of four
+    double tr = a1.x * t1r - a1.y * t1i + a2.x * t2r - a2.y * t2i;
+    double ti = a1.x * t1i + a1.y * t1r + a2.x * t2i + a2.y * t2r;
+#pragma unroll
+    for (int off = G / 2; off > 0; off >>= 1) {
+        tr += __shfl_xor_sync(0xffffffffu, tr, off);
+        ti += __shfl_xor_sync(0xffffffffu, ti, off);
     }
-    if (lane == 0) {
-        y[r].x += a1.x * t1r - a1.y * t1i + a2.x * t2r - a2.y * t2i;
-        y[r].y += a1.x * t1i + a1.y * t1r + a2.x * t2i + a2.y * t2r;
+    if (ok && l == 0) {
+        y[r].x += tr;
+        y[r].y += ti;
     }
 }
 
@@ -1128,42 +1034,47 @@ static sie_status apply_Z(sie_op* op, const double2* H, double2* E, double* nest
     return SIE_OK;
 }
 
-// node -> stencil entries map of the exterior grid (built once, on the host,
-// from the stencil bases; the operator build calls it before any capture)
+// node -> stencil entries map of the exterior grid, entries of a node by triangle
+// (built once, on the host, from the stencil bases, by the operator build)
 sie_status proj_map_ready(sie_op* op)
 {
-    if (op->pm_node) return SIE_OK;
+    if (op->pm_ptr) return SIE_OK;
     cudaStream_t st = op->mesh->ctx->stream;
     const GridDesc& g = op->ext.g;
     const int Mp = g.M + 1, S = Mp * Mp * Mp;
-    const int64_t nt = op->mesh->h.nt;
+    const int64_t nt = op->mesh->h.nt, Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
+    if (nt * S > INT32_MAX || Ng > INT32_MAX) {
+        set_error("projection map: more than 2^31 stencil entries or grid nodes");
+        return SIE_ERR_UNSUPPORTED;
+    }
     std::vector<int32_t> hb(3 * nt);
     SIE_CUDA_TRY(cudaMemcpyAsync(hb.data(), op->base, sizeof(int32_t) * 3 * nt, cudaMemcpyDeviceToHost, st));
     SIE_CUDA_TRY(cudaStreamSynchronize(st));
-    std::vector<std::pair<int64_t, int32_t>> e(nt * S);
+    auto node = [&](int64_t t, int u) {
+        const int nx = hb[3 * t] + u % Mp, ny = hb[3 * t + 1] + (u / Mp) % Mp, nz = hb[3 * t + 2] + u / (Mp * Mp);
+        return ((int64_t)nz * g.N[1] + ny) * g.N[0] + nx;
+    };
+    std::vector<int32_t> cnt(Ng, 0), nodes;
     for (int64_t t = 0; t < nt; t++)
-        for (int u = 0; u < S; u++) {
-            int nx = hb[3 * t] + u % Mp, ny = hb[3 * t + 1] + (u / Mp) % Mp, nz = hb[3 * t + 2] + u / (Mp * Mp);
-            e[t * S + u] = {((int64_t)nz * g.N[1] + ny) * g.N[0] + nx, (int32_t)(t * S + u)};
-        }
-    std::sort(e.begin(), e.end());
-    std::vector<int64_t> node, ptr(1, 0);
-    std::vector<int32_t> ent(e.size());
-    for (size_t k = 0; k < e.size(); k++) {
-        if (k == 0 || e[k].first != e[k - 1].first) {
-            if (k) ptr.push_back((int64_t)k);
-            node.push_back(e[k].first);
-        }
-        ent[k] = e[k].second;
+        for (int u = 0; u < S; u++)
+            if (cnt[node(t, u)]++ == 0) nodes.push_back((int32_t)node(t, u));
+    // by falling number of entries, then by node
+    std::sort(nodes.begin(), nodes.end(),
+              [&](int32_t a, int32_t b) { return cnt[a] != cnt[b] ? cnt[a] > cnt[b] : a < b; });
+    std::vector<int32_t> ptr(nodes.size() + 1, 0), at(Ng, 0), ent(nt * S);
+    for (size_t v = 0; v < nodes.size(); v++) {
+        at[nodes[v]] = ptr[v];
+        ptr[v + 1] = ptr[v] + cnt[nodes[v]];
     }
-    ptr.push_back((int64_t)e.size());
-    op->pm_nnode = (int64_t)node.size();
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_node, sizeof(int64_t) * node.size(), st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_ptr, sizeof(int64_t) * ptr.size(), st));
+    for (int64_t t = 0; t < nt; t++)
+        for (int u = 0; u < S; u++) ent[at[node(t, u)]++] = (int32_t)(t * S + u);
+    op->pm_nnode = (int64_t)nodes.size();
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_node, sizeof(int32_t) * nodes.size(), st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_ptr, sizeof(int32_t) * ptr.size(), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_ent, sizeof(int32_t) * ent.size(), st));
+    SIE_CUDA_TRY(cudaMemcpyAsync(op->pm_node, nodes.data(), sizeof(int32_t) * nodes.size(), cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pm_tc, sizeof(double2) * 9 * nt, st));
-    SIE_CUDA_TRY(cudaMemcpyAsync(op->pm_node, node.data(), sizeof(int64_t) * node.size(), cudaMemcpyHostToDevice, st));
-    SIE_CUDA_TRY(cudaMemcpyAsync(op->pm_ptr, ptr.data(), sizeof(int64_t) * ptr.size(), cudaMemcpyHostToDevice, st));
+    SIE_CUDA_TRY(cudaMemcpyAsync(op->pm_ptr, ptr.data(), sizeof(int32_t) * ptr.size(), cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaMemcpyAsync(op->pm_ent, ent.data(), sizeof(int32_t) * ent.size(), cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaStreamSynchronize(st));
     return SIE_OK;
@@ -1201,11 +1112,10 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
         float2* buf = reinterpret_cast<float2*>(op->ws.bufs);
         {
             Stage s_(c, "project_sys32");
-            SIE_TRY(proj_map_ready(op));
-            SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(float2) * 7 * Ng, st));
             float2* tc = reinterpret_cast<float2*>(op->pm_tc);
-            k_tri_coef<float2><<<nb(M.nt), 256, 0, st>>>(M.nt, M, H, E, rho, tc);
-            k_project_gather<float2, float><<<nb(op->pm_nnode), 256, 0, st>>>(
+            k_tri_coef<float2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, E, rho, tc);
+            SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(float2) * 7 * Ng, st));
+            k_project_gather<float2, float><<<gio_blocks(op->pm_nnode, 8), 256, 0, st>>>(
                 op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W32, tc, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
@@ -1222,7 +1132,12 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
         }
         {
             Stage s_(c, "interp32");
-            k_interp32<<<(M.nt + 3) / 4, 128, 0, st>>>(M.nt, S, g.M, M, op->base, op->W32, src, g, Ng, y1);
+            if (M.nt <= GIO_WIDE)
+                k_interp<32, float2, float, 4><<<gio_blocks(M.nt, 32, GIO_SMALL), GIO_SMALL, 0, st>>>(
+                    M.nt, S, g.M, M, op->base, op->W32, src, g, make_double2(1.0, 0.0), Ng, y1, 0);
+            else
+                k_interp<4, float2, float, 4><<<gio_blocks(M.nt, 4), 256, 0, st>>>(
+                    M.nt, S, g.M, M, op->base, op->W32, src, g, make_double2(1.0, 0.0), Ng, y1, 0);
             SIE_CUDA_TRY(cudaGetLastError());
         }
     } else {
@@ -1230,10 +1145,9 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
         double2* buf = op->ws.bufs;
         {
             Stage s_(c, "project_sys");
-            SIE_TRY(proj_map_ready(op));
+            k_tri_coef<double2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, E, rho, op->pm_tc);
             SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(double2) * 7 * Ng, st));
-            k_tri_coef<double2><<<nb(M.nt), 256, 0, st>>>(M.nt, M, H, E, rho, op->pm_tc);
-            k_project_gather<double2, double><<<nb(op->pm_nnode), 256, 0, st>>>(
+            k_project_gather<double2, double><<<gio_blocks(op->pm_nnode, 8), 256, 0, st>>>(
                 op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W, op->pm_tc, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
@@ -1250,7 +1164,7 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
         }
         {
             Stage s_(c, "interp");
-            SIE_TRY(aim_interp(op, src, 1, make_double2(1.0, 0.0), y1));
+            SIE_TRY(aim_interp(op, src, 1, make_double2(1.0, 0.0), y1, 0, 1));
         }
     }
     {
@@ -1263,10 +1177,14 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
                 k_spmv2_c64<<<(unsigned)((ne + 3) / 4), 128, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLK32,
                                                                        op->pk_he, make_double2(0.0, op->k0),
                                                                        make_double2(-1.0, 0.0), y1);
-            else
-                k_spmv2<<<(unsigned)((ne + 3) / 4), 128, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLA, H,
-                                                                   make_double2(0.0, op->k0), X.valK, E,
-                                                                   make_double2(-1.0, 0.0), y1);
+            else {
+                const bool small = ne <= 8192;
+                auto f = small ? k_spmv2<32> : k_spmv2<8>;
+                const int T = small ? 64 : 256;  // small: over more SMs' FP64 lanes
+                f<<<nb(ne * (small ? 32 : 8), T), T, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLA, H,
+                                                              make_double2(0.0, op->k0), X.valK, E,
+                                                              make_double2(-1.0, 0.0), y1);
+            }
             SIE_CUDA_TRY(cudaGetLastError());
         }
         Stage s_(c, "spmv_sys_rest");
