@@ -683,9 +683,17 @@ __device__ __forceinline__ void z_product(const C* __restrict__ spec, int64_t i,
     }
 }
 
+// CTAs per SM the register count must allow: 16 warps at 128 registers (complex128), 28 at 72
 template <int N, class P, int MODE>
-__global__ void __launch_bounds__(ZMode<MODE>::NI* z_pb<N, P, MODE>() * Plan<N>::R2,
-                                  512 / (ZMode<MODE>::NI * z_pb<N, P, MODE>() * Plan<N>::R2) + 1 - (sizeof(typename P::G) / 16))
+__host__ __device__ constexpr int z_ctas()
+{
+    const int warps = (ZMode<MODE>::NI * z_pb<N, P, MODE>() * Plan<N>::R2 + 31) / 32;
+    const int n = (sizeof(typename P::G) == 16 ? 16 : 28) / warps;
+    return n < 1 ? 1 : n;
+}
+
+template <int N, class P, int MODE>
+__global__ void __launch_bounds__(ZMode<MODE>::NI* z_pb<N, P, MODE>() * Plan<N>::R2, z_ctas<N, P, MODE>())
     k_fft_z(typename P::G* __restrict__ buf, const typename P::G* __restrict__ spec,
             const typename P::TW* __restrict__ tw, int nz_phys, int64_t ncol, int64_t plane, int64_t bnn,
             int64_t batch, typename P::R k0)
@@ -849,7 +857,8 @@ sie_status fft_z_n(cudaStream_t st, typename P::G* buf, const typename P::G* spe
                                                     int64_t, int64_t, int, float, const float2*);
 
 // the lengths up to 256
-#define SIE_FFT_LENGTHS(X) X(16) X(32) X(64) X(128) X(256)
+#define SIE_FFT_LENGTHS(X) \
+    X(16) X(20) X(24) X(32) X(40) X(48) X(64) X(80) X(96) X(128) X(160) X(192) X(256)
 #define SIE_FFT_EXTERN(N) SIE_FFT_INSTANCES(N, extern)
 
 }  // namespace sie

@@ -58,7 +58,7 @@ struct GridDesc {
     double o[3];
     double h;
     int N[3];     // physical nodes per axis
-    int n[3];     // FFT lengths (powers of two >= 2N-1)
+    int n[3];     // FFT lengths >= 2N-1 (fft_length in host.cpp)
     int M;        // Lagrange order
     int Rnear;    // near radius (nodes)
 };

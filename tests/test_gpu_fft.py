@@ -28,7 +28,9 @@ def _mesh(kind, n):
     return box([1e-3 * v for v in d], d)
 
 
-@pytest.mark.parametrize("kind,n", [("sphere", 0), ("sphere", 20), ("sphere", 33), ("sphere", 64), ("sphere", 65),
+@pytest.mark.parametrize("kind,n", [("sphere", 0), ("sphere", 17), ("sphere", 20), ("sphere", 24), ("sphere", 33),
+                                    ("sphere", 40), ("sphere", 48), ("sphere", 64), ("sphere", 65), ("sphere", 81),
+                                    ("sphere", 96), ("x", 2), ("x", 5), ("x", 60), ("z", 2), ("z", 5), ("z", 60),
                                     ("x", 3), ("x", 30), ("x", 80), ("y", 45), ("z", 22), ("z", 45), ("z", 80)])
 def test_grid_products_match_oracle(lib, ctx, kind, n):
     V, T = _mesh(kind, n)
