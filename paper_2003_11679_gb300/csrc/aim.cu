@@ -356,13 +356,13 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
 
 static void free_aim(AimOp& a)
 {
-    void* ptrs[] = {a.spec, a.spec32, a.pairs, a.row_ptr, a.col, a.valL, a.valK, a.valLA, a.dLA, a.dL,
+    void* ptrs[] = {a.spec, a.spec32, a.pairs, a.row_ptr, a.col, a.valL, a.valK, a.valLA, a.dLA, a.dL, a.idLA,
                     a.tri_row_ptr, a.tri_col, a.valLphi, a.valLphiNR, a.valM, a.valLK32, a.valLphi32,
                     a.obj_k, a.obj_ik2};
     a.obj_k = a.obj_ik2 = nullptr;
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    a.valLA = a.dLA = a.dL = a.valLphi = a.valLphiNR = a.valM = nullptr;
+    a.valLA = a.dLA = a.dL = a.idLA = a.valLphi = a.valLphiNR = a.valM = nullptr;
     a.valLK32 = nullptr;
     a.valLphi32 = nullptr;
     a.tri_row_ptr = nullptr;

@@ -23,7 +23,7 @@ struct ConSys {
     int nt, ne;
     DevMesh M;
     const double *elen;
-    const double2* dLA;
+    const double2* idLA;        // 1 / diag(LA)
     const int64_t* rp;          // triangle CSR of Lphi_NR
     const int32_t* col;
     const double2* val;
@@ -35,12 +35,6 @@ struct ConSys {
     double2 *v1, *b, *q;        // scratch per right-hand side: ne, nt, nt
     double* stat;               // largest iteration count and residual
 };
-
-__device__ __forceinline__ double2 c_div(double2 a, double2 d)
-{
-    const double den = d.x * d.x + d.y * d.y;
-    return make_double2((a.x * d.x + a.y * d.y) / den, (a.y * d.x - a.x * d.y) / den);
-}
 
 struct ConClu {
     const ConSys& s;
@@ -105,7 +99,7 @@ struct ConClu {
     // o = z - kappa D Dg^-1 D^T phi on own triangle t
     __device__ __forceinline__ double2 charge(int t, double2 z) const
     {
-        const double2 d = dsum(t, [&](int e) { return c_div(dt(e, M.xv), s.dLA[e]); });
+        const double2 d = dsum(t, [&](int e) { return r_cm(s.idLA[e], dt(e, M.xv)); });
         const double2 kd = r_cm(s.kappa, d);
         return make_double2(z.x - kd.x, z.y - kd.y);
     }
@@ -187,7 +181,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, 
     };
     for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) v1[e] = v1p(e);
     for (int k = threadIdx.x; k < rows; k += blockDim.x) {
-        const double2 r = ops.dsum((int)r0 + k, [&](int e) { return c_div(v1p(e), s.dLA[e]); });
+        const double2 r = ops.dsum((int)r0 + k, [&](int e) { return r_cm(s.idLA[e], v1p(e)); });
         M.w[k] = r;
         b[r0 + k] = r;
         sol[r0 + k] = make_double2(0, 0);
@@ -228,7 +222,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, 
         // y = Dg^-1 (v1' + kappa D^T Lphi q) [/ (j k0)]; v1' of other CTAs' edges is complete since the first barriers
         auto y_of = [&](int e) {
             const double2 k = r_cm(s.kappa, ops.dt(e, M.xv)), v = __ldcg(v1 + e);
-            const double2 y = c_div(make_double2(v.x + k.x, v.y + k.y), s.dLA[e]);
+            const double2 y = r_cm(s.idLA[e], make_double2(v.x + k.x, v.y + k.y));
             return s.ext ? r_cm(s.ijk0, y) : y;
         };
         for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) y1[e] = y_of(e);
@@ -250,15 +244,15 @@ bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, in
 {
     const int nt = (int)op->mesh->h.nt, ne = (int)op->mesh->h.ne;
     if (!a.lu || !a.lu->Xinv || nt > CLU_MAXN || w.m != restart) return false;
-    const int C = clu_ctas(nt);
+    const int C = clu_pick((const void*)k_constraint, nt, a.npairs, w.m, R, sizeof(float2) * (nt + 1));
+    if (!C) return false;
     const size_t smem = clu_smem(nt, w.m, C) + sizeof(float2) * (nt + 1);
-    if (smem > 200 * 1024 || !clu_fits((const void*)k_constraint, C, R, smem)) return false;
     cudaStream_t st = op->mesh->ctx->stream;
     ConSys s{};
     s.nt = nt, s.ne = ne;
     s.M = op->mesh->d;
     s.elen = op->elen;
-    s.dLA = a.dLA;
+    s.idLA = a.idLA;
     s.rp = a.tri_row_ptr, s.col = a.tri_col, s.val = a.valLphiNR;
     s.X = a.lu->Xinv;
     s.kappa = kappa;

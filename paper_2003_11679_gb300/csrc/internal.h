@@ -156,6 +156,7 @@ struct AimOp {
     double2* valLA = nullptr;       // near-corrected LA (vector potential part)
     double2* dLA = nullptr;         // exact diagonal of LA
     double2* dL = nullptr;          // exact diagonal of L
+    double2* idLA = nullptr;        // 1 / dLA
     // triangle CSR of the near-corrected Lphi (pairs in (t, s) order)
     std::vector<int64_t> tri_row_ptr_h;
     std::vector<int32_t> tri_col_h;
@@ -310,12 +311,12 @@ struct sie_op {
     double2* bal = nullptr;         // weighted right-hand side and preconditioner input (2 (ne + nt))
     double lu_ms = 0;               // wall time of the dense constraint-preconditioner factorisations
     // surface impedance boundary condition (interior_model = SIE_SIBC): RWG Gram
-    // matrix as edge CSR, its diagonal, and eta_i / eta0
+    // matrix as edge CSR and eta_i / eta0
     int64_t* gr_row_ptr = nullptr;
     int64_t gr_nnz = 0;
     int32_t* gr_col = nullptr;
     double2* gr_val = nullptr;
-    double2* gr_diag = nullptr;
+    double* gr_idiag = nullptr;     // reciprocal of its (real) diagonal
     double eta_re = 0, eta_im = 0;
     // projection of the system product as a gather: grid nodes with stencil entries, CSR
     // of those entries (t * S + u), per-triangle coefficients

@@ -987,6 +987,14 @@ __global__ void k_csr_fill(int ne, const int64_t* __restrict__ row_ptr, const in
     }
 }
 
+__global__ void k_recip(int n, const double2* __restrict__ d, double2* __restrict__ r)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const cd v = cdivc(mk(1.0, 0.0), mk(d[i].x, d[i].y));
+    r[i] = make_double2(v.re, v.im);
+}
+
 __global__ void k_lphi_vals(int64_t np, const double2* __restrict__ loc, double2* __restrict__ v,
                             double2* __restrict__ vnr)
 {
@@ -1050,6 +1058,9 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q)
                                                            make_double2(ik2.real(), ik2.imag()), a.obj_ik2, a.valL,
                                                            a.valK,
                                                            a.valLA, a.dLA, a.dL);
+    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&a.idLA, sizeof(double2) * H.ne, st));
+    k_recip<<<(unsigned)((H.ne + 255) / 256), 256, 0, st>>>((int)H.ne, a.dLA, a.idLA);
     SIE_CUDA_TRY(cudaGetLastError());
     // triangle CSR of Lphi (exact - grid): rows = pair blocks, columns = s
     a.tri_row_ptr_h = pstart;

@@ -16,7 +16,8 @@ struct NestSys {
     int64_t ne;
     const int64_t *ix_rp, *a_rp;
     const int32_t *ix_col, *a_col;
-    const double2 *ix_val, *a_val, *k_val, *m_val, *diag;  // k_val, m_val: GIBC; diag: SIBC
+    const double2 *ix_val, *a_val, *k_val, *m_val;  // k_val, m_val: GIBC
+    const double* idiag;                            // SIBC: 1 / diag(G)
     const double2* H;      // R vectors, ldh apart
     double2* E;            // R vectors, lde apart
     int64_t ldh, lde;
@@ -39,9 +40,9 @@ struct NestOps {
         for (int t = threadIdx.x; t < K.R * rows; t += blockDim.x) {
             const int q = t / rows;
             const int64_t k = r0 + t % rows, at = ((int64_t)j * K.R + q) * K.n + k;
-            const double2 d = s.diag[k], v = K.V[at];
-            const double den = d.x * d.x + d.y * d.y;
-            if (j < K.m) K.Z[at] = make_double2((v.x * d.x + v.y * d.y) / den, (v.y * d.x - v.x * d.y) / den);
+            const double d = s.idiag[k];
+            const double2 v = K.V[at];
+            if (j < K.m) K.Z[at] = make_double2(v.x * d, v.y * d);
         }
     }
     __device__ void product(const double2* val, const double2* x, double2* y)
@@ -127,9 +128,8 @@ struct NestClu {
             M.xv[r0 + k] = v;
             return;
         }
-        const double2 d = s.diag[r0 + k];
-        const double den = d.x * d.x + d.y * d.y;
-        const double2 z = make_double2((v.x * d.x + v.y * d.y) / den, (v.y * d.x - v.x * d.y) / den);
+        const double d = s.idiag[r0 + k];
+        const double2 z = make_double2(v.x * d, v.y * d);
         if (j < K.m) Z[(int64_t)j * K.n + r0 + k] = z;
         M.xz[r0 + k] = z;
     }
@@ -211,9 +211,6 @@ int res_ctas(int64_t work)
     return (int)std::max<int64_t>(1, std::min<int64_t>(sms, (work + 63) / 64));
 }
 
-// CTAs of a cluster: 8 (portable) up to 1,024 rows, then 16
-int clu_ctas(int64_t n) { return n <= 1024 ? 8 : CLU_MAXC; }
-
 // lanes per row: as many as the CTA's threads and half the mean row allow
 int res_group(int64_t rows, int64_t nrow, int64_t nnz)
 {
@@ -274,6 +271,22 @@ bool clu_fits(const void* fn, int C, int R, size_t smem)
     return n >= R;
 }
 
+// CTAs of a cluster (0: the R clusters do not run at once).  8 (portable) for up to
+// 1,024 rows and 16,384 entries, else 16: a bar's 504 rows of 64 entries take 14,000
+// cycles a product on 8 SMs' FP64 lanes, 7,000 on 16.  Clusters of 16 fit a GPU region
+// once only: 8 of them may not run at once, and 8 clusters of 8 take 210 ms for a solve
+// of the bar with 8 right-hand sides, the forms without clusters 430.
+int clu_pick(const void* fn, int64_t n, int64_t nnz, int m, int R, size_t extra)
+{
+    if (n > CLU_MAXN) return 0;
+    const bool small = n <= 1024;
+    for (int C = small && nnz <= 16384 ? 8 : CLU_MAXC; C >= (small ? 8 : CLU_MAXC); C >>= 1) {
+        const size_t smem = clu_smem(n, m, C) + extra;
+        if (smem <= 200 * 1024 && clu_fits(fn, C, R, smem)) return C;
+    }
+    return 0;
+}
+
 // Rows per right-hand side up to which the cluster form is taken (CLU_MAXN): its
 // gather vectors have to fit, and 16 SMs do the arithmetic of all rows.
 sie_status nested_solve(sie_op* op, int R, const double2* H, int64_t ldh, double2* E, int64_t lde, double2 f,
@@ -291,7 +304,7 @@ sie_status nested_solve(sie_op* op, int R, const double2* H, int64_t ldh, double
     s.a_val = sibc ? op->gr_val : I.valL;
     s.k_val = sibc ? nullptr : I.valK;
     s.m_val = sibc ? nullptr : I.valM;
-    s.diag = sibc ? op->gr_diag : nullptr;
+    s.idiag = sibc ? op->gr_idiag : nullptr;
     s.H = H, s.ldh = ldh, s.E = E, s.lde = lde;
     s.f = f;
     s.zf = op->edge_zf;
@@ -303,8 +316,7 @@ sie_status nested_solve(sie_op* op, int R, const double2* H, int64_t ldh, double
     K.stat = op->gstat;
     unsigned* cnt = op->res_bar;
     int* err = (int*)(op->res_bar + 1);
-    const int C = clu_ctas(ne);
-    if (ne <= CLU_MAXN && clu_fits((const void*)k_nested_clu, C, R, clu_smem(ne, w.m, C))) {
+    if (const int C = clu_pick((const void*)k_nested_clu, ne, sibc ? op->gr_nnz : I.nnz, w.m, R, 0)) {
         const int64_t rows = (ne + C - 1) / C;
         int G = res_group(rows, ne, sibc ? op->gr_nnz : I.nnz), Gx = sibc ? res_group(rows, ne, op->ix_nnz) : G;
         CluLock lock;

@@ -155,18 +155,19 @@ __device__ __forceinline__ void res_update(const ResKrylov& K, int64_t r0, int64
     __syncthreads();
 }
 
-// 2^-exponent of v (1 for zero, infinity and NaN)
-__device__ __forceinline__ double res_unscale(double v)
+// 2^-exponent of the largest of three magnitudes (1 for zero, infinity and NaN)
+__device__ __forceinline__ double res_unscale(double a, double b, double c)
 {
-    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    const int m = max(max(__double2hiint(a) & 0x7fffffff, __double2hiint(b) & 0x7fffffff), __double2hiint(c) & 0x7fffffff);
+    const int e = m >> 20;
     return (e == 0 || e == 0x7ff) ? 1.0 : __hiloint2double((2046 - min(e, 2045)) << 20, 0);
 }
 
 // column j of one right-hand side (one thread): h1 + h2 and the norm hn through
 // the previous rotations, rotation j (c real), g; the rotated column to Hq when
-// store; gabs = |g_j| becomes |g_{j+1}|.  One chain of dependent FP64 operations:
-// two reciprocal square roots instead of three hypot and six divisions (13,600
-// cycles an iteration with those, a third of it)
+// store; gabs = |g_j| becomes |g_{j+1}|.  One chain of FP64 operations of one warp,
+// 64 cycles or more each: two reciprocal square roots instead of three hypot and six
+// divisions (13,600 cycles an iteration with those, a third of it)
 __device__ __forceinline__ void res_givens(int j, int m, const double2* a1, const double2* a2, double hn, double2* c_,
                                            double2* s_, double2* g_, double2* Hq, bool store, double& gabs)
 {
@@ -178,7 +179,7 @@ __device__ __forceinline__ void res_givens(int j, int m, const double2* a1, cons
         a = make_double2(c_[i].x * b.x - ta.x, c_[i].x * b.y - ta.y);
     }
     // scaled by a power of two: no square overflows or underflows
-    const double sc = res_unscale(fmax(fmax(fabs(a.x), fabs(a.y)), hn));
+    const double sc = res_unscale(a.x, a.y, hn);
     const double ax = a.x * sc, ay = a.y * sc, b = hn * sc, u = ax * ax + ay * ay, t = u + b * b;
     const double ru = u > 0 ? rsqrt(u) : 0.0, rt = t > 0 ? rsqrt(t) : (t == t ? 0.0 : t), sn = b * rt;
     double2 c, s, d;  // d = c a + s hn
@@ -230,15 +231,35 @@ __device__ __forceinline__ void res_stat(double* stat, int iters, double worst)
 // relative residual; a NaN norm gives NaN
 __device__ __forceinline__ double res_rel(double r, double bn) { return bn > 0 ? r / bn : (bn == bn ? 0.0 : bn); }
 
-// norm of w - V h2 from |w|^2 = h2[nv] and h2[0 .. nv), by one warp; in every lane
-__device__ __forceinline__ double res_norm(const double2* h2, int nv, int lane)
+// squared norm of w - V h2 from |w|^2 = h2[nv] and h2[0 .. nv), by one warp; in every
+// lane.  |h2|^2 is left out where it cannot change the result (exponents 30 apart)
+__device__ __forceinline__ double res_norm2(const double2* h2, int nv, int lane)
 {
+    int e = 0;
+    for (int i = lane; i < nv; i += 32)
+        e = max(e, max(__double2hiint(h2[i].x) & 0x7fffffff, __double2hiint(h2[i].y) & 0x7fffffff));
+    e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e) >> 20;
+    const double ww = h2[nv].x;
+    const int ew = (__double2hiint(ww) & 0x7fffffff) >> 20;
+    // |h2|^2 < 2 nv 4^(e - 1022) <= 2^(2 e - 2044 + 8), |w|^2 >= 2^(ew - 1023)
+    if (2 * e - 2036 < ew - 1023 - 60) return ww;
     double s = 0;
     for (int i = lane; i < nv; i += 32) s += h2[i].x * h2[i].x + h2[i].y * h2[i].y;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    s = h2[nv].x - s;
-    return s != s ? s : sqrt(fmax(s, 0.0));
+    s = ww - s;
+    return s != s ? s : fmax(s, 0.0);
+}
+// norm and its reciprocal (0 for 0) from the squared norm
+__device__ __forceinline__ void res_root(double s, double& norm, double& inv)
+{
+    if (s > 0 && s < 1e300) {
+        inv = rsqrt(s);
+        norm = s * inv;
+    } else {
+        norm = s != s ? s : sqrt(s);
+        inv = norm > 0 ? 1.0 / norm : 0.0;
+    }
 }
 
 // The FGMRES cycle (zero initial guess, at most K.m iterations) on the residual
@@ -298,9 +319,10 @@ __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* sm
         res_reduce(K, j + 2, P2, ld, h2, ld);
         if ((threadIdx.x >> 5) < R) {
             const int q = threadIdx.x >> 5;
-            const double hn = res_norm(h2 + q * ld, j + 1, threadIdx.x & 31);
+            const double hh = res_norm2(h2 + q * ld, j + 1, threadIdx.x & 31);
             if ((threadIdx.x & 31) == 0) {
-                wn[q] = hn > 0 ? 1.0 / hn : 0.0;
+                double hn;
+                res_root(hh, hn, wn[q]);
                 res_givens(j, m, h1 + q * ld, h2 + q * ld, hn, cs + q * ld, sn + q * ld, g + q * ld, K.H + q * K.ldh,
                            blockIdx.x == 0, gabs[q]);
                 rel[q] = res_rel(gabs[q], bnorm[q]);
@@ -347,7 +369,7 @@ constexpr int CLU_MAXC = 16;
 
 // one right-hand side per cluster; shared memory of a CTA:
 //   x[2][n] gather vectors (v, z), w[rows], pr[2][C][m + 2] partial sums, cs, sn, g, h1, h2 [m + 2]
-int clu_ctas(int64_t n);
+int clu_pick(const void* fn, int64_t n, int64_t nnz, int m, int R, size_t extra);
 int res_group(int64_t rows, int64_t nrow, int64_t nnz);
 bool clu_fits(const void* fn, int C, int R, size_t smem);
 sie_status clu_launch(const void* fn, int C, int R, size_t smem, void** args, cudaStream_t st);
@@ -406,25 +428,22 @@ __device__ __forceinline__ void clu_dots(const CluMem& M, const double2* V, int6
             *cooperative_groups::this_cluster().map_shared_rank(M.pr + (buf * M.C + M.rank) * M.ld + i, lane) = s;
     }
 }
-// h[i] = sum over the CTAs (8 or 16), four chains
+// h[i] = sum over the CTAs (8 or 16): a warp per column, a half for each component
+// (4 FP64 additions; a thread per column took 2,200 cycles in a chain of them)
 __device__ __forceinline__ void clu_reduce(const CluMem& M, int cols, int buf, double2* h)
 {
-    for (int i = threadIdx.x; i < cols; i += blockDim.x) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5, c = lane & 15;
+    for (int i = warp; i < cols; i += nw) {
         const double2* p = M.pr + buf * M.C * M.ld + i;
-        double2 s[4];
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const double2 a = p[c * M.ld], b = p[(c + 4) * M.ld];
-            s[c] = make_double2(a.x + b.x, a.y + b.y);
+        double v = 0;
+        if (c < M.C) {
+            const double2 a = p[c * M.ld];
+            v = lane < 16 ? a.x : a.y;
         }
-        if (M.C > 8)
 #pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const double2 a = p[(c + 8) * M.ld], b = p[(c + 12) * M.ld];
-                s[c].x += a.x + b.x;
-                s[c].y += a.y + b.y;
-            }
-        h[i] = make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
+        for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        const double y = __shfl_xor_sync(0xffffffffu, v, 16);
+        if (lane == 0) h[i] = make_double2(v, y);
     }
     __syncthreads();
 }
@@ -488,7 +507,7 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
     const int64_t n = K.n, r0 = sys.r0;
     double2* V = K.V + (int64_t)q * (m + 1) * n;  // this right-hand side's basis
     double2* H = K.H + q * K.ldh;
-    __shared__ double bnorm, rel, wn, gabs;
+    __shared__ double bnorm, tolb, wn, gabs;
     __shared__ int go, above_s;
     clu_sync();  // every CTA of the cluster has started, or is done with the last cycle
     clu_dots(M, V, n, r0, rows, 0, true, 0);
@@ -498,6 +517,7 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
         const double d2 = M.h1[0].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
         bnorm = run.bnorm < 0 ? b : run.bnorm;
         gabs = b;
+        tolb = bnorm > 0 ? K.tol * bnorm : 1e300;  // a zero right-hand side is solved
         wn = b > 0 ? 1.0 / b : 0.0;
         M.g[0] = make_double2(b, 0);
     }
@@ -531,15 +551,25 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
         clu_dots(M, V, n, r0, rows, j + 1, true, 1);
         clu_sync();
         clu_reduce(M, j + 2, 1, M.h2);
-        double hn = 0;
-        if (threadIdx.x < 32) hn = res_norm(M.h2, j + 1, threadIdx.x);
+        // warp 0: norm, rotation and decision; the others meanwhile subtract V h2
+        double hh = 0;
+        if (threadIdx.x < 32) {
+            hh = res_norm2(M.h2, j + 1, threadIdx.x);
+        } else {
+            for (int k = threadIdx.x - 32; k < rows; k += blockDim.x - 32) {
+                double2 s = make_double2(0, 0);
+                for (int i = 0; i <= j; i++) r_fma(s, V[(int64_t)i * n + r0 + k], M.h2[i]);
+                M.w[k] = make_double2(M.w[k].x - s.x, M.w[k].y - s.y);
+            }
+        }
         if (threadIdx.x == 0) {
-            wn = hn > 0 ? 1.0 / hn : 0.0;
+            double hn;
+            res_root(hh, hn, wn);
             res_givens(j, m, M.h1, M.h2, hn, M.cs, M.sn, M.g, H, M.rank == 0, gabs);
-            rel = res_rel(gabs, bnorm);
-            int more = rel >= K.tol;
+            // NaN stops here (rel, below, reports it); tolb = tol |b|
+            int more = gabs >= tolb;
             if (lock.R > 1) {
-                more = clu_vote(lock, q, run.it + j, rel >= K.tol, M.rank == 0);
+                more = clu_vote(lock, q, run.it + j, more, M.rank == 0);
             } else if (!more && extra > 0) {
                 extra--;
                 more = 1;
@@ -560,16 +590,11 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
         }
         if (decide < 0) return -1;
         if (!decide) break;
-        for (int k = threadIdx.x; k < rows; k += blockDim.x) {
-            double2 s = make_double2(0, 0);
-            for (int i = 0; i <= j; i++) r_fma(s, V[(int64_t)i * n + r0 + k], M.h2[i]);
-            M.w[k] = make_double2(M.w[k].x - s.x, M.w[k].y - s.y);
-        }
         set_v(j + 1);
     }
     clu_sync();  // rank 0's H
     if (threadIdx.x < 32) res_backsub(j, m, H, M.g, threadIdx.x);
-    run.rel = rel;
+    run.rel = res_rel(gabs, bnorm);
     run.above = above_s != 0;
     run.it += j + 1;
     __syncthreads();

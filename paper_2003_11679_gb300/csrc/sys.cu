@@ -1506,7 +1506,7 @@ static sie_status gram_prepare(sie_op* op)
     cudaStream_t st = op->mesh->ctx->stream;
     const HostMesh& h = op->mesh->h;
     std::vector<std::vector<std::pair<int32_t, double>>> rows(h.ne);
-    std::vector<double2> diag(h.ne, make_double2(0.0, 0.0));
+    std::vector<double> diag(h.ne, 0.0);
     for (int64_t t = 0; t < h.nt; t++) {
         double l2 = 0;
         for (int i = 0; i < 3; i++) {
@@ -1521,12 +1521,13 @@ static sie_status gram_prepare(sie_op* op)
                 double v = h.coef[3 * t + i] * h.coef[3 * t + j] * h.area[t] *
                            (l2 / 36.0 + qi[0] * qj[0] + qi[1] * qj[1] + qi[2] * qj[2]);
                 rows[h.tri_edge[3 * t + i]].push_back({h.tri_edge[3 * t + j], v});
-                if (h.tri_edge[3 * t + i] == h.tri_edge[3 * t + j]) diag[h.tri_edge[3 * t + i]].x += v;
+                if (h.tri_edge[3 * t + i] == h.tri_edge[3 * t + j]) diag[h.tri_edge[3 * t + i]] += v;
             }
     }
     SIE_TRY(upload_rows(st, rows, &op->gr_row_ptr, &op->gr_col, &op->gr_val, &op->gr_nnz));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gr_diag, sizeof(double2) * h.ne, st));
-    SIE_CUDA_TRY(cudaMemcpyAsync(op->gr_diag, diag.data(), sizeof(double2) * h.ne, cudaMemcpyHostToDevice, st));
+    for (double& d : diag) d = 1.0 / d;
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gr_idiag, sizeof(double) * h.ne, st));
+    SIE_CUDA_TRY(cudaMemcpyAsync(op->gr_idiag, diag.data(), sizeof(double) * h.ne, cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaStreamSynchronize(st));
     return SIE_OK;
 }
@@ -1657,7 +1658,7 @@ void sys_release(sie_op* op)
     op->mscr = op->ir_multi = op->mvec = op->con_scr = nullptr;
     op->kcs_in.release(st);
     op->kcs_out.release(st);
-    for (void* p : {(void*)op->gr_row_ptr, (void*)op->gr_col, (void*)op->gr_val, (void*)op->gr_diag,
+    for (void* p : {(void*)op->gr_row_ptr, (void*)op->gr_col, (void*)op->gr_val, (void*)op->gr_idiag,
                     (void*)op->pm_node, (void*)op->pm_ptr, (void*)op->pm_ent, (void*)op->pm_tc,
                     (void*)op->pk_he, (void*)op->pk_sig, (void*)op->bal})
         if (p) cudaFreeAsync(p, st);
