@@ -278,7 +278,7 @@ struct sie_op {
     double2* ix_val = nullptr;
     double* elen = nullptr;         // edge lengths
     double2* sys_E = nullptr;       // E' = Z' H (ne)
-    double2* sys_tmp = nullptr;     // ne + 2 nt scratch
+    double2* sys_tmp = nullptr;     // 2 (ne + nt) scratch
     double2* sys_vec = nullptr;     // 4 (ne + nt) scratch for host-pointer calls
     float4* pk_he = nullptr;        // mixed near product: complex64 (H, E) side by side (ne)
     float2* pk_sig = nullptr;       // mixed near product: complex64 triangle charges (nt)
@@ -299,7 +299,8 @@ struct sie_op {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one per precision (SIE_FP64, SIE_MIXED)
     bool gfailed = false;           // capture or instantiation failed: stream path only
     bool capturing = false;         // apply_Z emits the device-controlled nested solve
-    cudaStream_t gs[2] = {nullptr, nullptr};  // capture streams: graph, while-loop body
+    cudaStream_t gs[2] = {nullptr, nullptr};  // capture streams: main chain, branch beside it
+    cudaEvent_t gev[3] = {nullptr, nullptr, nullptr};  // fork, E known, join
     double2* g_io = nullptr;        // graph input x and output y, 2 (ne + nt)
     // device (6): largest nested iteration count and residual since cleared, those of the
     // the last nested solve (residual, count)

@@ -1080,33 +1080,75 @@ sie_status proj_map_ready(sie_op* op)
     return SIE_OK;
 }
 
-// y = SYS x, x = [H (ne); c0 rho (nt)]
-// the system product after the interior impedance: y = SYS [H; rho] with
-// E = Z' H already computed (every step of Eq. sys but the nested solve)
-static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E, const double2* rho, double2* y);
-
-static sie_status apply_sys(sie_op* op, const double2* x, double2* y)
+// The charge rows y2 of y = SYS [H; rho] and yb = the scalar-potential term: all that
+// needs neither E nor the grid
+static sie_status sys_charge(sie_op* op, cudaStream_t st, const double2* H, const double2* rho, double2* yb,
+                             double2* y2)
 {
-    const int64_t ne = op->mesh->h.ne;
-    double2* E = op->sys_E;
-    SIE_TRY(apply_Z(op, x, E, nullptr));
-    return apply_sys_rest(op, x, E, x + ne, y);
+    sie_ctx* c = op->mesh->ctx;
+    const DevMesh& M = op->mesh->d;
+    const int64_t ne = M.ne, nt = M.nt;
+    AimOp& X = op->ext;
+    const bool c64 = op->p.precision == SIE_MIXED && X.valLK32;
+    SIE_CUDA_TRY(cudaMemsetAsync(yb, 0, sizeof(double2) * ne, st));
+    Stage s_(c, "spmv_sys_rest");
+    double2* sig = op->sys_tmp + ne;  // apply_Z uses the first ne
+    double2* phi = sig + nt;
+    if (c64) {
+        k_sigma32<<<nb(nt), 256, 0, st>>>((int)nt, M.area, rho, op->pk_sig);
+        SIE_CUDA_TRY(csr_launch(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphi32, op->pk_sig,
+                                make_double2(1.0, 0.0), false, phi));
+    } else {
+        k_sigma<<<nb(nt), 256, 0, st>>>((int)nt, M.area, rho, sig);
+        SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphi, sig, cplx(1.0, 0.0), phi, false));
+    }
+    k_dt<<<nb(ne), 256, 0, st>>>((int)ne, M.edge_tri, op->elen, phi, yb);
+    k_row2<<<nb(nt), 256, 0, st>>>((int)nt, M, H, rho, op->k0, y2);
+    SIE_CUDA_TRY(cudaGetLastError());
+    return SIE_OK;
 }
 
-static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E, const double2* rho, double2* y)
+// yb += the near-region products of H and E and the term in E alone
+static sie_status sys_near(sie_op* op, cudaStream_t st, const double2* H, const double2* E, double2* yb)
+{
+    sie_ctx* c = op->mesh->ctx;
+    const int64_t ne = op->mesh->h.ne;
+    AimOp& X = op->ext;
+    const bool c64 = op->p.precision == SIE_MIXED && X.valLK32;
+    if (c64) k_pack_he32<<<nb(ne), 256, 0, st>>>((int)ne, H, E, op->pk_he);
+    {
+        // the exterior near-region product alone (one kernel)
+        Stage s1_(c, "spmv_near_ext");
+        if (c64)
+            k_spmv2_c64<<<(unsigned)((ne + 3) / 4), 128, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLK32, op->pk_he,
+                                                                   make_double2(0.0, op->k0), make_double2(-1.0, 0.0),
+                                                                   yb);
+        else {
+            const bool small = ne <= 8192;
+            auto f = small ? k_spmv2<32> : k_spmv2<8>;
+            const int T = small ? 64 : 256;  // small: over more SMs' FP64 lanes
+            f<<<nb(ne * (small ? 32 : 8), T), T, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLA, H,
+                                                          make_double2(0.0, op->k0), X.valK, E,
+                                                          make_double2(-1.0, 0.0), yb);
+        }
+        SIE_CUDA_TRY(cudaGetLastError());
+    }
+    Stage s_(c, "spmv_sys_rest");
+    return spmv(st, (int)ne, op->ix_nnz, op->ix_row_ptr, op->ix_col, op->ix_val, E, cplx(-0.5, 0.0), yb);
+}
+
+// y1 = the grid part.  The interpolation adds two triangles' values to an edge of zeros
+// (in either order the same sum); yb is added after it.
+static sie_status sys_grid(sie_op* op, const double2* H, const double2* E, const double2* rho, double2* y1)
 {
     sie_ctx* c = op->mesh->ctx;
     cudaStream_t st = c->stream;
     const DevMesh& M = op->mesh->d;
-    const int64_t ne = M.ne, nt = M.nt;
-    double2* y1 = y;
-    double2* y2 = y + ne;
     AimOp& X = op->ext;
     const GridDesc& g = X.g;
     int S = (g.M + 1) * (g.M + 1) * (g.M + 1);
     int64_t Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
     int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    SIE_CUDA_TRY(cudaMemsetAsync(y1, 0, sizeof(double2) * ne, st));
     if (op->p.precision == SIE_MIXED) {
         float2* src = reinterpret_cast<float2*>(op->ws.src);
         float2* buf = reinterpret_cast<float2*>(op->ws.bufs);
@@ -1167,44 +1209,47 @@ static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E,
             SIE_TRY(aim_interp(op, src, 1, make_double2(1.0, 0.0), y1, 0, 1));
         }
     }
-    {
-        const bool c64 = op->p.precision == SIE_MIXED && X.valLK32;
-        if (c64) k_pack_he32<<<nb(ne), 256, 0, st>>>((int)ne, H, E, op->pk_he);
-        {
-            // the exterior near-region product alone (one kernel)
-            Stage s1_(c, "spmv_near_ext");
-            if (c64)
-                k_spmv2_c64<<<(unsigned)((ne + 3) / 4), 128, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLK32,
-                                                                       op->pk_he, make_double2(0.0, op->k0),
-                                                                       make_double2(-1.0, 0.0), y1);
-            else {
-                const bool small = ne <= 8192;
-                auto f = small ? k_spmv2<32> : k_spmv2<8>;
-                const int T = small ? 64 : 256;  // small: over more SMs' FP64 lanes
-                f<<<nb(ne * (small ? 32 : 8), T), T, 0, st>>>((int)ne, X.row_ptr, X.col, X.valLA, H,
-                                                              make_double2(0.0, op->k0), X.valK, E,
-                                                              make_double2(-1.0, 0.0), y1);
-            }
-            SIE_CUDA_TRY(cudaGetLastError());
-        }
-        Stage s_(c, "spmv_sys_rest");
-        SIE_TRY(spmv(st, (int)ne, op->ix_nnz, op->ix_row_ptr, op->ix_col, op->ix_val, E, cplx(-0.5, 0.0), y1));
-        double2* phi = op->sys_tmp + nt;
-        if (c64) {
-            k_sigma32<<<nb(nt), 256, 0, st>>>((int)nt, M.area, rho, op->pk_sig);
-            SIE_CUDA_TRY(csr_launch(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphi32, op->pk_sig,
-                                    make_double2(1.0, 0.0), false, phi));
-        } else {
-            double2* sig = op->sys_tmp;
-            k_sigma<<<nb(nt), 256, 0, st>>>((int)nt, M.area, rho, sig);
-            SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphi, sig, cplx(1.0, 0.0), phi,
-                         false));
-        }
-        k_dt<<<nb(ne), 256, 0, st>>>((int)ne, M.edge_tri, op->elen, phi, y1);
-        k_row2<<<nb(nt), 256, 0, st>>>((int)nt, M, H, rho, op->k0, y2);
-        SIE_CUDA_TRY(cudaGetLastError());
-    }
     return SIE_OK;
+}
+
+// the system product after the interior impedance: y = SYS [H; rho] with
+// E = Z' H already computed (every step of Eq. sys but the nested solve)
+static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E, const double2* rho, double2* y)
+{
+    cudaStream_t st = op->mesh->ctx->stream;
+    const int64_t ne = op->mesh->h.ne;
+    double2* yb = op->sys_tmp + ne + 2 * op->mesh->h.nt;
+    SIE_TRY(sys_charge(op, st, H, rho, yb, y + ne));
+    SIE_TRY(sys_near(op, st, H, E, yb));
+    SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * ne, st));
+    SIE_TRY(sys_grid(op, H, E, rho, y));
+    return axpby(st, ne, 1.0, yb, 1.0, y);
+}
+
+// y = SYS x, x = [H (ne); c0 rho (nt)].  Captured into a graph, the charge part runs
+// beside the nested solve and the near part beside the transforms, on a branch.
+static sie_status apply_sys(sie_op* op, const double2* x, double2* y)
+{
+    const int64_t ne = op->mesh->h.ne;
+    double2* E = op->sys_E;
+    if (!op->capturing) {
+        SIE_TRY(apply_Z(op, x, E, nullptr));
+        return apply_sys_rest(op, x, E, x + ne, y);
+    }
+    cudaStream_t st = op->mesh->ctx->stream, sb = op->gs[1];
+    double2* yb = op->sys_tmp + ne + 2 * op->mesh->h.nt;
+    SIE_CUDA_TRY(cudaEventRecord(op->gev[0], st));
+    SIE_CUDA_TRY(cudaStreamWaitEvent(sb, op->gev[0], 0));
+    SIE_TRY(sys_charge(op, sb, x, x + ne, yb, y + ne));
+    SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * ne, st));
+    SIE_TRY(apply_Z(op, x, E, nullptr));
+    SIE_CUDA_TRY(cudaEventRecord(op->gev[1], st));
+    SIE_CUDA_TRY(cudaStreamWaitEvent(sb, op->gev[1], 0));
+    SIE_TRY(sys_near(op, sb, x, E, yb));
+    SIE_CUDA_TRY(cudaEventRecord(op->gev[2], sb));
+    SIE_TRY(sys_grid(op, x, E, x + ne, y));
+    SIE_CUDA_TRY(cudaStreamWaitEvent(st, op->gev[2], 0));
+    return axpby(st, ne, 1.0, yb, 1.0, y);
 }
 
 // ------------------------------------------------------------------ graph of the system product
@@ -1237,8 +1282,12 @@ static sie_status build_sys_graph(sie_op* op)
     // everything the product touches exists before the capture starts
     SIE_TRY(op->kin.alloc(c->stream, ne, inner_m(op)));
     if (!op->g_io) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->g_io, sizeof(double2) * 2 * n, c->stream));
-    for (int i = 0; i < 2; i++)
-        if (!op->gs[i]) SIE_CUDA_TRY(cudaStreamCreateWithFlags(&op->gs[i], cudaStreamNonBlocking));
+    int lo = 0, hi = 0;
+    SIE_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    for (int i = 0; i < 2; i++)  // the branch gives way to the main chain
+        if (!op->gs[i]) SIE_CUDA_TRY(cudaStreamCreateWithPriority(&op->gs[i], cudaStreamNonBlocking, i ? lo : hi));
+    for (cudaEvent_t& ev : op->gev)
+        if (!ev) SIE_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     SIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
     cudaStream_t saved = c->stream;
     c->stream = op->gs[0];
@@ -1610,7 +1659,7 @@ sie_status sys_prepare(sie_op* op)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->elen, sizeof(double) * h.ne, st));
     SIE_CUDA_TRY(cudaMemcpyAsync(op->elen, h.edge_len.data(), sizeof(double) * h.ne, cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_E, sizeof(double2) * h.ne, st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_tmp, sizeof(double2) * (h.ne + 2 * h.nt), st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_tmp, sizeof(double2) * 2 * (h.ne + h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_vec, sizeof(double2) * 4 * (h.ne + h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * 6, st));
     SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
@@ -1632,6 +1681,10 @@ void sys_release(sie_op* op)
     sys_graph_reset(op);
     cudaStreamSynchronize(st);
     constraint_lu_release(op);
+    for (cudaEvent_t& ev : op->gev) {
+        if (ev) cudaEventDestroy(ev);
+        ev = nullptr;
+    }
     for (cudaStream_t& g : op->gs)
         if (g) {
             cudaStreamDestroy(g);
