@@ -38,7 +38,8 @@
  * Errors: every call returns a sie_status; nothing aborts or exits.
  * sie_last_error() returns a message for the last failing call on the
  * calling thread.  Calls on one context must not overlap in time (one host
- * thread at a time); all device work is issued on the context's stream.
+ * thread at a time); all device work is issued on the context's stream, or on
+ * branches that leave it and join it again within the call.
  */
 #ifndef SIE_H
 #define SIE_H
@@ -229,8 +230,8 @@ sie_status sie_op_stats(const sie_op* op, double out[6]);
  * near region, [15] host-side pair lists; [16] system-product CUDA graph
  * (near-region-only interiors): +1 captured for SIE_FP64, +2 for SIE_MIXED,
  * +4 capture failed (the stream path is used); [17] nodes of the last
- * captured graph outside the nested loop (kernels, memsets, copies and the
- * loop node), [18] nodes of the loop body (run once per nested iteration);
+ * captured graph (kernels, memsets, copies; the nested solve is one kernel),
+ * [18] 0 (no node runs once per nested iteration);
  * [19] wall time in ms of the dense factorisations of the constraint
  * preconditioners' triangle systems (0 when they are solved iteratively,
  * minus the sie_status when the factorisation could not be made, e.g. -3 for
@@ -256,9 +257,10 @@ sie_status sie_op_grid(const sie_op* op, double origin[3], double* h, int64_t N[
  * synchronise and report it through sie_op_stats.
  * When the interior operator is near-region only and profiling is off, the
  * SYS product (nested solve included) is captured on first use into a CUDA
- * graph, one per precision, and replayed; the nested iterations are then a
- * loop the device ends itself, with the same iteration limit as the stream
- * path.  The environment variable SIE_GRAPH=0 selects the stream path.  The
+ * graph, one per precision, and replayed; the nested solve is one kernel
+ * that ends its own iterations, as on the stream path (a wait inside it that
+ * runs out is SIE_ERR_TIMEOUT, reported like an inexact nested solve).  The
+ * environment variable SIE_GRAPH=0 selects the stream path.  The
  * graph is dropped when tol_inner or inner_maxit change (sie_op_set_solver). */
 sie_status sie_matvec(sie_op* op, int which, const double* x, double* y, int nrhs, int flags);
 

@@ -315,8 +315,14 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
     sie_ctx* pc = op->mesh->ctx;
     cudaStream_t st = pc->stream;
     const DevMesh& M = op->mesh->d;
+    // the near part first: it writes every y, the grid part adds
+    {
+        Stage s_(pc, a.has_grid ? "spmv_aim" : "spmv_near_only");
+        const double2* v = which_LK == 0 ? a.valL : a.valK;
+        SIE_CUDA_TRY(csr_launch(st, M.ne, a.nnz, a.row_ptr, a.col, v, x, make_double2(1.0, 0.0), false, y));
+        SIE_CUDA_TRY(cudaGetLastError());
+    }
     if (a.has_grid) {
-        SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * M.ne, st));
         const GridDesc& g = a.g;
         int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
         int ngrid = which_LK == 0 ? 4 : 3;
@@ -343,13 +349,6 @@ sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, doubl
             Stage s_(pc, "interp");
             SIE_TRY(aim_interp(op, src, which_LK == 0, make_double2(sc.real(), sc.imag()), y, M.ne, 1));
         }
-    }
-    {
-        Stage s_(pc, a.has_grid ? "spmv_aim" : "spmv_near_only");
-        // near-only operators have no grid term: the product overwrites y
-        const double2* v = which_LK == 0 ? a.valL : a.valK;
-        SIE_CUDA_TRY(csr_launch(st, M.ne, a.nnz, a.row_ptr, a.col, v, x, make_double2(1.0, 0.0), a.has_grid, y));
-        SIE_CUDA_TRY(cudaGetLastError());
     }
     return SIE_OK;
 }

@@ -44,7 +44,7 @@ __global__ void k_specmul_b(int mode, int nr, const double2* __restrict__ spec, 
     }
 }
 
-// Y[r] (+)= A X[r] for r < nr <= GL: a warp per row.  GL lanes share an entry, one
+// Y[r] = A X[r] for r < nr <= GL: a warp per row.  GL lanes share an entry, one
 // right-hand side each, so 32 / GL entries are in work at a time; the value is one
 // broadcast load and the vectors, interleaved by k_pack_rhs, one coalesced row of GL
 // per entry (rhs-major vectors cost nr scattered 16-byte gathers).  Only the 32 / GL
@@ -54,7 +54,7 @@ __global__ void k_specmul_b(int mode, int nr, const double2* __restrict__ spec, 
 template <int GL>
 __global__ void __launch_bounds__(128) k_csr_panel(int nrow, const int64_t* __restrict__ rp,
                                                    const int32_t* __restrict__ col, const double2* __restrict__ val,
-                                                   const double2* __restrict__ Xp, int nr, int acc,
+                                                   const double2* __restrict__ Xp, int nr,
                                                    double2* __restrict__ Y, int64_t ldy)
 {
     const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
@@ -93,14 +93,7 @@ __global__ void __launch_bounds__(128) k_csr_panel(int nrow, const int64_t* __re
         yr += __shfl_xor_sync(0xffffffffu, yr, off);
         yi += __shfl_xor_sync(0xffffffffu, yi, off);
     }
-    if (sl == 0 && r < nr) {
-        double2* o = Y + r * ldy + row;
-        if (acc) {
-            yr += o->x;
-            yi += o->y;
-        }
-        *o = make_double2(yr, yi);
-    }
+    if (sl == 0 && r < nr) Y[r * ldy + row] = make_double2(yr, yi);
 }
 
 // Xp[c GL + r] = X[r ldx + c], zero for r >= nr
@@ -114,23 +107,21 @@ __global__ void k_pack_rhs(int64_t n, int nr, int GL, const double2* __restrict_
     Xp[i] = r < nr ? X[r * ldx + c] : make_double2(0, 0);
 }
 
-// Y = A X (acc: Y += A X) for nr <= RB vectors of an edge CSR matrix, rhs-major; the
-// values read once for all nr
-static sie_status csr_panel(sie_op* op, const int64_t* rp, const int32_t* col, const double2* val, const double2* X,
-                            int nr, bool acc, double2* Y)
+// Y = A X for nr <= RB vectors of an edge CSR matrix, rhs-major, on st; the values
+// read once for all nr
+static sie_status csr_panel(sie_op* op, cudaStream_t st, const int64_t* rp, const int32_t* col, const double2* val,
+                            const double2* X, int nr, double2* Y)
 {
-    cudaStream_t st = op->mesh->ctx->stream;
     const int ne = op->mesh->d.ne;
-    if (!op->bws_xp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_xp, sizeof(double2) * RB * ne, st));
     const int GL = nr > 4 ? 8 : (nr > 2 ? 4 : 2);
     k_pack_rhs<<<(unsigned)(((int64_t)ne * GL + 255) / 256), 256, 0, st>>>(ne, nr, GL, X, ne, op->bws_xp);
     const unsigned blocks = (unsigned)((ne + 3) / 4);
     if (GL == 8)
-        k_csr_panel<8><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
+        k_csr_panel<8><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, Y, ne);
     else if (GL == 4)
-        k_csr_panel<4><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
+        k_csr_panel<4><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, Y, ne);
     else
-        k_csr_panel<2><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, acc, Y, ne);
+        k_csr_panel<2><<<blocks, 128, 0, st>>>(ne, rp, col, val, op->bws_xp, nr, Y, ne);
     SIE_CUDA_TRY(cudaGetLastError());
     return SIE_OK;
 }
@@ -151,6 +142,11 @@ static sie_status batch_workspace(sie_op* op, double2** bufs, double2** src)
     return SIE_OK;
 }
 
+// entries x right-hand sides from which a branch for the near part pays for its events
+// (about 8 us; 2 M entries take 15 us).  K at 1,280 triangles, eight right-hand sides:
+// 317 -> 299 us; L at 20,480: 3,457 -> 3,409 us (both parts then bound by issue)
+constexpr int64_t BRANCH_MIN = 2000000;
+
 // Y = A X for nr vectors (nr <= RB, rhs-major, length N_e), A = L (which_LK 0)
 // or K (1) of operator a
 sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X, double2* Y, int nr)
@@ -163,8 +159,16 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
         set_error("aim_apply_block: block size out of range");
         return SIE_ERR_ARG;
     }
+    if (!op->bws_xp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_xp, sizeof(double2) * RB * ne, st));
+    // the near part (FP64 products) beside the grid part (atomics and integer transforms)
+    Branch br(op, a.has_grid && !pc->prof.on && a.nnz * nr >= BRANCH_MIN);
+    {
+        SIE_CUDA_TRY(br.follow());
+        Stage s_(pc, a.has_grid ? "spmv_block" : "spmv_near_only_block");
+        const double2* v = which_LK == 0 ? a.valL : a.valK;
+        SIE_TRY(csr_panel(op, br.st(), a.row_ptr, a.col, v, X, nr, Y));
+    }
     if (a.has_grid) {
-        SIE_CUDA_TRY(cudaMemsetAsync(Y, 0, sizeof(double2) * ne * nr, st));
         const GridDesc& g = a.g;
         const int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
         const int ngrid = which_LK == 0 ? 4 : 3;
@@ -188,14 +192,10 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
         std::complex<double> kk(a.kr, a.ki);
         std::complex<double> sc = which_LK == 0 ? -1.0 / (kk * kk) : std::complex<double>(0.0);
         {
+            SIE_CUDA_TRY(br.join());
             Stage s_(pc, "interp_block");
             SIE_TRY(aim_interp(op, src, which_LK == 0, make_double2(sc.real(), sc.imag()), Y, ne, nr));
         }
-    }
-    {
-        Stage s_(pc, a.has_grid ? "spmv_block" : "spmv_near_only_block");
-        const double2* v = which_LK == 0 ? a.valL : a.valK;
-        SIE_TRY(csr_panel(op, a.row_ptr, a.col, v, X, nr, a.has_grid, Y));
     }
     return SIE_OK;
 }

@@ -286,7 +286,7 @@ struct sie_op {
     sie::PanelWork kmulti;          // lockstep solves: one Krylov basis per right-hand side
     sie::PanelWork kcs_multi;       // ... and per triangle system of their constraint preconditioner
     sie::PanelWork kzp;             // lockstep block products: the nested interior solves of the block
-    double2* zp = nullptr;          // block products: H, E, rhs and scratch panels (4 x 8 ne)
+    double2* zp = nullptr;          // block products: H, E and branch sum panels (3 x 8 ne)
     double2* mscr = nullptr;        // lockstep solves: per right-hand side scratch (8 blocks)
     double2* ir_multi = nullptr;    // lockstep refinement: residuals, corrections, products (3 x 8 (ne + nt))
     double2* con_scr = nullptr;     // their constraint preconditioner in one kernel: 8 (ne + 2 nt)
@@ -294,19 +294,18 @@ struct sie_op {
     double2 *cs_e = nullptr, *cs_t = nullptr, *pc_e = nullptr, *pc_t = nullptr;  // preconditioner scratch
     // last solve: outer iters, relres; max nested iters, relres; max constraint iters, relres
     double stats[6] = {0, 0, 0, 0, 0, 0};
-    // CUDA graph of the system product (near-only interior, profiling off): the
-    // nested solve is a device-controlled while loop inside the graph
+    // CUDA graph of the system product (near-only interior, profiling off)
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one per precision (SIE_FP64, SIE_MIXED)
     bool gfailed = false;           // capture or instantiation failed: stream path only
-    bool capturing = false;         // apply_Z emits the device-controlled nested solve
-    cudaStream_t gs[2] = {nullptr, nullptr};  // capture streams: main chain, branch beside it
-    cudaEvent_t gev[3] = {nullptr, nullptr, nullptr};  // fork, E known, join
+    bool capturing = false;         // apply_sys is being captured
+    cudaStream_t gs[2] = {nullptr, nullptr};  // capture of the product; branch beside the main chain
+    cudaEvent_t gev[2] = {nullptr, nullptr};  // main -> branch, branch -> main
     double2* g_io = nullptr;        // graph input x and output y, 2 (ne + nt)
     // device (6): largest nested iteration count and residual since cleared, those of the
     // the last nested solve (residual, count)
     double* gstat = nullptr;
     unsigned* res_bar = nullptr;    // resident kernels: barrier counter, error flag, lockstep flags (RES_WORDS)
-    size_t gnodes[2] = {0, 0};      // nodes of the last captured graph: outside the loop, loop body
+    size_t gnodes[2] = {0, 0};      // nodes of the last captured graph; 0
     double2* ir_buf = nullptr;      // iterative refinement: residual, correction, product (3 (ne + nt))
     double q_w = 0.0;               // charge-row weight of the GMRES residual norm (0: not yet computed)
     double2* bal = nullptr;         // weighted right-hand side and preconditioner input (2 (ne + nt))
@@ -358,6 +357,35 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q);
 sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, double2* y);
 // Y = A X for nr <= 8 vectors at once (spectra, weights and near values read once)
 sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X, double2* Y, int nr);
+// Work beside the context's stream: st() is the operator's branch stream between
+// follow() (it waits for the main stream's work so far) and join() (the main stream
+// waits for it; also on destruction, so no call returns with unordered work).  off:
+// st() is the context's stream and nothing is forked.
+class Branch {
+public:
+    Branch(sie_op* op, bool on) : op_(op), on_(on && op->gs[1]) {}
+    ~Branch() { join(); }
+    cudaStream_t st() const { return on_ ? op_->gs[1] : op_->mesh->ctx->stream; }
+    cudaError_t follow()
+    {
+        if (!on_) return cudaSuccess;
+        open_ = true;
+        const cudaError_t e = cudaEventRecord(op_->gev[0], op_->mesh->ctx->stream);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(op_->gs[1], op_->gev[0], 0);
+    }
+    cudaError_t join()
+    {
+        if (!open_) return cudaSuccess;
+        open_ = false;
+        const cudaError_t e = cudaEventRecord(op_->gev[1], op_->gs[1]);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(op_->mesh->ctx->stream, op_->gev[1], 0);
+    }
+
+private:
+    sie_op* op_;
+    bool on_, open_ = false;
+};
+
 sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y, int64_t ldy, int nr);
 sie_status aim_project(sie_op* op, const double2* x, int64_t ldx, int nr, int ngrid, double2* tc, double2* src);
 sie_status sys_prepare(sie_op* op);

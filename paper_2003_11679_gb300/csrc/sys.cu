@@ -951,8 +951,7 @@ static GL8 gl_rule(int n)
 static sie_status constraint_solve(sie_op* op, AimOp& a, cplx kappa, KrylovWork& K, double tol, const double2* v,
                                    double2* y);
 
-// Krylov basis of the nested solve: it runs without restart, so the graph's
-// device-ended loop and the stream path take the same iterations
+// Krylov basis of the nested solve: it runs without restart, in and outside a graph
 constexpr int INNER_BASIS_MAX = 128;
 static int inner_m(const sie_op* op) { return std::max(1, std::min(op->p.inner_maxit, INNER_BASIS_MAX)); }
 
@@ -1212,50 +1211,33 @@ static sie_status sys_grid(sie_op* op, const double2* H, const double2* E, const
     return SIE_OK;
 }
 
-// the system product after the interior impedance: y = SYS [H; rho] with
-// E = Z' H already computed (every step of Eq. sys but the nested solve)
-static sie_status apply_sys_rest(sie_op* op, const double2* H, const double2* E, const double2* rho, double2* y)
-{
-    cudaStream_t st = op->mesh->ctx->stream;
-    const int64_t ne = op->mesh->h.ne;
-    double2* yb = op->sys_tmp + ne + 2 * op->mesh->h.nt;
-    SIE_TRY(sys_charge(op, st, H, rho, yb, y + ne));
-    SIE_TRY(sys_near(op, st, H, E, yb));
-    SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * ne, st));
-    SIE_TRY(sys_grid(op, H, E, rho, y));
-    return axpby(st, ne, 1.0, yb, 1.0, y);
-}
-
-// y = SYS x, x = [H (ne); c0 rho (nt)].  Captured into a graph, the charge part runs
-// beside the nested solve and the near part beside the transforms, on a branch.
+// y = SYS x, x = [H (ne); c0 rho (nt)].  The charge part runs beside the nested solve
+// and the near part (FP64 products) beside the transforms (integer), on a branch when
+// the product is captured: a bar of 336 triangles 154 -> 142 us, 20,480 triangles
+// 1,265 -> 1,177 us.  The interpolation adds two triangles' values to an edge of zeros,
+// the branch sums into yb: every sum keeps a fixed order.
 static sie_status apply_sys(sie_op* op, const double2* x, double2* y)
 {
     const int64_t ne = op->mesh->h.ne;
     double2* E = op->sys_E;
-    if (!op->capturing) {
-        SIE_TRY(apply_Z(op, x, E, nullptr));
-        return apply_sys_rest(op, x, E, x + ne, y);
-    }
-    cudaStream_t st = op->mesh->ctx->stream, sb = op->gs[1];
     double2* yb = op->sys_tmp + ne + 2 * op->mesh->h.nt;
-    SIE_CUDA_TRY(cudaEventRecord(op->gev[0], st));
-    SIE_CUDA_TRY(cudaStreamWaitEvent(sb, op->gev[0], 0));
-    SIE_TRY(sys_charge(op, sb, x, x + ne, yb, y + ne));
+    Branch br(op, op->capturing);
+    SIE_CUDA_TRY(br.follow());
+    SIE_TRY(sys_charge(op, br.st(), x, x + ne, yb, y + ne));
+    cudaStream_t st = op->mesh->ctx->stream;
     SIE_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(double2) * ne, st));
     SIE_TRY(apply_Z(op, x, E, nullptr));
-    SIE_CUDA_TRY(cudaEventRecord(op->gev[1], st));
-    SIE_CUDA_TRY(cudaStreamWaitEvent(sb, op->gev[1], 0));
-    SIE_TRY(sys_near(op, sb, x, E, yb));
-    SIE_CUDA_TRY(cudaEventRecord(op->gev[2], sb));
+    SIE_CUDA_TRY(br.follow());
+    SIE_TRY(sys_near(op, br.st(), x, E, yb));
     SIE_TRY(sys_grid(op, x, E, x + ne, y));
-    SIE_CUDA_TRY(cudaStreamWaitEvent(st, op->gev[2], 0));
+    SIE_CUDA_TRY(br.join());
     return axpby(st, ne, 1.0, yb, 1.0, y);
 }
 
 // ------------------------------------------------------------------ graph of the system product
 // For a near-region-only interior the whole product (nested solve included)
-// is captured once into a CUDA graph: one launch per product instead of ~80,
-// and the nested iteration count is decided on the device.  One graph per
+// is captured once into a CUDA graph: one launch per product instead of about 20,
+// and no host wait for the nested solve, which is one kernel.  One graph per
 // precision; dropped when the nested-solve settings change.  SIE_GRAPH=0 in the
 // environment keeps the stream path (for comparison).
 static bool graph_enabled()
@@ -1282,12 +1264,6 @@ static sie_status build_sys_graph(sie_op* op)
     // everything the product touches exists before the capture starts
     SIE_TRY(op->kin.alloc(c->stream, ne, inner_m(op)));
     if (!op->g_io) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->g_io, sizeof(double2) * 2 * n, c->stream));
-    int lo = 0, hi = 0;
-    SIE_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-    for (int i = 0; i < 2; i++)  // the branch gives way to the main chain
-        if (!op->gs[i]) SIE_CUDA_TRY(cudaStreamCreateWithPriority(&op->gs[i], cudaStreamNonBlocking, i ? lo : hi));
-    for (cudaEvent_t& ev : op->gev)
-        if (!ev) SIE_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     SIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
     cudaStream_t saved = c->stream;
     c->stream = op->gs[0];
@@ -1659,6 +1635,12 @@ sie_status sys_prepare(sie_op* op)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->elen, sizeof(double) * h.ne, st));
     SIE_CUDA_TRY(cudaMemcpyAsync(op->elen, h.edge_len.data(), sizeof(double) * h.ne, cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_E, sizeof(double2) * h.ne, st));
+    int lo = 0, hi = 0;
+    SIE_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    for (int i = 0; i < 2; i++)  // the branch gives way to the main chain
+        if (!op->gs[i]) SIE_CUDA_TRY(cudaStreamCreateWithPriority(&op->gs[i], cudaStreamNonBlocking, i ? lo : hi));
+    for (cudaEvent_t& ev : op->gev)
+        if (!ev) SIE_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_tmp, sizeof(double2) * 2 * (h.ne + h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_vec, sizeof(double2) * 4 * (h.ne + h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * 6, st));
@@ -2078,13 +2060,24 @@ static sie_status apply_sys_multi(sie_op* op, int R, const double2* const* x, do
     }
     cudaStream_t st = op->mesh->ctx->stream;
     const int64_t ne = op->mesh->h.ne;
-    if (!op->zp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->zp, sizeof(double2) * 4 * MULTI_RHS * ne, st));
+    if (!op->zp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->zp, sizeof(double2) * 3 * MULTI_RHS * ne, st));
     double2* Hp = op->zp;
     double2* Ep = op->zp + MULTI_RHS * ne;
+    double2* Bp = op->zp + 2 * MULTI_RHS * ne;
+    Branch br(op, !op->mesh->ctx->prof.on);  // as in apply_sys
+    SIE_CUDA_TRY(br.follow());
+    for (int q = 0; q < R; q++) SIE_TRY(sys_charge(op, br.st(), x[q], x[q] + ne, Bp + q * ne, y[q] + ne));
     for (int q = 0; q < R; q++)
         SIE_CUDA_TRY(cudaMemcpyAsync(Hp + q * ne, x[q], sizeof(double2) * ne, cudaMemcpyDeviceToDevice, st));
     SIE_TRY(apply_Z_panel(op, R, Hp, Ep));
-    for (int q = 0; q < R; q++) SIE_TRY(apply_sys_rest(op, x[q], Ep + q * ne, x[q] + ne, y[q]));
+    SIE_CUDA_TRY(br.follow());
+    for (int q = 0; q < R; q++) SIE_TRY(sys_near(op, br.st(), x[q], Ep + q * ne, Bp + q * ne));
+    for (int q = 0; q < R; q++) {
+        SIE_CUDA_TRY(cudaMemsetAsync(y[q], 0, sizeof(double2) * ne, st));
+        SIE_TRY(sys_grid(op, x[q], Ep + q * ne, x[q] + ne, y[q]));
+    }
+    SIE_CUDA_TRY(br.join());
+    for (int q = 0; q < R; q++) SIE_TRY(axpby(st, ne, 1.0, Bp + q * ne, 1.0, y[q]));
     return SIE_OK;
 }
 
