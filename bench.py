@@ -209,15 +209,16 @@ def stage_model(stage, info, ne, nt, nnz_ext, nnz_int):
     return r
 
 
-# grids per FFT launch in the system product: 7 forward (H, E, rho sources), 4 inverse
-FFT_GRIDS = {"fft_fwd_x": 7, "fft_fwd_y": 7, "fft_fwd_z": 7, "fft_inv_z": 4, "fft_inv_y": 4, "fft_inv_x": 4}
+# grids per FFT launch in the system product: 7 forward (H, E, rho sources), 4 inverse;
+# the rest of the sparse products is recorded in two parts (charge rows, I-cross E)
+FFT_GRIDS = {"spmv_sys_rest": 0.5, "fft_fwd_x": 7, "fft_fwd_y": 7, "fft_fwd_z": 7, "fft_inv_z": 4, "fft_inv_y": 4, "fft_inv_x": 4}
 
 # DRAM bytes (read + write) per launch of a stage's kernel from one ncu capture,
 # with the hash of the library sources it was taken on (stale once they change).
 # k_fft_z<128,Fx,ZM_SYS> on the 128^3 FFT grid: the grid part has the same
 # size at every mesh level of the copper workload, so the capture on the
 # 480-RWG mesh holds per launch for the 30,720-RWG one.
-TRAFFIC = {("fft_z_specmul", "fp64"): (249870080 + 47390208, "f124e1ac95d297f3")}
+TRAFFIC = {("fft_z_specmul", "fp64"): (250122496 + 46384128, "710465e61225b3dc")}
 
 
 # stages whose FP64 form computes in 64-bit block fixed point (integer multiply-adds)
