@@ -214,14 +214,21 @@ __global__ void k_to_c64(const double2* __restrict__ a, float2* __restrict__ b, 
     if (i < n) b[i] = make_float2((float)a[i].x, (float)a[i].y);
 }
 
+sie_status aim_sample(cudaStream_t st, const GridDesc& g, double kr, double ki, double2* spec)
+{
+    const int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    k_sample<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(g, kr, ki, spec, nn);
+    SIE_CUDA_TRY(cudaGetLastError());
+    return SIE_OK;
+}
+
 sie_status aim_spectra(sie_op* op, AimOp& a)
 {
     cudaStream_t st = op->mesh->ctx->stream;
     const GridDesc& g = a.g;
     int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2];
     SIE_CUDA_TRY(cudaMallocAsync((void**)&a.spec, sizeof(double2) * 4 * nn, st));
-    k_sample<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(g, a.kr, a.ki, a.spec, nn);
-    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_TRY(aim_sample(st, g, a.kr, a.ki, a.spec));
     SIE_TRY(fft3d(st, a.spec, (const double2*)nullptr, g, -1, 0, nullptr, 4));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&a.spec32, sizeof(float2) * 4 * nn, st));
     k_to_c64<<<(unsigned)((4 * nn + 255) / 256), 256, 0, st>>>(a.spec, a.spec32, 4 * nn);
@@ -469,6 +476,9 @@ sie_status sie_op_build(sie_mesh* mesh, double freq_hz, double eps_r, double mu_
     op->ext.kr = op->k0;
     op->ext.ki = 0.0;
     op->ext.has_grid = true;
+    // interior operator (Sec. III-C): near-only when every pair inside the skin-depth
+    // cutoff is a near pair, else AIM on the object grid; none for SIE_SIBC
+    op->inn.has_grid = op->p.interior_model != SIE_SIBC && nobj == 1 && om[0].cut > (g.Rnear - g.M) * g.h;
     auto now = [] { return std::chrono::steady_clock::now(); };
     auto ms = [](std::chrono::steady_clock::time_point a, std::chrono::steady_clock::time_point b) {
         return std::chrono::duration<double, std::milli>(b - a).count();
@@ -494,13 +504,10 @@ sie_status sie_op_build(sie_mesh* mesh, double freq_hz, double eps_r, double mu_
     }
     auto t3 = now();
     op->build_ms[1] = ms(t2, t3);
-    // interior operator (Sec. III-C): near-only when every pair inside the
-    // skin-depth cutoff is a near pair, else AIM on the object grid (shared
-    // with the exterior grid for a single object)
+    // interior operator (an interior grid is shared with the exterior's)
     op->inn.kr = ki.real();
     op->inn.ki = ki.imag();
     op->inn.g = g;
-    const double cut = om[0].cut;
     op->eta_re = om[0].eta.real();
     op->eta_im = om[0].eta.imag();
     if (nobj > 1) {
@@ -515,7 +522,7 @@ sie_status sie_op_build(sie_mesh* mesh, double freq_hz, double eps_r, double mu_
         if ((s = up(st, &op->edge_zf, zf.data(), zf.size())) != SIE_OK) return fail(s);
     }
     if (op->p.interior_model == SIE_SIBC) {
-        op->inn.has_grid = false;  // no interior operators: Z' comes from the Gram system
+        // no interior operators: Z' comes from the Gram system
     } else if (nobj > 1) {
         for (int o = 0; o < nobj; o++)
             if (om[o].cut > (g.Rnear - g.M) * g.h) {
@@ -524,7 +531,6 @@ sie_status sie_op_build(sie_mesh* mesh, double freq_hz, double eps_r, double mu_
                           "(5 skin depths inside the near region) or interior_model = SIE_SIBC");
                 return fail(SIE_ERR_UNSUPPORTED);
             }
-        op->inn.has_grid = false;
         std::vector<double> cuts(nobj);
         std::vector<double2> kk(nobj), ik2(nobj);
         for (int o = 0; o < nobj; o++) {
@@ -536,11 +542,9 @@ sie_status sie_op_build(sie_mesh* mesh, double freq_hz, double eps_r, double mu_
         near_pairs_cutoff_objects(mesh->h, cuts, op->inn.hpairs);
         if ((s = up(st, &op->inn.obj_k, kk.data(), kk.size())) != SIE_OK) return fail(s);
         if ((s = up(st, &op->inn.obj_ik2, ik2.data(), ik2.size())) != SIE_OK) return fail(s);
-    } else if (cut <= (g.Rnear - g.M) * g.h) {
-        op->inn.has_grid = false;
-        near_pairs_cutoff(mesh->h, cut, op->inn.hpairs);
+    } else if (!op->inn.has_grid) {
+        near_pairs_cutoff(mesh->h, om[0].cut, op->inn.hpairs);
     } else {
-        op->inn.has_grid = true;
         if ((s = aim_spectra(op, op->inn)) != SIE_OK) return fail(s);
         op->inn.hpairs = op->ext.hpairs;
     }

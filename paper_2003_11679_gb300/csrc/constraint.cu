@@ -1,5 +1,5 @@
-// Constraint preconditioners as one kernel per application, a cluster per
-// right-hand side (resident.cuh, CluMem):
+// Constraint preconditioners as one kernel per application, a cluster of CTAs
+// (resident.cuh, CluMem):
 //   (Dg - kappa D^T Lphi_NR D) y = v             (Eq. nest2pc, nested)
 // by block elimination on the charges q = D y,
 //   (I - kappa D Dg^-1 D^T Lphi_NR) q = D Dg^-1 v,  y = Dg^-1 (v + kappa D^T Lphi_NR q),
@@ -8,9 +8,8 @@
 // restarted FGMRES preconditioned by the explicit complex64 inverse: FP32 products
 // and per-lane sums, row sums in FP64.
 // The work is small and was latency-bound: 14 launches an iteration and a host
-// check took 118 us (320 triangles) to 220 us (1,280) an application, 2.8 ms for
-// eight right-hand sides of a 336-triangle bar one after another.  One application
-// takes 42 and 125 us now.  An iteration meets at 5 cluster barriers; the inverse is read by 8 or 16 SMs
+// check took 118 us (320 triangles) to 220 us (1,280) an application; 42 and 125 us
+// now.  An iteration meets at 5 cluster barriers; the inverse is read by 8 or 16 SMs
 // (1,280 triangles: 13 MB, about 6 us), which bounds the size it is taken for
 // (CLU_MAXN triangles).
 #include <algorithm>
@@ -30,9 +29,9 @@ struct ConSys {
     const float2* X;            // explicit inverse, nt x nt
     double2 kappa, ijk0;        // ijk0 = 1 / (j k0)
     int ext;                    // 1: the exterior AEFIE preconditioner of [x1; x2]
-    const double2* x[8];        // ne, or ne + nt
-    double2* y[8];
-    double2 *v1, *b, *q;        // scratch per right-hand side: ne, nt, nt
+    const double2* x;           // ne, or ne + nt
+    double2* y;
+    double2 *v1, *b, *q;        // scratch: ne, nt, nt
     double* stat;               // largest iteration count and residual
 };
 
@@ -44,7 +43,6 @@ struct ConClu {
     int G;
     int64_t r0;
     int rows;
-    double2* Z;
 
     // l_e (phi_T+ - phi_T-)
     __device__ __forceinline__ double2 dt(int e, const double2* phi) const
@@ -134,7 +132,7 @@ struct ConClu {
                 }
             }
             const double2 z = warp_sum(make_double2((double)ar + br, (double)ai + bi));
-            if (lane == 0) Z[(int64_t)j * K.n + r0 + k] = z;
+            if (lane == 0) K.Z[(int64_t)j * K.n + r0 + k] = z;
             if (lane < M.C) *cooperative_groups::this_cluster().map_shared_rank(M.xz + r0 + k, lane) = z;
         }
         return true;
@@ -147,19 +145,18 @@ struct ConClu {
     }
 };
 
-__global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, CluLock lock, int maxit, int G)
+__global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, int maxit, int G)
 {
     extern __shared__ __align__(16) double2 rs_smem[];
     CluMem M(rs_smem, K.n, K.m);
     float2* xf = reinterpret_cast<float2*>(M.h2 + M.ld);
-    const int q = (int)blockIdx.x / M.C;
     const int64_t len = (s.nt + M.C - 1) / M.C, r0 = min((int64_t)s.nt, M.rank * len);
     const int rows = (int)(min((int64_t)s.nt, r0 + len) - r0);
     const int elen = (s.ne + M.C - 1) / M.C, e0 = min(s.ne, M.rank * elen), e1 = min(s.ne, e0 + elen);
-    ConClu ops{s, K, M, xf, G, r0, rows, K.Z + (int64_t)q * K.m * K.n};
-    const double2 *x1 = s.x[q], *x2 = s.x[q] + s.ne;
-    double2 *y1 = s.y[q], *y2 = s.y[q] + s.ne;
-    double2 *v1 = s.v1 + (int64_t)q * s.ne, *b = s.b + (int64_t)q * s.nt, *sol = s.q + (int64_t)q * s.nt;
+    ConClu ops{s, K, M, xf, G, r0, rows};
+    const double2 *x1 = s.x, *x2 = s.x + s.ne;
+    double2 *y1 = s.y, *y2 = s.y + s.ne;
+    double2 *v1 = s.v1, *b = s.b, *sol = s.q;
     clu_sync();  // every CTA has started: distributed shared memory may be written
     // v1' = v1 - (j k0)^-1 D^T Lphi B v2, B v2 = -A v2
     if (s.ext) {
@@ -189,16 +186,11 @@ __global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, 
     __syncthreads();
     CluRun run;
     run.maxit = maxit;
-    bool lost = false;
     for (;;) {
-        const int jend = clu_fgmres(ops, K, M, q, lock, run);
-        if (jend < 0) {
-            lost = true;
-            break;
-        }
+        const int jend = clu_fgmres(ops, K, M, run);
         for (int k = threadIdx.x; k < rows; k += blockDim.x) {
             double2 x = sol[r0 + k];
-            for (int i = 0; i <= jend; i++) r_fma(x, ops.Z[(int64_t)i * K.n + r0 + k], M.g[i]);
+            for (int i = 0; i <= jend; i++) r_fma(x, K.Z[(int64_t)i * K.n + r0 + k], M.g[i]);
             sol[r0 + k] = x;
             M.xz[r0 + k] = x;
         }
@@ -215,39 +207,33 @@ __global__ void __launch_bounds__(RES_T, 1) k_constraint(ConSys s, ResKrylov K, 
         }
         __syncthreads();
     }
-    if (lost) {
-        if (threadIdx.x == 0) s.stat[1] = __longlong_as_double(0x7ff0000000000000ll);
-    } else {
-        if (M.rank == 0 && threadIdx.x == 0) res_stat_max(s.stat, run.it, run.rel);
-        // y = Dg^-1 (v1' + kappa D^T Lphi q) [/ (j k0)]; v1' of other CTAs' edges is complete since the first barriers
-        auto y_of = [&](int e) {
-            const double2 k = r_cm(s.kappa, ops.dt(e, M.xv)), v = __ldcg(v1 + e);
-            const double2 y = r_cm(s.idLA[e], make_double2(v.x + k.x, v.y + k.y));
-            return s.ext ? r_cm(s.ijk0, y) : y;
-        };
-        for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) y1[e] = y_of(e);
-        if (s.ext)
-            for (int k = threadIdx.x; k < rows; k += blockDim.x) {
-                const int t = (int)r0 + k;
-                const double2 d = ops.dsum(t, y_of), v = x2[t];
-                const double a = s.M.area[t];
-                y2[t] = r_cm(s.ijk0, make_double2(v.x - d.x / a, v.y - d.y / a));
-            }
-    }
+    if (M.rank == 0 && threadIdx.x == 0) res_stat_max(s.stat, run.it, run.rel);
+    // y = Dg^-1 (v1' + kappa D^T Lphi q) [/ (j k0)]; v1' of other CTAs' edges is complete since the first barriers
+    auto y_of = [&](int e) {
+        const double2 k = r_cm(s.kappa, ops.dt(e, M.xv)), v = __ldcg(v1 + e);
+        const double2 y = r_cm(s.idLA[e], make_double2(v.x + k.x, v.y + k.y));
+        return s.ext ? r_cm(s.ijk0, y) : y;
+    };
+    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) y1[e] = y_of(e);
+    if (s.ext)
+        for (int k = threadIdx.x; k < rows; k += blockDim.x) {
+            const int t = (int)r0 + k;
+            const double2 d = ops.dsum(t, y_of), v = x2[t];
+            const double a = s.M.area[t];
+            y2[t] = r_cm(s.ijk0, make_double2(v.x - d.x / a, v.y - d.y / a));
+        }
     clu_sync();  // no CTA leaves while another may still write to its shared memory
 }
 
 // true: applied by the cluster kernel (and *st_out is its launch status)
-bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, int R, const double2* const* x,
-                         double2* const* y, double tol, int maxit, int restart, const ResWork& w, double2* v1, double2* b,
-                         double2* q, sie_status* st_out)
+bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, const double2* x, double2* y, double tol,
+                         int maxit, const ResWork& w, double2* v1, double2* b, double2* q, sie_status* st_out)
 {
     const int nt = (int)op->mesh->h.nt, ne = (int)op->mesh->h.ne;
-    if (!a.lu || !a.lu->Xinv || nt > CLU_MAXN || w.m != restart) return false;
-    const int C = clu_pick((const void*)k_constraint, nt, a.npairs, w.m, R, sizeof(float2) * (nt + 1));
+    if (!a.lu || !a.lu->Xinv || nt > CLU_MAXN) return false;
+    const int C = clu_pick((const void*)k_constraint, nt, a.npairs, w.m, sizeof(float2) * (nt + 1));
     if (!C) return false;
     const size_t smem = clu_smem(nt, w.m, C) + sizeof(float2) * (nt + 1);
-    cudaStream_t st = op->mesh->ctx->stream;
     ConSys s{};
     s.nt = nt, s.ne = ne;
     s.M = op->mesh->d;
@@ -258,24 +244,17 @@ bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, in
     s.kappa = kappa;
     s.ijk0 = make_double2(0.0, -1.0 / op->k0);
     s.ext = ext;
-    for (int r = 0; r < R; r++) s.x[r] = x[r], s.y[r] = y[r];
+    s.x = x, s.y = y;
     s.v1 = v1, s.b = b, s.q = q;
     s.stat = op->gstat + 4;
     ResKrylov K{};
-    K.n = nt, K.m = w.m, K.R = R;
-    K.V = w.V, K.Z = w.Z, K.H = w.H, K.ldh = w.ldh;
+    K.n = nt, K.m = w.m;
+    K.V = w.V, K.Z = w.Z, K.H = w.H;
     K.tol = tol;
     K.stat = s.stat;
-    CluLock lock;
-    lock.R = R, lock.lag = 0, lock.flag = op->res_bar + 2, lock.err = (int*)(op->res_bar + 1);
-    auto run = [&]() -> sie_status {
-        if (R > 1) SIE_CUDA_TRY(cudaMemsetAsync(lock.flag, 0, sizeof(unsigned) * 8 * CLU_RING, st));
-        const int64_t rows = (nt + C - 1) / C;
-        int G = res_group(rows, nt, a.npairs), mi = maxit;
-        void* args[] = {&s, &K, &lock, &mi, &G};
-        return clu_launch((const void*)k_constraint, C, R, smem, args, st);
-    };
-    *st_out = run();
+    int G = res_group((nt + C - 1) / C, nt, a.npairs);
+    void* args[] = {&s, &K, &maxit, &G};
+    *st_out = clu_launch((const void*)k_constraint, C, smem, args, op->mesh->ctx->stream);
     return true;
 }
 

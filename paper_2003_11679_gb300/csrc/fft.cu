@@ -1,7 +1,9 @@
 // FFTs of the AIM grid path: twiddle tables, pass dispatch by length, pruned 3D
 // transforms and the grid products (forward, spectral product, inverse).
 // Lengths to 256 take the two-pass kernels of fft.cuh (fixed point for
-// complex128), 512 and 1024 the Stockham kernel below.
+// complex128), 512 and 1024 the Stockham kernel below, and so do all (power-of-two)
+// lengths of the lockstep block product, whose FP64 butterflies are part of what its
+// solutions are to the last bit (block.cu).
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -18,7 +20,7 @@ SIE_FFT_LENGTHS(SIE_FFT_EXTERN)
 // first use (guarded: contexts may run in threads) and kept for the process
 constexpr int TW_MAXDEV = 64, TW_MAXLEN = 1024;
 struct TwTab {
-    double2* d = nullptr;  // (cos, -sin)
+    double2* d = nullptr;  // (cos, -sin); powers of two
     float2* f = nullptr;   // n <= 256: (cos, sin); else (cos, -sin)
     twq* q = nullptr;      // n <= 256
 };
@@ -56,17 +58,15 @@ static sie_status twiddles(int n, TwTab* out)
             const auto q = [](long double v) { return to_q62((long long)llroundl(ldexpl(v, 62))); };
             hq[m] = twq{q(c), q(c + s), q(s - c)};
         }
-        if (small)
-            SIE_TRY(tw_upload(&t.q, hq));
-        else
-            SIE_TRY(tw_upload(&t.d, hd));
+        if (small) SIE_TRY(tw_upload(&t.q, hq));
+        if ((n & (n - 1)) == 0) SIE_TRY(tw_upload(&t.d, hd));
         SIE_TRY(tw_upload(&t.f, hf));
     }
     *out = t;
     return SIE_OK;
 }
 
-// ------------------------------------------------------------------ lengths 512 and 1024: Stockham FFT (register radix-8, FP64 / FP32)
+// ------------------------------------------------------------------ powers of two: Stockham FFT (register radix-8, FP64 / FP32)
 // Self-sorting Stockham formulation (Govindaraju et al., SC'08): pass p with
 // current span Ns and radix R: thread j loads a[r] = x[j + r n/R], multiplies
 // by exp(-+2 pi i (j mod Ns) r / (Ns R)), does an R-point DFT in registers and
@@ -281,11 +281,11 @@ __global__ void __launch_bounds__(PB*(1 << LOGN) / 8) k_fft_stockham(const C* in
                                              nullptr, tw);
 }
 
-template <int LOGN, class C>
-static sie_status launch_stockham(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, const C* tw,
+template <int LOGN, int PB, class C>
+static sie_status launch_stockham_pb(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, const C* tw,
                                   int nbatch)
 {
-    constexpr int n = 1 << LOGN, PB = 2048 / n;  // 256 threads, n / 8 per pencil
+    constexpr int n = 1 << LOGN;
     const size_t smem = sizeof(C) * 2 * PB * (n + 1);
     // once per instantiation (thread-safe static initialisation)
     static const cudaError_t attr = [smem] {
@@ -305,6 +305,16 @@ static sie_status launch_stockham(cudaStream_t st, const C* in, C* out, int inv,
     return SIE_OK;
 }
 
+// 256 threads, n / 8 per pencil; half of that where it would leave less than 4 CTAs an SM
+template <int LOGN, class C>
+static sie_status launch_stockham(cudaStream_t st, const C* in, C* out, int inv, const PassGeom& G, const C* tw,
+                                  int nbatch)
+{
+    constexpr int PB = 2048 >> LOGN;
+    if (G.npencil * nbatch / PB >= 4LL * 152) return launch_stockham_pb<LOGN, PB, C>(st, in, out, inv, G, tw, nbatch);
+    return launch_stockham_pb<LOGN, PB / 2, C>(st, in, out, inv, G, tw, nbatch);
+}
+
 // ------------------------------------------------------------------ dispatch by length
 template <class C>
 struct PolicyOf;
@@ -322,7 +332,7 @@ struct PolicyOf<float2> {
 };
 
 template <class C>
-static sie_status launch_pass(cudaStream_t st, int n, const C* in, C* out, int inv, const PassGeom& G, int nb = 1)
+static sie_status launch_pass(cudaStream_t st, int n, const C* in, C* out, int inv, const PassGeom& G, int nb)
 {
     using PO = PolicyOf<C>;
     using P = typename PO::P;
@@ -335,6 +345,25 @@ static sie_status launch_pass(cudaStream_t st, int n, const C* in, C* out, int i
 #undef SIE_CASE
         case 512: return launch_stockham<9, C>(st, in, out, inv, G, PO::tws(t), nb);
         case 1024: return launch_stockham<10, C>(st, in, out, inv, G, PO::tws(t), nb);
+    }
+    set_error("unsupported FFT length");
+    return SIE_ERR_UNSUPPORTED;
+}
+
+// FP64 butterflies at any power of two
+static sie_status launch_pass_p2(cudaStream_t st, int n, const double2* in, double2* out, int inv, const PassGeom& G,
+                                 int nb)
+{
+    TwTab t;
+    SIE_TRY(twiddles(n, &t));
+    switch (n) {
+        case 16: return launch_stockham<4, double2>(st, in, out, inv, G, t.d, nb);
+        case 32: return launch_stockham<5, double2>(st, in, out, inv, G, t.d, nb);
+        case 64: return launch_stockham<6, double2>(st, in, out, inv, G, t.d, nb);
+        case 128: return launch_stockham<7, double2>(st, in, out, inv, G, t.d, nb);
+        case 256: return launch_stockham<8, double2>(st, in, out, inv, G, t.d, nb);
+        case 512: return launch_stockham<9, double2>(st, in, out, inv, G, t.d, nb);
+        case 1024: return launch_stockham<10, double2>(st, in, out, inv, G, t.d, nb);
     }
     set_error("unsupported FFT length");
     return SIE_ERR_UNSUPPORTED;
@@ -364,8 +393,8 @@ static sie_status launch_z(cudaStream_t st, int n, C* buf, const C* spec, int nz
 // dir = +1: inverse of the spectrum in buf; prune = 1 writes only the physical
 // N box into the compact array `src` (used as output), prune = 0 keeps n^3 in buf.
 // nbatch grids at once: grid k at buf + k n^3 and (compact) src + k N^3
-template <class C>
-static sie_status fft3d_t(cudaStream_t st, C* buf, const C* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
+template <class C, class PASS>
+static sie_status fft3d_t(PASS pass, cudaStream_t st, C* buf, const C* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
                           int nbatch)
 {
     const int64_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -378,37 +407,37 @@ static sie_status fft3d_t(cudaStream_t st, C* buf, const C* src, const GridDesc&
                    prune ? bNg : bnn, bnn};
         {
             Stage s_(pc, "fft_fwd_x");
-            SIE_TRY(launch_pass<C>(st, (int)nx, prune ? src : buf, buf, 0, X, nbatch));
+            SIE_TRY(pass(st, (int)nx, prune ? src : buf, buf, 0, X, nbatch));
         }
         // y pass: pencils (x < nx, z < Nz)
         PassGeom Y{(int)Ny, (int)ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
         {
             Stage s_(pc, "fft_fwd_y");
-            SIE_TRY(launch_pass<C>(st, (int)ny, buf, buf, 0, Y, nbatch));
+            SIE_TRY(pass(st, (int)ny, buf, buf, 0, Y, nbatch));
         }
         // z pass: pencils (x < nx, y < ny)
         PassGeom Z{(int)Nz, (int)nz, nx * ny, (int)nx, 1, nx, pyz, 1, nx, pyz, 0, bnn, bnn};
         {
             Stage s_(pc, "fft_fwd_z");
-            SIE_TRY(launch_pass<C>(st, (int)nz, buf, buf, 0, Z, nbatch));
+            SIE_TRY(pass(st, (int)nz, buf, buf, 0, Z, nbatch));
         }
     } else {
         PassGeom Z{(int)nz, (int)Nz, nx * ny, (int)nx, 1, nx, pyz, 1, nx, pyz, 0, bnn, bnn};
         {
             Stage s_(pc, "fft_inv_z");
-            SIE_TRY(launch_pass<C>(st, (int)nz, buf, buf, 1, Z, nbatch));
+            SIE_TRY(pass(st, (int)nz, buf, buf, 1, Z, nbatch));
         }
         PassGeom Y{(int)ny, (int)Ny, nx * Nz, (int)nx, 1, pyz, nx, 1, pyz, nx, 0, bnn, bnn};
         {
             Stage s_(pc, "fft_inv_y");
-            SIE_TRY(launch_pass<C>(st, (int)ny, buf, buf, 1, Y, nbatch));
+            SIE_TRY(pass(st, (int)ny, buf, buf, 1, Y, nbatch));
         }
         C* dst = prune ? const_cast<C*>(src) : buf;
         PassGeom X{(int)nx, (int)Nx, Ny * Nz, (int)Ny, nx, pyz, 1, prune ? Nx : nx, prune ? Nx * Ny : pyz, 1, 1,
                    bnn, prune ? bNg : bnn};
         {
             Stage s_(pc, "fft_inv_x");
-            SIE_TRY(launch_pass<C>(st, (int)nx, buf, dst, 1, X, nbatch));
+            SIE_TRY(pass(st, (int)nx, buf, dst, 1, X, nbatch));
         }
     }
     return SIE_OK;
@@ -417,13 +446,19 @@ static sie_status fft3d_t(cudaStream_t st, C* buf, const C* src, const GridDesc&
 sie_status fft3d(cudaStream_t st, double2* buf, const double2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
                  int nbatch)
 {
-    return fft3d_t(st, buf, src, g, dir, prune, pc, nbatch);
+    return fft3d_t(launch_pass<double2>, st, buf, src, g, dir, prune, pc, nbatch);
 }
 
 sie_status fft3d(cudaStream_t st, float2* buf, const float2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
                  int nbatch)
 {
-    return fft3d_t(st, buf, src, g, dir, prune, pc, nbatch);
+    return fft3d_t(launch_pass<float2>, st, buf, src, g, dir, prune, pc, nbatch);
+}
+
+sie_status fft3d_p2(cudaStream_t st, double2* buf, const double2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
+                    int nbatch)
+{
+    return fft3d_t(launch_pass_p2, st, buf, src, g, dir, prune, pc, nbatch);
 }
 
 // Grid product with the fused z stage: forward x and y passes of the compact

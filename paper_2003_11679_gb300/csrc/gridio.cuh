@@ -23,6 +23,10 @@ __device__ __forceinline__ R gio_sum(R v)
 __device__ __forceinline__ double gio_fma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float gio_fma(float a, float b, float c) { return fmaf(a, b, c); }
 
+// products that are not to be contracted with the sum they go into
+__device__ __forceinline__ double gio_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float gio_mul(float a, float b) { return __fmul_rn(a, b); }
+
 // the four weights (w0, w1) of a stencil entry: 16-byte loads
 __device__ __forceinline__ void gio_w(const double* w, double& w0, double* w1)
 {
@@ -108,6 +112,49 @@ __global__ void __launch_bounds__(256) k_interp(int nt, int S, int Mord, DevMesh
     atomicAdd(&d->y, c * vi);
 }
 
+template <class C>
+__device__ __forceinline__ C cmk(double a, double b)
+{
+    C c;
+    c.x = a;
+    c.y = b;
+    return c;
+}
+
+// tc: per triangle 9 values: alpha_H, beta_H[3], alpha_E, beta_E[3], -c0rho; vector
+// blockIdx.y: H, E and rho ldh, lde and ldr apart, tc 9 nt apart
+template <class C>
+__global__ void k_tri_coef(int nt, DevMesh M, const double2* __restrict__ H, int64_t ldh, const double2* __restrict__ E,
+                           int64_t lde, const double2* __restrict__ rho, int64_t ldr, C* __restrict__ tc)
+{
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nt) return;
+    H += blockIdx.y * ldh;
+    E += blockIdx.y * lde;
+    rho += blockIdx.y * ldr;
+    double ar[2] = {0, 0}, ai[2] = {0, 0}, br[2][3] = {{0, 0, 0}, {0, 0, 0}}, bi[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    for (int i = 0; i < 3; i++) {
+        const int e = M.tri_edge[3 * t + i];
+        const double c = M.coef[3 * t + i];
+        const double2 xs[2] = {H[e], E[e]};
+        for (int f = 0; f < 2; f++) {
+            ar[f] += c * xs[f].x;
+            ai[f] += c * xs[f].y;
+            for (int a = 0; a < 3; a++) {
+                const double qq = c * M.q[9 * t + 3 * i + a];
+                br[f][a] += qq * xs[f].x;
+                bi[f][a] += qq * xs[f].y;
+            }
+        }
+    }
+    C* o = tc + 9 * (blockIdx.y * (int64_t)nt + t);
+    for (int f = 0; f < 2; f++) {
+        o[4 * f] = cmk<C>(ar[f], ai[f]);
+        for (int a = 0; a < 3; a++) o[4 * f + 1 + a] = cmk<C>(br[f][a], bi[f][a]);
+    }
+    o[8] = cmk<C>(-rho[t].x, -rho[t].y);
+}
+
 // Projection of the system product as a gather (deterministic, no atomics): per
 // triangle t the current on t is alpha (r - c_t) + beta (alpha = sum_i c_i x_i,
 // beta_a = sum_i c_i q_ia x_i) for x = H and x = E', and the charge grid takes
@@ -121,17 +168,21 @@ __global__ void __launch_bounds__(256) k_interp(int nt, int S, int Mord, DevMesh
 // one chain.  Gathers from L2 and FP64 products bound it.  20,480 triangles: 148 us with
 // a thread per node in grid order, 118 us with every node in one unsorted list, 60 us
 // now (FP32: 44, 50, 34 us); a bar of 336: 40 us, 19 us now.
-template <class C, class R>
+// Vector blockIdx.y: tc 9 nt and src 7 Ng apart.  CHAIN: an entry's two products are
+// chained into the sum; else added up first (block.cu; the roundings are spelled out).
+template <class C, class R, bool CHAIN = true>
 __global__ void __launch_bounds__(256) k_project_gather(int64_t nnode, const int32_t* __restrict__ node,
                                                         const int32_t* __restrict__ ptr,
                                                         const int32_t* __restrict__ ent, int S,
-                                                        const R* __restrict__ W, const C* __restrict__ tc,
+                                                        const R* __restrict__ W, const C* __restrict__ tc, int nt,
                                                         C* __restrict__ src, int64_t Ng)
 {
     constexpr int U = 4;
     const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8;
     const int o = threadIdx.x % 8;
     if (v >= nnode || o >= 7) return;
+    tc += blockIdx.y * 9 * (int64_t)nt;
+    src += blockIdx.y * 7 * Ng;
     // grid o: al w1[a] + be w0; the charge: c0rho w0
     const bool rho = o == 6;
     const int f = o >= 3 ? 1 : 0, a = rho ? 0 : o - 3 * f, ia = 4 * f, ib = rho ? 8 : 4 * f + 1 + a;
@@ -161,8 +212,13 @@ __global__ void __launch_bounds__(256) k_project_gather(int64_t nnode, const int
 #pragma unroll
         for (int u = 0; u < U; u++)
             if (id[u] >= 0) {
-                ar = gio_fma(al[u].x, w1[u], gio_fma(be[u].x, w0[u], ar));
-                ai = gio_fma(al[u].y, w1[u], gio_fma(be[u].y, w0[u], ai));
+                if (CHAIN || rho) {
+                    ar = gio_fma(al[u].x, w1[u], gio_fma(be[u].x, w0[u], ar));
+                    ai = gio_fma(al[u].y, w1[u], gio_fma(be[u].y, w0[u], ai));
+                } else {
+                    ar += gio_fma(be[u].x, w0[u], gio_mul(al[u].x, w1[u]));
+                    ai += gio_fma(be[u].y, w0[u], gio_mul(al[u].y, w1[u]));
+                }
             }
     }
     C z;

@@ -229,6 +229,14 @@ struct sie_mesh {
 };
 
 namespace sie {
+// grids of the lockstep block product (block.cu), made on first use: R vectors at a
+// time (0: not made), power-of-two lengths g.n, kernel spectra, padded and compact
+// grids, triangle coefficients, charges and potentials of 8 vectors
+struct BlockWork {
+    int R = 0;
+    GridDesc g{};
+    double2 *spec = nullptr, *buf = nullptr, *src = nullptr, *tc = nullptr, *tri = nullptr;
+};
 // Krylov workspace of one restarted FGMRES (basis V, preconditioned basis Z)
 struct KrylovWork {
     int64_t n = 0;
@@ -243,8 +251,8 @@ struct KrylovWork {
     void release(cudaStream_t st);
 };
 // Krylov workspace of R right-hand sides, each with its own basis (V: R of m + 1
-// vectors, Z: R of m; the cooperative grid form keeps them V[j][q][n]); one launch
-// per Gram-Schmidt step serves all of them (gridDim.y = R)
+// vectors, Z: R of m); one launch per Gram-Schmidt step serves all of them
+// (gridDim.y = R)
 struct PanelWork {
     int64_t n = 0;
     int m = 0, R = 0;
@@ -286,10 +294,10 @@ struct sie_op {
     sie::PanelWork kmulti;          // lockstep solves: one Krylov basis per right-hand side
     sie::PanelWork kcs_multi;       // ... and per triangle system of their constraint preconditioner
     sie::PanelWork kzp;             // lockstep block products: the nested interior solves of the block
-    double2* zp = nullptr;          // block products: H, E and branch sum panels (3 x 8 ne)
+    double2* zp = nullptr;          // block products: E, nested right-hand sides and scratch (3 x 8 ne)
+    sie::BlockWork blk;             // block products: grids
     double2* mscr = nullptr;        // lockstep solves: per right-hand side scratch (8 blocks)
     double2* ir_multi = nullptr;    // lockstep refinement: residuals, corrections, products (3 x 8 (ne + nt))
-    double2* con_scr = nullptr;     // their constraint preconditioner in one kernel: 8 (ne + 2 nt)
     double2* mvec = nullptr;        // lockstep solves from host buffers: 2 x 8 (ne + nt)
     double2 *cs_e = nullptr, *cs_t = nullptr, *pc_e = nullptr, *pc_t = nullptr;  // preconditioner scratch
     // last solve: outer iters, relres; max nested iters, relres; max constraint iters, relres
@@ -316,6 +324,7 @@ struct sie_op {
     int64_t gr_nnz = 0;
     int32_t* gr_col = nullptr;
     double2* gr_val = nullptr;
+    double2* gr_diag = nullptr;     // its diagonal
     double* gr_idiag = nullptr;     // reciprocal of its (real) diagonal
     double eta_re = 0, eta_im = 0;
     // projection of the system product as a gather: grid nodes with stencil entries, CSR
@@ -332,26 +341,35 @@ struct sie_op {
 
 // ------------------------------------------------------------------ launchers (aim.cu, near.cu)
 namespace sie {
-// Krylov workspace of a grid-resident solve (resident.cuh) of R vectors
+// Krylov workspace of a resident solve (resident.cuh)
 struct ResWork {
     int m = 0;
     double2 *V = nullptr, *Z = nullptr, *W = nullptr, *H = nullptr, *part = nullptr;
-    int64_t ldh = 0;
 };
-// constraint preconditioner (ext: the exterior AEFIE form) of R vectors in one
-// cluster kernel (constraint.cu); v1, b, q: scratch of R ne, R nt, R nt.  false: not
-// taken (no dense inverse, too many triangles); *st_out: launch status
-bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, int R, const double2* const* x,
-                         double2* const* y, double tol, int maxit, int restart, const ResWork& w, double2* v1, double2* b,
-                         double2* q, sie_status* st_out);
-// E_q = f (or per edge) A^-1 b(H_q), q < R <= 8: nested interior solves of
-// near-region-only and SIBC operators (nested.cu); extra: iterations run past
-// the tolerance; statistics in op->gstat
-sie_status nested_solve(sie_op* op, int R, const double2* H, int64_t ldh, double2* E, int64_t lde, double2 f,
-                        int extra, const ResWork& w);
+// constraint preconditioner (ext: the exterior AEFIE form) in one cluster kernel
+// (constraint.cu); v1, b, q: scratch of ne, nt, nt.  false: not taken (no dense
+// inverse, too many triangles); *st_out: launch status
+bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, const double2* x, double2* y, double tol,
+                         int maxit, const ResWork& w, double2* v1, double2* b, double2* q, sie_status* st_out);
+// E = f (or per edge) A^-1 b(H): nested interior solve of near-region-only and SIBC
+// operators (nested.cu); extra: iterations run past the tolerance; statistics in op->gstat
+sie_status nested_solve(sie_op* op, const double2* H, double2* E, double2 f, int extra, const ResWork& w);
+// lanes per row of the lockstep solves' products with I_x (5 entries a row) and the
+// triangle matrices (about 100): fixed, since their sums depend on them and a measured
+// choice (csr_autotune) on chance
+constexpr int BLK_IX_LANES = 4, BLK_TRI_LANES = 32;
+// block products (block.cu) of R <= 8 vectors, one distance apart: Y_q = A X_q of a CSR
+// matrix, and SYS x_q given E_q = Z' H_q
+sie_status blk_csr(cudaStream_t st, int nrow, const int64_t* rp, const int32_t* col, const double2* val,
+                   const double2* X, int64_t ldx, int R, double2* Y, int64_t ldy);
+sie_status blk_sys_rest(sie_op* op, int R, const double2* x, int64_t ldx, const double2* E, int64_t lde, double2* y,
+                        int64_t ldy);
+void blk_release(sie_op* op);
 sie_status dev_upload_mesh(sie_mesh* m);
 sie_status dev_free_mesh(sie_mesh* m);
 sie_status aim_weights(sie_op* op);
+// kernel samples (G, dG/dx, dG/dy, dG/dz) of g's FFT box into spec (4 n^3)
+sie_status aim_sample(cudaStream_t st, const GridDesc& g, double kr, double ki, double2* spec);
 sie_status aim_spectra(sie_op* op, AimOp& a);
 sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q);
 sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, double2* y);
@@ -434,6 +452,9 @@ sie_status fft_sys(cudaStream_t st, float2* buf, float2* src, const GridDesc& g,
                    sie_ctx* pc);
 sie_status fft3d(cudaStream_t st, double2* buf, const double2* src, const GridDesc& g, int dir, int prune,
                  sie_ctx* prof_ctx, int nbatch = 1);
+// FP64 butterflies at power-of-two lengths (block.cu)
+sie_status fft3d_p2(cudaStream_t st, double2* buf, const double2* src, const GridDesc& g, int dir, int prune, sie_ctx* pc,
+                    int nbatch);
 sie_status fft3d(cudaStream_t st, float2* buf, const float2* src, const GridDesc& g, int dir, int prune,
                  sie_ctx* prof_ctx, int nbatch = 1);
 }  // namespace sie

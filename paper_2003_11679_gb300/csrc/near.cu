@@ -300,20 +300,19 @@ __device__ __forceinline__ void store_moments(cd* acc, int lane, double2* __rest
         for (int i = 0; i < 14; i++) mom[i] = make_double2(acc[i].re, acc[i].im);
 }
 
+}  // namespace sie
+#include "near_points.cuh"
+namespace sie {
+
 // far pairs: one warp per pair, a lane per outer point
 __global__ void __launch_bounds__(128) k_near_far(const int32_t* __restrict__ pairs, int64_t np,
                                                   const uint8_t* __restrict__ cls, DevMesh M, double kr, double ki,
-                                                  const double2* __restrict__ obj_k, double2* __restrict__ mom)
+                                                  double2* __restrict__ mom)
 {
     const int64_t p = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (p >= np || cls[p] != PC_FAR) return;
     const int t = pairs[2 * p], s = pairs[2 * p + 1];
-    if (obj_k) {
-        const double2 ko = obj_k[M.obj[t]];
-        kr = ko.x;
-        ki = ko.y;
-    }
     const v3 a = ld3(M.V + 3 * M.T[3 * t]), b = ld3(M.V + 3 * M.T[3 * t + 1]), c = ld3(M.V + 3 * M.T[3 * t + 2]);
     const v3 a2 = ld3(M.V + 3 * M.T[3 * s]), b2 = ld3(M.V + 3 * M.T[3 * s + 1]), c2 = ld3(M.V + 3 * M.T[3 * s + 2]);
     const v3 ct = ld3(M.cen + 3 * t);
@@ -375,8 +374,7 @@ template <bool REALK>
 __global__ void __launch_bounds__(32 * NC_W, 4) k_near_close(const int2* __restrict__ unit, int nunit, int npts,
                                                           const int32_t* __restrict__ pairs,
                                                           const uint8_t* __restrict__ cls, DevMesh M, double kr,
-                                                          double ki, const double2* __restrict__ obj_k,
-                                                          double2* __restrict__ part)
+                                                          double ki, double2* __restrict__ part)
 {
     __shared__ CloseSm sm_[NC_W];
     const int un = blockIdx.x * NC_W + threadIdx.x / 32;
@@ -385,11 +383,6 @@ __global__ void __launch_bounds__(32 * NC_W, 4) k_near_close(const int2* __restr
     CloseSm& S = sm_[threadIdx.x / 32];
     const int p = unit[un].x, q_lo = unit[un].y;
     const int t = pairs[2 * (int64_t)p], s = pairs[2 * (int64_t)p + 1], kind = cls[p];
-    if (!REALK && obj_k) {
-        const double2 ko = obj_k[M.obj[t]];
-        kr = ko.x;
-        ki = ko.y;
-    }
     const cd k = mk(kr, REALK ? 0.0 : ki);
     const double kabs = REALK ? kr : sqrt(kr * kr + ki * ki);
     const cd mjk = mk(k.im, -k.re);  // -j k
@@ -724,25 +717,40 @@ __global__ void k_near_sum(int n, const int3* __restrict__ own, const double2* _
     mom[14 * (int64_t)o.x + i] = s;
 }
 
-// moments of all near pairs of a
-static sie_status near_moments(sie_op* op, const AimOp& a, const QuadDev& q, double2* mom)
+// outer points of a pair class, as on the device
+static void outer_counts(const QuadDev& q, int nout[5])
+{
+    const int ge = q.opan * q.n[QR_OLAM] * 2 * q.emupan * q.n[QR_EMU], gv = q.opan * q.n[QR_OLAM] * q.n[QR_OMU];
+    nout[PC_FAR] = q.n[QR_FAR] * q.n[QR_FAR], nout[PC_PLAIN] = q.n[QR_OUT] * q.n[QR_OUT];
+    nout[PC_VERTEX] = gv, nout[PC_EDGE] = ge, nout[PC_SELF] = 3 * ge;
+}
+
+// scratch of a build, given back to the stream's pool on every return
+struct Scratch {
+    cudaStream_t st;
+    std::vector<void*> p;
+    explicit Scratch(cudaStream_t s) : st(s) {}
+    ~Scratch()
+    {
+        for (void* v : p) cudaFreeAsync(v, st);
+    }
+    template <class T>
+    cudaError_t get(T** d, size_t n)
+    {
+        const cudaError_t e = cudaMallocAsync((void**)d, sizeof(T) * n, st);
+        if (e == cudaSuccess) p.push_back(*d);
+        return e;
+    }
+};
+
+// moments by the panel rule (single objects): far pairs, then the units of the close ones
+static sie_status moments_panels(sie_op* op, const AimOp& a, const std::vector<uint8_t>& hc, const int nout[5],
+                                 const uint8_t* cls, double2* mom)
 {
     cudaStream_t st = op->mesh->ctx->stream;
-    const DevMesh& M = op->mesh->d;
     const int64_t np = a.npairs;
-    if (np <= 0) return SIE_OK;
-    uint8_t* cls = nullptr;
-    std::vector<uint8_t> hc(np);
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&cls, np, st));
-    k_pair_class<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a.pairs, np, M, a.kr, a.ki, a.obj_k, cls);
+    k_near_far<<<(unsigned)((np + 3) / 4), 128, 0, st>>>(a.pairs, np, cls, op->mesh->d, a.kr, a.ki, mom);
     SIE_CUDA_TRY(cudaGetLastError());
-    SIE_CUDA_TRY(cudaMemcpyAsync(hc.data(), cls, np, cudaMemcpyDeviceToHost, st));
-    k_near_far<<<(unsigned)((np + 3) / 4), 128, 0, st>>>(a.pairs, np, cls, M, a.kr, a.ki, a.obj_k, mom);
-    SIE_CUDA_TRY(cudaGetLastError());
-    SIE_CUDA_TRY(cudaStreamSynchronize(st));
-    // outer points of a class, as graded_count() on the device
-    const int ge = q.opan * q.n[QR_OLAM] * 2 * q.emupan * q.n[QR_EMU], gv = q.opan * q.n[QR_OLAM] * q.n[QR_OMU];
-    const int nout[5] = {0, q.n[QR_OUT] * q.n[QR_OUT], gv, ge, 3 * ge};
     int64_t count[5] = {0, 0, 0, 0, 0}, total = 0;
     for (int64_t p = 0; p < np; p++) count[hc[p]]++;
     for (int c = 1; c < 5; c++) total += count[c] * ((nout[c] + 31) / 32);
@@ -757,32 +765,93 @@ static sie_status near_moments(sie_op* op, const AimOp& a, const QuadDev& q, dou
                 for (int o = 0; o < nout[c]; o += npts) unit.push_back(make_int2((int)p, o));
                 own.push_back(make_int3((int)p, first, (int)unit.size() - first));
             }
-    if (!unit.empty()) {
-        int2* du = nullptr;
-        int3* dow = nullptr;
-        double2* part = nullptr;
+    if (unit.empty()) return SIE_OK;
+    Scratch mem(st);
+    int2* du = nullptr;
+    int3* dow = nullptr;
+    double2* part = nullptr;
+    const int nu = (int)unit.size(), no = (int)own.size();
+    SIE_CUDA_TRY(mem.get(&du, nu));
+    SIE_CUDA_TRY(mem.get(&dow, no));
+    SIE_CUDA_TRY(mem.get(&part, 14 * (size_t)nu));
+    SIE_CUDA_TRY(cudaMemcpyAsync(du, unit.data(), sizeof(int2) * nu, cudaMemcpyHostToDevice, st));
+    SIE_CUDA_TRY(cudaMemcpyAsync(dow, own.data(), sizeof(int3) * no, cudaMemcpyHostToDevice, st));
+    const unsigned blocks = (unsigned)((nu + NC_W - 1) / NC_W);
+    if (a.ki == 0.0)
+        k_near_close<true><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, op->mesh->d, a.kr, 0.0, part);
+    else
+        k_near_close<false><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, op->mesh->d, a.kr, a.ki, part);
+    SIE_CUDA_TRY(cudaGetLastError());
+    k_near_sum<<<(14 * no + 127) / 128, 128, 0, st>>>(no, dow, part, mom);
+    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_CUDA_TRY(cudaStreamSynchronize(st));  // the host lists outlive the copies
+    return SIE_OK;
+}
+
+// moments from every outer point by itself, in runs of pairs whose points fit the scratch
+static sie_status moments_points(sie_op* op, const AimOp& a, const std::vector<uint8_t>& hc, const int nout[5],
+                                 double2* mom)
+{
+    cudaStream_t st = op->mesh->ctx->stream;
+    const int64_t np = a.npairs;
+    std::vector<int64_t> order;  // by falling work per point
+    for (int c = 4; c >= 0; c--)
+        for (int64_t p = 0; p < np; p++)
+            if (hc[p] == c) order.push_back(p);
+    int64_t all = 0;
+    for (int64_t p : order) all += (nout[hc[p]] + 31) / 32;
+    int most = 0;
+    for (int c = 0; c < 5; c++) most = std::max(most, (nout[c] + 31) / 32);
+    const int64_t cap = std::min<int64_t>(all, std::max<int64_t>(pt::PT_UNITS, most));
+    Scratch mem(st);
+    int2* du = nullptr;
+    int3* dow = nullptr;
+    double* pts = nullptr;
+    SIE_CUDA_TRY(mem.get(&du, cap));
+    SIE_CUDA_TRY(mem.get(&dow, cap));
+    SIE_CUDA_TRY(mem.get(&pts, pt::PT_N * 32 * (size_t)cap));
+    std::vector<int2> unit;
+    std::vector<int3> own;
+    for (size_t at = 0; at < order.size();) {
+        unit.clear();
+        own.clear();
+        for (; at < order.size(); at++) {
+            const int p = (int)order[at], n = nout[hc[p]], nu = (n + 31) / 32;
+            if ((int64_t)unit.size() + nu > cap) break;
+            own.push_back(make_int3(p, (int)unit.size(), n));
+            for (int o = 0; o < n; o += 32) unit.push_back(make_int2(p, o));
+        }
         const int nu = (int)unit.size(), no = (int)own.size();
-        SIE_CUDA_TRY(cudaMallocAsync((void**)&du, sizeof(int2) * nu, st));
-        SIE_CUDA_TRY(cudaMallocAsync((void**)&dow, sizeof(int3) * no, st));
-        SIE_CUDA_TRY(cudaMallocAsync((void**)&part, sizeof(double2) * 14 * nu, st));
         SIE_CUDA_TRY(cudaMemcpyAsync(du, unit.data(), sizeof(int2) * nu, cudaMemcpyHostToDevice, st));
         SIE_CUDA_TRY(cudaMemcpyAsync(dow, own.data(), sizeof(int3) * no, cudaMemcpyHostToDevice, st));
-        const unsigned blocks = (unsigned)((nu + NC_W - 1) / NC_W);
-        if (!a.obj_k && a.ki == 0.0)
-            k_near_close<true><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, M, a.kr, 0.0, nullptr, part);
-        else
-            k_near_close<false><<<blocks, 32 * NC_W, 0, st>>>(du, nu, npts, a.pairs, cls, M, a.kr, a.ki, a.obj_k,
-                                                              part);
+        pt::k_near_points<<<(nu + pt::PT_W - 1) / pt::PT_W, 32 * pt::PT_W, 0, st>>>(
+            du, nu, a.pairs, op->mesh->d, a.kr, a.ki, a.obj_k, pts, 32 * cap);
         SIE_CUDA_TRY(cudaGetLastError());
-        k_near_sum<<<(14 * no + 127) / 128, 128, 0, st>>>(no, dow, part, mom);
+        pt::k_near_gather<<<(no + 3) / 4, 128, 0, st>>>(no, dow, a.pairs, pts, 32 * cap, mom);
         SIE_CUDA_TRY(cudaGetLastError());
         SIE_CUDA_TRY(cudaStreamSynchronize(st));  // the host lists outlive the copies
-        cudaFreeAsync(du, st);
-        cudaFreeAsync(dow, st);
-        cudaFreeAsync(part, st);
     }
-    cudaFreeAsync(cls, st);
     return SIE_OK;
+}
+
+// moments of all near pairs of a; points: every outer point by itself (near_points.cuh)
+static sie_status near_moments(sie_op* op, const AimOp& a, const QuadDev& q, bool points, double2* mom)
+{
+    cudaStream_t st = op->mesh->ctx->stream;
+    const DevMesh& M = op->mesh->d;
+    const int64_t np = a.npairs;
+    if (np <= 0) return SIE_OK;
+    Scratch mem(st);
+    uint8_t* cls = nullptr;
+    std::vector<uint8_t> hc(np);
+    SIE_CUDA_TRY(mem.get(&cls, np));
+    k_pair_class<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a.pairs, np, M, a.kr, a.ki, a.obj_k, cls);
+    SIE_CUDA_TRY(cudaGetLastError());
+    SIE_CUDA_TRY(cudaMemcpyAsync(hc.data(), cls, np, cudaMemcpyDeviceToHost, st));
+    SIE_CUDA_TRY(cudaStreamSynchronize(st));
+    int nout[5];
+    outer_counts(q, nout);
+    return points ? moments_points(op, a, hc, nout, mom) : moments_panels(op, a, hc, nout, cls, mom);
 }
 
 // kernel values at integer lags |l_d| <= Lm: (G, dG/dx, dG/dy, dG/dz), zero at lag 0
@@ -1018,7 +1087,9 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&mom, sizeof(double2) * 14 * std::max<int64_t>(a.npairs, 1), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&loc, sizeof(double2) * NLOC * std::max<int64_t>(a.npairs, 1), st));
     const int wpb = 4;
-    SIE_TRY(near_moments(op, a, q, mom));
+    // operators without an interior grid: lockstep block products (near_points.cuh)
+    const bool points = !op->inn.has_grid;
+    SIE_TRY(near_moments(op, a, q, points, mom));
     int Lm = a.g.Rnear + a.g.M;
     int S = (a.g.M + 1) * (a.g.M + 1) * (a.g.M + 1);
     if (a.has_grid) {
@@ -1028,7 +1099,8 @@ sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q)
         SIE_CUDA_TRY(cudaGetLastError());
     }
     if (a.npairs > 0) {
-        k_near_local<<<(unsigned)((a.npairs + wpb - 1) / wpb), 32 * wpb, 0, st>>>(
+        auto local = points ? pt::k_near_local : k_near_local;
+        local<<<(unsigned)((a.npairs + wpb - 1) / wpb), 32 * wpb, 0, st>>>(
             a.pairs, a.npairs, M, mom, a.has_grid ? 1 : 0, S, a.g.M, op->base, op->W, tab, Lm, loc);
         SIE_CUDA_TRY(cudaGetLastError());
     }

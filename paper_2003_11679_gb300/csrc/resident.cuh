@@ -3,12 +3,11 @@
 // charge system) need a few microseconds of arithmetic per iteration; as a graph
 // loop of nine kernels an iteration took 45 to 50 us.  Two forms:
 //
-//  * clu_fgmres (up to CLU_MAXN rows): a thread-block cluster of 8 or 16 CTAs per
-//    right-hand side.  The vector that the next product gathers from sits whole
-//    in every CTA's shared memory, written by its owners through distributed
-//    shared memory; so are the CTAs' partial sums.  An iteration meets at 3 or 4
-//    hardware cluster barriers (0.2 to 0.3 us) and reads no other memory than the
-//    matrix rows (L1) and own rows of the basis;
+//  * clu_fgmres (up to CLU_MAXN rows): a thread-block cluster of 8 or 16 CTAs.  The
+//    vector that the next product gathers from sits whole in every CTA's shared
+//    memory, written by its owners through distributed shared memory; so are the CTAs'
+//    partial sums.  An iteration meets at 3 or 4 hardware cluster barriers (0.2 to 0.3
+//    us) and reads no other memory than the matrix rows (L1) and own rows of the basis;
 //  * res_fgmres (more rows): a cooperative grid of up to one CTA per SM with
 //    barriers in global memory (about 1.5 us); what other CTAs wrote is read past
 //    L1 (ld.cg).  On 8 CTAs a copper bar's 504-row solve took 186 us this way.
@@ -33,7 +32,7 @@ namespace sie {
 
 constexpr int RES_T = 512;              // threads per CTA
 constexpr int RES_MAXCTA = 160;         // partial-sum slots
-constexpr int RES_WORDS = 2 + 8 * 16;   // counter, error flag, ring of lockstep flags
+constexpr int RES_WORDS = 2;            // counter, error flag
 constexpr int RES_SPIN = 1 << 20;       // polls of a barrier before it gives up (under a second)
 
 __device__ __forceinline__ double2 r_cm(double2 a, double2 b)
@@ -75,21 +74,20 @@ __device__ __forceinline__ bool res_barrier(ResBar& b)
     return !bad;
 }
 
-// Krylov arrays: vector q of step j at V + (j R + q) n; part: per-CTA sums
+// Krylov arrays; part: per-CTA sums
 struct ResKrylov {
     int64_t n;
-    int m, R;           // largest cycle length, right-hand sides
-    double2 *V, *Z, *W; // (m + 1) R n, m R n, R n
-    double2* H;         // rotated Hessenberg columns: per right-hand side (m + 1) m
-    int64_t ldh;        // stride of H between right-hand sides
-    double2* part;      // RES_MAXCTA R 2 (m + 2)
+    int m;              // largest cycle length
+    double2 *V, *Z, *W; // (m + 1) n, m n, n
+    double2* H;         // rotated Hessenberg columns, (m + 1) m
+    double2* part;      // RES_MAXCTA 2 (m + 2)
     double tol;
-    int extra;          // iterations run after every residual is below tol (host-checked cycles ran one)
+    int extra;          // iterations run after the residual is below tol (host-checked cycles ran one)
     double* stat;       // 0, 1: largest iteration count and residual so far; 2, 3: this run's residual and count
 };
 
 // dynamic shared memory of res_fgmres
-inline size_t res_smem(int m, int R) { return sizeof(double2) * (size_t)R * 5 * (m + 2); }
+inline size_t res_smem(int m) { return sizeof(double2) * (size_t)5 * (m + 2); }
 
 // sums of both components over the warp, in every lane: the halves of the warp
 // take one component each after the first exchange (6 FP64 additions, not 10)
@@ -104,53 +102,44 @@ __device__ __forceinline__ double2 warp_sum(double2 s)
     return up ? make_double2(other, keep) : make_double2(keep, other);
 }
 
-// part[(c R + q) ld + i] = sum over own rows of conj(V_i) w, i < nv, and of |w|^2 (slot nv) when norm
+// part[c ld + i] = sum over own rows of conj(V_i) w, i < nv, and of |w|^2 (slot nv) when norm
 __device__ __forceinline__ void res_dots(const ResKrylov& K, int64_t r0, int64_t r1, int nv, bool norm, double2* part,
                                          int ld)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int cols = nv + (norm ? 1 : 0);
-    for (int t = warp; t < K.R * cols; t += nw) {
-        const int q = t / cols, i = t % cols;
-        const double2* w = K.W + q * K.n;
-        const double2* v = i < nv ? K.V + ((int64_t)i * K.R + q) * K.n : w;
+    for (int i = warp; i < nv + (norm ? 1 : 0); i += nw) {
+        const double2* v = i < nv ? K.V + (int64_t)i * K.n : K.W;
         double2 s = make_double2(0, 0);
-        for (int64_t k = r0 + lane; k < r1; k += 32) r_fma(s, r_cj(v[k]), w[k]);
+        for (int64_t k = r0 + lane; k < r1; k += 32) r_fma(s, r_cj(v[k]), K.W[k]);
         s = warp_sum(s);
-        if (lane == 0) part[((int64_t)blockIdx.x * K.R + q) * ld + i] = s;
+        if (lane == 0) part[(int64_t)blockIdx.x * ld + i] = s;
     }
 }
 
-// h[q ldh + i] = sum over the CTAs of part (in CTA order per lane, then a fixed tree)
-__device__ __forceinline__ void res_reduce(const ResKrylov& K, int cols, const double2* part, int ld, double2* h, int ldh)
+// h[i] = sum over the CTAs of part (in CTA order per lane, then a fixed tree)
+__device__ __forceinline__ void res_reduce(int cols, const double2* part, int ld, double2* h)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int t = warp; t < K.R * cols; t += nw) {
-        const int q = t / cols, i = t % cols;
+    for (int i = warp; i < cols; i += nw) {
         double2 s = make_double2(0, 0);
         for (int c = lane; c < (int)gridDim.x; c += 32) {
-            const double2 p = __ldcg(part + ((int64_t)c * K.R + q) * ld + i);
+            const double2 p = __ldcg(part + (int64_t)c * ld + i);
             s.x += p.x;
             s.y += p.y;
         }
         s = warp_sum(s);
-        if (lane == 0) h[q * ldh + i] = s;
+        if (lane == 0) h[i] = s;
     }
     __syncthreads();
 }
 
 // w -= sum_i V_i h_i on own rows
-__device__ __forceinline__ void res_update(const ResKrylov& K, int64_t r0, int64_t r1, int nv, const double2* h, int ldh)
+__device__ __forceinline__ void res_update(const ResKrylov& K, int64_t r0, int64_t r1, int nv, const double2* h)
 {
-    const int rows = (int)(r1 - r0);
-    for (int t = threadIdx.x; t < K.R * rows; t += blockDim.x) {
-        const int q = t / rows;
-        const int64_t k = r0 + t % rows;
+    for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x) {
         double2 s = make_double2(0, 0);
-        const double2* v = K.V + (int64_t)q * K.n + k;
-        for (int i = 0; i < nv; i++) r_fma(s, v[(int64_t)i * K.R * K.n], h[q * ldh + i]);
-        double2* w = K.W + q * K.n + k;
-        *w = make_double2(w->x - s.x, w->y - s.y);
+        for (int i = 0; i < nv; i++) r_fma(s, K.V[(int64_t)i * K.n + k], h[i]);
+        K.W[k] = make_double2(K.W[k].x - s.x, K.W[k].y - s.y);
     }
     __syncthreads();
 }
@@ -163,7 +152,7 @@ __device__ __forceinline__ double res_unscale(double a, double b, double c)
     return (e == 0 || e == 0x7ff) ? 1.0 : __hiloint2double((2046 - min(e, 2045)) << 20, 0);
 }
 
-// column j of one right-hand side (one thread): h1 + h2 and the norm hn through
+// column j (one thread): h1 + h2 and the norm hn through
 // the previous rotations, rotation j (c real), g; the rotated column to Hq when
 // store; gabs = |g_j| becomes |g_{j+1}|.  One chain of FP64 operations of one warp,
 // 64 cycles or more each: two reciprocal square roots instead of three hypot and six
@@ -263,44 +252,37 @@ __device__ __forceinline__ void res_root(double s, double& norm, double& inv)
 }
 
 // The FGMRES cycle (zero initial guess, at most K.m iterations) on the residual
-// panel already in K.W (own rows, after a __syncthreads).  sys: rows r0, r1 of
-// this CTA; precond(j, bar): Z_j = M V_j, with the barrier that ends it; apply(j):
-// W = A Z_j on own rows; after_v(j): own rows of V_j are set (for a pointwise
-// preconditioner).  After it, the solutions' combinations: x_q = sum_i Z_i y_i,
-// y in shared memory at y[q (m + 2) + i], i <= jend.  Returns jend, -1 when a wait
-// ran out.
+// already in K.W (own rows, after a __syncthreads).  sys: rows r0, r1 of this CTA;
+// precond(j, bar): Z_j = M V_j, with the barrier that ends it; apply(j): W = A Z_j on
+// own rows; after_v(j): own rows of V_j are set (for a pointwise preconditioner).
+// After it, the solution's combination: x = sum_i Z_i y_i, y in shared memory,
+// i <= jend.  Returns jend, -1 when a wait ran out.
 template <class SYS>
 __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* smem, double2** y_out)
 {
-    const int m = K.m, R = K.R, ld = m + 2;
+    const int m = K.m, ld = m + 2;
     const int64_t n = K.n, r0 = sys.r0, r1 = sys.r1;
-    const int rows = (int)(r1 - r0);
     double2* cs = smem;
-    double2* sn = cs + R * ld;
-    double2* g = sn + R * ld;
-    double2* h1 = g + R * ld;
-    double2* h2 = h1 + R * ld;
-    __shared__ double bnorm[8], rel[8], wn[8], gabs[8];
-    __shared__ double2 nr[8];
+    double2* sn = cs + ld;
+    double2* g = sn + ld;
+    double2* h1 = g + ld;
+    double2* h2 = h1 + ld;
+    __shared__ double bnorm, rel, wn, gabs;
     double2* P1 = K.part;
-    double2* P2 = P1 + (int64_t)RES_MAXCTA * R * ld;
+    double2* P2 = P1 + (int64_t)RES_MAXCTA * ld;
     res_dots(K, r0, r1, 0, true, P1, ld);
     if (!res_barrier(bar)) return -1;
-    res_reduce(K, 1, P1, ld, nr, 1);
-    if (threadIdx.x < R) {
-        const double d2 = nr[threadIdx.x].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
-        bnorm[threadIdx.x] = gabs[threadIdx.x] = b;
-        wn[threadIdx.x] = b > 0 ? 1.0 / b : 0.0;
-        g[threadIdx.x * ld] = make_double2(b, 0);
+    res_reduce(1, P1, ld, h1);
+    if (threadIdx.x == 0) {
+        const double d2 = h1[0].x, b = d2 != d2 ? d2 : sqrt(fmax(d2, 0.0));  // a NaN norm stays NaN
+        bnorm = gabs = b;
+        wn = b > 0 ? 1.0 / b : 0.0;
+        g[0] = make_double2(b, 0);
     }
     __syncthreads();
     auto set_v = [&](int j) {
-        for (int t = threadIdx.x; t < R * rows; t += blockDim.x) {
-            const int q = t / rows;
-            const int64_t k = r0 + t % rows;
-            const double2 w = K.W[q * n + k];
-            K.V[((int64_t)j * R + q) * n + k] = make_double2(w.x * wn[q], w.y * wn[q]);
-        }
+        for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x)
+            K.V[(int64_t)j * n + k] = make_double2(K.W[k].x * wn, K.W[k].y * wn);
         sys.after_v(j);
     };
     set_v(0);
@@ -312,50 +294,42 @@ __device__ int res_fgmres(SYS& sys, const ResKrylov& K, ResBar& bar, double2* sm
         __syncthreads();
         res_dots(K, r0, r1, j + 1, false, P1, ld);
         if (!res_barrier(bar)) return -1;
-        res_reduce(K, j + 1, P1, ld, h1, ld);
-        res_update(K, r0, r1, j + 1, h1, ld);
+        res_reduce(j + 1, P1, ld, h1);
+        res_update(K, r0, r1, j + 1, h1);
         res_dots(K, r0, r1, j + 1, true, P2, ld);
         if (!res_barrier(bar)) return -1;
-        res_reduce(K, j + 2, P2, ld, h2, ld);
-        if ((threadIdx.x >> 5) < R) {
-            const int q = threadIdx.x >> 5;
-            const double hh = res_norm2(h2 + q * ld, j + 1, threadIdx.x & 31);
-            if ((threadIdx.x & 31) == 0) {
+        res_reduce(j + 2, P2, ld, h2);
+        if (threadIdx.x < 32) {
+            const double hh = res_norm2(h2, j + 1, threadIdx.x);
+            if (threadIdx.x == 0) {
                 double hn;
-                res_root(hh, hn, wn[q]);
-                res_givens(j, m, h1 + q * ld, h2 + q * ld, hn, cs + q * ld, sn + q * ld, g + q * ld, K.H + q * K.ldh,
-                           blockIdx.x == 0, gabs[q]);
-                rel[q] = res_rel(gabs[q], bnorm[q]);
+                res_root(hh, hn, wn);
+                res_givens(j, m, h1, h2, hn, cs, sn, g, K.H, blockIdx.x == 0, gabs);
+                rel = res_rel(gabs, bnorm);
             }
         }
         __syncthreads();
-        bool more = false;
-        for (int q = 0; q < R; q++) more = more || rel[q] >= K.tol;
+        bool more = rel >= K.tol;
         if (!more && extra > 0) {
             extra--;
             more = true;
         }
         more = more && j + 1 < m;
         if (!more) break;
-        res_update(K, r0, r1, j + 1, h2, ld);
+        res_update(K, r0, r1, j + 1, h2);
         set_v(j + 1);
         if (!res_barrier(bar)) return -1;
     }
-    // y = R^-1 g: a warp per right-hand side (CTA 0's H is complete after a barrier)
+    // y = R^-1 g (CTA 0's H is complete after a barrier)
     if (!res_barrier(bar)) return -1;
-    if ((threadIdx.x >> 5) < R)
-        res_backsub(j, m, K.H + (threadIdx.x >> 5) * K.ldh, g + (threadIdx.x >> 5) * ld, threadIdx.x & 31);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double worst = 0;
-        for (int q = 0; q < R; q++) worst = rel[q] != rel[q] ? rel[q] : (worst != worst ? worst : fmax(worst, rel[q]));
-        res_stat(K.stat, j + 1, worst);
-    }
+    if (threadIdx.x < 32) res_backsub(j, m, K.H, g, threadIdx.x);
+    if (blockIdx.x == 0 && threadIdx.x == 0) res_stat(K.stat, j + 1, rel);
     __syncthreads();
     *y_out = g;
     return j;
 }
 
-// the same from several clusters: maxima of nonnegative doubles by their bits (a NaN's exceed all)
+// the same as maxima of nonnegative doubles by their bits (a NaN's exceed all)
 __device__ __forceinline__ void res_stat_max(double* stat, int iters, double rel)
 {
     unsigned long long* st = (unsigned long long*)stat;
@@ -367,12 +341,11 @@ __device__ __forceinline__ void res_stat_max(double* stat, int iters, double rel
 constexpr int CLU_MAXN = 2048;  // rows: two gather vectors take 64 KB of shared memory then
 constexpr int CLU_MAXC = 16;
 
-// one right-hand side per cluster; shared memory of a CTA:
+// shared memory of a CTA:
 //   x[2][n] gather vectors (v, z), w[rows], pr[2][C][m + 2] partial sums, cs, sn, g, h1, h2 [m + 2]
-int clu_pick(const void* fn, int64_t n, int64_t nnz, int m, int R, size_t extra);
+int clu_pick(const void* fn, int64_t n, int64_t nnz, int m, size_t extra);
 int res_group(int64_t rows, int64_t nrow, int64_t nnz);
-bool clu_fits(const void* fn, int C, int R, size_t smem);
-sie_status clu_launch(const void* fn, int C, int R, size_t smem, void** args, cudaStream_t st);
+sie_status clu_launch(const void* fn, int C, size_t smem, void** args, cudaStream_t st);
 inline size_t clu_smem(int64_t n, int m, int C)
 {
     return sizeof(double2) * (size_t)(2 * n + (n + C - 1) / C + 2 * C * (m + 2) + 5 * (m + 2));
@@ -448,50 +421,10 @@ __device__ __forceinline__ void clu_reduce(const CluMem& M, int cols, int buf, d
     __syncthreads();
 }
 
-// coupling of the clusters of a lockstep block: a cluster goes on while any
-// right-hand side was above tol lag iterations ago (lag 1: the flags it reads
-// were written an iteration ago, nothing waits).  flag: a ring of CLU_RING
-// iterations x 8 right-hand sides, zero at the launch, holding 2 (iteration + 1) +
-// (above tol); the clusters are never two iterations apart.
-constexpr int CLU_RING = 16;
-struct CluLock {
-    int R = 1, lag = 1;
-    unsigned* flag = nullptr;
-    int* err = nullptr;
-};
-// publish iteration it of right-hand side q (one CTA of its cluster); then 1: go on, 0: all below, -1: a wait ran out
-__device__ __forceinline__ int clu_vote(const CluLock& lock, int q, int it, bool above, bool publish)
-{
-    if (publish)
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(lock.flag + (it % CLU_RING) * 8 + q),
-                     "r"(2u * (unsigned)(it + 1) + (above ? 1u : 0u))
-                     : "memory");
-    const int at = it - lock.lag;
-    if (at < 0) return 1;
-    int more = 0;
-    for (int p = 0; p < lock.R; p++) {
-        unsigned v = 0;
-        int n = 0;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
-                         : "=r"(v)
-                         : "l"(lock.flag + (at % CLU_RING) * 8 + p)
-                         : "memory");
-        } while ((int)(v >> 1) < at + 1 && ++n < RES_SPIN);
-        if ((int)(v >> 1) < at + 1) {
-            atomicExch(lock.err, 1);
-            return -1;
-        }
-        if (v & 1) more = 1;
-    }
-    return more;
-}
-
-// The cycle for this cluster's right-hand side, whose residual is in M.w (own
-// rows, after a __syncthreads).  sys: r0, rows; precond(j): from M.xv, Z_j (own
+// The cycle of a cluster; the residual is in M.w (own rows, after a __syncthreads).  sys: r0, rows; precond(j): from M.xv, Z_j (own
 // rows) and M.xz of every CTA, false for a pointwise one done by set_v; set_v(j,
 // k, v): own row k of V_j is v (sets own row of what the next product gathers, which
-// share() then copies to the other CTAs); apply(j): M.w = A z from M.xz.  After it y in M.g; returns jend, -1 when a wait ran out.
+// share() then copies to the other CTAs); apply(j): M.w = A z from M.xz.  After it y in M.g; returns jend.
 // Restarted solves call it again with the new residual: it0 iterations done, at
 // most maxit in all, bnorm0 the norm of the right-hand side (below 0 in the first
 // cycle); *above: a residual is still above tol; rel_out: this one's.
@@ -501,12 +434,12 @@ struct CluRun {
     bool above = true;
 };
 template <class SYS>
-__device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const CluLock& lock, CluRun& run)
+__device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, CluRun& run)
 {
     const int m = K.m, rows = sys.rows;
     const int64_t n = K.n, r0 = sys.r0;
-    double2* V = K.V + (int64_t)q * (m + 1) * n;  // this right-hand side's basis
-    double2* H = K.H + q * K.ldh;
+    double2* V = K.V;
+    double2* H = K.H;
     __shared__ double bnorm, tolb, wn, gabs;
     __shared__ int go, above_s;
     clu_sync();  // every CTA of the cluster has started, or is done with the last cycle
@@ -567,29 +500,16 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
             res_root(hh, hn, wn);
             res_givens(j, m, M.h1, M.h2, hn, M.cs, M.sn, M.g, H, M.rank == 0, gabs);
             // NaN stops here (rel, below, reports it); tolb = tol |b|
-            int more = gabs >= tolb;
-            if (lock.R > 1) {
-                more = clu_vote(lock, q, run.it + j, more, M.rank == 0);
-            } else if (!more && extra > 0) {
+            bool more = gabs >= tolb;
+            if (!more && extra > 0) {
                 extra--;
-                more = 1;
+                more = true;
             }
-            above_s = more > 0;
-            go = more > 0 && j + 1 < m && run.it + j + 1 < run.maxit ? 1 : (more < 0 ? -1 : 0);
+            above_s = more;
+            go = more && j + 1 < m && run.it + j + 1 < run.maxit;
         }
         __syncthreads();
-        // the CTAs of a cluster read the same flags, but one of them may give up alone: agree first
-        int decide = go;
-        if (lock.R > 1) {
-            if (threadIdx.x < M.C)
-                *cooperative_groups::this_cluster().map_shared_rank(
-                    M.pr + M.rank * M.ld, threadIdx.x) = make_double2((double)go, 0);
-            clu_sync();
-            for (int c = 0; c < M.C; c++)
-                if (M.pr[c * M.ld].x < 0) decide = -1;
-        }
-        if (decide < 0) return -1;
-        if (!decide) break;
+        if (!go) break;  // every CTA of the cluster decides from the same numbers
         set_v(j + 1);
     }
     clu_sync();  // rank 0's H
@@ -601,44 +521,35 @@ __device__ int clu_fgmres(SYS& sys, const ResKrylov& K, CluMem& M, int q, const 
     return j;
 }
 
-// sum over a CSR row of val x (x of R vectors ldx apart), by the G lanes of a
-// group: every lane ends with the sums.  CG: x was written by other CTAs of this
-// kernel.  All lanes of the warp call it (rows beyond the end with e0 = e1).
-template <int RM, bool CG>
-__device__ __forceinline__ void res_row(int64_t e0, int64_t e1, const int32_t* __restrict__ col,
-                                        const double2* __restrict__ val, const double2* x, int64_t ldx, int R, int l,
-                                        int G, double2* s)
+// sum over a CSR row of val x by the G lanes of a group: every lane ends with it.
+// CG: x was written by other CTAs of this kernel.  All lanes of the warp call it (rows
+// beyond the end with e0 = e1).
+template <bool CG>
+__device__ __forceinline__ double2 res_row(int64_t e0, int64_t e1, const int32_t* __restrict__ col,
+                                           const double2* __restrict__ val, const double2* x, int l, int G)
 {
-#pragma unroll
-    for (int q = 0; q < RM; q++) s[q] = make_double2(0, 0);
+    double2 s = make_double2(0, 0);
     int64_t e = e0 + l;
-    if constexpr (RM == 1) {
-        for (; e + 3 * G < e1; e += 4 * G) {  // four loads in flight
-            double2 v[4], xv[4];
+    for (; e + 3 * G < e1; e += 4 * G) {  // four loads in flight
+        double2 v[4], xv[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int c = __ldg(col + e + u * G);
-                v[u] = __ldg(val + e + u * G);
-                xv[u] = CG ? __ldcg(x + c) : x[c];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; u++) r_fma(s[0], v[u], xv[u]);
+        for (int u = 0; u < 4; u++) {
+            const int c = __ldg(col + e + u * G);
+            v[u] = __ldg(val + e + u * G);
+            xv[u] = CG ? __ldcg(x + c) : x[c];
         }
+#pragma unroll
+        for (int u = 0; u < 4; u++) r_fma(s, v[u], xv[u]);
     }
     for (; e < e1; e += G) {
         const int c = __ldg(col + e);
-        const double2 v = __ldg(val + e);
-#pragma unroll
-        for (int q = 0; q < RM; q++)
-            if (q < R) r_fma(s[q], v, CG ? __ldcg(x + q * ldx + c) : x[q * ldx + c]);
+        r_fma(s, __ldg(val + e), CG ? __ldcg(x + c) : x[c]);
     }
-#pragma unroll
-    for (int q = 0; q < RM; q++)
-        if (q < R)
-            for (int off = G >> 1; off > 0; off >>= 1) {
-                s[q].x += __shfl_xor_sync(0xffffffffu, s[q].x, off);
-                s[q].y += __shfl_xor_sync(0xffffffffu, s[q].y, off);
-            }
+    for (int off = G >> 1; off > 0; off >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    return s;
 }
 
 // for the rows [r0, r1) by groups of G lanes: body(row or -1, lane in group); all lanes of a warp run together

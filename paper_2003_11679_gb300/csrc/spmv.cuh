@@ -74,15 +74,18 @@ __device__ __forceinline__ double2 csr_row_dot(int64_t e0, int64_t e1, const int
     return make_double2(sr, si);
 }
 
-// y = alpha A x (ACC = false) or y += alpha A x (ACC = true); up to 256 threads
+// y = alpha A x (ACC = false) or y += alpha A x (ACC = true); up to 256 threads.  Vector
+// blockIdx.y: x and y ldx and ldy apart
 template <int G, bool ACC, class VT, class XT>
 __global__ void __launch_bounds__(256) k_csr(int nrow, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                              const VT* __restrict__ val, const XT* __restrict__ x,
-                                             double2 alpha, double2* __restrict__ y)
+                                             double2 alpha, double2* __restrict__ y, int64_t ldx, int64_t ldy)
 {
     const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G);
     const int l = threadIdx.x % G;
     const bool ok = r < nrow;
+    x += blockIdx.y * ldx;
+    y += blockIdx.y * ldy;
     // rows past the end still take part in the shuffles, with an empty range
     const int64_t e0 = ok ? __ldg(rp + r) : 0, e1 = ok ? __ldg(rp + r + 1) : 0;
     const double2 s = csr_row_dot<G, VT, XT>(e0, e1, col, val, x, l);
@@ -126,7 +129,8 @@ inline int csr_group_for(const int64_t* rp, int nrow, int64_t nnz, int vbytes)
 
 template <class VT, class XT>
 inline cudaError_t csr_launch_g(cudaStream_t st, int G, int nrow, const int64_t* rp, const int32_t* col,
-                                const VT* val, const XT* x, double2 alpha, bool acc, double2* y);
+                                const VT* val, const XT* x, double2 alpha, bool acc, double2* y, int nr = 1,
+                                int64_t ldx = 0, int64_t ldy = 0);
 
 template <class VT, class XT>
 inline cudaError_t csr_launch(cudaStream_t st, int nrow, int64_t nnz, const int64_t* rp, const int32_t* col,
@@ -136,27 +140,28 @@ inline cudaError_t csr_launch(cudaStream_t st, int nrow, int64_t nnz, const int6
     return csr_launch_g(st, csr_group_for(rp, nrow, nnz, (int)sizeof(VT)), nrow, rp, col, val, x, alpha, acc, y);
 }
 
-// the product with G lanes per row (4, 8, 16 or 32)
+// the product with G lanes per row (4, 8, 16 or 32) of nr vectors, ldx and ldy apart
 template <class VT, class XT>
 inline cudaError_t csr_launch_g(cudaStream_t st, int G, int nrow, const int64_t* rp, const int32_t* col,
-                                const VT* val, const XT* x, double2 alpha, bool acc, double2* y)
+                                const VT* val, const XT* x, double2 alpha, bool acc, double2* y, int nr, int64_t ldx,
+                                int64_t ldy)
 {
     // CTAs of 64 threads when 256 would not fill the SMs twice: FP64 runs at 2 lanes per
     // SM, so a small product gains from more SMs
     const int T = (int64_t)nrow * G < 256 * 304 ? 64 : 256;
-    const unsigned blocks = (unsigned)(((int64_t)nrow * G + T - 1) / T);
+    const dim3 blocks((unsigned)(((int64_t)nrow * G + T - 1) / T), nr);
     if (G == 4) {
-        if (acc) k_csr<4, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<4, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<4, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
+        else k_csr<4, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
     } else if (G == 8) {
-        if (acc) k_csr<8, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<8, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<8, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
+        else k_csr<8, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
     } else if (G == 16) {
-        if (acc) k_csr<16, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<16, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<16, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
+        else k_csr<16, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
     } else {
-        if (acc) k_csr<32, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
-        else k_csr<32, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y);
+        if (acc) k_csr<32, true, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
+        else k_csr<32, false, VT, XT><<<blocks, T, 0, st>>>(nrow, rp, col, val, x, alpha, y, ldx, ldy);
     }
     return cudaGetLastError();
 }

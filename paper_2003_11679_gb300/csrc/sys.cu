@@ -559,45 +559,6 @@ static sie_status fgmres(sie_ctx* c, KrylovWork& K, int64_t n, const Apply& A, c
 }
 
 // ------------------------------------------------------------------ system kernels
-template <class C>
-__device__ __forceinline__ C cmk(double a, double b)
-{
-    C c;
-    c.x = a;
-    c.y = b;
-    return c;
-}
-
-// tc: per triangle 9 values: alpha_H, beta_H[3], alpha_E, beta_E[3], -c0rho
-template <class C>
-__global__ void k_tri_coef(int nt, DevMesh M, const double2* __restrict__ H, const double2* __restrict__ E,
-                           const double2* __restrict__ rho, C* __restrict__ tc)
-{
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nt) return;
-    double ar[2] = {0, 0}, ai[2] = {0, 0}, br[2][3] = {{0, 0, 0}, {0, 0, 0}}, bi[2][3] = {{0, 0, 0}, {0, 0, 0}};
-    for (int i = 0; i < 3; i++) {
-        const int e = M.tri_edge[3 * t + i];
-        const double c = M.coef[3 * t + i];
-        const double2 xs[2] = {H[e], E[e]};
-        for (int f = 0; f < 2; f++) {
-            ar[f] += c * xs[f].x;
-            ai[f] += c * xs[f].y;
-            for (int a = 0; a < 3; a++) {
-                const double qq = c * M.q[9 * t + 3 * i + a];
-                br[f][a] += qq * xs[f].x;
-                bi[f][a] += qq * xs[f].y;
-            }
-        }
-    }
-    C* o = tc + 9 * (int64_t)t;
-    for (int f = 0; f < 2; f++) {
-        o[4 * f] = cmk<C>(ar[f], ai[f]);
-        for (int a = 0; a < 3; a++) o[4 * f + 1 + a] = cmk<C>(br[f][a], bi[f][a]);
-    }
-    o[8] = cmk<C>(-rho[t].x, -rho[t].y);
-}
-
 __global__ void k_specmul_sys32(const float2* __restrict__ spec, float2* __restrict__ buf, int64_t nn, float k0)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -975,7 +936,7 @@ static sie_status apply_Z_resident(sie_op* op, const double2* H, double2* E, dou
     {
         Stage s_(c, "inner_solve");
         // one iteration past the tolerance outside the graph, as fgmres with its lagged check
-        SIE_TRY(nested_solve(op, 1, H, ne, E, ne, make_double2(f.real(), f.imag()), op->capturing ? 0 : 1, w));
+        SIE_TRY(nested_solve(op, H, E, make_double2(f.real(), f.imag()), op->capturing ? 0 : 1, w));
     }
     if (op->capturing) return SIE_OK;
     SIE_CUDA_TRY(cudaMemcpyAsync(K.resid_h, op->gstat + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1154,10 +1115,10 @@ static sie_status sys_grid(sie_op* op, const double2* H, const double2* E, const
         {
             Stage s_(c, "project_sys32");
             float2* tc = reinterpret_cast<float2*>(op->pm_tc);
-            k_tri_coef<float2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, E, rho, tc);
+            k_tri_coef<float2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, 0, E, 0, rho, 0, tc);
             SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(float2) * 7 * Ng, st));
             k_project_gather<float2, float><<<gio_blocks(op->pm_nnode, 8), 256, 0, st>>>(
-                op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W32, tc, src, Ng);
+                op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W32, tc, M.nt, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
         if (fused_z() && fft_fused_z(g)) {
@@ -1186,10 +1147,10 @@ static sie_status sys_grid(sie_op* op, const double2* H, const double2* E, const
         double2* buf = op->ws.bufs;
         {
             Stage s_(c, "project_sys");
-            k_tri_coef<double2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, E, rho, op->pm_tc);
+            k_tri_coef<double2><<<nb(M.nt, 128), 128, 0, st>>>(M.nt, M, H, 0, E, 0, rho, 0, op->pm_tc);
             SIE_CUDA_TRY(cudaMemsetAsync(src, 0, sizeof(double2) * 7 * Ng, st));
             k_project_gather<double2, double><<<gio_blocks(op->pm_nnode, 8), 256, 0, st>>>(
-                op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W, op->pm_tc, src, Ng);
+                op->pm_nnode, op->pm_node, op->pm_ptr, op->pm_ent, S, op->W, op->pm_tc, M.nt, src, Ng);
             SIE_CUDA_TRY(cudaGetLastError());
         }
         if (fused_z() && fft_fused_z(g)) {
@@ -1346,8 +1307,8 @@ static sie_status constraint_solve(sie_op* op, AimOp& a, cplx kappa, KrylovWork&
         w.m = K.m, w.V = K.V, w.Z = K.Z, w.H = K.Hd;
         sie_status s = SIE_OK;
         Stage s_(c, "constraint_solve");
-        if (constraint_resident(op, a, make_double2(kappa.real(), kappa.imag()), false, 1, &v, &y, tol,
-                                op->p.constraint_maxit, op->p.constraint_restart, w, t1, rq, q, &s))
+        if (constraint_resident(op, a, make_double2(kappa.real(), kappa.imag()), false, v, y, tol, op->p.constraint_maxit,
+                                w, t1, rq, q, &s))
             return s;
     }
     k_jacobi<<<nb(ne), 256, 0, st>>>(ne, v, a.dLA, make_double2(1.0, 0.0), t1);
@@ -1421,8 +1382,8 @@ static sie_status precond_sys(sie_op* op, const double2* x, double2* y)
         w.m = K.m, w.V = K.V, w.Z = K.Z, w.H = K.Hd;
         sie_status s = SIE_OK;
         Stage s_(op->mesh->ctx, "constraint_solve");
-        if (constraint_resident(op, X, make_double2(1.0 / (op->k0 * op->k0), 0.0), true, 1, &x, &y, op->p.tol_constraint,
-                                op->p.constraint_maxit, op->p.constraint_restart, w, v1p, op->cs_t, op->cs_t + nt, &s))
+        if (constraint_resident(op, X, make_double2(1.0 / (op->k0 * op->k0), 0.0), true, x, y, op->p.tol_constraint,
+                                op->p.constraint_maxit, w, v1p, op->cs_t, op->cs_t + nt, &s))
             return s;
     }
     // v1' = v1 - (j k0)^-1 D^T Lphi B v2,  B v2 = -A v2
@@ -1550,7 +1511,11 @@ static sie_status gram_prepare(sie_op* op)
             }
     }
     SIE_TRY(upload_rows(st, rows, &op->gr_row_ptr, &op->gr_col, &op->gr_val, &op->gr_nnz));
+    std::vector<double2> dc(h.ne);
+    for (int64_t m = 0; m < h.ne; m++) dc[m] = make_double2(diag[m], 0.0);
     for (double& d : diag) d = 1.0 / d;
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gr_diag, sizeof(double2) * h.ne, st));
+    SIE_CUDA_TRY(cudaMemcpyAsync(op->gr_diag, dc.data(), sizeof(double2) * h.ne, cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gr_idiag, sizeof(double) * h.ne, st));
     SIE_CUDA_TRY(cudaMemcpyAsync(op->gr_idiag, diag.data(), sizeof(double) * h.ne, cudaMemcpyHostToDevice, st));
     SIE_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1689,11 +1654,11 @@ void sys_release(sie_op* op)
     op->zp = nullptr;
     for (void* p : {(void*)op->mscr, (void*)op->ir_multi, (void*)op->mvec})
         if (p) cudaFreeAsync(p, st);
-    if (op->con_scr) cudaFreeAsync(op->con_scr, st);
-    op->mscr = op->ir_multi = op->mvec = op->con_scr = nullptr;
+    op->mscr = op->ir_multi = op->mvec = nullptr;
+    blk_release(op);
     op->kcs_in.release(st);
     op->kcs_out.release(st);
-    for (void* p : {(void*)op->gr_row_ptr, (void*)op->gr_col, (void*)op->gr_val, (void*)op->gr_idiag,
+    for (void* p : {(void*)op->gr_row_ptr, (void*)op->gr_col, (void*)op->gr_val, (void*)op->gr_idiag, (void*)op->gr_diag,
                     (void*)op->pm_node, (void*)op->pm_ptr, (void*)op->pm_ent, (void*)op->pm_tc,
                     (void*)op->pk_he, (void*)op->pk_sig, (void*)op->bal})
         if (p) cudaFreeAsync(p, st);
@@ -2030,57 +1995,6 @@ void PanelWork::release(cudaStream_t st)
     m = R = 0;
 }
 
-// E = Z' H for a panel of R vectors (near-region-only or SIBC interiors), one
-// grid-resident kernel; Hp, Ep: R x ne.  Does not wait: its statistics stay in op->gstat.
-static sie_status apply_Z_panel(sie_op* op, int R, const double2* Hp, double2* Ep)
-{
-    sie_ctx* c = op->mesh->ctx;
-    const int64_t ne = op->mesh->h.ne;
-    cplx f;
-    if (op->p.interior_model == SIE_SIBC)
-        f = cplx(op->eta_re, op->eta_im);
-    else
-        f = -1.0 / cplx(op->sigma * ETA0, op->k0 * op->eps_r);
-    PanelWork& K = op->kzp;
-    SIE_TRY(K.alloc(c->stream, ne, inner_m(op), R));
-    ResWork w;
-    w.m = K.m, w.V = K.V, w.Z = K.Z, w.W = K.W, w.H = K.Hd, w.ldh = pw_d(K.m), w.part = K.P;
-    Stage s_(c, "inner_solve");
-    return nested_solve(op, R, Hp, ne, Ep, ne, make_double2(f.real(), f.imag()), 1, w);
-}
-
-// y_q = SYS x_q for R vectors (block product): the R nested interior solves as
-// one panel solve (near-region-only and SIBC interiors; AIM interiors solve
-// each through apply_Z), then the rest of the product per vector.
-static sie_status apply_sys_multi(sie_op* op, int R, const double2* const* x, double2* const* y)
-{
-    if (op->inn.has_grid && op->p.interior_model != SIE_SIBC) {
-        for (int q = 0; q < R; q++) SIE_TRY(apply_sys(op, x[q], y[q]));
-        return SIE_OK;
-    }
-    cudaStream_t st = op->mesh->ctx->stream;
-    const int64_t ne = op->mesh->h.ne;
-    if (!op->zp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->zp, sizeof(double2) * 3 * MULTI_RHS * ne, st));
-    double2* Hp = op->zp;
-    double2* Ep = op->zp + MULTI_RHS * ne;
-    double2* Bp = op->zp + 2 * MULTI_RHS * ne;
-    Branch br(op, !op->mesh->ctx->prof.on);  // as in apply_sys
-    SIE_CUDA_TRY(br.follow());
-    for (int q = 0; q < R; q++) SIE_TRY(sys_charge(op, br.st(), x[q], x[q] + ne, Bp + q * ne, y[q] + ne));
-    for (int q = 0; q < R; q++)
-        SIE_CUDA_TRY(cudaMemcpyAsync(Hp + q * ne, x[q], sizeof(double2) * ne, cudaMemcpyDeviceToDevice, st));
-    SIE_TRY(apply_Z_panel(op, R, Hp, Ep));
-    SIE_CUDA_TRY(br.follow());
-    for (int q = 0; q < R; q++) SIE_TRY(sys_near(op, br.st(), x[q], Ep + q * ne, Bp + q * ne));
-    for (int q = 0; q < R; q++) {
-        SIE_CUDA_TRY(cudaMemsetAsync(y[q], 0, sizeof(double2) * ne, st));
-        SIE_TRY(sys_grid(op, x[q], Ep + q * ne, x[q] + ne, y[q]));
-    }
-    SIE_CUDA_TRY(br.join());
-    for (int q = 0; q < R; q++) SIE_TRY(axpby(st, ne, 1.0, Bp + q * ne, 1.0, y[q]));
-    return SIE_OK;
-}
-
 // ------------------------------------------------------------------ several right-hand sides in lockstep
 // y_q = Op x_q for q < R: a non-owning reference to a block operator
 class BlockApply {
@@ -2220,6 +2134,98 @@ static sie_status fgmres_multi(sie_ctx* c, PanelWork& K, int R, int64_t n, const
     return all_below(rel) ? SIE_OK : SIE_ERR_NOT_CONVERGED;
 }
 
+// E_q = Z' H_q for R vectors (near-region-only or SIBC interiors; H_q ldh apart, E_q
+// ne apart): right-hand sides and products as CSR x panel products (block.cu), the
+// iterations in lockstep (near-only: A = L_i,NR, M = its sparse approximate inverse;
+// SIBC: A = Gram, M = Jacobi), then the impedance factor
+static sie_status apply_Z_panel(sie_op* op, int R, const double2* H, int64_t ldh, double2* E)
+{
+    sie_ctx* c = op->mesh->ctx;
+    cudaStream_t st = c->stream;
+    const int64_t ne = op->mesh->h.ne;
+    AimOp& I = op->inn;
+    const bool sibc = op->p.interior_model == SIE_SIBC;
+    double2* a = op->zp + MULTI_RHS * ne;      // right-hand sides
+    double2* t = op->zp + 2 * MULTI_RHS * ne;  // scratch
+    // I-cross H (weight -1/2 for GIBC, +1 for SIBC)
+    SIE_TRY(blk_csr(st, (int)ne, op->ix_row_ptr, op->ix_col, op->ix_val, H, ldh, R, sibc ? a : t, ne));
+    if (!sibc) {
+        SIE_TRY(blk_csr(st, (int)ne, I.row_ptr, I.col, I.valK, H, ldh, R, a, ne));
+        SIE_TRY(axpby(st, R * ne, -0.5, t, 1.0, a));
+    }
+    // the R vectors of a block lie one distance apart
+    auto product = [&](const int64_t* rp, const int32_t* col, const double2* val, const double2* const* x,
+                       double2* const* y) {
+        return blk_csr(st, (int)ne, rp, col, val, x[0], R > 1 ? x[1] - x[0] : 0, R, y[0], R > 1 ? y[1] - y[0] : 0);
+    };
+    auto A = [&](int, const double2* const* x, double2* const* y) {
+        return sibc ? product(op->gr_row_ptr, op->gr_col, op->gr_val, x, y) : product(I.row_ptr, I.col, I.valL, x, y);
+    };
+    auto M = [&](int, const double2* const* x, double2* const* y) -> sie_status {
+        if (!sibc) return product(I.row_ptr, I.col, I.valM, x, y);
+        for (int q = 0; q < R; q++)
+            k_jacobi<<<nb(ne), 256, 0, st>>>(ne, x[q], op->gr_diag, make_double2(1.0, 0.0), y[q]);
+        SIE_CUDA_TRY(cudaGetLastError());
+        return SIE_OK;
+    };
+    const double2* b[MULTI_RHS];
+    double2* e[MULTI_RHS];
+    for (int q = 0; q < R; q++) b[q] = a + q * ne, e[q] = E + q * ne;
+    const int m_in = inner_m(op);
+    int it[MULTI_RHS];
+    double rr[MULTI_RHS];
+    {
+        Stage s_(c, "inner_solve");
+        const sie_status s = fgmres_multi(c, op->kzp, R, ne, A, M, b, e, op->p.tol_inner, m_in, m_in, it, rr);
+        if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
+    }
+    for (int q = 0; q < R; q++) {
+        op->stats[2] = std::max(op->stats[2], (double)it[q]);
+        op->stats[3] = std::max(op->stats[3], rr[q]);
+    }
+    if (op->edge_zf) {
+        for (int q = 0; q < R; q++) k_scale_edges<<<nb(ne), 256, 0, st>>>(ne, op->edge_zf, e[q]);
+        SIE_CUDA_TRY(cudaGetLastError());
+        return SIE_OK;
+    }
+    cplx f;
+    if (sibc) {
+        f = cplx(op->eta_re, op->eta_im);
+    } else {
+        cplx zs(0.0, op->k0 * op->eps_r);
+        zs += op->sigma * ETA0;
+        f = -1.0 / zs;
+    }
+    return axpby(st, R * ne, f, E, 0.0, E);
+}
+
+// y_q = SYS x_q for R vectors: near-region-only and SIBC interiors as one block
+// product (block.cu), the complex64 product and AIM interiors one vector at a time
+static sie_status apply_sys_multi(sie_op* op, int R, const double2* const* x, double2* const* y)
+{
+    if (op->inn.has_grid) {
+        for (int q = 0; q < R; q++) SIE_TRY(apply_sys(op, x[q], y[q]));
+        return SIE_OK;
+    }
+    cudaStream_t st = op->mesh->ctx->stream;
+    const int64_t ne = op->mesh->h.ne;
+    if (!op->zp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->zp, sizeof(double2) * 3 * MULTI_RHS * ne, st));
+    double2* Ep = op->zp;
+    // the R vectors of a block lie one distance apart
+    const int64_t ldx = R > 1 ? x[1] - x[0] : 0, ldy = R > 1 ? y[1] - y[0] : 0;
+    SIE_TRY(apply_Z_panel(op, R, x[0], ldx, Ep));
+    if (op->p.precision != SIE_MIXED) return blk_sys_rest(op, R, x[0], ldx, Ep, ne, y[0], ldy);
+    double2* yb = op->sys_tmp + ne + 2 * op->mesh->h.nt;
+    for (int q = 0; q < R; q++) {
+        SIE_TRY(sys_charge(op, st, x[q], x[q] + ne, yb, y[q] + ne));
+        SIE_TRY(sys_near(op, st, x[q], Ep + q * ne, yb));
+        SIE_CUDA_TRY(cudaMemsetAsync(y[q], 0, sizeof(double2) * ne, st));
+        SIE_TRY(sys_grid(op, x[q], Ep + q * ne, x[q] + ne, y[q]));
+        SIE_TRY(axpby(st, ne, 1.0, yb, 1.0, y[q]));
+    }
+    return SIE_OK;
+}
+
 // scratch of the lockstep solves: per right-hand side the weighted input of
 // the preconditioner, the weighted right-hand side and the preconditioner's
 // vectors (ne: v1', t1, te and the triangle operator's te; nt: sigma, phi,
@@ -2236,20 +2242,18 @@ static sie_status multi_scratch(sie_op* op)
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->mscr, sizeof(double2) * MULTI_RHS * multi_stride(op),
                                  op->mesh->ctx->stream));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->ir_multi, sizeof(double2) * 3 * MULTI_RHS * n, op->mesh->ctx->stream));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->con_scr,
-                                 sizeof(double2) * MULTI_RHS * (op->mesh->h.ne + 2 * op->mesh->h.nt),
-                                 op->mesh->ctx->stream));
     return SIE_OK;
 }
 
 // the constraint preconditioner (precond_sys) for R vectors: the sparse
 // steps per vector, the R triangle systems by lockstep GMRES whose
 // preconditioner is one pass over the dense inverse for all of them
-// (DenseLU::solve_multi); without a factorisation, precond_sys for each
+// (DenseLU::solve_multi); without a factorisation, and for penetrable objects, whose
+// products are made one vector at a time anyway, precond_sys for each
 static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, double2* const* y)
 {
     AimOp& X = op->ext;
-    if (!X.lu) {
+    if (!X.lu || (op->inn.has_grid && op->mesh->h.nt <= CLU_MAXN)) {
         for (int q = 0; q < R; q++) SIE_TRY(precond_sys(op, x[q], y[q]));
         return SIE_OK;
     }
@@ -2259,19 +2263,11 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
     const int64_t ne = M.ne, nt = M.nt, n = ne + nt;
     const cplx jk0(0.0, op->k0);
     const cplx kappa = 1.0 / (op->k0 * op->k0);
-    const int m = std::min(op->p.constraint_restart, 20);
-    {
-        PanelWork& K = op->kcs_multi;
-        SIE_TRY(K.alloc(st, nt, m, R));
-        ResWork w;
-        w.m = m, w.V = K.V, w.Z = K.Z, w.H = K.Hd, w.ldh = pw_d(m);
-        double2* v1 = op->con_scr;
-        sie_status s = SIE_OK;
-        Stage s_(c, "constraint_solve");
-        if (constraint_resident(op, X, make_double2(kappa.real(), kappa.imag()), true, R, x, y, op->p.tol_constraint,
-                                op->p.constraint_maxit, m, w, v1, v1 + R * ne, v1 + R * (ne + nt), &s))
-            return s;
-    }
+    auto lphi = [&](const double2* u, double2* v) {
+        SIE_CUDA_TRY(csr_launch_g(st, BLK_TRI_LANES, (int)nt, X.tri_row_ptr, X.tri_col, X.valLphiNR, u,
+                                  make_double2(1.0, 0.0), false, v));
+        return SIE_OK;
+    };
     double2 *v1p[MULTI_RHS], *t1[MULTI_RHS], *te[MULTI_RHS], *sig[MULTI_RHS], *ph[MULTI_RHS];
     double2 *rq[MULTI_RHS], *qv[MULTI_RHS], *ste[MULTI_RHS], *sph[MULTI_RHS];
     for (int q = 0; q < R; q++) {
@@ -2289,7 +2285,7 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
     for (int q = 0; q < R; q++) {
         // v1' = v1 - (j k0)^-1 D^T Lphi B v2, then the charge right-hand side D Dg^-1 v1'
         k_sigma<<<nb(nt), 256, 0, st>>>((int)nt, M.area, x[q] + ne, sig[q]);
-        SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphiNR, sig[q], 1.0, ph[q], false));
+        SIE_TRY(lphi(sig[q], ph[q]));
         SIE_CUDA_TRY(cudaMemsetAsync(v1p[q], 0, sizeof(double2) * ne, st));
         k_dt<<<nb(ne), 256, 0, st>>>((int)ne, M.edge_tri, op->elen, ph[q], v1p[q]);
         SIE_TRY(axpby(st, ne, 1.0, x[q], -1.0 / jk0, v1p[q]));
@@ -2300,7 +2296,7 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
     // triangle operator S q = q - kappa D Dg^-1 D^T Lphi q for each vector
     auto S = [&](int Rn, const double2* const* u, double2* const* v) {
         for (int q = 0; q < Rn; q++) {
-            SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphiNR, u[q], 1.0, sph[q], false));
+            SIE_TRY(lphi(u[q], sph[q]));
             SIE_CUDA_TRY(cudaMemsetAsync(ste[q], 0, sizeof(double2) * ne, st));
             k_dt<<<nb(ne), 256, 0, st>>>((int)ne, M.edge_tri, op->elen, sph[q], ste[q]);
             k_jacobi<<<nb(ne), 256, 0, st>>>(ne, ste[q], X.dLA, make_double2(1.0, 0.0), ste[q]);
@@ -2319,7 +2315,7 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
         double rr[MULTI_RHS];
         Stage s_(c, "constraint_solve");
         sie_status s = fgmres_multi(c, op->kcs_multi, R, nt, S, LU, rq, qv, op->p.tol_constraint,
-                                    op->p.constraint_maxit, m, it, rr, 0);
+                                    op->p.constraint_maxit, std::min(op->p.constraint_restart, 20), it, rr, 0);
         if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
         for (int q = 0; q < R; q++) {
             op->stats[4] = std::max(op->stats[4], (double)it[q]);
@@ -2328,7 +2324,7 @@ static sie_status precond_sys_multi(sie_op* op, int R, const double2* const* x, 
     }
     for (int q = 0; q < R; q++) {
         // y1 = (j k0)^-1 Dg^-1 (v1' + kappa D^T Lphi q)
-        SIE_TRY(spmv(st, (int)nt, tri_nnz(X), X.tri_row_ptr, X.tri_col, X.valLphiNR, qv[q], 1.0, ph[q], false));
+        SIE_TRY(lphi(qv[q], ph[q]));
         SIE_CUDA_TRY(cudaMemsetAsync(te[q], 0, sizeof(double2) * ne, st));
         k_dt<<<nb(ne), 256, 0, st>>>((int)ne, M.edge_tri, op->elen, ph[q], te[q]);
         SIE_TRY(axpby(st, ne, kappa, te[q], 0.0, te[q]));
