@@ -11,6 +11,7 @@
 // rows (10); now 104 us on a cluster of 16 and 294 us on the whole GPU.
 #include <algorithm>
 
+#include "limits.h"
 #include "resident.cuh"
 
 namespace sie {
@@ -172,12 +173,10 @@ __global__ void __launch_bounds__(RES_T, 1) k_nested_clu(NestSys s, ResKrylov K,
 // CTAs of a resident kernel: about 64 rows each, at most one per SM
 int res_ctas(int64_t work)
 {
-    static const int sms = [] {
-        int dev = 0, v = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        return std::max(1, std::min(v, RES_MAXCTA));
-    }();
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = std::max(1, std::min(v, RES_MAXCTA));
     return (int)std::max<int64_t>(1, std::min<int64_t>(sms, (work + 63) / 64));
 }
 
@@ -192,7 +191,7 @@ int res_group(int64_t rows, int64_t nrow, int64_t nnz)
 
 sie_status res_launch(const void* fn, int ctas, size_t smem, void** args, cudaStream_t st)
 {
-    SIE_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SIE_CUDA_TRY(kernel_limit(fn, smem));
     SIE_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(RES_T), args, smem, st));
     return SIE_OK;
 }
@@ -212,8 +211,7 @@ static void clu_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int C, 
 
 sie_status clu_launch(const void* fn, int C, size_t smem, void** args, cudaStream_t st)
 {
-    SIE_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (C > 8) SIE_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    SIE_CUDA_TRY(kernel_limit(fn, smem, C > 8));
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     clu_config(cfg, &at, C, smem);
@@ -225,13 +223,11 @@ sie_status clu_launch(const void* fn, int C, size_t smem, void** args, cudaStrea
 // whether the GPU runs a cluster of C CTAs
 static bool clu_fits(const void* fn, int C, size_t smem)
 {
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (C > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     clu_config(cfg, &at, C, smem);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+    if (kernel_limit(fn, smem, C > 8) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
