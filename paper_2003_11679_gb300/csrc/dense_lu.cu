@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "limits.h"
 
 namespace sie {
 
@@ -291,9 +292,7 @@ static sie_status cgemm(cudaStream_t st, int M, int N, int K, const float2* A, i
                         int64_t ldb, float2* C, int64_t ldc, int sub)
 {
     if (M <= 0 || N <= 0) return SIE_OK;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_cgemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem());
-    SIE_CUDA_TRY(attr);
+    SIE_CUDA_TRY(kernel_limit((const void*)k_cgemm, gemm_smem()));
     dim3 grid((N + GEMM_BN - 1) / GEMM_BN, (M + GEMM_BM - 1) / GEMM_BM);
     k_cgemm<<<grid, 256, gemm_smem(), st>>>(M, N, K, A, lda, B, ldb, C, ldc, sub);
     SIE_CUDA_TRY(cudaGetLastError());
@@ -729,9 +728,7 @@ sie_status DenseLU::solve_multi(cudaStream_t st, int R, const double2* const* b,
         o.p[q] = x[q];
     }
     const size_t smem = sizeof(float4) * MULTI_R * MR_CHUNK;  // 64 KB
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_cgemm_inv_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    SIE_CUDA_TRY(attr);
+    SIE_CUDA_TRY(kernel_limit((const void*)k_cgemm_inv_multi, smem));
     k_cgemm_inv_multi<<<(unsigned)((n + MR_ROWS - 1) / MR_ROWS), 256, smem, st>>>(
         n, R, reinterpret_cast<const float4*>(Xinv), reinterpret_cast<const float4*>(bpack), o);
     SIE_CUDA_TRY(cudaGetLastError());

@@ -287,20 +287,10 @@ static sie_status launch_stockham_pb(cudaStream_t st, const C* in, C* out, int i
 {
     constexpr int n = 1 << LOGN;
     const size_t smem = sizeof(C) * 2 * PB * (n + 1);
-    // once per instantiation (thread-safe static initialisation)
-    static const cudaError_t attr = [smem] {
-        cudaError_t e = cudaFuncSetAttribute(k_fft_stockham<LOGN, PB, C, 0>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(k_fft_stockham<LOGN, PB, C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
-    }();
-    SIE_CUDA_TRY(attr);
+    const auto fn = inv ? k_fft_stockham<LOGN, PB, C, 1> : k_fft_stockham<LOGN, PB, C, 0>;
+    SIE_CUDA_TRY(kernel_limit((const void*)fn, smem));
     const unsigned blocks = (unsigned)((G.npencil + PB - 1) / PB);
-    if (inv)
-        k_fft_stockham<LOGN, PB, C, 1><<<dim3(blocks, nbatch), PB * n / 8, smem, st>>>(in, out, tw, G);
-    else
-        k_fft_stockham<LOGN, PB, C, 0><<<dim3(blocks, nbatch), PB * n / 8, smem, st>>>(in, out, tw, G);
+    fn<<<dim3(blocks, nbatch), PB * n / 8, smem, st>>>(in, out, tw, G);
     SIE_CUDA_TRY(cudaGetLastError());
     return SIE_OK;
 }

@@ -27,6 +27,7 @@
 #include <stdint.h>
 
 #include "internal.h"
+#include "limits.h"
 #include "sysmul.cuh"
 
 namespace sie {
@@ -823,9 +824,7 @@ sie_status fft_z_n(cudaStream_t st, typename P::G* buf, const typename P::G* spe
 {
     constexpr int PB = z_pb<N, P, MODE>();
     constexpr size_t smem = sizeof(typename P::V) * ZMode<MODE>::NI * PB * fft_pitch<N>(PB);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_fft_z<N, P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    SIE_CUDA_TRY(attr);
+    SIE_CUDA_TRY(kernel_limit((const void*)k_fft_z<N, P, MODE>, smem));
     const dim3 grid((unsigned)((ncol + PB - 1) / PB), nb);
     k_fft_z<N, P, MODE>
         <<<grid, ZMode<MODE>::NI * PB * Plan<N>::R2, smem, st>>>(buf, spec, tw, nz_phys, ncol, plane, bnn, batch, k0);

@@ -42,3 +42,10 @@ def test_refused_sizes_change_nothing(probe):
     out = (ctypes.c_int * 2)()
     assert probe.limits_refused(out) == 0
     assert list(out) == [-1, 70000]
+
+
+def test_no_kernel_sets_its_limits_elsewhere():
+    csrc = os.path.join(ROOT, "paper_2003_11679_gb300", "csrc")
+    for f in os.listdir(csrc):
+        if f != "limits.cpp":
+            assert "cudaFuncSetAttribute" not in open(os.path.join(csrc, f)).read(), f
