@@ -258,8 +258,12 @@ sie_status sie_op_grid(const sie_op* op, double origin[3], double* h, int64_t N[
  * When the interior operator is near-region only and profiling is off, the
  * SYS product (nested solve included) is captured on first use into a CUDA
  * graph, one per precision, and replayed; the nested solve is one kernel
- * that ends its own iterations, as on the stream path (a wait inside it that
- * runs out is SIE_ERR_TIMEOUT, reported like an inexact nested solve).  The
+ * that ends its own iterations, as on the stream path.  A wait inside it that
+ * runs out is SIE_ERR_TIMEOUT: from host-pointer products, RCS and solves
+ * (before SIE_ERR_NOT_CONVERGED, whatever the solve made of the unwritten
+ * product); device-pointer products leave an infinite nested residual in
+ * sie_op_stats.  SIE_WAIT_POLLS in the environment lowers the number of polls
+ * of a wait (read when a nested solve is launched or captured).  The
  * environment variable SIE_GRAPH=0 selects the stream path.  The
  * graph is dropped when tol_inner or inner_maxit change (sie_op_set_solver). */
 sie_status sie_matvec(sie_op* op, int which, const double* x, double* y, int nrhs, int flags);

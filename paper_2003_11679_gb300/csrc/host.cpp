@@ -681,7 +681,7 @@ sie_status sie_op_set_solver(sie_op* op, const sie_params* p)
 sie_status sie_op_stats(const sie_op* op, double out[6])
 {
     if (!op || !out) return SIE_ERR_ARG;
-    sie::sys_stats_fold(const_cast<sie_op*>(op));  // nested-solve counts of graph runs
+    (void)sie::sys_stats_fold(const_cast<sie_op*>(op));  // nested-solve counts of graph runs
     for (int i = 0; i < 6; i++) out[i] = op->stats[i];
     return SIE_OK;
 }

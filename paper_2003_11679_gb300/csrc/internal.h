@@ -309,10 +309,14 @@ struct sie_op {
     cudaStream_t gs[2] = {nullptr, nullptr};  // capture of the product; branch beside the main chain
     cudaEvent_t gev[2] = {nullptr, nullptr};  // main -> branch, branch -> main
     double2* g_io = nullptr;        // graph input x and output y, 2 (ne + nt)
-    // device (6): largest nested iteration count and residual since cleared, those of the
-    // the last nested solve (residual, count)
+    // device (GSTAT): largest nested iteration count and residual since cleared, residual and
+    // count of the last nested solve, largest constraint iteration count and residual,
+    // and (as an int) whether a wait of a resident kernel ran out
+    static constexpr int GSTAT = 7;
     double* gstat = nullptr;
-    unsigned* res_bar = nullptr;    // resident kernels: barrier counter, error flag, lockstep flags (RES_WORDS)
+    bool wait_lost = false;         // host copy of that mark (sys_stats_fold)
+    double last_nested = 0;         // residual of the last resident nested solve when it was read
+    unsigned* res_bar = nullptr;    // resident kernels: barrier counter
     size_t gnodes[2] = {0, 0};      // nodes of the last captured graph; 0
     double2* ir_buf = nullptr;      // iterative refinement: residual, correction, product (3 (ne + nt))
     double q_w = 0.0;               // charge-row weight of the GMRES residual norm (0: not yet computed)
@@ -423,7 +427,7 @@ bool sys_z_workspace_ready(const sie_op* op);
 // drop the captured system-product graph (solver settings changed)
 void sys_graph_reset(sie_op* op);
 // fold the nested-solve statistics of graph runs into op->stats (synchronises)
-void sys_stats_fold(sie_op* op);
+sie_status sys_stats_fold(sie_op* op);
 sie_status sys_far_sums(sie_op* op, const double2* x, const double* rhat_d, int ndir, double2* sums,
                         double* nested_res);
 // nested-solve statistics: clear them, or fold the graph's copy and return

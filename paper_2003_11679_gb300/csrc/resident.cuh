@@ -19,7 +19,8 @@
 // level, so nothing cancels), which saves a reduction.
 //
 // Waits in global memory are bounded: a CTA that gives up sets *err and returns,
-// the others run out at their next wait, and the host reports SIE_ERR_TIMEOUT.
+// the others run out at their next wait, and the call that reads the status reports
+// SIE_ERR_TIMEOUT whatever else came of the unwritten result.
 // Launches whose CTAs wait on one another that way are cooperative.
 #pragma once
 #include <cooperative_groups.h>
@@ -32,7 +33,6 @@ namespace sie {
 
 constexpr int RES_T = 512;              // threads per CTA
 constexpr int RES_MAXCTA = 160;         // partial-sum slots
-constexpr int RES_WORDS = 2;            // counter, error flag
 constexpr int RES_SPIN = 1 << 20;       // polls of a barrier before it gives up (under a second)
 
 __device__ __forceinline__ double2 r_cm(double2 a, double2 b)
@@ -50,6 +50,7 @@ __device__ __forceinline__ void r_fma(double2& c, double2 a, double2 b)
 struct ResBar {
     unsigned* cnt;   // zero at the launch
     int* err;
+    int polls;
     unsigned target;
 };
 // false: the wait ran out
@@ -65,7 +66,7 @@ __device__ __forceinline__ bool res_barrier(ResBar& b)
         int it = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(b.cnt) : "memory");
-            if (++it > RES_SPIN) ok = 0;
+            if (++it > b.polls) ok = 0;
         } while (ok && v < b.target);
         if (!ok) atomicExch(b.err, 1);
         bad = !ok;

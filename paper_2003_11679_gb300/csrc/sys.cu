@@ -10,6 +10,7 @@
 #include <cmath>
 #include <complex>
 #include <cstring>
+#include <limits>
 #include <vector>
 
 #include "gridio.cuh"
@@ -939,13 +940,13 @@ static sie_status apply_Z_resident(sie_op* op, const double2* H, double2* E, dou
         SIE_TRY(nested_solve(op, H, E, make_double2(f.real(), f.imag()), op->capturing ? 0 : 1, w));
     }
     if (op->capturing) return SIE_OK;
-    SIE_CUDA_TRY(cudaMemcpyAsync(K.resid_h, op->gstat + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    SIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    const double rr = K.resid_h[0];
-    if (std::isinf(rr)) {
+    SIE_TRY(sys_stats_fold(op));
+    if (op->wait_lost) {
+        SIE_TRY(nested_clear(op));
         set_error("nested interior solve: a grid barrier's wait ran out");
         return SIE_ERR_TIMEOUT;
     }
+    const double rr = op->last_nested;
     if (!std::isfinite(rr)) {
         set_error("GMRES: the residual is not finite (non-finite right-hand side or operator)");
         return SIE_ERR_ARG;
@@ -1267,17 +1268,25 @@ static sie_status apply_sys_fast(sie_op* op, const double2* x, double2* y)
     return SIE_OK;
 }
 
-void sys_stats_fold(sie_op* op)
+sie_status sys_stats_fold(sie_op* op)
 {
-    if (!op->gstat) return;
-    double h[6] = {0, 0, 0, 0, 0, 0};
+    if (!op->gstat) return SIE_OK;
+    double h[sie_op::GSTAT] = {0, 0, 0, 0, 0, 0, 0};
     cudaStream_t st = op->mesh->ctx->stream;
-    if (cudaMemcpyAsync(h, op->gstat, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess) return;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return;
+    SIE_CUDA_TRY(cudaMemcpyAsync(h, op->gstat, sizeof(h), cudaMemcpyDeviceToHost, st));
+    SIE_CUDA_TRY(cudaStreamSynchronize(st));
     op->stats[2] = std::max(op->stats[2], h[0]);
     op->stats[3] = std::max(op->stats[3], h[1]);
     op->stats[4] = std::max(op->stats[4], h[4]);
     op->stats[5] = std::max(op->stats[5], h[5]);
+    op->last_nested = h[2];
+    int lost = 0;
+    std::memcpy(&lost, &h[6], sizeof(lost));
+    if (lost) {
+        op->wait_lost = true;
+        op->stats[3] = std::numeric_limits<double>::infinity();  // what device-pointer callers see
+    }
+    return SIE_OK;
 }
 
 // Constraint preconditioner (the near-region form of the AEFIE constraint
@@ -1608,10 +1617,9 @@ sie_status sys_prepare(sie_op* op)
         if (!ev) SIE_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_tmp, sizeof(double2) * 2 * (h.ne + h.nt), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->sys_vec, sizeof(double2) * 4 * (h.ne + h.nt), st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * 6, st));
-    SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
-    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->res_bar, sizeof(unsigned) * RES_WORDS, st));
-    SIE_CUDA_TRY(cudaMemsetAsync(op->res_bar, 0, sizeof(unsigned) * RES_WORDS, st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->gstat, sizeof(double) * sie_op::GSTAT, st));
+    SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * sie_op::GSTAT, st));
+    SIE_CUDA_TRY(cudaMallocAsync((void**)&op->res_bar, sizeof(unsigned), st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pk_he, sizeof(float4) * h.ne, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->pk_sig, sizeof(float2) * h.nt, st));
     SIE_CUDA_TRY(cudaMallocAsync((void**)&op->cs_e, sizeof(double2) * 2 * h.ne, st));
@@ -1678,17 +1686,14 @@ sie_status sys_matvec(sie_op* op, int which, const double2* x, double2* y)
     return apply_Z(op, x, y, nullptr);
 }
 
-// SIE_ERR_NOT_CONVERGED when a nested (interior) solve of the products since
-// the statistics were last cleared ended above tol_inner (synchronises)
+// SIE_ERR_TIMEOUT when a wait ran out in a nested (interior) solve of the products
+// since the statistics were last cleared, SIE_ERR_NOT_CONVERGED when one ended above
+// tol_inner (synchronises)
 sie_status nested_check(sie_op* op, const char* who)
 {
-    sys_stats_fold(op);
-    if (std::isinf(op->stats[3])) {
+    SIE_TRY(sys_stats_fold(op));
+    if (op->wait_lost) {
         set_error(std::string(who) + ": a grid barrier's wait ran out in a nested interior solve");
-        return SIE_ERR_TIMEOUT;
-    }
-    if (std::isinf(op->stats[5])) {
-        set_error(std::string(who) + ": a wait ran out in a constraint preconditioner");
         return SIE_ERR_TIMEOUT;
     }
     if (op->stats[3] >= op->p.tol_inner) {
@@ -1700,11 +1705,28 @@ sie_status nested_check(sie_op* op, const char* who)
     return SIE_OK;
 }
 
-// clear the nested-solve statistics (host and graph copies)
+// The status of an outer solve that ended with s: products whose nested solve gave up
+// leave their result unwritten, and whatever the outer iteration made of it (no
+// convergence, numbers that are not finite) is not the reason
+static sie_status solve_status(sie_op* op, sie_status s, const char* who)
+{
+    if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED && s != SIE_ERR_ARG) return s;
+    const sie_status n = nested_check(op, who);
+    if (n == SIE_ERR_TIMEOUT) {
+        SIE_TRY(nested_clear(op));
+        return n;
+    }
+    return s == SIE_OK ? n : s;
+}
+
+// clear the nested-solve statistics (host and device copies; the constraint entries of
+// the device copy are in the host's since the solve that made them)
 sie_status nested_clear(sie_op* op)
 {
     op->stats[2] = op->stats[3] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 2, op->mesh->ctx->stream));
+    op->wait_lost = false;
+    if (op->gstat)
+        SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * sie_op::GSTAT, op->mesh->ctx->stream));
     return SIE_OK;
 }
 
@@ -1756,8 +1778,8 @@ sie_status sys_solve(sie_op* op, const double2* b, double2* x, int* iters, doubl
         SIE_TRY(weight_rows(op, u, tw, true));
         return precond_sys(op, tw, v);
     };
-    for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, op->mesh->ctx->stream));
+    op->stats[4] = op->stats[5] = 0;
+    SIE_TRY(nested_clear(op));
     SIE_TRY(weight_rows(op, b, bw, false));
     int it = 0;
     double rr = 0;
@@ -1767,7 +1789,7 @@ sie_status sys_solve(sie_op* op, const double2* b, double2* x, int* iters, doubl
     op->stats[1] = rr;
     if (iters) *iters = it;
     if (relres) *relres = rr;
-    if (s == SIE_OK) s = nested_check(op, "sie_solve");
+    s = solve_status(op, s, "sie_solve");
     if (s == SIE_OK || s == SIE_ERR_NOT_CONVERGED) SIE_TRY(constraint_lu_check(op));
     return s;
 }
@@ -1816,8 +1838,8 @@ sie_status sys_solve_refined(sie_op* op, const double2* b, double2* x, int* iter
         SIE_TRY(weight_rows(op, u, tw, true));
         return precond_sys(op, tw, v);
     };
-    for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
+    op->stats[4] = op->stats[5] = 0;
+    SIE_TRY(nested_clear(op));
     SIE_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double2) * n, st));
     double bn = 0, rel = 1.0;
     SIE_TRY(weight_rows(op, b, op->bal, false));
@@ -1859,14 +1881,15 @@ sie_status sys_solve_refined(sie_op* op, const double2* b, double2* x, int* iter
         if ((s = axpby(st, n, 1.0, d, 1.0, x)) != SIE_OK) break;
     }
     op->p.precision = saved;
-    if (s != SIE_OK) return s;
-    op->stats[0] = total;
-    op->stats[1] = rel;
-    if (iters) *iters = total;
-    if (relres) *relres = rel;
-    SIE_TRY(constraint_lu_check(op));
-    if (!(rel < op->p.tol_outer)) return SIE_ERR_NOT_CONVERGED;
-    return nested_check(op, "sie_solve (refined)");
+    if (s == SIE_OK) {
+        op->stats[0] = total;
+        op->stats[1] = rel;
+        if (iters) *iters = total;
+        if (relres) *relres = rel;
+        SIE_TRY(constraint_lu_check(op));
+        if (!(rel < op->p.tol_outer)) s = SIE_ERR_NOT_CONVERGED;
+    }
+    return solve_status(op, s, "sie_solve (refined)");
 }
 
 sie_status sys_rhs(sie_op* op, const double* khat, const double* epol, double2* b)
@@ -2381,15 +2404,15 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
         for (int q = 0; q < Rn; q++) SIE_TRY(weight_rows(op, u[q], tw[q], true));
         return precond_sys_multi(op, Rn, tw, v);
     };
-    for (int i = 2; i < 6; i++) op->stats[i] = 0;
-    if (op->gstat) SIE_CUDA_TRY(cudaMemsetAsync(op->gstat, 0, sizeof(double) * 6, st));
+    op->stats[4] = op->stats[5] = 0;
+    SIE_TRY(nested_clear(op));
     for (int q = 0; q < R; q++) SIE_TRY(weight_rows(op, b[q], bw[q], false));
     int it[MULTI_RHS];
     double rr[MULTI_RHS];
     sie_status s = SIE_OK;
     if (!refine) {
         s = fgmres_multi(c, op->kmulti, R, n, A, Minv, bw, x, op->p.tol_outer, op->p.maxit, op->p.restart, it, rr);
-        if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return s;
+        if (s != SIE_OK && s != SIE_ERR_NOT_CONVERGED) return solve_status(op, s, "sie_solve");
     } else {
         double2 *r[MULTI_RHS], *d[MULTI_RHS], *t[MULTI_RHS];
         for (int q = 0; q < R; q++) {
@@ -2434,7 +2457,7 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
             if (s != SIE_OK) break;
         }
         op->p.precision = saved;
-        if (s != SIE_OK) return s;
+        if (s != SIE_OK) return solve_status(op, s, "sie_solve");
         for (int q = 0; q < R; q++) {
             it[q] = total;
             rr[q] = rel[q];
@@ -2452,7 +2475,7 @@ sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* 
     }
     op->stats[0] = itmax;
     op->stats[1] = rrmax;
-    if (s == SIE_OK) s = nested_check(op, "sie_solve");
+    s = solve_status(op, s, "sie_solve");
     if (s == SIE_OK || s == SIE_ERR_NOT_CONVERGED) SIE_TRY(constraint_lu_check(op));
     return s;
 }
