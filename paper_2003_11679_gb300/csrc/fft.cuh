@@ -18,13 +18,15 @@
 // runs with two more bits, rounded off in its twiddle products.  The
 // error is relative to the pencil's norm, as that of an FP64 FFT is, and smaller:
 // 0.5e-16 to 0.7e-16 at every length, most of it the rounding of the stored
-// result, where FP64 butterflies give 1e-16 to 2e-16.  A pencil with a NaN or an
-// infinity gives NaNs, as the sums of an FP64 transform do.
+// result, where FP64 butterflies give 1e-16 to 2e-16.  Below the normal range results
+// are rounded once to a multiple of 2^-1074 (gradual underflow).  A pencil with a NaN
+// or an infinity gives NaNs, as the sums of an FP64 transform do.
 //
 // The complex64 path uses the same passes in FP32.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "internal.h"
 #include "limits.h"
@@ -406,25 +408,67 @@ SIE_HD long long fx_from(unsigned hi, unsigned lo, int s0)
     const long long f = (long long)(m >> s), sg = (long long)(int)hi >> 63;  // sg 0 or -1
     return (f ^ sg) - sg;
 }
-// f 2^(E - bits + 1) as a double; x0 = emax - bits.  Conversion on the FP64 pipe,
-// which the transforms leave idle, then the exponent by an integer addition.
-SIE_HD double fx_to(long long f, int x0)
+// bits of a double and back
+SIE_HD unsigned long long fx_bits(double d)
 {
 #ifdef __CUDA_ARCH__
-    const double d = __ll2double_rn(f);
-    const int hi = __double2hiint(d), e = ((hi >> 20) & 0x7ff) + (x0 - 1022);  // biased exponent of the result
-    int oh = hi + ((x0 - 1022) << 20), ol = __double2loint(d);
-    if (f == 0 || e <= 0) oh = hi & 0x80000000, ol = 0;               // zero, or below the normal range
-    if (e >= 2047) oh = (hi & 0x80000000) | 0x7ff00000, ol = 0;
-    return __hiloint2double(oh, ol);
+    return (unsigned long long)__double_as_longlong(d);
 #else
-    return ldexp((double)f, x0 - 1022);
+    unsigned long long r;
+    memcpy(&r, &d, 8);
+    return r;
 #endif
+}
+SIE_HD double fx_double(unsigned long long r)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)r);
+#else
+    double d;
+    memcpy(&d, &r, 8);
+    return d;
+#endif
+}
+// f 2^(x0 - 1022) where it may lie below the normal range: by integer operations,
+// rounded once at the place of its last bit
+SIE_HD double fx_to_low(long long f, int x0)
+{
+    const long long sg = f >> 63;
+    const unsigned long long a = (unsigned long long)((f ^ sg) - sg);
+    if (a == 0) return 0.0;
+#ifdef __CUDA_ARCH__
+    const int lz = __clzll((long long)a);
+#else
+    const int lz = __builtin_clzll(a);
+#endif
+    const int e = 63 + x0 - lz, sh = e < 0 ? 10 - e : 10;  // biased exponent less one
+    unsigned long long r = sh > 63 ? 0 : ((a << (lz - 1)) + (1ull << (sh - 1))) >> sh;
+    if (e > 0) r += (unsigned long long)(unsigned)e << 52;  // bit 52 of r adds one
+    return fx_double(r | ((unsigned long long)sg & 0x8000000000000000ull));
+}
+// f 2^(E - bits + 1) as a double; x0 = emax - bits.  Conversion on the FP64 pipe,
+// which the transforms leave idle, then the exponent by an integer addition.  From
+// x0 = 0 on no result is below the normal range (f is a whole number).
+SIE_HD double fx_to(long long f, int x0)
+{
+    if (x0 < 0) return fx_to_low(f, x0);
+#ifdef __CUDA_ARCH__
+    const double d = __ll2double_rn(f);
+#else
+    const double d = (double)f;
+#endif
+    const unsigned long long b = fx_bits(d);
+    const int hi = (int)(b >> 32), e = ((hi >> 20) & 0x7ff) + (x0 - 1022);  // biased exponent of the result
+    unsigned oh = (unsigned)hi + ((unsigned)(x0 - 1022) << 20), ol = (unsigned)b;
+    if (f == 0) oh = 0, ol = 0;
+    if (f != 0 && e >= 2047) oh = ((unsigned)hi & 0x80000000u) | 0x7ff00000u, ol = 0;
+    return fx_double(((unsigned long long)oh << 32) | ol);
 }
 
 // the same by integer operations alone, where the FP64 pipe is busy
 SIE_HD double fx_to_int(long long f, int x0)
 {
+    if (x0 < 0) return fx_to_low(f, x0);
     const long long sg = f >> 63;
     const unsigned long long a = (unsigned long long)((f ^ sg) - sg);
 #ifdef __CUDA_ARCH__
@@ -435,16 +479,9 @@ SIE_HD double fx_to_int(long long f, int x0)
     const int e = 63 + x0 - lz;  // biased exponent less one
     unsigned long long r = ((a << (lz - 1)) + 0x200) >> 10;  // |f| < 2^62: lz >= 2; bit 52 set (a carry moves up)
     r += (unsigned long long)(unsigned)e << 52;
-    if (a == 0 || e < 0) r = 0;
-    if (e >= 2046) r = 0x7ff0000000000000ull;
-    r |= (unsigned long long)sg & 0x8000000000000000ull;
-#ifdef __CUDA_ARCH__
-    return __longlong_as_double((long long)r);
-#else
-    double d;
-    memcpy(&d, &r, 8);
-    return d;
-#endif
+    if (a == 0) r = 0;
+    if (a != 0 && e >= 2046) r = 0x7ff0000000000000ull;
+    return fx_double(r | ((unsigned long long)sg & 0x8000000000000000ull));
 }
 
 // ------------------------------------------------------------------ plans
