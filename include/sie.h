@@ -246,9 +246,8 @@ sie_status sie_op_grid(const sie_op* op, double origin[3], double* h, int64_t N[
  * x, y: complex128, length N_e (L0, K0, LI, KI, ZI) or N_e + N_t (SYS, the
  * AEFIE unknowns [H; c0 rho] of Eq. sys).  flags: SIE_DEVICE_PTRS or 0.
  * L0, K0, LI and KI with nrhs > 1 run in blocks of up to 8 right-hand sides:
- * the kernel spectra, the stencil weights and the near-region values are read
- * once per block (one projection, FFT pass, spectral multiply, interpolation
- * and CSR x panel launch per block).  The other operators loop over the
+ * one projection, FFT pass, spectral multiply, interpolation and CSR x panel
+ * launch per block, and the near-region values are read once for all of it.  The other operators loop over the
  * right-hand sides.
  * SYS and ZI contain the nested solve of Eq. (nest2): one unrestarted FGMRES
  * cycle of at most min(inner_maxit, 128) iterations to tol_inner.  When it

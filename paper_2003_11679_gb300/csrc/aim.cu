@@ -260,16 +260,6 @@ __global__ void k_specmul(int mode, const double2* __restrict__ spec, double2* _
     }
 }
 
-// ------------------------------------------------------------------ near CSR product
-// y[m] += sum_e val[e] x[col[e]]; one warp per row
-
-sie_status csr_mv(cudaStream_t st, int nrow, int64_t nnz, const int64_t* rp, const int32_t* col,
-                  const double2* val, const double2* x, double2* y)
-{
-    SIE_CUDA_TRY(csr_launch(st, nrow, nnz, rp, col, val, x, make_double2(1.0, 0.0), false, y));
-    return SIE_OK;
-}
-
 // y_r += W applied to the nr inverse-transformed products (4 grids each with the
 // scalar potential, else 3)
 sie_status aim_interp(sie_op* op, const double2* grids, int has_phi, double2 scal, double2* y, int64_t ldy, int nr)
@@ -595,7 +585,7 @@ sie_status sie_matvec(sie_op* op, int which, const double* x, double* y, int nrh
     bool dev = flags & SIE_DEVICE_PTRS;
     if (which >= SIE_OP_SYS) SIE_TRY(nested_clear(op));
     if (which < SIE_OP_SYS && nrhs > 1) {
-        // blocks of up to 8 right-hand sides: spectra, weights and near values read once per block
+        // blocks of up to 8 right-hand sides: one launch per step, near values read once per block
         AimOp& a = (which == SIE_OP_L0 || which == SIE_OP_K0) ? op->ext : op->inn;
         const int lk = (which == SIE_OP_L0 || which == SIE_OP_LI) ? 0 : 1;
         const int RBLK = 8;

@@ -1,10 +1,11 @@
 // Multi-right-hand-side AIM products (Eqs. AIM_Lin, AIM_Kin) for a block of up
-// to RB vectors: the kernel spectra, the stencil weights and the near-region
-// values are read once per block instead of once per vector.
+// to RB vectors: one launch per step for all of them, and the near-region values
+// are read once per block instead of once per vector.
 //   * projection: one grid of CTAs per right-hand side (gridio.cuh; weights from L2);
 //   * FFTs: one launch per pass over all grids of the block;
-//   * spectral multiply: G (or grad G) loaded once per node, applied to every
-//     vector of the block;
+//   * z transforms and spectral products: one row of CTAs per right-hand side, each
+//     reading the spectra of its columns (fft.cuh; mostly from L2); z lengths above
+//     256 multiply in a kernel of their own, which loads G (or grad G) once per node;
 //   * interpolation: one grid of CTAs per right-hand side;
 //   * near region: CSR x panel product, each (column, value) pair loaded once.
 // Vectors are rhs-major (vector r at r * len), as everywhere in the ABI.

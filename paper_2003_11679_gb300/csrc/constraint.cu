@@ -113,23 +113,16 @@ struct ConClu {
         for (int k = warp; k < rows; k += nw) {
             const float2* row = s.X + (r0 + k) * (int64_t)n;
             float ar = 0, ai = 0, br = 0, bi = 0;
-            if (n % 2 == 0) {  // 16-byte aligned rows
-                const float4* r4 = reinterpret_cast<const float4*>(row);
-                const float4* x4 = reinterpret_cast<const float4*>(xf);
+            // n is even (constraint_resident): 16-byte aligned rows
+            const float4* r4 = reinterpret_cast<const float4*>(row);
+            const float4* x4 = reinterpret_cast<const float4*>(xf);
 #pragma unroll 4
-                for (int c = lane; c < n / 2; c += 32) {
-                    const float4 a = __ldg(r4 + c), v = x4[c];
-                    ar = fmaf(a.x, v.x, fmaf(-a.y, v.y, ar));
-                    ai = fmaf(a.x, v.y, fmaf(a.y, v.x, ai));
-                    br = fmaf(a.z, v.z, fmaf(-a.w, v.w, br));
-                    bi = fmaf(a.z, v.w, fmaf(a.w, v.z, bi));
-                }
-            } else {
-                for (int c = lane; c < n; c += 32) {
-                    const float2 a = __ldg(row + c), v = xf[c];
-                    ar = fmaf(a.x, v.x, fmaf(-a.y, v.y, ar));
-                    ai = fmaf(a.x, v.y, fmaf(a.y, v.x, ai));
-                }
+            for (int c = lane; c < n / 2; c += 32) {
+                const float4 a = __ldg(r4 + c), v = x4[c];
+                ar = fmaf(a.x, v.x, fmaf(-a.y, v.y, ar));
+                ai = fmaf(a.x, v.y, fmaf(a.y, v.x, ai));
+                br = fmaf(a.z, v.z, fmaf(-a.w, v.w, br));
+                bi = fmaf(a.z, v.w, fmaf(a.w, v.z, bi));
             }
             const double2 z = warp_sum(make_double2((double)ar + br, (double)ai + bi));
             if (lane == 0) K.Z[(int64_t)j * K.n + r0 + k] = z;
@@ -230,7 +223,7 @@ bool constraint_resident(sie_op* op, const AimOp& a, double2 kappa, bool ext, co
                          int maxit, const ResWork& w, double2* v1, double2* b, double2* q, sie_status* st_out)
 {
     const int nt = (int)op->mesh->h.nt, ne = (int)op->mesh->h.ne;
-    if (!a.lu || !a.lu->Xinv || nt > CLU_MAXN) return false;
+    if (!a.lu || !a.lu->Xinv || nt > CLU_MAXN || nt % 2) return false;  // closed meshes have 3 nt = 2 ne: even
     const int C = clu_pick((const void*)k_constraint, nt, a.npairs, w.m, sizeof(float2) * (nt + 1));
     if (!C) return false;
     const size_t smem = clu_smem(nt, w.m, C) + sizeof(float2) * (nt + 1);

@@ -155,8 +155,8 @@ static sie_status set_objects(HostMesh& m, const int32_t* obj)
 
 // ------------------------------------------------------------------ grid (Sec. III-A, Sec. IV)
 // shortest supported FFT length >= n (-1: none): lengths with factors 3 and 5 fill
-// the gaps of the powers of two, so a dimension's padding is at most a third
-// instead of almost all of it.  A 19-node cube transforms on 40^3 instead of 64^3, a
+// the gaps of the powers of two up to 256, so that up to there a dimension's padding is
+// at most a third instead of almost all of it (257 still takes 512).  A 19-node cube transforms on 40^3 instead of 64^3, a
 // bar of 41 x 9 x 9 nodes on 96 x 20 x 20 instead of 128 x 32 x 32.
 static int fft_length(int n)
 {

@@ -377,7 +377,7 @@ sie_status aim_sample(cudaStream_t st, const GridDesc& g, double kr, double ki, 
 sie_status aim_spectra(sie_op* op, AimOp& a);
 sie_status near_build(sie_op* op, AimOp& a, const QuadDev& q);
 sie_status aim_apply(sie_op* op, AimOp& a, int which_LK, const double2* x, double2* y);
-// Y = A X for nr <= 8 vectors at once (spectra, weights and near values read once)
+// Y = A X for nr <= 8 vectors at once (one launch per step, near values read once)
 sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X, double2* Y, int nr);
 // Work beside the context's stream: st() is the operator's branch stream between
 // follow() (it waits for the main stream's work so far) and join() (the main stream
@@ -419,9 +419,6 @@ sie_status sys_solve_refined(sie_op* op, const double2* b, double2* x, int* iter
 sie_status sys_solve_multi(sie_op* op, int R, const double2* const* b, double2* const* x, int* iters, double* relres,
                            bool refine);
 sie_status sys_rhs(sie_op* op, const double* khat, const double* epol, double2* b);
-// y = A x for an edge CSR matrix (overwrites y)
-sie_status csr_mv(cudaStream_t st, int nrow, int64_t nnz, const int64_t* rp, const int32_t* col,
-                  const double2* val, const double2* x, double2* y);
 sie_status sys_rcs(sie_op* op, const double2* x, const double* rhat, int ndir, double* rcs);
 bool sys_z_workspace_ready(const sie_op* op);
 // drop the captured system-product graph (solver settings changed)
