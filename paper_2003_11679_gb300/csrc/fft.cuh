@@ -18,13 +18,14 @@
 // runs with two more bits, rounded off in its twiddle products.  The
 // error is relative to the pencil's norm, as that of an FP64 FFT is, and smaller:
 // 0.5e-16 to 0.7e-16 at every length, most of it the rounding of the stored
-// result, where FP64 butterflies give 1e-16 to 2e-16.  Below the normal range results
-// are rounded once to a multiple of 2^-1074 (gradual underflow).  A pencil with a NaN
-// or an infinity gives NaNs, as the sums of an FP64 transform do.
+// result, where FP64 butterflies give 1e-16 to 2e-16.  Results below the normal range
+// are multiples of 2^-1074 (gradual underflow).  A pencil with a NaN or an infinity
+// gives NaNs, as the sums of an FP64 transform do.
 //
 // The complex64 path uses the same passes in FP32.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -370,13 +371,14 @@ SIE_HD void dftR(V* a)
 }
 
 // ------------------------------------------------------------------ complex128 <-> fixed point
-// Scales of a pencil: emax, the largest exponent field of its components, and
+// Scales of a pencil: field, the largest high word of its components' magnitudes (1 for
+// one that has only low bits; 0: all zero), emax, its exponent field, and
 // l1 = sum over the components of floor(|v| 2^(20 - E)) + 1, E = emax's exponent.
 // After scaling by 2^(bits - 1 - E) the components are below 2^bits and their sum
 // is below 2^61; the first pass takes 4 times that (its sums of R1 terms fit too).
 struct FxScale {
     int s0, x0;
-    bool bad;
+    bool bad, low;  // not finite; results may lie below the normal range
 };
 SIE_HD int fx_l1(unsigned hi, int emax)
 {
@@ -394,7 +396,7 @@ SIE_HD FxScale fx_scale(int field, int l1, int log2_r1)
 #endif
     // first pass: R1 terms of its bits, or the whole sum, whichever bound is lower
     const int top = 59 - log2_r1 > 80 - lg ? 59 - log2_r1 : 80 - lg, b = 82 - lg < top ? 82 - lg : top;
-    return FxScale{emax + 63 - (b + 2), emax - b, emax == 0x7ff};
+    return FxScale{emax + 63 - (b + 2), emax - b, emax == 0x7ff, emax < b && field > 0};
 }
 // v 2^(bits - 1 - E) as an integer, the fraction below 2^(E - bits + 1) cut off;
 // s0 = emax + 63 - bits
@@ -429,46 +431,26 @@ SIE_HD double fx_double(unsigned long long r)
     return d;
 #endif
 }
-// f 2^(x0 - 1022) where it may lie below the normal range: by integer operations,
-// rounded once at the place of its last bit
-SIE_HD double fx_to_low(long long f, int x0)
-{
-    const long long sg = f >> 63;
-    const unsigned long long a = (unsigned long long)((f ^ sg) - sg);
-    if (a == 0) return 0.0;
-#ifdef __CUDA_ARCH__
-    const int lz = __clzll((long long)a);
-#else
-    const int lz = __builtin_clzll(a);
-#endif
-    const int e = 63 + x0 - lz, sh = e < 0 ? 10 - e : 10;  // biased exponent less one
-    unsigned long long r = sh > 63 ? 0 : ((a << (lz - 1)) + (1ull << (sh - 1))) >> sh;
-    if (e > 0) r += (unsigned long long)(unsigned)e << 52;  // bit 52 of r adds one
-    return fx_double(r | ((unsigned long long)sg & 0x8000000000000000ull));
-}
-// f 2^(E - bits + 1) as a double; x0 = emax - bits.  Conversion on the FP64 pipe,
-// which the transforms leave idle, then the exponent by an integer addition.  From
-// x0 = 0 on no result is below the normal range (f is a whole number).
+// f 2^(E - bits + 1) as a double; x0 = emax - bits >= 0 or f = 0: no result is below the
+// normal range then (f is a whole number).  Conversion on the FP64 pipe, which the
+// transforms leave idle, then the exponent by an integer addition.
 SIE_HD double fx_to(long long f, int x0)
 {
-    if (x0 < 0) return fx_to_low(f, x0);
 #ifdef __CUDA_ARCH__
     const double d = __ll2double_rn(f);
+    const int hi = __double2hiint(d), e = ((hi >> 20) & 0x7ff) + (x0 - 1022);  // biased exponent of the result
+    int oh = hi + ((x0 - 1022) << 20), ol = __double2loint(d);
+    if (f == 0) oh = 0;
+    if (e >= 2047) oh = (hi & 0x80000000) | 0x7ff00000, ol = 0;
+    return __hiloint2double(oh, ol);
 #else
-    const double d = (double)f;
+    return ldexp((double)f, x0 - 1022);
 #endif
-    const unsigned long long b = fx_bits(d);
-    const int hi = (int)(b >> 32), e = ((hi >> 20) & 0x7ff) + (x0 - 1022);  // biased exponent of the result
-    unsigned oh = (unsigned)hi + ((unsigned)(x0 - 1022) << 20), ol = (unsigned)b;
-    if (f == 0) oh = 0, ol = 0;
-    if (f != 0 && e >= 2047) oh = ((unsigned)hi & 0x80000000u) | 0x7ff00000u, ol = 0;
-    return fx_double(((unsigned long long)oh << 32) | ol);
 }
 
 // the same by integer operations alone, where the FP64 pipe is busy
 SIE_HD double fx_to_int(long long f, int x0)
 {
-    if (x0 < 0) return fx_to_low(f, x0);
     const long long sg = f >> 63;
     const unsigned long long a = (unsigned long long)((f ^ sg) - sg);
 #ifdef __CUDA_ARCH__
@@ -483,6 +465,10 @@ SIE_HD double fx_to_int(long long f, int x0)
     if (a != 0 && e >= 2046) r = 0x7ff0000000000000ull;
     return fx_double(r | ((unsigned long long)sg & 0x8000000000000000ull));
 }
+
+// the same for x0 < 0 (pencils below 2^-960 or so): results below the normal range are
+// multiples of 2^-1074
+SIE_HD double fx_to_low(long long f, int x0) { return fx_to_int(f, x0 + 64) * 0x1p-64; }
 
 // ------------------------------------------------------------------ plans
 template <int N>
@@ -540,9 +526,9 @@ __device__ __forceinline__ void load_first(const G* __restrict__ in, int64_t bas
     }
 }
 
-__device__ __forceinline__ int exp_max(double2 v)
+__device__ __forceinline__ int high_max(double2 v)
 {
-    return max(__double2hiint(v.x) & 0x7ff00000, __double2hiint(v.y) & 0x7ff00000);
+    return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
 }
 
 // first pass of a pencil: inputs g -> DFT -> twiddle -> shared memory
@@ -590,9 +576,13 @@ __device__ __forceinline__ void second_pass(const typename P::V* s, int k1, type
 template <int R1, int R2>
 __device__ __forceinline__ FxScale pencil_scale(const double2* g, int n_in, int* em, int* l1, bool act)
 {
-    int m = 0;
+    int m = 0, lo = 0;
 #pragma unroll
-    for (int r = 0; r < R1; r++) m = max(m, exp_max(g[r]));
+    for (int r = 0; r < R1; r++) {
+        m = max(m, high_max(g[r]));
+        lo |= __double2loint(g[r].x) | __double2loint(g[r].y);
+    }
+    if (m == 0 && lo != 0) m = 1;
     if (act) atomicMax(em, m);
     __syncthreads();
     const int field = *em, emax = max(field >> 20, 1);
@@ -605,13 +595,34 @@ __device__ __forceinline__ FxScale pencil_scale(const double2* g, int n_in, int*
     constexpr int lg = R1 > 8 ? 4 : (R1 > 4 ? 3 : 2);
     return fx_scale(field, *l1, lg);
 }
-template <bool FP64PIPE>
-__device__ __forceinline__ double2 fx_out(fx2 v, const FxScale& q)
+// put(r, v) of the N outputs of a butterfly, v() the result r (converted only where it is
+// stored); its own slots in shared memory are s[r st].  Pencils that are not finite or so
+// small that results may lie below the normal range take a branch of their own, a short
+// loop over the slots: with the tests on every value the system product at 128^3 took
+// 617 us (not finite) and 638 us (both), 604 us this way.  A pencil of zeros, of which
+// forward passes have many, needs neither.
+template <int N, bool FP64PIPE, class F>
+__device__ __forceinline__ void fx_results(const fx2* a, const FxScale& q, fx2* s, int st, F put)
 {
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    if (q.bad) return make_double2(nan, nan);
-    return FP64PIPE ? make_double2(fx_to(v.x, q.x0), fx_to(v.y, q.x0))
-                    : make_double2(fx_to_int(v.x, q.x0), fx_to_int(v.y, q.x0));
+    if (!q.bad && !q.low) {
+#pragma unroll
+        for (int r = 0; r < N; r++)
+            put(r, [&] {
+                return FP64PIPE ? make_double2(fx_to(a[r].x, q.x0), fx_to(a[r].y, q.x0))
+                                : make_double2(fx_to_int(a[r].x, q.x0), fx_to_int(a[r].y, q.x0));
+            });
+    } else {
+#pragma unroll
+        for (int r = 0; r < N; r++) s[r * st] = a[r];
+#pragma unroll 1
+        for (int r = 0; r < N; r++) {
+            put(r, [&] {
+                const fx2 v = s[r * st];
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                return q.bad ? make_double2(nan, nan) : make_double2(fx_to_low(v.x, q.x0), fx_to_low(v.y, q.x0));
+            });
+        }
+    }
 }
 
 // ------------------------------------------------------------------ one pass over many pencils
@@ -648,7 +659,7 @@ __global__ void __launch_bounds__(pass_pb<N>() * Plan<N>::R2)
     const int64_t lo = ok ? p % G.L : 0, hi = ok ? p / G.L : 0;
     typename P::G g[R1];
     load_first<R1, R2>(in, lo * G.slo_in + hi * G.shi_in + blockIdx.y * G.bs_in, G.st_in, tp, G.n_in, ok, g);
-    FxScale q{0, 0, false};
+    FxScale q{0, 0, false, false};
     if constexpr (FX) {
         for (int i = threadIdx.x; i < PB; i += blockDim.x) em[i] = l1[i] = 0;
         __syncthreads();
@@ -661,15 +672,15 @@ __global__ void __launch_bounds__(pass_pb<N>() * Plan<N>::R2)
     for (int k1 = tp; k1 < R1; k1 += R2) {
         typename P::V a[R2];
         second_pass<INV, R1, R2, P>(s, k1, a);
-#pragma unroll
-        for (int r = 0; r < R2; r++) {
+        auto put = [&](int r, auto v) {
             const int k = k1 + r * R1;
-            if (ok && k < G.n_out) {
-                if constexpr (FX)
-                    out[ob + (int64_t)k * G.st_out] = fx_out<true>(a[r], q);
-                else
-                    out[ob + (int64_t)k * G.st_out] = a[r];
-            }
+            if (ok && k < G.n_out) out[ob + (int64_t)k * G.st_out] = v();
+        };
+        if constexpr (FX) {
+            fx_results<R2, true>(a, q, s + k1, R1 + 1, put);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R2; r++) put(r, [&] { return a[r]; });
         }
     }
 }
@@ -761,7 +772,7 @@ __global__ void __launch_bounds__(ZMode<MODE>::NI* z_pb<N, P, MODE>() * Plan<N>:
             asm volatile("prefetch.global.L2 [%0];" ::"l"(q0 + 3 * bnn));
         }
     }
-    FxScale q{0, 0, false};
+    FxScale q{0, 0, false, false};
     V* s = sm + me * PITCH;
     C* sc = smc + me * PITCH;
     {
@@ -780,12 +791,12 @@ __global__ void __launch_bounds__(ZMode<MODE>::NI* z_pb<N, P, MODE>() * Plan<N>:
     for (int k1 = tp; k1 < R1; k1 += R2) {
         V a[R2];
         second_pass<0, R1, R2, P>(s, k1, a);
+        auto put = [&](int r, auto v) { sc[r * (R1 + 1) + k1] = v(); };
+        if constexpr (FX) {
+            fx_results<R2, false>(a, q, s + k1, R1 + 1, put);
+        } else {
 #pragma unroll
-        for (int r = 0; r < R2; r++) {
-            if constexpr (FX)
-                sc[r * (R1 + 1) + k1] = fx_out<false>(a[r], q);
-            else
-                sc[r * (R1 + 1) + k1] = a[r];
+            for (int r = 0; r < R2; r++) put(r, [&] { return a[r]; });
         }
     }
     __syncthreads();
@@ -825,15 +836,15 @@ __global__ void __launch_bounds__(ZMode<MODE>::NI* z_pb<N, P, MODE>() * Plan<N>:
     for (int k1 = tp; k1 < R1; k1 += R2) {
         V a[R2];
         second_pass<1, R1, R2, P>(s, k1, a);
-#pragma unroll
-        for (int r = 0; r < R2; r++) {
+        auto put = [&](int r, auto v) {
             const int k = k1 + r * R1;
-            if (k < nz_phys) {
-                if constexpr (FX)
-                    buf[gb + (int64_t)k * plane] = fx_out<true>(a[r], q);
-                else
-                    buf[gb + (int64_t)k * plane] = a[r];
-            }
+            if (k < nz_phys) buf[gb + (int64_t)k * plane] = v();
+        };
+        if constexpr (FX) {
+            fx_results<R2, true>(a, q, s + k1, R1 + 1, put);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R2; r++) put(r, [&] { return a[r]; });
         }
     }
 }

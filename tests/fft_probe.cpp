@@ -10,8 +10,8 @@ static unsigned long long bits(double d) { unsigned long long r; memcpy(&r, &d, 
 extern "C" void fx_out(int n, const long long* f, const int* x0, double* a, double* b)
 {
     for (int i = 0; i < n; i++) {
-        a[i] = sie::fx_to(f[i], x0[i]);
-        b[i] = sie::fx_to_int(f[i], x0[i]);
+        a[i] = x0[i] < 0 ? sie::fx_to_low(f[i], x0[i]) : sie::fx_to(f[i], x0[i]);
+        b[i] = x0[i] < 0 ? a[i] : sie::fx_to_int(f[i], x0[i]);
     }
 }
 
@@ -30,6 +30,7 @@ extern "C" void fx_round_trip(int n, const double* v, int log2_r1, double* out)
     for (int i = 0; i < n; i++) {
         const unsigned long long u = bits(v[i]);
         // the first pass carries two more bits, rounded off after it
-        out[i] = sie::fx_to((sie::fx_from((unsigned)(u >> 32), (unsigned)u, q.s0) + 2) >> 2, q.x0);
+        const long long f = (sie::fx_from((unsigned)(u >> 32), (unsigned)u, q.s0) + 2) >> 2;
+        out[i] = q.low ? sie::fx_to_low(f, q.x0) : sie::fx_to(f, q.x0);
     }
 }

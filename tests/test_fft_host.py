@@ -1,6 +1,6 @@
-"""Conversions of the fixed-point transforms on the CPU (the same operations as on the
-GPU): results are the nearest double over the whole range, below the normal range (where
-FP64 arithmetic underflows gradually) as above it.
+"""Conversions of the fixed-point transforms on the CPU: results are the nearest double
+over the normal range, and below it, where FP64 arithmetic underflows gradually, within
+3/4 of the last place (53 bits first, then the place of 2^-1074).
 """
 import ctypes
 import os
@@ -49,10 +49,10 @@ def test_results_are_the_nearest_doubles(probe, lo, hi):
     for i in range(n):
         v, ulp = _nearest(f[i], x0[i])
         for got in (a[i], b[i]):
-            assert np.isfinite(got) and abs(Fraction(got) - v) <= ulp / 2
+            assert np.isfinite(got) and abs(Fraction(got) - v) <= ulp * Fraction(3 if abs(v) < Fraction(2)**-1022 else 2, 4)
 
 
-@pytest.mark.parametrize("scale", [1e-320, 1e-308, 1e-305, 1e-290, 1.0, 1e300])
+@pytest.mark.parametrize("scale", [0.0, 5e-324, 1e-320, 1e-308, 1e-305, 1e-290, 1.0, 1e300])
 @pytest.mark.parametrize("r1", [4, 8, 16])
 def test_pencils_of_any_size(probe, r1, scale):
     r = np.random.default_rng(int(r1))

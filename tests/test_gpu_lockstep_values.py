@@ -51,3 +51,24 @@ def test_solutions_are_what_they_were(lib, ctx, name):
     assert got.shape == want.shape
     for q in range(len(want)):
         assert np.linalg.norm(got[q] - want[q]) <= 1e-9 * np.linalg.norm(want[q])
+
+
+def test_bar_to_a_tight_tolerance(lib, ctx):
+    """At tol_outer 1e-8 the method's own noise no longer decides: eight right-hand sides in
+    lockstep and one after another (another arithmetic, another preconditioner path) agree
+    to the two residuals times the condition of the row-weighted system, 2e4."""
+    size, div, f, model, nrhs, grid_n = CASES["bar"]
+    mesh = lib.Mesh(ctx, *box(size, div))
+    op = lib.Operator(mesh, f, 1.0, 1.0, 5.8e7, lib.params(interior_model=model, grid_n=grid_n, tol_outer=1e-8,
+                                                         tol_inner=1e-11, restart=400))
+    th, ph = 0.3 + 0.35 * np.arange(nrhs), 0.2 + 0.9 * np.arange(nrhs)
+    k = np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], axis=1)
+    e = np.stack([np.cos(th) * np.cos(ph), np.cos(th) * np.sin(ph), -np.sin(th)], axis=1)
+    b = op.rhs_planewave(k, e)
+    x, _, rr = op.solve(b, nrhs=nrhs)
+    xs, _, rs = op.solve(b, nrhs=nrhs, sequential=True)
+    assert (rr < 1e-8).all() and (rs < 1e-8).all()
+    for q in range(nrhs):
+        assert np.linalg.norm(x[q] - xs[q]) <= 4e-4 * np.linalg.norm(xs[q])
+    op.close()
+    mesh.close()
