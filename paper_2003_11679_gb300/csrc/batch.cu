@@ -143,11 +143,6 @@ static sie_status batch_workspace(sie_op* op, double2** bufs, double2** src)
     return SIE_OK;
 }
 
-// entries x right-hand sides from which a branch for the near part pays for its events
-// (about 8 us; 2 M entries take 15 us).  K at 1,280 triangles, eight right-hand sides:
-// 317 -> 299 us; L at 20,480: 3,457 -> 3,409 us (both parts then bound by issue)
-constexpr int64_t BRANCH_MIN = 2000000;
-
 // Y = A X for nr vectors (nr <= RB, rhs-major, length N_e), A = L (which_LK 0)
 // or K (1) of operator a
 sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X, double2* Y, int nr)
@@ -161,8 +156,11 @@ sie_status aim_apply_block(sie_op* op, AimOp& a, int which_LK, const double2* X,
         return SIE_ERR_ARG;
     }
     if (!op->bws_xp) SIE_CUDA_TRY(cudaMallocAsync((void**)&op->bws_xp, sizeof(double2) * RB * ne, st));
-    // the near part (FP64 products) beside the grid part (atomics and integer transforms)
-    Branch br(op, a.has_grid && !pc->prof.on && a.nnz * nr >= BRANCH_MIN);
+    // the near part (FP64 products) on a branch beside the grid part (atomics and integer
+    // transforms), at every size: K of two and eight right-hand sides 65 -> 57 and 89 -> 77 us
+    // at 80 triangles, eight at 1,280 308 -> 293 us, L at 20,480 3,457 -> 3,409 us (both parts
+    // wait for issue slots there).  The stage timers need one stream.
+    Branch br(op, a.has_grid && !pc->prof.on);
     {
         SIE_CUDA_TRY(br.follow());
         Stage s_(pc, a.has_grid ? "spmv_block" : "spmv_near_only_block");

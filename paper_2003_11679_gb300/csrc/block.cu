@@ -228,7 +228,7 @@ sie_status blk_sys_rest(sie_op* op, int R, const double2* x, int64_t ldx, const 
     const GridDesc& g = w.g;
     const int ne = M.ne, nt = M.nt, S = (g.M + 1) * (g.M + 1) * (g.M + 1);
     const int64_t nn = (int64_t)g.n[0] * g.n[1] * g.n[2], Ng = (int64_t)g.N[0] * g.N[1] * g.N[2];
-    SIE_CUDA_TRY(cudaMemset2DAsync(y, sizeof(double2) * ldy, 0, sizeof(double2) * ne, R, st));
+    SIE_CUDA_TRY(cudaMemset2DAsync(y, sizeof(double2) * std::max<int64_t>(ldy, ne), 0, sizeof(double2) * ne, R, st));
     for (int q0 = 0; q0 < R; q0 += w.R) {
         const int r = std::min(w.R, R - q0);
         const double2 *xq = x + q0 * ldx, *Eq = E + q0 * lde;

@@ -43,13 +43,13 @@ __device__ __forceinline__ void gio_w(const float* w, float& w0, float* w1)
 // S1 = sum_u w1 . A(u), T0 = sum_u w0 A(u), P0 = sum_u w0 Phi(u) over its stencil.
 // Right-hand side blockIdx.y: grids out + y NG Ng, vector y + y ldy.  NG: 4 grids
 // (A, Phi) or 3 (A).  FP32 grids (C = float2): FP32 gathers and sums, FP64 from the
-// edge coefficients on.  G lanes per triangle: 4, or all 32 up to 4,096 triangles and
-// right-hand sides together, where one gather latency counts and not the additions (80
-// triangles: 9 us against 15 us).  L2 gathers and FP64 additions bound it: 20,480
-// triangles took 105 us (eight right-hand sides 785 us) with 32 lanes, 33 us (157 us)
-// with 4.
+// edge coefficients on.  G lanes per triangle: 4, or all 32 up to 2,048 triangles and
+// right-hand sides together, where one gather latency counts and not the additions: with
+// 32 and 4 lanes 9.1 and 14.9 us at 320, 13.7 and 15.4 at 1,280, 16.4 and 16.6 at 2,000,
+// 20.4 and 15.4 at 2,560.  L2 gathers and FP64 additions bound it beyond: 20,480 triangles
+// take 105 us (eight right-hand sides 785 us) with 32 lanes, 34 us (157 us) with 4.
 // With 32 lanes CTAs have 64 threads: a small mesh then spreads over more SMs' FP64 lanes.
-constexpr int64_t GIO_WIDE = 4096;
+constexpr int64_t GIO_WIDE = 2048;
 constexpr int GIO_SMALL = 64;
 template <int G, class C, class R, int NG>
 __global__ void __launch_bounds__(256) k_interp(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
@@ -232,7 +232,9 @@ __global__ void __launch_bounds__(256) k_project_gather(int64_t nnode, const int
 // triangles): J and, with 4 grids, rho = 2 alpha w0.  A thread per (triangle, stencil
 // node); alpha and beta from tc (k_tri_coef1), or from x where tc is null: few
 // triangles, one launch less.  Right-hand side blockIdx.y: x + y ldx, src + y ngrid Ng.
-// With tc 14 FP64 operations an entry instead of 47: 168 us.
+// With tc 14 FP64 operations an entry instead of 47: 170 us.  The line is GIO_WIDE too:
+// without and with tc 12.8 and 15.3 us at 1,280 triangles and right-hand sides, 15.7 and
+// 14.9 at 2,304, 21.9 and 17.3 at 4,608.
 template <bool TC>
 __global__ void __launch_bounds__(256) k_project(int nt, int S, int Mord, DevMesh M, const int32_t* __restrict__ base,
                                                  const double* __restrict__ W, const double2* __restrict__ x,

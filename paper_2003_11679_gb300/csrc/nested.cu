@@ -233,14 +233,16 @@ static bool clu_fits(const void* fn, int C, size_t smem)
     return n >= 1;
 }
 
-// CTAs of a cluster (0: none).  8 (portable) for up to 1,024 rows and 16,384 entries,
-// else 16: a bar's 504 rows of 64 entries take 14,000 cycles a product on 8 SMs' FP64
-// lanes, 7,000 on 16.
+// CTAs of a cluster (0: none).  8 for up to 768 rows and 6,000 entries, whose barriers and
+// chains count more than their products (8 and 16 CTAs: 450 rows of 5 entries 190 and 194
+// us, 648 rows 192 and 196, 96 rows of 58 81 and 82), else 16 (882 rows of 5: 220 and 195
+// us; 168 rows of 62: 89 and 83; a bar's 504 rows of 65: 118 and 102).  Up to 1,024 rows 8
+// (portable) where 16 do not run.
 int clu_pick(const void* fn, int64_t n, int64_t nnz, int m, size_t extra)
 {
     if (n > CLU_MAXN) return 0;
-    const bool small = n <= 1024;
-    for (int C = small && nnz <= 16384 ? 8 : CLU_MAXC; C >= (small ? 8 : CLU_MAXC); C >>= 1) {
+    const bool portable = n <= 1024;
+    for (int C = n <= 768 && nnz <= 6000 ? 8 : CLU_MAXC; C >= (portable ? 8 : CLU_MAXC); C >>= 1) {
         const size_t smem = clu_smem(n, m, C) + extra;
         if (smem <= 200 * 1024 && clu_fits(fn, C, smem)) return C;
     }

@@ -650,7 +650,8 @@ __global__ void __launch_bounds__(128) k_spmv2_c64(int nrow, const int64_t* __re
 // lane.  FP64 arithmetic bounds large meshes: with 8 lanes the warp-wide additions of
 // a row's sums are shared by four rows (15.0 M entries, 190 us of products: 453 us
 // with 32 lanes, 274 us with 8).  Up to 8,192 rows the GPU is not full and a row's
-// chain counts: 32 lanes (504 rows: 12 us against 22 us).
+// chain counts: with 32 and 8 lanes 11 and 23 us at 480 rows, 28 and 33 at 3,456, 40 and
+// 39 at 7,680, 130 and 109 at 30,720 (4.8 M entries).
 template <int G>
 __global__ void __launch_bounds__(256) k_spmv2(int nrow, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                                const double2* __restrict__ v1, const double2* __restrict__ x1, double2 a1,
