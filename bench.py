@@ -218,7 +218,7 @@ FFT_GRIDS = {"spmv_sys_rest": 0.5, "fft_fwd_x": 7, "fft_fwd_y": 7, "fft_fwd_z": 
 # k_fft_z<128,Fx,ZM_SYS> on the 128^3 FFT grid: the grid part has the same
 # size at every mesh level of the copper workload, so the capture on the
 # 480-RWG mesh holds per launch for the 30,720-RWG one.
-TRAFFIC = {("fft_z_specmul", "fp64"): (250122496 + 46384128, "710465e61225b3dc")}
+TRAFFIC = {("fft_z_specmul", "fp64"): (249940480 + 46186752, "540d6868261e2657")}
 
 
 # stages whose FP64 form computes in 64-bit block fixed point (integer multiply-adds)

@@ -8,7 +8,7 @@
 // restarted FGMRES preconditioned by the explicit complex64 inverse: FP32 products
 // and per-lane sums, row sums in FP64.
 // The work is small and was latency-bound: 14 launches an iteration and a host
-// check took 118 us (320 triangles) to 220 us (1,280) an application; 42 and 125 us
+// check took 118 us (320 triangles) to 220 us (1,280) an application; 42 and 121 us
 // now.  An iteration meets at 5 cluster barriers; the inverse is read by 8 or 16 SMs
 // (1,280 triangles: 13 MB, about 6 us), which bounds the size it is taken for
 // (CLU_MAXN triangles).

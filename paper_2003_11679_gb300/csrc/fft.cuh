@@ -629,7 +629,7 @@ __device__ __forceinline__ void fx_results(const fx2* a, const FxScale& q, fx2* 
 // PB pencils per CTA, R2 threads per pencil; in and out may alias (a pencil is
 // read completely before any of it is written).  128 points, 7 grids of 8,064
 // pencils (the y pass of the system product at 63^3): FP64 Stockham radix 8 took
-// 292 us at 82% of the FP64 pipe; 73 us now, the integer (ALU) pipe 60% busy, and
+// 292 us at 82% of the FP64 pipe; 69 us now, the integer (ALU) pipe 61% busy, and
 // 20 us in complex64 (47 us before).
 template <int N>
 __host__ __device__ constexpr int pass_pb()
@@ -692,10 +692,10 @@ __global__ void __launch_bounds__(pass_pb<N>() * Plan<N>::R2)
 // grids, writes z < nz_phys of grids 0 .. NO - 1 in place (the inverse y pass
 // reads nothing else).  Threads: grid, then column fastest.
 // System product at 128^3, 16,384 columns: FP64 transforms took 1,091 us, the FP64
-// pipe 85% busy; 351 us now.  Its spectral products alone keep that pipe busy for
-// 140 us, so the forward outputs are converted by integer operations; the rest is
-// integer issue and the barriers between phases (two to four CTAs an SM).  In
-// complex64: 158 us before, 76 us now.
+// pipe 85% busy; 347 us now, FP64 46% and ALU 42% busy.  Its spectral products alone keep
+// the FP64 pipe busy for 140 us, so the forward outputs are converted by integer
+// operations; the rest is integer issue and the barriers between phases (two to four
+// CTAs an SM).  In complex64: 158 us before, 70 us now.
 enum { ZM_SYS = 0, ZM_L = 1, ZM_K = 2 };
 template <int MODE>
 struct ZMode {

@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(128) k_near_far(const int32_t* __restrict__ pa
 //  * units of self and edge pairs come first, so no long unit ends the launch.
 // One warp per pair with the outer points split over lanes, 27 orders with a
 // division each and separate cosh, tanh, phi1 per direction took 364 ms for the
-// exterior near region of an 80-triangle sphere at 3 GHz; 27 ms now, 37 million
-// directions at 286 FP64 operations, the FP64 pipe 88% busy.
+// exterior near region of an 80-triangle sphere at 3 GHz; 28 ms now, 37 million
+// directions at 286 FP64 operations, the FP64 pipe 87% busy.
 constexpr int NC_W = 2;     // warps per CTA (42 KB of shared memory)
 constexpr int NC_NT = 24;   // largest order: 1 / 24! < 2e-24
 constexpr int NC_NA = 8;    // angular nodes with tabulated exp(+-ds x_q); more are evaluated

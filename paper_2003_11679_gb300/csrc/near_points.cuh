@@ -14,7 +14,8 @@
 // tree over the lanes.  With one warp per pair and its points in a loop, the 1,680 points
 // of a self pair were a chain of 53 rounds on a nearly empty GPU: build of a copper cube
 // of 48 triangles 1,907 -> 356 ms, exterior near region of 1,280 triangles 2,259 -> 1,717
-// ms (FP64 arithmetic bounds it: 2,300 operations a direction, the panel rule has 286).
+// ms (FP64 arithmetic bounds it, the pipe is 82 to 85% busy: 2,300 operations a
+// direction, the panel rule has 286).
 //
 // A compiler may fuse either product of a sum of two, and decides from the code around
 // it: k_near_points keeps the statements of a point together for that reason.

@@ -5,10 +5,9 @@
 //         E' = -(j k0 eps_r + sigma eta0)^-1 A^-1 b;
 //   SIBC: b = I_x H, A = Gram matrix G, M = diag(G)^-1, E' = (eta_i / eta0) A^-1 b.
 // Latency bounds it: an iteration is 4 (SIBC) or 5 (GIBC) barriers and chains of FP64
-// operations.  SIBC
-// needs no barrier for M: Z_j is written beside V_j.  As a graph loop of nine kernels
-// an iteration, 310 us for a copper bar's 504 rows (4 iterations) and 500 us for 30,720
-// rows (10); now 104 us on a cluster of 16 and 294 us on the whole GPU.
+// operations.  SIBC needs no barrier for M: Z_j is written beside V_j.  As a graph loop
+// of nine kernels an iteration, 310 us for a copper bar's 504 rows (4 iterations) and
+// 500 us for 30,720 rows (10); now 102 us on a cluster of 16 and 284 us on the whole GPU.
 #include <algorithm>
 #include <cstdlib>
 
