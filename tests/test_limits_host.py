@@ -21,7 +21,8 @@ def probe(tmp_path_factory):
     if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
         pytest.skip("g++ or the CUDA headers are missing")
     so = str(tmp_path_factory.mktemp("limits") / "liblimits_probe.so")
-    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", os.path.join(CUDA, "include"),
+    # -Bsymbolic: the stand-in, not a CUDA runtime that another test has loaded
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", os.path.join(CUDA, "include"),
                     os.path.join(ROOT, "tests", "limits_probe.cpp"),
                     os.path.join(ROOT, "paper_2003_11679_gb300", "csrc", "limits.cpp"), "-o", so, "-lpthread"],
                    check=True, capture_output=True)
